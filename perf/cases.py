@@ -220,6 +220,34 @@ def work(case):
     return {"bytes": float(n * V * (4 if case["dtype"] == "f32" else 2) + small), "flops": 4.0 * n * V}
 
 
+def exact(case, seed):
+    """The normalisers of the drafting step and the intermediates of "block_ex" (p_i, S_i, h_i, log-normalisers) in
+    64 bits, from the inputs as stored; tokens and lengths have no such value."""
+    kind, T = case["kind"], case["temperature"]
+    if kind not in ("sample", "block_ex"):
+        return None
+    s = prepare(case, seed)
+    if kind == "sample":
+        z = s["logits"]
+        return None, torch.cat([torch.logsumexp(z[b:b + 16].double() / T, dim=-1) for b in range(0, z.shape[0], 16)])
+    B, g = s["tokens"].shape
+    f = lambda *shape: torch.empty(shape, dtype=torch.float64, device="cuda")
+    p, S, h, lse_t, lse_d = f(B, g + 1), f(B, g), f(B, g + 1), f(B, g + 1), f(B, g)
+    for b in range(B):
+        P, Q = (torch.log_softmax(s[k][b].double() / T, dim=-1) for k in ("target", "draft"))
+        lse_t[b] = torch.logsumexp(s["target"][b].double() / T, dim=-1)
+        lse_d[b] = torch.logsumexp(s["draft"][b].double() / T, dim=-1)
+        x = s["tokens"][b].long().unsqueeze(1)
+        ratio = (P[:g].gather(1, x) - Q.gather(1, x)).exp().squeeze(1)
+        p[b, 0] = 1.0
+        for i in range(g):
+            p[b, i + 1] = (p[b, i] * ratio[i]).clamp(max=1.0)
+        S[b] = (p[b, :g, None] * P[:g].exp() - Q.exp()).clamp_(min=0.0).sum(dim=-1)
+    h[:, :g] = torch.where(S > 0.0, S / (S + 1.0 - p[:, :g]), torch.zeros_like(S))
+    h[:, 0], h[:, g] = 1.0, p[:, g]
+    return None, None, dict(p=p, S=S, h=h, lse_t=lse_t, lse_d=lse_d)
+
+
 def tolerance(case):
     """Whole values: sums in another order move the edges of the sampler's cells, and a uniform that close to one of
     the V edges picks the neighbour.  1e-4 + 2e-8 V of the draws is the bound that the library's tests use (seen
