@@ -76,10 +76,9 @@ enum { BV_NOALLOC_SCRATCH_BYTES = 8 * 1024 * 1024 };
  *   out_tokens    [B, gamma+1] int32: X_1..X_tau, Y, then -1
  *   out_len       [B] int32: tau + 1, or -1 for a sequence with a data fault
  *   stream        a cudaStream_t (NULL = the default stream)
- * Rows whose byte length is a multiple of 16 with 16-byte aligned bases use the
- * 128-bit path; any other V >= 1 is served by an element-wise path.
- * Since S_i <= p_i, h_i <= p_i: on the 128-bit path S_i is evaluated only for
- * positions with eta_i <= p_i, from the highest down to the first one that passes
+ * Rows of any V >= 1 at any alignment are read 16 bytes at a time.
+ * Since S_i <= p_i, h_i <= p_i: S_i is evaluated only for
+ * positions with eta_i <= p_i that can still be the highest one to pass
  * eta_i <= h_i; tau and Y are those of the full evaluation (bv_verify_ex does the
  * full evaluation).  The cost of a call therefore depends on how many drafted
  * tokens are accepted.
@@ -317,10 +316,10 @@ int bv_stream_status(void* stream);
 
 /*
  * Tuning and test options, process-wide, read by every later call (0 restores the default choice):
- *   "kernel"        1 flow, 2 cluster, 3 element-wise streaming kernel, 4 small-batch kernel (for the shapes
- *                   each admits; the default picks the small-batch kernel for up to 32 sequences whose
- *                   logits are few enough to make the launch a matter of latency - up to 16 sequences for
- *                   the entry points on probabilities -, else the flow kernel)
+ *   "kernel"        1 flow, 2 cluster, 3 element-wise streaming kernel, 4 small-batch kernel, 5 phase kernel (for
+ *                   the shapes each admits; the default picks the small-batch kernel for up to 32 sequences
+ *                   whose logits are few enough to make the launch a matter of latency, the phase kernel for
+ *                   middling batches and for rows that are not whole 16-byte vectors, else the flow kernel)
  *   "small_bytes"   logit megabytes up to which the small-batch kernel is the default
  *   "cluster"       cluster width of the cluster / streaming kernels (1, 2, 4, 8)
  *   "max_clusters"  cap on the clusters those kernels launch
@@ -333,9 +332,9 @@ int bv_stream_status(void* stream);
  *                   chunks that last target rows get, so that the launch ends on short items (default 0:
  *                   none; it helped only where most drafted tokens are accepted)
  *   "wait_limit"    polls after which a bounded device-side wait gives up (tests)
- *   "never_signal"  tests: the flow kernel's workers never report an item as swept, so its waits
+ *   "never_signal"  tests: the kernels' workers never report what they have swept, so the waits
  *                   run out and the call ends with BV_ERR_TIMEOUT
- * Their first values come from the environment variables BV_KERNEL (flow / cluster / stream / small),
+ * Their first values come from the environment variables BV_KERNEL (flow / cluster / stream / small / phase),
  * BV_CLUSTER, BV_MAX_CLUSTERS, BV_FLOW_CHUNKS, BV_FLOW_PIECES, BV_FLOW_CTAS, BV_FLOW_DEPTH, read once.
  * Returns BV_ERR_INVALID_ARG for an unknown name.
  */
@@ -347,7 +346,7 @@ int bv_release(void);
 /* Number of kernel launches the last device-path call on this thread enqueued. */
 int bv_last_launch_count(void);
 /* Which kernel the last bv_verify / tv_verify (or _ex, _lse, _probs, gbv_, _host) call on this thread launched, in the
- * codes of the "kernel" option: 1 flow, 2 cluster, 3 element-wise streaming, 4 small-batch; 0 if it launched none. */
+ * codes of the "kernel" option: 1 flow, 2 cluster, 3 element-wise streaming, 4 small-batch, 5 phase; 0 if it launched none. */
 int bv_last_kernel(void);
 /* cudaError_t value of the last failing runtime call on this thread (0 if none). */
 int bv_last_cuda_error(void);

@@ -86,7 +86,7 @@ def bv_last_launch_count() -> int:
 
 def bv_last_kernel() -> int:
     """Code of the kernel the last verification call on this thread launched (1 flow, 2 cluster,
-    3 element-wise streaming, 4 small-batch)."""
+    3 element-wise streaming, 4 small-batch, 5 phase)."""
     return int(load_library().bv_last_kernel())
 
 

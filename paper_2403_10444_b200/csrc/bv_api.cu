@@ -19,11 +19,26 @@ constexpr int kTicketSlots = 64;  // concurrent calls of the cluster kernels on 
 // V = 152064, B <= 32: Algorithm 2 gains up to about 90 MB at low and high acceptance alike, Algorithm 1,
 // whose one residual sweep per sequence is cheap, up to about 160 MB)
 constexpr long long kSmallBytes[2] = {160LL << 20, 90LL << 20};   // [algo]
+// Logit bytes between which the phase kernel is the default for rows of 16-byte vectors ({Algorithm 1, Algorithms 2 and 4,
+// Algorithm 2 with supplied normalisers}), and the sequences from which it is on probabilities.  Measured at V = 128256 bf16,
+// gamma = 8, drafts of noise 0.1 / 0.7 / 1.5, against the kernel that ran there before:
+//   Algorithm 2, B = 8 (35 MB): 50 / 52 / 47 us against 39 / 34 / 31 (small-batch); 16: 53 / 53 / 50 against 62 / 55 / 48;
+//   33: 65 / 62 / 60 against 86 / 80 / 77 (flow); 128: 144 / 145 / 136 against 168 / 154 / 140; 200 (874 MB): 202 / 208 / 194
+//   against 230 / 218 / 195; the 2.2 GB of B = 256, V = 256000: 432 against 416 (the flow kernel overlaps the two sweeps)
+//   supplied normalisers, noise 0.7, B = 8 / 16 / 33 / 128 / 256: 46 / 48 / 52 / 101 / 164 us against 33 / 55 / 67 / 121 / 184
+//   Algorithm 1, noise 0.7, B = 16 / 33 / 64 / 128: 47 / 57 / 82 / 132 us against 46 / 77 / 90 / 115 (it reads all rows, the
+//   flow kernel the ones the tests need)
+//   probabilities, noise 0.7, B = 8 / 16 / 33 / 128 / 256: 26 / 29 / 31 / 49 / 72 us against 21 / 31 / 39 / 65 / 120
+constexpr long long kPhaseBytes[3][2] = {{64LL << 20, 320LL << 20}, {64LL << 20, 1000LL << 20}, {48LL << 20, 1400LL << 20}};
+constexpr int kPhaseProbsB = 12;
+constexpr size_t kSlotHead = 16384;   // leading bytes of a stream's workspace: status word, barrier words, the phase kernel's counters
+constexpr size_t kSlotPhase = 256;    // ... the last of these from here on
+static_assert(kSlotPhase + bv::kPhaseCounterWords * sizeof(unsigned) <= kSlotHead, "the counters fit in the head");
 constexpr int kStreamSlots = 32;  // streams per device that keep a workspace of their own
 
 // Tuning and test options (bv_set_option); their first values come from the environment, read once.
 struct Options {
-    int kernel = 0;        // 0: chosen by shape; 1 flow, 2 cluster, 3 stream, 4 small-batch
+    int kernel = 0;        // 0: chosen by shape; 1 flow, 2 cluster, 3 stream, 4 small-batch, 5 phase
     int small_bytes = 0;   // logit bytes (in MB) up to which the small-batch kernel is chosen; 0: the built-in limit
     int cluster = 0;       // cluster width of the cluster / stream kernels (1, 2, 4, 8); 0: chosen by shape
     int max_clusters = 0;  // cap on the clusters launched; 0: none
@@ -46,6 +61,7 @@ int kernel_code(const char* v) {
     if (!std::strcmp(v, "cluster")) return 2;
     if (!std::strcmp(v, "stream")) return 3;
     if (!std::strcmp(v, "small")) return 4;
+    if (!std::strcmp(v, "phase")) return 5;
     return 0;
 }
 void load_env_options() {
@@ -64,9 +80,9 @@ void load_env_options() {
 struct StreamSlot {
     cudaStream_t stream = nullptr;
     bool used = false;
-    void* ws = nullptr;        // [status word, 256 bytes][flow scratch]
+    void* ws = nullptr;        // [head: zero between calls, but for the status word][scratch]
     size_t bytes = 0;
-    size_t clean = 0;          // leading bytes of the flow scratch known to be zero between calls
+    size_t clean = 0;          // leading bytes of the scratch known to be zero between calls
     unsigned long long stamp = 0;
 };
 
@@ -82,6 +98,7 @@ struct DeviceState {
     unsigned long long clock = 0;
     int flow_ctas_per_sm[2] = {};
     int small_ctas[2] = {};            // small-batch kernel: CTAs of a launch per dtype (0: not asked yet)
+    int phase_ctas[2] = {};            // the phase kernel's
     // staging for the host-buffer entry points
     void* stage = nullptr;
     size_t stage_bytes = 0;
@@ -120,7 +137,7 @@ int device_state(DeviceState** out) {
     return BV_OK;
 }
 
-// The workspace of `stream` with room for `need` bytes of flow scratch behind its status word.
+// The workspace of `stream` with room for `need` bytes of scratch behind its head.
 // A stream seen for the first time takes a free entry, or the one used longest ago (whose area is
 // freed in its own stream's order).
 int stream_slot(DeviceState& d, cudaStream_t stream, size_t need, StreamSlot** out) {
@@ -139,12 +156,12 @@ int stream_slot(DeviceState& d, cudaStream_t stream, size_t need, StreamSlot** o
         s->stream = stream;
     }
     s->stamp = ++d.clock;
-    const size_t total = 256 + need;
+    const size_t total = kSlotHead + need;
     if (s->bytes < total) {
         if (s->ws && (e = cudaFreeAsync(s->ws, stream)) != cudaSuccess) return cuda_fail(e);
         s->ws = nullptr; s->bytes = 0; s->clean = 0;
         if ((e = cudaMallocAsync(&s->ws, total, stream)) != cudaSuccess) return cuda_fail(e);
-        if ((e = cudaMemsetAsync(s->ws, 0, 256, stream)) != cudaSuccess) return cuda_fail(e);   // the status word
+        if ((e = cudaMemsetAsync(s->ws, 0, kSlotHead, stream)) != cudaSuccess) return cuda_fail(e);
         s->bytes = total;
     }
     *out = s;
@@ -165,6 +182,78 @@ int pick_cluster(const DeviceState& d, const Options& opt, int B, size_t row_byt
     // cheaper exchanges) win: measured 0.43 against 0.57 ms at B = 256, gamma = 8, V = 152064.
     if (c == 8 && static_cast<long long>(B) * c >= 8LL * d.sm_count) c = 4;
     return c;
+}
+
+// Is there room for `need` bytes of scratch in the stream's workspace, or may it grow now?  Not while the stream is
+// captured: what is allocated then belongs to the graph.
+bool slot_can_hold(const DeviceState& d, cudaStream_t stream, size_t need) {
+    for (const StreamSlot& c : d.slots)
+        if (c.used && c.stream == stream && c.bytes >= kSlotHead + need) return true;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) { cudaGetLastError(); return false; }
+    return cap == cudaStreamCaptureStatusNone;
+}
+
+// Where the phase kernel is the default for rows of 16-byte vectors.
+bool phase_pays(int algo, const bv::Params& prm, const Options& opt, long long logit_bytes) {
+    const bool small = bv::small_fits(prm.B, prm.gamma);
+    if (prm.probs) return !small || prm.B >= kPhaseProbsB;
+    const int which = algo == bv::kTokenVerify ? 0 : (prm.lse_d != nullptr ? 2 : 1);
+    const long long least = opt.small_bytes > 0 ? static_cast<long long>(opt.small_bytes) << 20 : kPhaseBytes[which][0];
+    return (!small || logit_bytes > least) && logit_bytes <= kPhaseBytes[which][1];
+}
+
+// The phase kernel for the call in `prm`: BV_OK, an error, or 1 if it does not take the call.  Rows at any alignment have no
+// other kernel of this speed, so a batch of more sequences than it takes goes through it in parts.
+int run_phase(DeviceState& d, const bv::Params& prm, int dtype, bool vec, cudaStream_t stream) {
+    int& nc = d.phase_ctas[dtype];
+    if (nc == 0) {
+        nc = bv::phase_max_ctas(dtype, d.sm_count);
+        if (nc <= 0) nc = -1;
+    }
+    if (nc < 0) return 1;
+    const int g = prm.gamma;
+    int part = prm.B;
+    bv::PhasePlan plan = bv::phase_plan(prm.V, dtype, vec, part, g, prm.lse_d != nullptr, nc);
+    while (!plan.fits && !vec && part > 1) {
+        part = part > bv::kPhaseMaxB ? bv::kPhaseMaxB : part / 2;
+        plan = bv::phase_plan(prm.V, dtype, vec, part, g, prm.lse_d != nullptr, nc);
+    }
+    if (!plan.fits) return 1;
+    bv::PhaseScratch ps;
+    const size_t need = bv::phase_scratch(nullptr, nullptr, part, g, plan, &ps);
+    if (!slot_can_hold(d, stream, need)) return 1;
+    StreamSlot* slot = nullptr;
+    const int rc = stream_slot(d, stream, need, &slot);
+    if (rc != BV_OK) return rc;
+    slot->clean = 0;                // (the area the flow kernel expects to find zero is written here)
+    const size_t row_bytes = static_cast<size_t>(prm.V) * (dtype == BV_DTYPE_F32 ? 4 : 2);
+    int launches = 0;
+    for (int b0 = 0; b0 < prm.B; b0 += part, ++launches) {
+        bv::Params p = prm;
+        const size_t b = static_cast<size_t>(b0);
+        p.B = prm.B - b0 < part ? prm.B - b0 : part;
+        p.tgt = static_cast<const char*>(prm.tgt) + b * (g + 1) * row_bytes;
+        p.drf = static_cast<const char*>(prm.drf) + b * g * row_bytes;
+        p.tok = prm.tok + b * g;
+        p.uni = prm.uni + b * (g + 2);
+        if (prm.lse_d) p.lse_d = prm.lse_d + b * g;
+        p.out_tokens = prm.out_tokens + b * (g + 1);
+        p.out_len = prm.out_len + b;
+        if (prm.out_p) p.out_p = prm.out_p + b * (g + 1);
+        if (prm.out_S) p.out_S = prm.out_S + b * g;
+        if (prm.out_h) p.out_h = prm.out_h + b * (g + 1);
+        if (prm.out_lse_t) p.out_lse_t = prm.out_lse_t + b * (g + 1);
+        if (prm.out_lse_d) p.out_lse_d = prm.out_lse_d + b * g;
+        p.status = static_cast<int*>(slot->ws);
+        if (p.B != part) plan = bv::phase_plan(p.V, dtype, vec, p.B, g, p.lse_d != nullptr, nc);
+        bv::phase_scratch(static_cast<char*>(slot->ws) + kSlotHead, reinterpret_cast<unsigned*>(static_cast<char*>(slot->ws) + kSlotPhase),
+                          p.B, g, plan, &ps);
+        const cudaError_t e = bv::launch_phase(p, ps, dtype, vec, nc, stream);
+        if (e != cudaSuccess) return cuda_fail(e);
+    }
+    t_last_launches = launches; t_last_kernel = 5;
+    return BV_OK;
 }
 
 struct Extra {              // what only some entry points pass
@@ -209,11 +298,18 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
     prm.never_signal = opt.never_signal;
 
     prm.algo = algo;
+    const long long logit_bytes = static_cast<long long>(B) * (2 * gamma + 1) * static_cast<long long>(row_bytes);
     const bool flow_ok = vec && (opt.kernel == 0 || opt.kernel == 1);
+
+    // Both sweeps split over all warps, with the folds between them: between the small-batch kernel's sizes and the flow
+    // kernel's, and for rows at any alignment.
+    const bool only_vec = prm.lse_d != nullptr || prm.greedy || prm.probs;      // (entry points without an element-wise path)
+    if (opt.kernel == 5 ? vec || !only_vec : opt.kernel == 0 && (vec ? phase_pays(algo, prm, opt, logit_bytes) : !only_vec)) {
+        if ((rc = run_phase(*d, prm, dtype, vec, stream)) <= BV_OK) return rc;
+    }
 
     // A few sequences whose logits fit in L2: the launch is a matter of latency, and the kernel with two
     // grid-wide barriers instead of queues takes half the time of the flow kernel or less.
-    const long long logit_bytes = static_cast<long long>(B) * (2 * gamma + 1) * static_cast<long long>(row_bytes);
     const long long small_limit = opt.small_bytes > 0 ? static_cast<long long>(opt.small_bytes) << 20 : kSmallBytes[algo == bv::kBlockVerify ? 1 : 0];
     // (given probabilities only a few row pairs per sequence are read whatever the size of the rest: there the
     // small-batch kernel wins up to 16 sequences, 17 against 33 us for one, 33 against 38 us for sixteen)
@@ -230,8 +326,8 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
             if ((rc = stream_slot(*d, stream, bv::small_scratch_bytes(B, gamma, plan), &slot)) != BV_OK) return rc;
             slot->clean = 0;                // (the area the flow kernel expects to find zero is written here)
             bv::SmallScratch sc;
-            // the barrier words share the 256-byte block of the status word: zero since it was allocated
-            bv::small_scratch_layout(static_cast<char*>(slot->ws) + 256, reinterpret_cast<unsigned*>(static_cast<char*>(slot->ws) + 128),
+            // the barrier words are in the head: zero since it was allocated
+            bv::small_scratch_layout(static_cast<char*>(slot->ws) + kSlotHead, reinterpret_cast<unsigned*>(static_cast<char*>(slot->ws) + 128),
                                      B, gamma, plan, &sc);
             prm.ticket = nullptr;
             prm.nclusters = 0;
@@ -243,7 +339,7 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
         }
     }
 
-    // (only the two kernels above and below serve these entry points)
+    // (only the kernels above and below serve these entry points)
     if ((prm.lse_d != nullptr || prm.greedy || prm.probs) && !flow_ok) return BV_ERR_UNSUPPORTED;
 
     // 16-byte rows: the flow of independent work items (both algorithms)
@@ -266,7 +362,7 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
             const size_t need = bv::flow_scratch_bytes(B, gamma, plan, &zero_bytes);
             StreamSlot* slot = nullptr;
             if ((rc = stream_slot(*d, stream, need, &slot)) != BV_OK) return rc;
-            char* scratch = static_cast<char*>(slot->ws) + 256;
+            char* scratch = static_cast<char*>(slot->ws) + kSlotHead;
             bv::FlowScratch fl;
             bv::flow_scratch_layout(scratch, B, gamma, plan, &fl);
             // (with every position swept the second sweeps are the larger half of the launch and never wait for one another: deeper measured better)

@@ -266,22 +266,6 @@ __device__ __forceinline__ void f_step_sweep1_pair(const float (&vp)[EPV], const
     sP += vsP;
     sQ += vsQ;
 }
-// First sweep, two consecutive vectors of one row; the running sum in double.
-template <int EPV>
-__device__ __forceinline__ void f_step_sweep1_single(const float (&va)[EPV], const float (&vb)[EPV], float kf,
-                                                     float& MPw, double& sP) {
-    float vsA = f_exp_sum<EPV>(va, kf, -MPw);
-    float vsB = f_exp_sum<EPV>(vb, kf, -MPw);
-    if (__any_sync(0xffffffffu, fmaxf(vsA, vsB) > kRaiseBound)) {
-        const float y = rintf(warp_max(fmaxf(vec_max<EPV>(va), vec_max<EPV>(vb))) * kf);
-        if (y > MPw) { sP *= static_cast<double>(ref_scale(MPw, y)); MPw = y; }
-        vsA = f_exp_sum<EPV>(va, kf, -MPw);
-        vsB = f_exp_sum<EPV>(vb, kf, -MPw);
-    }
-    sP += static_cast<double>(vsA);
-    sP += static_cast<double>(vsB);
-}
-
 // PROBS: the rows hold probabilities (used as stored) instead of logits: no row has a first sweep,
 // the blocks are folded by the post warps when the launch starts, and the residual terms are formed
 // from the stored numbers.

@@ -88,6 +88,21 @@ __device__ __forceinline__ float f_pair_sum(const float (&vp)[EPV], const float 
     }
     return f_sum<EPV>(t);
 }
+// First sweep, two consecutive vectors of one row; the running sum in double where a token may be drawn from it.
+template <int EPV, class Sum>
+__device__ __forceinline__ void f_step_sweep1_single(const float (&va)[EPV], const float (&vb)[EPV], float kf,
+                                                     float& MPw, Sum& sP) {
+    float vsA = f_exp_sum<EPV>(va, kf, -MPw);
+    float vsB = f_exp_sum<EPV>(vb, kf, -MPw);
+    if (__any_sync(0xffffffffu, fmaxf(vsA, vsB) > kRaiseBound)) {
+        const float y = rintf(warp_max(fmaxf(vec_max<EPV>(va), vec_max<EPV>(vb))) * kf);
+        if (y > MPw) { sP *= static_cast<Sum>(ref_scale(MPw, y)); MPw = y; }
+        vsA = f_exp_sum<EPV>(va, kf, -MPw);
+        vsB = f_exp_sum<EPV>(vb, kf, -MPw);
+    }
+    sP += static_cast<Sum>(vsA);
+    sP += static_cast<Sum>(vsB);
+}
 template <int DT> __device__ __forceinline__ void f_load(const char* row, int i, float (&v)[Raw<DT>::EPV]) {
     Raw<DT>::unpack(ld_stream_v4(row + static_cast<size_t>(i) * 16), v);
 }
@@ -124,13 +139,13 @@ struct FlowCtx {
     double kd;
 };
 
-// One warp walks segment [w0, w1) of a row pair in index order and returns the first element
+// One warp walks vectors [w0, w1) of a row pair in index order and returns the first element
 // whose running residual mass exceeds tw (else the last element with positive mass, else -1).
-template <int DT, bool PROBS = false, int kAhead = 4>      // kAhead: runs of 32 vectors whose loads are in flight together
-__device__ int f_rescan(const char* rowP, const char* rowQ, int w0, int w1, int lane, float kf, float cp,
-                        float nMP, float nMQ, double tw) {
+// load(i, in, rp, rq): vector i of both rows, or what weighs nothing if it is not `in` the range.
+template <int DT, bool PROBS, int kAhead, class LoadFn>    // kAhead: runs of 32 vectors whose loads are in flight together
+__device__ __forceinline__ int f_rescan_with(LoadFn load, bool have_q, int w0, int w1, int lane, float kf, float cp,
+                                             float nMP, float nMQ, double tw) {
     constexpr int EPV = Raw<DT>::EPV;
-    constexpr uint32_t kPad = PROBS ? 0u : Raw<DT>::kNegInf;   // an element beyond the segment weighs nothing
     // The terms are the fp32 values of the sweeps; their running sum, which decides the token, is
     // kept in fp64 (a cell of the distribution can be far narrower than fp32 resolves next to the
     // mass before it).
@@ -143,9 +158,7 @@ __device__ int f_rescan(const char* rowP, const char* rowQ, int w0, int w1, int 
 #pragma unroll
         for (int a = 0; a < kAhead; ++a) {
             const int i = base0 + 32 * a + lane;
-            const bool ok = i < w1;
-            rp[a] = ok ? ld_stream_v4(rowP + static_cast<size_t>(i) * 16) : make_uint4(kPad, kPad, kPad, kPad);
-            rq[a] = (ok && rowQ) ? ld_stream_v4(rowQ + static_cast<size_t>(i) * 16) : make_uint4(kPad, kPad, kPad, kPad);
+            load(i, i < w1, rp[a], rq[a]);
         }
 #pragma unroll
         for (int a = 0; a < kAhead; ++a) {
@@ -155,7 +168,7 @@ __device__ int f_rescan(const char* rowP, const char* rowQ, int w0, int w1, int 
             float vp[EPV], vq[EPV], tt[EPV];
             Raw<DT>::unpack(rp[a], vp);
             Raw<DT>::unpack(rq[a], vq);
-            if (rowQ) f_pair_sum<EPV, true, PROBS>(vp, vq, kf, cp, nMP, nMQ, tt);
+            if (have_q) f_pair_sum<EPV, true, PROBS>(vp, vq, kf, cp, nMP, nMQ, tt);
             else f_pair_sum<EPV, false, PROBS>(vp, vq, kf, cp, nMP, nMQ, tt);
             double ls = 0.0;
 #pragma unroll
@@ -195,6 +208,17 @@ __device__ int f_rescan(const char* rowP, const char* rowQ, int w0, int w1, int 
         found = last_pos;
     }
     return found;
+}
+
+// ... of rows of whole 16-byte vectors
+template <int DT, bool PROBS = false, int kAhead = 4>
+__device__ int f_rescan(const char* rowP, const char* rowQ, int w0, int w1, int lane, float kf, float cp,
+                        float nMP, float nMQ, double tw) {
+    constexpr uint32_t kPad = PROBS ? 0u : Raw<DT>::kNegInf;   // an element beyond the segment weighs nothing
+    return f_rescan_with<DT, PROBS, kAhead>([&](int i, bool in, uint4& rp, uint4& rq) {
+        rp = in ? ld_stream_v4(rowP + static_cast<size_t>(i) * 16) : make_uint4(kPad, kPad, kPad, kPad);
+        rq = (in && rowQ) ? ld_stream_v4(rowQ + static_cast<size_t>(i) * 16) : make_uint4(kPad, kPad, kPad, kPad);
+    }, rowQ != nullptr, w0, w1, lane, kf, cp, nMP, nMQ, tw);
 }
 
 // Acceptance weight of position 0 < i < gamma from p_i and S_i: Eq. "pacc_block",

@@ -113,4 +113,38 @@ void small_scratch_layout(void* base, unsigned* barrier, int B, int gamma, const
 int small_max_ctas(int dtype, int sm_count);
 cudaError_t launch_small(const Params& prm, const SmallScratch& sc, int dtype, int nctas, cudaStream_t stream);
 
+// Phase kernel (bv_phase.cu): a cooperative launch of one CTA per SM, both sweeps split statically over all warps.
+constexpr int kPhaseMaxB = 768;       // sequences (a CTA's threads look at one each)
+constexpr int kPhaseCounterWords = 72 + 2 * kPhaseMaxB;
+enum : int { kPhFolded = 0, kPhExited = 32 };
+struct PhPos { float cp, nMP, nMQ, pad; double p, ZQ; };   // p_c Z_Q / Z_P, minus the row references, p_c, Z_Q
+struct PhasePlan {
+    int rows;             // rows of a sequence in the first sweep: 2 gamma, or gamma with supplied draft normalisers
+    int units;            // units of 64 vectors in a row
+    int n1;               // units of the first sweep
+    int per1;             // ... of which each warp takes this many
+    int slots;            // warps that may hold some of one row, at most
+    bool fits;            // few enough sequences, units and tokens for the kernel's counters and indexes
+};
+struct PhaseScratch {
+    unsigned* ctr;        // [kPhFolded] sequences folded, [kPhExited] CTAs that have left; zero between launches, like the next three
+    unsigned* done;       // [2 rounds] sequences whose listed second sweeps are in; in the high half: those that go on
+    unsigned* cnt1;       // [B] units of the first sweep that are in, and one for the drafted tokens' logits
+    unsigned* cnt2;       // [B] units of the round's second sweeps that are in
+    double2* part;        // [B rows][slots] {reference, sum} of each warp's piece of the row
+    float2* drafted;      // [B gamma] the drafted tokens' logits in the target and the draft row
+    PhPos* pos;           // [B (gamma+1)]
+    uint4* sel;           // [2 rounds, 1 unread][B] candidates: positions 0 .. 31, 32 .. 63, position gamma, data fault
+    uint2* rest;          // [B] candidates below one that passes unless its residual is empty
+    float* seg_M;         // [B][units] references of the last target row's units
+    double* seg;          // [B (gamma+1)][units] unit totals of the second sweeps
+    int n1, rows, units, per1, slots;
+    unsigned zero_words;
+};
+PhasePlan phase_plan(int V, int dtype, bool aligned, int B, int gamma, bool lse, int nctas);
+// Lays the scratch out from `base` on; returns the bytes it takes (base may be null for that).
+size_t phase_scratch(void* base, unsigned* counters, int B, int gamma, const PhasePlan& pl, PhaseScratch* ps);
+int phase_max_ctas(int dtype, int sm_count);
+cudaError_t launch_phase(const Params& prm, const PhaseScratch& ps, int dtype, bool aligned, int nctas, cudaStream_t stream);
+
 }  // namespace bv
