@@ -194,13 +194,13 @@ bool slot_can_hold(const DeviceState& d, cudaStream_t stream, size_t need) {
     return cap == cudaStreamCaptureStatusNone;
 }
 
-// Where the phase kernel is the default for rows of 16-byte vectors.
-bool phase_pays(int algo, const bv::Params& prm, const Options& opt, long long logit_bytes) {
+// Where the phase kernel is the default.  (Rows that are not whole 16-byte vectors: wherever the small-batch kernel is not.)
+bool phase_pays(int algo, const bv::Params& prm, const Options& opt, bool vec, long long logit_bytes) {
     const bool small = bv::small_fits(prm.B, prm.gamma);
     if (prm.probs) return !small || prm.B >= kPhaseProbsB;
     const int which = algo == bv::kTokenVerify ? 0 : (prm.lse_d != nullptr ? 2 : 1);
     const long long least = opt.small_bytes > 0 ? static_cast<long long>(opt.small_bytes) << 20 : kPhaseBytes[which][0];
-    return (!small || logit_bytes > least) && logit_bytes <= kPhaseBytes[which][1];
+    return (!small || logit_bytes > least) && (!vec || logit_bytes <= kPhaseBytes[which][1]);
 }
 
 // The phase kernel for the call in `prm`: BV_OK, an error, or 1 if it does not take the call.  Rows at any alignment have no
@@ -304,7 +304,7 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
     // Both sweeps split over all warps, with the folds between them: between the small-batch kernel's sizes and the flow
     // kernel's, and for rows at any alignment.
     const bool only_vec = prm.lse_d != nullptr || prm.greedy || prm.probs;      // (entry points without an element-wise path)
-    if (opt.kernel == 5 ? vec || !only_vec : opt.kernel == 0 && (vec ? phase_pays(algo, prm, opt, logit_bytes) : !only_vec)) {
+    if ((vec || !only_vec) && (opt.kernel == 5 || (opt.kernel == 0 && phase_pays(algo, prm, opt, vec, logit_bytes)))) {
         if ((rc = run_phase(*d, prm, dtype, vec, stream)) <= BV_OK) return rc;
     }
 
@@ -313,15 +313,17 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
     const long long small_limit = opt.small_bytes > 0 ? static_cast<long long>(opt.small_bytes) << 20 : kSmallBytes[algo == bv::kBlockVerify ? 1 : 0];
     // (given probabilities only a few row pairs per sequence are read whatever the size of the rest: there the
     // small-batch kernel wins up to 16 sequences, 17 against 33 us for one, 33 against 38 us for sixteen)
-    if (vec && bv::small_fits(B, gamma) &&
+    if ((vec || !only_vec) && bv::small_fits(B, gamma) &&
         (opt.kernel == 4 || (opt.kernel == 0 && (prm.probs ? B <= 16 : logit_bytes <= small_limit)))) {
         int& nc = d->small_ctas[dtype];
         if (nc == 0) {
             nc = bv::small_max_ctas(dtype, d->sm_count);
             if (nc <= 0) nc = -1;
         }
-        if (nc > 0) {
-            const bv::SmallPlan plan = bv::small_plan(static_cast<long long>(row_bytes / 16), B, gamma, nc);
+        // (a row that starts inside a vector lies in one more)
+        const long long vecs = vec ? static_cast<long long>(row_bytes / 16) : (static_cast<long long>(row_bytes) + 30) / 16;
+        const bv::SmallPlan plan = bv::small_plan(vecs, B, gamma, nc > 0 ? nc : 1);
+        if (nc > 0 && (vec || (V <= (1 << 30) && slot_can_hold(*d, stream, bv::small_scratch_bytes(B, gamma, plan))))) {
             StreamSlot* slot = nullptr;
             if ((rc = stream_slot(*d, stream, bv::small_scratch_bytes(B, gamma, plan), &slot)) != BV_OK) return rc;
             slot->clean = 0;                // (the area the flow kernel expects to find zero is written here)
@@ -332,7 +334,7 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
             prm.ticket = nullptr;
             prm.nclusters = 0;
             prm.status = static_cast<int*>(slot->ws);
-            cudaError_t e = bv::launch_small(prm, sc, dtype, nc, stream);
+            cudaError_t e = bv::launch_small(prm, sc, dtype, vec, nc, stream);
             if (e != cudaSuccess) return cuda_fail(e);
             t_last_launches = 1; t_last_kernel = 4;
             return BV_OK;

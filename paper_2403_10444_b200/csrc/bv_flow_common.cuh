@@ -221,6 +221,59 @@ __device__ int f_rescan(const char* rowP, const char* rowQ, int w0, int w1, int 
     }, rowQ != nullptr, w0, w1, lane, kf, cp, nMP, nMQ, tw);
 }
 
+// ---- rows at any alignment: a row is read as the aligned vectors that its bytes lie in; what of the first and the last
+// of them belongs to its neighbours weighs nothing ----
+// row start -> first 16-byte vector, elements of it that belong to the row before, vectors
+// (AL: rows of whole 16-byte vectors on 16-byte aligned bases)
+template <int DT, bool AL>
+__device__ __forceinline__ void row_grid(const char* row, int V, const char*& base, int& h, int& nv) {
+    constexpr int EPV = Raw<DT>::EPV;
+    constexpr int ESZ = (DT == kF32) ? 4 : 2;
+    if (AL) { base = row; h = 0; nv = V / EPV; return; }
+    const unsigned off = static_cast<unsigned>(reinterpret_cast<uintptr_t>(row) & 15u);
+    base = row - off; h = static_cast<int>(off) / ESZ; nv = (h + V + EPV - 1) / EPV;
+}
+// elements of vector i (on the row's 16-byte grid, h elements into the vector before) outside [0, V) weigh nothing
+template <int EPV> __device__ __forceinline__ void row_mask(float (&v)[EPV], int i, int h, int V, float pad) {
+#pragma unroll
+    for (int e = 0; e < EPV; ++e) {
+        const int x = i * EPV + e - h;
+        if (x < 0 || x >= V) v[e] = pad;
+    }
+}
+// Sixteen bytes of a row from element x0 on, elements outside [0, V) as `pad` (rows at any alignment, one at a time).
+template <int DT>
+__device__ __forceinline__ uint4 row_elements(const char* row, int x0, int V, uint32_t pad) {
+    uint32_t w[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (DT == kF32) {
+            const int x = x0 + j;
+            w[j] = x >= 0 && x < V ? __ldg(reinterpret_cast<const unsigned*>(row) + x) : pad;
+        } else {
+            const int x = x0 + 2 * j;
+            const uint32_t l = x >= 0 && x < V ? __ldg(reinterpret_cast<const unsigned short*>(row) + x) : (pad & 0xffffu);
+            const uint32_t h = x + 1 >= 0 && x + 1 < V ? __ldg(reinterpret_cast<const unsigned short*>(row) + x + 1) : (pad & 0xffffu);
+            w[j] = l | (h << 16);
+        }
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+// ... the rescan: vectors [w0, w1) on the target row's grid
+template <int DT, bool PROBS, int kAhead>
+__device__ int f_rescan_any(const char* rowP, const char* rowQ, int V, int w0, int w1, int lane, float kf, float cp,
+                            float nMP, float nMQ, double tw) {
+    constexpr uint32_t kPad = PROBS ? 0u : Raw<DT>::kNegInf;
+    constexpr int EPV = Raw<DT>::EPV;
+    const char* base; int h, nv;
+    row_grid<DT, false>(rowP, V, base, h, nv);
+    const int found = f_rescan_with<DT, PROBS, kAhead>([&](int i, bool in, uint4& rp, uint4& rq) {
+        rp = in ? row_elements<DT>(rowP, i * EPV - h, V, kPad) : make_uint4(kPad, kPad, kPad, kPad);
+        rq = in && rowQ ? row_elements<DT>(rowQ, i * EPV - h, V, kPad) : make_uint4(kPad, kPad, kPad, kPad);
+    }, rowQ != nullptr, w0, w1 < nv ? w1 : nv, lane, kf, cp, nMP, nMQ, tw);
+    return found >= 0 ? found - h : found;
+}
+
 // Acceptance weight of position 0 < i < gamma from p_i and S_i: Eq. "pacc_block",
 // h_i = S_i / (S_i + 1 - p_i), and 0 for an empty residual.  Algorithm 4 prints its h_i as
 // sum_x max(pt_i P_i - Q_i, 0) / sum_x max(Q_i - pt_i P_i, 0); both rows sum to one, so the second

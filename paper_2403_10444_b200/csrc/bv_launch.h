@@ -111,7 +111,7 @@ SmallPlan small_plan(long long units, int B, int gamma, int nctas);
 size_t small_scratch_bytes(int B, int gamma, const SmallPlan& pl);
 void small_scratch_layout(void* base, unsigned* barrier, int B, int gamma, const SmallPlan& pl, SmallScratch* sc);
 int small_max_ctas(int dtype, int sm_count);
-cudaError_t launch_small(const Params& prm, const SmallScratch& sc, int dtype, int nctas, cudaStream_t stream);
+cudaError_t launch_small(const Params& prm, const SmallScratch& sc, int dtype, bool aligned, int nctas, cudaStream_t stream);
 
 // Phase kernel (bv_phase.cu): a cooperative launch of one CTA per SM, both sweeps split statically over all warps.
 constexpr int kPhaseMaxB = 768;       // sequences (a CTA's threads look at one each)

@@ -335,25 +335,6 @@ static __device__ __noinline__ void ph_fold_probs(const Params& prm, const Phase
     ph_decide(prm, ps, b, lane, M, Z, M, Z, rat, badrow, eta, eta_g, false);
 }
 
-// Sixteen bytes of a row from element x0 on, elements outside [0, V) as `pad` (rows at any alignment, one at a time).
-template <int DT>
-__device__ __forceinline__ uint4 ph_elements(const char* row, int x0, int V, uint32_t pad) {
-    uint32_t w[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        if (DT == kF32) {
-            const int x = x0 + j;
-            w[j] = x >= 0 && x < V ? __ldg(reinterpret_cast<const unsigned*>(row) + x) : pad;
-        } else {
-            const int x = x0 + 2 * j;
-            const uint32_t l = x >= 0 && x < V ? __ldg(reinterpret_cast<const unsigned short*>(row) + x) : (pad & 0xffffu);
-            const uint32_t h = x + 1 >= 0 && x + 1 < V ? __ldg(reinterpret_cast<const unsigned short*>(row) + x + 1) : (pad & 0xffffu);
-            w[j] = l | (h << 16);
-        }
-    }
-    return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
 // Unit totals of a position as a warp looks at them: lane l speaks for `per` consecutive ones.
 template <class At> __device__ __forceinline__ double ph_lane_sum(At at, int per, int lane) {
     double s = 0.0;
@@ -411,7 +392,6 @@ static __device__ __noinline__ void ph_finalize(const Params& prm, const PhaseSc
     const bool all = f_all_positions(prm) && !dry, tv = prm.algo == kTokenVerify;
     constexpr size_t ESZ = (DT == kF32) ? 4 : 2;
     constexpr int EPV = Raw<DT>::EPV;
-    constexpr uint32_t kPad = PROBS ? 0u : Raw<DT>::kNegInf;
     const size_t row_bytes = static_cast<size_t>(prm.V) * ESZ;
     const size_t row0 = static_cast<size_t>(b) * (g + 1);
     const float* u = prm.uni + static_cast<size_t>(b) * (g + 2);
@@ -480,12 +460,7 @@ static __device__ __noinline__ void ph_finalize(const Params& prm, const PhaseSc
                 found = f_rescan<DT, PROBS, 2>(rowP, rowQ, w0, min(w0 + kPhUnit, prm.V / EPV), lane, prm.kf, q.cp, q.nMP, q.nMQ, rem);
             } else {
                 // (the units are cut on the 16-byte vectors that the target row's bytes lie in)
-                const int h = static_cast<int>((reinterpret_cast<uintptr_t>(rowP) & 15u) / ESZ), nv = (h + prm.V + EPV - 1) / EPV;
-                found = f_rescan_with<DT, PROBS, 2>([&](int i, bool in, uint4& rp, uint4& rq) {
-                    rp = in ? ph_elements<DT>(rowP, i * EPV - h, prm.V, kPad) : make_uint4(kPad, kPad, kPad, kPad);
-                    rq = in && rowQ ? ph_elements<DT>(rowQ, i * EPV - h, prm.V, kPad) : make_uint4(kPad, kPad, kPad, kPad);
-                }, rowQ != nullptr, w0, min(w0 + kPhUnit, nv), lane, prm.kf, q.cp, q.nMP, q.nMQ, rem);
-                if (found >= 0) found -= h;
+                found = f_rescan_any<DT, PROBS, 2>(rowP, rowQ, prm.V, w0, w0 + kPhUnit, lane, prm.kf, q.cp, q.nMP, q.nMQ, rem);
             }
         }
         if (!all) break;
@@ -527,20 +502,11 @@ __device__ __forceinline__ void ph_fetch_edge(uint32_t cell, const char* p, bool
             constexpr int ESZ = (DT == kF32) ? 4 : 2;
             const int first = p < lo ? static_cast<int>((lo - p) / ESZ) : 0;
             const int n = static_cast<int>((hi - p) / ESZ);
-            v = ph_elements<DT>(p + first * ESZ, -first, n - first, pad);
+            v = row_elements<DT>(p + first * ESZ, -first, n - first, pad);
         }
         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cell), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
     }
 }
-// elements of vector i (on the row's 16-byte grid, h elements into the vector before) outside [0, V) weigh nothing
-template <int EPV> __device__ __forceinline__ void ph_mask(float (&v)[EPV], int i, int h, int V, float pad) {
-#pragma unroll
-    for (int e = 0; e < EPV; ++e) {
-        const int x = i * EPV + e - h;
-        if (x < 0 || x >= V) v[e] = pad;
-    }
-}
-
 // AL: rows of whole 16-byte vectors on 16-byte aligned bases.  Otherwise a row is read as the aligned vectors that its
 // bytes lie in, and what of the first and the last of them belongs to its neighbours weighs nothing; in a second sweep
 // the draft row's elements are shifted onto the target row's grid between two neighbouring cells of the ring.
@@ -583,12 +549,6 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
     bool i_single = true;
     const char* iAlo = nullptr; const char* iAhi = nullptr;   // unaligned: bounds of the tensor that cell A is read from
     int iq = 0, i_nvq = 0;                // unaligned pairs: this lane's vector of the draft row, and how many there are
-    // row start -> first 16-byte vector, elements of it that belong to the row before, vectors
-    auto grid_of = [&](const char* row, const char*& base, int& h, int& nv) {
-        if (AL) { base = row; h = 0; nv = V / EPV; return; }
-        const unsigned off = static_cast<unsigned>(reinterpret_cast<uintptr_t>(row) & 15u);
-        base = row - off; h = static_cast<int>(off) / ESZ; nv = (h + V + EPV - 1) / EPV;
-    };
     auto issue_step = [&](uint32_t cell) {
         if (AL) {
             const int adv = i_single ? 64 : 32;
@@ -623,7 +583,7 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
     // units k .. k+n-1 of the row that starts at `row`
     auto open_row = [&](const char* row, int k, int n, PhRun& q) {
         const char* base; int h, nv;
-        grid_of(row, base, h, nv);
+        row_grid<DT, AL>(row, V, base, h, nv);
         const int v0 = k * kPhUnit, v1 = min((k + n) * kPhUnit, nv);
         iA = base + static_cast<size_t>(v0 + lane) * 16;
         iB = iA + 512;
@@ -691,7 +651,7 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
                 float va[EPV], vb[EPV];
                 R::unpack(lds128(rp), va);
                 R::unpack(lds128(rp + 512), vb);
-                if (!AL && (v == 0 || v + 64 >= nv)) { ph_mask<EPV>(va, v + lane, h, V, kPadF); ph_mask<EPV>(vb, v + 32 + lane, h, V, kPadF); }
+                if (!AL && (v == 0 || v + 64 >= nv)) { row_mask<EPV>(va, v + lane, h, V, kPadF); row_mask<EPV>(vb, v + 32 + lane, h, V, kPadF); }
                 // (the run's reference comes from the first vectors of every lane)
                 if (st == 0) M = fmaxf(rintf(warp_max(fmaxf(vec_max<EPV>(va), vec_max<EPV>(vb))) * kf), kNoRef);
                 const float was = M;
@@ -765,7 +725,7 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
                 const int h = open_row(tgt + ri * row_bytes, k_i, n, q);
                 if (!i_single) {
                     const char* baseQ; int hQ, nvQ;
-                    grid_of(drf + (static_cast<size_t>(i_b) * g + i_c) * row_bytes, baseQ, hQ, nvQ);
+                    row_grid<DT, AL>(drf + (static_cast<size_t>(i_b) * g + i_c) * row_bytes, V, baseQ, hQ, nvQ);
                     int dq = 0, shift = hQ - h;
                     if (!AL && shift < 0) { shift += EPV; dq = -1; }
                     iq = k_i * kPhUnit + lane + dq;
@@ -813,7 +773,7 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
                         float va[EPV], vb[EPV];
                         R::unpack(lds128(rp), va);
                         R::unpack(lds128(rp + 512), vb);
-                        if (!AL && (v == 0 || v + 64 >= nv)) { ph_mask<EPV>(va, v + lane, h, V, kPadF); ph_mask<EPV>(vb, v + 32 + lane, h, V, kPadF); }
+                        if (!AL && (v == 0 || v + 64 >= nv)) { row_mask<EPV>(va, v + lane, h, V, kPadF); row_mask<EPV>(vb, v + 32 + lane, h, V, kPadF); }
                         acc = 0.0;
                         if (PROBS) {
                             acc = static_cast<double>(f_sum<EPV>(va)) + static_cast<double>(f_sum<EPV>(vb));
@@ -859,7 +819,7 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
                         }
                         if (!AL) {
                             __syncwarp();                     // (every lane has read its neighbours' cells)
-                            if (v == 0 || v + 32 >= nv) { ph_mask<EPV>(va, v + lane, h, V, kPadF); ph_mask<EPV>(vb, v + lane, h, V, kPadF); }
+                            if (v == 0 || v + 32 >= nv) { row_mask<EPV>(va, v + lane, h, V, kPadF); row_mask<EPV>(vb, v + lane, h, V, kPadF); }
                         }
                         acc += static_cast<double>(f_pair_sum<EPV, true, PROBS>(va, vb, kf, cp, nMP, nMQ, t));
                         if ((v & 32) || v + 32 >= v1) {       // the end of a unit

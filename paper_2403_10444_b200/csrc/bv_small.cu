@@ -27,7 +27,7 @@ constexpr int kSmAllThreads = kSmThreads + 32;
 constexpr int kSmMaxRows = 1056;      // rows B (2 gamma + 1) whose normalisers a CTA keeps in shared memory
 constexpr int kSmMaxPos = 560;        // positions B (gamma + 1)
 constexpr int kSmInFlight = 8;        // 16-byte loads a thread has in flight in the first phase
-constexpr int kSmPairsInFlight = 5;   // pairs of them in the second
+constexpr int kSmPairsInFlight = 5;   // pairs of them in the second (unaligned rows: three of one and two)
 constexpr int kSmMaxUni = kSmMaxPos + kSmallMaxB;   // uniforms B (gamma + 2)
 
 struct SmallShared {
@@ -80,17 +80,43 @@ __device__ __forceinline__ const char* small_row(const Params& prm, size_t row_b
                   : static_cast<const char*>(prm.drf) + (static_cast<size_t>(b) * g + (j - g - 1)) * row_bytes;
 }
 
+// vector i of the nv that a row's bytes lie in, from `base` on; [lo, hi): the tensor
+template <int DT, bool AL>
+__device__ __forceinline__ uint4 small_load(const char* base, int i, int nv, const char* lo, const char* hi, uint32_t pad) {
+    const char* p = base + static_cast<long long>(i) * 16;
+    if (i < 0 || i >= nv) return make_uint4(pad, pad, pad, pad);
+    if (AL || (p >= lo && p + 16 <= hi)) return ld_stream_v4(p);
+    constexpr int ESZ = (DT == kF32) ? 4 : 2;                // (it reaches outside the tensor: the elements inside)
+    const int first = p < lo ? static_cast<int>((lo - p) / ESZ) : 0;
+    return row_elements<DT>(p + first * ESZ, -first, static_cast<int>((hi - p) / ESZ) - first, pad);
+}
+// 16 bytes from byte 4 q + bits / 8 on of two neighbouring vectors
+__device__ __forceinline__ uint4 small_shift(const uint4& a, const uint4& b, int q, int bits) {
+    uint32_t w0 = a.x, w1 = a.y, w2 = a.z, w3 = a.w, w4 = b.x, w5 = b.y, w6 = b.z, w7 = b.w;
+    if (q & 2) { w0 = w2; w1 = w3; w2 = w4; w3 = w5; w4 = w6; w5 = w7; }
+    if (q & 1) { w0 = w1; w1 = w2; w2 = w3; w3 = w4; w4 = w5; }
+    return make_uint4(__funnelshift_r(w0, w1, bits), __funnelshift_r(w1, w2, bits), __funnelshift_r(w2, w3, bits), __funnelshift_r(w3, w4, bits));
+}
+
 // PROBS: the rows hold probabilities, used as stored: there is no first phase (and no first barrier).
-template <int DT, bool PROBS>
+// AL: rows of whole 16-byte vectors on 16-byte aligned bases.  Otherwise a row is read as the vectors its bytes lie in
+// (row_grid), and the draft row of a pair is put on the target row's grid from two neighbouring vectors.
+template <int DT, bool PROBS, bool AL>
 __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const Params prm, const SmallScratch sc) {
     using R = Raw<DT>;
     constexpr int EPV = R::EPV;
+    constexpr int kPairs = AL ? kSmPairsInFlight : 3;
+    const float kPadF = PROBS ? 0.f : -INFINITY;
     constexpr uint32_t kPad = PROBS ? 0u : R::kNegInf;       // what a lane beyond the end of a segment finds: no weight
     constexpr size_t ESZ = (DT == kF32) ? 4 : 2;
     __shared__ SmallShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int g = prm.gamma, B = prm.B, units = prm.V / EPV;
+    const int g = prm.gamma, B = prm.B, V = prm.V;
     const size_t row_bytes = static_cast<size_t>(prm.V) * ESZ;
+    const char* const tgt = static_cast<const char*>(prm.tgt);
+    const char* const drf = static_cast<const char*>(prm.drf);
+    const char* const tgt_end = tgt + static_cast<size_t>(B) * (g + 1) * row_bytes;
+    const char* const drf_end = drf + static_cast<size_t>(B) * g * row_bytes;
     const float kf = prm.kf;
     const int rpb = 2 * g + 1, nrows = B * rpb;
     const unsigned limit = prm.wait_limit ? prm.wait_limit : (1u << 22);
@@ -117,22 +143,28 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const Pa
         const int rid = item / nch, ch = item % nch;
         if (prm.lse_d != nullptr && rid % rpb > g) continue;      // (a draft row whose normaliser is supplied: nothing to learn)
         const char* row = small_row(prm, row_bytes, rid / rpb, rid % rpb);
-        int u0, u1;
-        small_seg_range(units, nch, ch, u0, u1);
+        const char* base16; int h, nv, u0, u1;
+        row_grid<DT, AL>(row, V, base16, h, nv);
+        const char* const lo = rid % rpb <= g ? tgt : drf;
+        const char* const hi = rid % rpb <= g ? tgt_end : drf_end;
+        small_seg_range(nv, nch, ch, u0, u1);
         float M = kNoRef, s = 0.f;
-        const uint4 ninf = make_uint4(R::kNegInf, R::kNegInf, R::kNegInf, R::kNegInf);
         for (int base = u0; warp < kSmWarps && base < u1; base += kSmThreads * kSmInFlight) {
             uint4 raw[kSmInFlight];
 #pragma unroll
             for (int j = 0; j < kSmInFlight; ++j) {
                 const int i = base + j * kSmThreads + tid;
-                raw[j] = i < u1 ? ld_stream_v4(row + static_cast<size_t>(i) * 16) : ninf;
+                raw[j] = small_load<DT, AL>(base16, i, u1, lo, hi, R::kNegInf);
             }
 #pragma unroll
             for (int j = 0; j < kSmInFlight; ++j) {
                 if (base + j * kSmThreads + (warp << 5) < u1) {          // (warp-uniform)
                     float v[EPV];
                     R::unpack(raw[j], v);
+                    if (!AL) {
+                        const int i = base + j * kSmThreads + tid;
+                        if (i == 0 || i == nv - 1) row_mask<EPV>(v, i, h, V, kPadF);
+                    }
                     f_accumulate<EPV>(v, kf, M, s);
                 }
             }
@@ -305,23 +337,35 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const Pa
             const char* rowQ = have_q ? small_row(prm, row_bytes, b, g + 1 + i) : nullptr;
             const float cp = sh.csc[b * (g + 1) + i];
             const float nMP = -sh.rowM[b * rpb + i], nMQ = have_q ? -sh.rowM[b * rpb + g + 1 + i] : 0.f;
-            int s0, s1;
-            small_seg_range(units, nseg, piece * kSmWarps + (warp < kSmWarps ? warp : 0), s0, s1);
+            int s0, s1, hP, nvP, hQ = 0, nvQ = 0;
+            const char* baseP;
+            const char* baseQ = nullptr;
+            row_grid<DT, AL>(rowP, V, baseP, hP, nvP);
+            if (have_q) row_grid<DT, AL>(rowQ, V, baseQ, hQ, nvQ);
+            int shift = hQ - hP, dq = 0;                      // the draft row's elements against the target row's grid
+            if (!AL && shift < 0) { shift += EPV; dq = -1; }
+            const int sq = shift * static_cast<int>(ESZ) >> 2, sbits = (shift * static_cast<int>(ESZ) & 3) * 8;
+            small_seg_range(nvP, nseg, piece * kSmWarps + (warp < kSmWarps ? warp : 0), s0, s1);
             double acc = 0.0;
-            for (int base = s0; warp < kSmWarps && base < s1; base += 32 * kSmPairsInFlight) {
-                uint4 rp[kSmPairsInFlight], rq[kSmPairsInFlight];
-                const uint4 ninf = make_uint4(kPad, kPad, kPad, kPad);
+            for (int base = s0; warp < kSmWarps && base < s1; base += 32 * kPairs) {
+                uint4 rp[kPairs], rq[kPairs], rx[AL ? 1 : kPairs];
 #pragma unroll
-                for (int j = 0; j < kSmPairsInFlight; ++j) {
+                for (int j = 0; j < kPairs; ++j) {
                     const int v = base + 32 * j + lane;
-                    rp[j] = v < s1 ? ld_stream_v4(rowP + static_cast<size_t>(v) * 16) : ninf;
-                    rq[j] = (v < s1 && have_q) ? ld_stream_v4(rowQ + static_cast<size_t>(v) * 16) : ninf;
+                    rp[j] = small_load<DT, AL>(baseP, v, s1, tgt, tgt_end, kPad);
+                    const int lim = v < s1 ? (AL ? s1 : nvQ) : 0;
+                    rq[j] = small_load<DT, AL>(baseQ, v + dq, have_q ? lim : 0, drf, drf_end, kPad);
+                    if (!AL) rx[AL ? 0 : j] = small_load<DT, AL>(baseQ, v + dq + 1, have_q ? lim : 0, drf, drf_end, kPad);
                 }
 #pragma unroll
-                for (int j = 0; j < kSmPairsInFlight; ++j) {
+                for (int j = 0; j < kPairs; ++j) {
                     float vp[EPV], vq[EPV], t[EPV];
                     R::unpack(rp[j], vp);
-                    R::unpack(rq[j], vq);
+                    R::unpack(AL ? rq[j] : small_shift(rq[j], rx[AL ? 0 : j], sq, sbits), vq);
+                    if (!AL) {
+                        const int v = base + 32 * j + lane;
+                        if (v == 0 || v >= nvP - 1) { row_mask<EPV>(vp, v, hP, V, kPadF); row_mask<EPV>(vq, v, hP, V, kPadF); }
+                    }
                     if (have_q) acc += static_cast<double>(f_pair_sum<EPV, true, PROBS>(vp, vq, kf, cp, nMP, nMQ, t));
                     else acc += static_cast<double>(f_pair_sum<EPV, false, PROBS>(vp, vq, kf, cp, nMP, nMQ, t));
                 }
@@ -408,11 +452,14 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const Pa
                 }
                 const int sel = __shfl_sync(0xffffffffu, 4 * lane + e, src);
                 const double before = shfl_d(bef, src);
-                int s0, s1;
-                small_seg_range(units, nseg, sel, s0, s1);
-                found = f_rescan<DT, PROBS, 5>(small_row(prm, row_bytes, b, tau), have_q ? small_row(prm, row_bytes, b, g + 1 + tau) : nullptr,
-                                     s0, s1, lane, kf, sh.csc[b * (g + 1) + tau], -sh.rowM[b * rpb + tau],
-                                     have_q ? -sh.rowM[b * rpb + g + 1 + tau] : 0.f, t - before);
+                const char* rowP = small_row(prm, row_bytes, b, tau);
+                const char* rowQ = have_q ? small_row(prm, row_bytes, b, g + 1 + tau) : nullptr;
+                const float cp = sh.csc[b * (g + 1) + tau], nMP = -sh.rowM[b * rpb + tau], nMQ = have_q ? -sh.rowM[b * rpb + g + 1 + tau] : 0.f;
+                const char* baseP; int h, nv, s0, s1;
+                row_grid<DT, AL>(rowP, V, baseP, h, nv);
+                small_seg_range(nv, nseg, sel, s0, s1);
+                found = AL ? f_rescan<DT, PROBS, 5>(rowP, rowQ, s0, s1, lane, kf, cp, nMP, nMQ, t - before)
+                           : f_rescan_any<DT, PROBS, 2>(rowP, rowQ, V, s0, s1, lane, kf, cp, nMP, nMQ, t - before);
             }
             const bool bad = sh.bad[b] != 0 || found < 0;      // (an empty residual where the algorithm must sample: a domain error)
             int32_t* ot = prm.out_tokens + static_cast<size_t>(b) * (g + 1);
@@ -507,26 +554,28 @@ void small_scratch_layout(void* base, unsigned* barrier, int B, int gamma, const
 }
 
 using SKernelFn = void (*)(const Params, const SmallScratch);
-static SKernelFn pick_small(int dtype, bool probs) {
-    if (probs) return dtype == kF32 ? verify_small_kernel<kF32, true> : verify_small_kernel<kBF16, true>;
-    return dtype == kF32 ? verify_small_kernel<kF32, false> : verify_small_kernel<kBF16, false>;
+static SKernelFn pick_small(int dtype, bool probs, bool aligned) {
+    if (probs) return dtype == kF32 ? verify_small_kernel<kF32, true, true> : verify_small_kernel<kBF16, true, true>;
+    if (aligned) return dtype == kF32 ? verify_small_kernel<kF32, false, true> : verify_small_kernel<kBF16, false, true>;
+    return dtype == kF32 ? verify_small_kernel<kF32, false, false> : verify_small_kernel<kBF16, false, false>;
 }
 
 int small_max_ctas(int dtype, int sm_count) {
-    int n = 0;
-    // (the variant on logits is the larger program)
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pick_small(dtype, false), kSmAllThreads, 0) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
+    for (int v = 0; v < 3; ++v) {
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pick_small(dtype, v == 2, v != 1), kSmAllThreads, 0) != cudaSuccess || n < 1) {
+            cudaGetLastError();
+            return 0;
+        }
     }
-    return n > 0 ? sm_count : 0;          // one CTA per SM: all of them resident at once, as the barriers need
+    return sm_count;          // one CTA per SM: all of them resident at once, as the barriers need
 }
 
-cudaError_t launch_small(const Params& prm, const SmallScratch& sc, int dtype, int nctas, cudaStream_t stream) {
+cudaError_t launch_small(const Params& prm, const SmallScratch& sc, int dtype, bool aligned, int nctas, cudaStream_t stream) {
     Params p = prm;
     SmallScratch s = sc;
     void* args[] = {&p, &s};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(pick_small(dtype, prm.probs != 0)), dim3(nctas), dim3(kSmAllThreads), args, 0, stream);
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(pick_small(dtype, prm.probs != 0, aligned)), dim3(nctas), dim3(kSmAllThreads), args, 0, stream);
 }
 
 }  // namespace bv

@@ -1,5 +1,5 @@
-"""The phase kernel at the edges of its work units, at every alignment of the rows, and where its second round runs,
-against the oracle by the rules of tests/parity.py (GPU)."""
+"""The phase kernel at the edges of its work units, at every alignment of the rows, and where its second round runs, and the
+small-batch kernel at every alignment, against the oracle by the rules of tests/parity.py (GPU)."""
 import pytest
 import torch
 
@@ -10,13 +10,13 @@ from parity import run_oracle, run_cuda, compare, assert_parity
 pytestmark = pytest.mark.gpu
 
 
-def check(inp, algos, offset=None):
+def check(inp, algos, kernel=5):
     import paper_2403_10444_b200 as bv
     for algo in algos:
         ref = run_oracle(algo, inp)
         for diag in (True, False):
             out = run_cuda(algo, inp, diagnostics=diag)
-            assert bv.bv_last_kernel() == 5 and bv.bv_stream_status() == 0
+            assert bv.bv_last_kernel() == kernel and bv.bv_stream_status() == 0
             assert_parity(compare(algo, ref, out[0], out[1], out[2] if diag else None, inp), diag)
 
 
@@ -27,10 +27,10 @@ def inputs(B, gamma, V, dtype, seed, sigma_d=0.5):
 # a unit is 64 vectors: 512 bf16 or 256 fp32 logits; rows one short of, at and one beyond whole units and vectors
 @pytest.mark.parametrize("dtype,V", [("bf16", v) for v in (1, 7, 8, 9, 505, 511, 512, 513, 519, 520, 1023, 1025, 8191, 50257)] +
                          [("f32", v) for v in (1, 3, 4, 5, 253, 255, 256, 257, 1021, 1023, 20003)])
-@pytest.mark.parametrize("B,gamma", [(1, 1), (3, 40), (50, 5)])
-def test_rows_around_whole_units(dtype, V, B, gamma, bv_options):
-    bv_options("kernel", 5)
-    check(inputs(B, gamma, V, dtype, V + B), (oracle.BLOCK_VERIFY, oracle.TOKEN_VERIFY))
+@pytest.mark.parametrize("B,gamma,kernel", [(1, 1, 5), (3, 40, 5), (50, 5, 5), (1, 1, 4), (3, 40, 4), (25, 5, 4)])
+def test_rows_around_whole_units(dtype, V, B, gamma, kernel, bv_options):
+    bv_options("kernel", kernel)
+    check(inputs(B, gamma, V, dtype, V + B), (oracle.BLOCK_VERIFY, oracle.TOKEN_VERIFY), kernel)
 
 
 @pytest.mark.parametrize("V,B,gamma", [(4096, 768, 1), (64, 768, 3), (1003, 2000, 2), (16, 769, 2)])
@@ -46,10 +46,12 @@ def test_as_many_sequences_as_it_takes_and_more(V, B, gamma, bv_options):
             assert_parity(compare(algo, ref, out[0], out[1], out[2] if diag else None, inp), diag)
 
 
+@pytest.mark.parametrize("kernel", [4, 5])
 @pytest.mark.parametrize("dtype,V", [("bf16", 4104), ("bf16", 3001), ("f32", 4100)])
-def test_tensors_that_start_inside_a_vector(dtype, V):
+def test_tensors_that_start_inside_a_vector(dtype, V, kernel, bv_options):
     # the first and the last row's outer vectors reach beyond the tensors
     import paper_2403_10444_b200 as bv
+    bv_options("kernel", kernel)
     inp = inputs(5, 3, V, dtype, V)
     t, d = inp["target_logits"], inp["draft_logits"]
     for ot, od in ((1, 0), (0, 3), (3, 2)):
@@ -61,7 +63,7 @@ def test_tensors_that_start_inside_a_vector(dtype, V):
         for algo, fn in ((oracle.BLOCK_VERIFY, bv.bv_verify), (oracle.TOKEN_VERIFY, bv.tv_verify)):
             ref = run_oracle(algo, inp)
             out = fn(dev["target_logits"], dev["draft_logits"], dev["draft_tokens"], dev["uniforms"], inp["temperature"])
-            assert bv.bv_last_kernel() == 5
+            assert bv.bv_last_kernel() == kernel
             assert_parity(compare(algo, ref, out[0], out[1], None, inp), False)
 
 
@@ -79,9 +81,9 @@ def test_candidates_below_an_empty_residual(V, bv_options):
     check(inp, (oracle.BLOCK_VERIFY, oracle.TOKEN_VERIFY))
 
 
-@pytest.mark.parametrize("V", [4096, 4097])
-def test_faults_are_per_sequence(V, bv_options):
-    bv_options("kernel", 5)
+@pytest.mark.parametrize("V,kernel", [(4096, 5), (4097, 5), (4097, 4)])
+def test_faults_are_per_sequence(V, kernel, bv_options):
+    bv_options("kernel", kernel)
     inp = inputs(12, 3, V, "f32", 3)
     t, d, x = inp["target_logits"], inp["draft_logits"], inp["draft_tokens"]
     t[1, 0, 3] = float("nan")
