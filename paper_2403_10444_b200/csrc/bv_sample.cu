@@ -33,48 +33,67 @@ __device__ __forceinline__ void named_bar_arrive(int id, int threads) {
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
-// vectors [a0, a1) of sub-segment `sub` of warp `warp` in a row of `units` vectors
+// A warp's part of a row of `units` vectors is cut into sub-segments of whole runs of 32 vectors, one load of a warp: at most
+// kSSub of them, `runs` runs each (the last ones of a short part are empty).
+// vectors [a0, a1) of sub-segment `sub` of warp `warp`
+__device__ __forceinline__ void s_part(int units, int warp, int& u0, int& u1, int& runs) {
+    u0 = static_cast<int>(static_cast<long long>(units) * warp / kSWarps);
+    u1 = static_cast<int>(static_cast<long long>(units) * (warp + 1) / kSWarps);
+    runs = ((u1 - u0 + 31) / 32 + kSSub - 1) / kSSub;
+    if (runs < 1) runs = 1;
+}
 __device__ __forceinline__ void s_range(int units, int warp, int sub, int& a0, int& a1) {
-    const int u0 = static_cast<int>(static_cast<long long>(units) * warp / kSWarps);
-    const int u1 = static_cast<int>(static_cast<long long>(units) * (warp + 1) / kSWarps);
-    a0 = u0 + static_cast<int>(static_cast<long long>(u1 - u0) * sub / kSSub);
-    a1 = u0 + static_cast<int>(static_cast<long long>(u1 - u0) * (sub + 1) / kSSub);
+    int u0, u1, runs;
+    s_part(units, warp, u0, u1, runs);
+    a0 = min(u0 + sub * runs * 32, u1);
+    a1 = min(a0 + runs * 32, u1);
 }
 
 // One streaming warp's pass over its sixteenth of a row: the {reference, sum} pair of each of its
-// sub-segments goes to sM / sS.
+// sub-segments goes to sM / sS.  The loads of kSInFlight runs are issued together whatever sub-segments they
+// belong to.  (With one sub-segment's loads at a time a row of 2048 vectors, 16 to a sub-segment, waited for memory eight
+// times: a step of a drafting chain, B = 128 sequences of 16384 bf16 logits, 13 us, now 5 us; 2048 rows of 128256 logits,
+// 125 vectors to a sub-segment, 140 us, now 113 us: 4.7 TB/s.)
 template <int DT>
 __device__ __forceinline__ void s_sweep_row(const char* row, int units, float kf, int warp, int lane, float* sM, float* sS) {
     using R = Raw<DT>;
     constexpr int EPV = R::EPV;
-    // ---- one pass over the warp's part of the row ----
     // (the warp's reference carries over from one sub-segment to the next: a sub-segment's pair is
     // its sum against the reference as it stood at its end, and only the first one has to find one)
-    float M = kNoRef;
-    for (int sub = 0; sub < kSSub; ++sub) {
-        int a0, a1;
-        s_range(units, warp, sub, a0, a1);
-        float s = 0.f;
-        const uint4 ninf = make_uint4(R::kNegInf, R::kNegInf, R::kNegInf, R::kNegInf);
-        for (int base = a0; base < a1; base += 32 * kSInFlight) {
-            uint4 raw[kSInFlight];                // all loads of the round are issued before any is used
+    float M = kNoRef, s = 0.f;
+    int u0, u1, runs;
+    s_part(units, warp, u0, u1, runs);
+    const uint4 ninf = make_uint4(R::kNegInf, R::kNegInf, R::kNegInf, R::kNegInf);
+    int sub = 0, left = runs;
+    for (int base = u0; base < u1; base += 32 * kSInFlight) {
+        uint4 raw[kSInFlight];                    // all loads of the round are issued before any is used
 #pragma unroll
-            for (int j = 0; j < kSInFlight; ++j) {
-                const int i = base + 32 * j + lane;
-                raw[j] = i < a1 ? ld_stream_v4(row + static_cast<size_t>(i) * 16) : ninf;
-            }
+        for (int j = 0; j < kSInFlight; ++j) {
+            const int i = base + 32 * j + lane;
+            raw[j] = i < u1 ? ld_stream_v4(row + static_cast<size_t>(i) * 16) : ninf;
+        }
 #pragma unroll
-            for (int j = 0; j < kSInFlight; ++j) {
-                if (base + 32 * j < a1) {
-                    float v[EPV];
-                    R::unpack(raw[j], v);
-                    f_accumulate<EPV>(v, kf, M, s);
+        for (int j = 0; j < kSInFlight; ++j) {
+            if (base + 32 * j < u1) {
+                float v[EPV];
+                R::unpack(raw[j], v);
+                f_accumulate<EPV>(v, kf, M, s);
+                if (--left == 0) {                // the end of a sub-segment
+                    s = warp_sum(s);
+                    if (lane == 0) { sM[warp * kSSub + sub] = M; sS[warp * kSSub + sub] = s; }
+                    ++sub;
+                    left = runs;
+                    s = 0.f;
                 }
             }
         }
+    }
+    if (left < runs) {
         s = warp_sum(s);
         if (lane == 0) { sM[warp * kSSub + sub] = M; sS[warp * kSSub + sub] = s; }
+        ++sub;
     }
+    if (lane >= sub && lane < kSSub) { sM[warp * kSSub + lane] = kNoRef; sS[warp * kSSub + lane] = 0.f; }
 }
 
 // The sampling warp's part: the row's normaliser from the 128 pairs and the token that the uniform u
@@ -83,7 +102,7 @@ __device__ __forceinline__ void s_sweep_row(const char* row, int units, float kf
 // read the pairs.
 template <int DT>
 __device__ __forceinline__ int s_draw_row(const char* row, int units, float kf, const float* sM, const float* sS, float u,
-                                          int lane, int release_pairs, float* lse_out) {
+                                          int lane, int release_pairs, double* norm) {
     // ---- normaliser and the sampled sub-segment (fp64 prefix sums, index order) ----
     float m[4], w[4];
 #pragma unroll
@@ -135,9 +154,13 @@ __device__ __forceinline__ int s_draw_row(const char* row, int units, float kf, 
         s_range(units, sel / kSSub, sel % kSSub, a0, a1);
         found = f_rescan<DT>(row, nullptr, a0, a1, lane, kf, 1.f, -Mrow, 0.f, t - before);
     }
-    *lse_out = found >= 0 ? static_cast<float>((static_cast<double>(Mrow) + log2(Z)) * 0.693147180559945309417232)
-                          : __int_as_float(0x7fc00000);
+    norm[0] = Mrow;
+    norm[1] = Z;
     return found;
+}
+// the row's log-normaliser from what s_draw_row left
+__device__ __forceinline__ float s_lse(int found, const double* norm) {
+    return found >= 0 ? static_cast<float>((norm[0] + log2(norm[1])) * 0.693147180559945309417232) : __int_as_float(0x7fc00000);
 }
 
 template <int DT>
@@ -172,13 +195,13 @@ sample_rows_kernel(const char* logits, const float* uni, int rows, int V, float 
         for (int it = 0; it < nmine; ++it) {
             named_bar_sync(kBarFull + (it & 1), kSAllThreads);
             const int r = blockIdx.x + it * gridDim.x;
-            float l;
+            double norm[2];
             // (row it + 2 waits for the release of this buffer; the last two rows have nobody waiting)
             const int found = s_draw_row<DT>(logits + static_cast<size_t>(r) * row_bytes, units, kf, sM2[it & 1], sS2[it & 1], uni[r],
-                                             lane, it + 2 < nmine ? kBarEmpty + (it & 1) : -1, &l);
+                                             lane, it + 2 < nmine ? kBarEmpty + (it & 1) : -1, norm);
             if (lane == 0) {
                 tokens[r] = found;
-                if (lse) lse[r] = l;
+                if (lse) lse[r] = s_lse(found, norm);
             }
         }
     }
@@ -201,27 +224,28 @@ draft_chain_kernel(const char* table, const int32_t* first, const float* uni, in
     const int units = V / EPV;
     const size_t row_bytes = static_cast<size_t>(V) * ESZ;
     __shared__ float sM[kSSegs], sS[kSSegs];
-    __shared__ int s_next;
+    __shared__ int s_next[2];
     for (int b = blockIdx.x; b < B; b += gridDim.x) {
         int last = first[b];
         for (int i = 0; i < gamma; ++i) {
             const bool ok = last >= 0 && last < V;
             const char* row = table + static_cast<size_t>(ok ? last : 0) * row_bytes;
             if (warp < kSWarps && ok) s_sweep_row<DT>(row, units, kf, warp, lane, sM, sS);
+            const float u = uni[static_cast<size_t>(i) * B + b];
             __syncthreads();
+            int found = -1;
+            double norm[2] = {0.0, 0.0};
             if (warp == kSWarps) {
-                float l = __int_as_float(0x7fc00000);
-                int found = -1;
-                if (ok) found = s_draw_row<DT>(row, units, kf, sM, sS, uni[static_cast<size_t>(i) * B + b], lane, -1, &l);
-                if (lane == 0) {
-                    tokens[static_cast<size_t>(b) * gamma + i] = found;
-                    if (lse) lse[static_cast<size_t>(b) * gamma + i] = l;
-                    s_next = found;
-                }
+                if (ok) found = s_draw_row<DT>(row, units, kf, sM, sS, u, lane, -1, norm);
+                if (lane == 0) s_next[i & 1] = found;
             }
             __syncthreads();
-            last = s_next;
-            __syncthreads();      // (s_next is written again in the next step)
+            last = s_next[i & 1];     // (written again two steps on, after another barrier)
+            // the streaming warps are on the next row already
+            if (warp == kSWarps && lane == 0) {
+                tokens[static_cast<size_t>(b) * gamma + i] = found;
+                if (lse) lse[static_cast<size_t>(b) * gamma + i] = s_lse(found, norm);
+            }
         }
     }
 }
