@@ -194,6 +194,17 @@ bool slot_can_hold(const DeviceState& d, cudaStream_t stream, size_t need) {
     return cap == cudaStreamCaptureStatusNone;
 }
 
+// Where the element-wise kernel is still the default: a few short unaligned rows a sequence, one sequence an SM at most,
+// whose dependent steps cost less than the phase kernel's waits for the whole batch.  Measured, V = 1001 / 2051 / 4099 bf16:
+// Algorithm 1, B = 100, gamma = 3: 24 / 26 / 30 us against 31 / 39 / 40; Algorithm 2, gamma = 2: 26 / 29 / 36 against 33 / 39 / 39
+// (gamma = 3: 32 / 36 / 46 against 34 / 41 / 40).  Where the small-batch kernel fits: Algorithm 1, B = 32, gamma = 2: 20 / 22 / 25
+// against 22 / 23 / 24 us; Algorithm 2: never by more than the runs differ.
+bool elements_pay(int algo, const bv::Params& prm, size_t row_bytes, int sm_count) {
+    if (prm.B > sm_count) return false;
+    if (algo == bv::kTokenVerify) return bv::small_fits(prm.B, prm.gamma) ? prm.gamma <= 2 && row_bytes <= 4200 : prm.gamma <= 3 && row_bytes <= 8200;
+    return !bv::small_fits(prm.B, prm.gamma) && prm.gamma <= 2 && row_bytes <= 8200;
+}
+
 // Where the phase kernel is the default.  (Rows that are not whole 16-byte vectors: wherever the small-batch kernel is not.)
 bool phase_pays(int algo, const bv::Params& prm, const Options& opt, bool vec, long long logit_bytes) {
     const bool small = bv::small_fits(prm.B, prm.gamma);
@@ -304,7 +315,8 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
     // Both sweeps split over all warps, with the folds between them: between the small-batch kernel's sizes and the flow
     // kernel's, and for rows at any alignment.
     const bool only_vec = prm.lse_d != nullptr || prm.greedy || prm.probs;      // (entry points without an element-wise path)
-    if ((vec || !only_vec) && (opt.kernel == 5 || (opt.kernel == 0 && phase_pays(algo, prm, opt, vec, logit_bytes)))) {
+    const bool elements = !vec && !only_vec && opt.kernel == 0 && elements_pay(algo, prm, row_bytes, d->sm_count);
+    if ((vec || !only_vec) && !elements && (opt.kernel == 5 || (opt.kernel == 0 && phase_pays(algo, prm, opt, vec, logit_bytes)))) {
         if ((rc = run_phase(*d, prm, dtype, vec, stream)) <= BV_OK) return rc;
     }
 
@@ -313,7 +325,7 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
     const long long small_limit = opt.small_bytes > 0 ? static_cast<long long>(opt.small_bytes) << 20 : kSmallBytes[algo == bv::kBlockVerify ? 1 : 0];
     // (given probabilities only a few row pairs per sequence are read whatever the size of the rest: there the
     // small-batch kernel wins up to 16 sequences, 17 against 33 us for one, 33 against 38 us for sixteen)
-    if ((vec || !only_vec) && bv::small_fits(B, gamma) &&
+    if ((vec || !only_vec) && !elements && bv::small_fits(B, gamma) &&
         (opt.kernel == 4 || (opt.kernel == 0 && (prm.probs ? B <= 16 : logit_bytes <= small_limit)))) {
         int& nc = d->small_ctas[dtype];
         if (nc == 0) {

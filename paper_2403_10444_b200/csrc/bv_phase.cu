@@ -199,6 +199,44 @@ static __device__ __forceinline__ void ph_decide(const Params& prm, const PhaseS
 static __device__ __forceinline__ void ph_reduce_rows(const PhaseScratch& ps, int g, int b, int lane, float (&MP)[2], double (&ZP)[2],
                                                       float (&MQ)[2], double (&ZQ)[2]) {
     const int slots = ps.slots, rows = ps.rows;
+    if (slots <= 32) {
+        // a lane per row: no step waits for another lane, and eight pieces are asked for at a time
+        for (int r0 = 0; r0 < rows; r0 += 32) {
+            const int r = r0 + lane;
+            const unsigned x = static_cast<unsigned>((b * rows + r) * ps.units);
+            const int np = r < rows ? static_cast<int>((x + ps.units - 1) / ps.per1 - x / ps.per1) + 1 : 0;
+            const double2* part = ps.part + (static_cast<size_t>(b) * rows + r) * slots;
+            float m = kNoRef;
+            double s = 0.0;
+            for (int p0 = 0; p0 < slots; p0 += 8) {
+                double2 v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = p0 + j < np ? __ldcg(&part[p0 + j]) : make_double2(kNoRef, 0.0);
+                float mm = m;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) mm = fmaxf(mm, static_cast<float>(v[j].x));
+                s *= static_cast<double>(ref_scale(m, mm));
+#pragma unroll
+                for (int j = 0; j < 8; ++j) s += v[j].y * static_cast<double>(ref_scale(static_cast<float>(v[j].x), mm));
+                m = mm;
+            }
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {                     // target rows c and c + 32, draft rows c and c + 32
+                if ((h & 1) && g <= 32) continue;
+                if (h >= 2 && rows == g) continue;
+                const int c = lane + 32 * (h & 1), src = c + (h < 2 ? 0 : g) - r0;
+                const bool here = c < g && src >= 0 && src < 32;
+                const float mq = __shfl_sync(0xffffffffu, m, here ? src : 0);
+                const double zq = shfl_d(s, here ? src : 0);
+                if (here) {
+                    if (h < 2) { MP[h & 1] = mq; ZP[h & 1] = zq; }
+                    else { MQ[h & 1] = mq; ZQ[h & 1] = zq; }
+                }
+            }
+        }
+        return;
+    }
+    // (few long rows, in many pieces: the lanes share a row)
     int L = 1;
     while (L < slots && L < 32) L <<= 1;  // lanes that look at one row
     const int rp = 32 / L, sub = lane / L, k = lane % L;
@@ -387,7 +425,7 @@ __device__ __forceinline__ int ph_locate(At at, int per, int lane, double mine, 
 // token and the end of the sequence; else what is left of its candidates goes into the next round.
 // (dry: walk the code on whatever the scratch holds, write nothing)
 template <int DT, bool PROBS, bool AL>
-static __device__ __noinline__ void ph_finalize(const Params& prm, const PhaseScratch& ps, int b, int round, int lane, bool dry) {
+static __device__ __noinline__ void ph_finalize(const Params& prm, const PhaseScratch& ps, int b, uint4 sel, int round, int lane, bool dry) {
     const int g = prm.gamma, units = ps.units, per = (units + 31) / 32;
     const bool all = f_all_positions(prm) && !dry, tv = prm.algo == kTokenVerify;
     constexpr size_t ESZ = (DT == kF32) ? 4 : 2;
@@ -395,10 +433,9 @@ static __device__ __noinline__ void ph_finalize(const Params& prm, const PhaseSc
     const size_t row_bytes = static_cast<size_t>(prm.V) * ESZ;
     const size_t row0 = static_cast<size_t>(b) * (g + 1);
     const float* u = prm.uni + static_cast<size_t>(b) * (g + 2);
-    uint4 sel = __ldcg(&ps.sel[static_cast<size_t>(round) * prm.B + b]);
-    if (dry) sel = make_uint4(1u, 0u, 0u, 0u);
     const double p_g = __ldcg(&ps.pos[row0 + g].p);
     const float u_res = u[g], u_last = u[g + 1], eta_g = u[g - 1];
+    const int X0 = lane < g ? prm.tok[static_cast<size_t>(b) * g + lane] : -1, X1 = lane + 32 < g ? prm.tok[static_cast<size_t>(b) * g + lane + 32] : -1;
     unsigned lo = sel.x, hi = sel.y;
     int last = static_cast<int>(sel.z);
     bool bad = sel.w != 0u;
@@ -477,8 +514,7 @@ static __device__ __noinline__ void ph_finalize(const Params& prm, const PhaseSc
     } else {
         bad = bad || found < 0;           // (an empty residual where the algorithm must sample: a domain error)
         int32_t* ot = prm.out_tokens + row0;
-        const int32_t* X = prm.tok + static_cast<size_t>(b) * g;
-        for (int i = lane; i <= g; i += 32) ot[i] = bad ? -1 : (i < tau ? X[i] : (i == tau ? found : -1));
+        for (int i = lane; i <= g; i += 32) ot[i] = bad ? -1 : (i < tau ? (i < 32 ? X0 : X1) : (i == tau ? found : -1));
         if (lane == 0) prm.out_len[b] = bad ? -1 : tau + 1;
     }
     if (lane == 0) {
@@ -606,7 +642,7 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
     if (helper) {
         if (!PROBS && blockIdx.x < B) drafted(blockIdx.x);
         if (!PROBS) ph_fold(prm, ps, blockIdx.x % B, lane, true);
-        ph_finalize<DT, PROBS, AL>(prm, ps, blockIdx.x % B, 0, lane, true);
+        ph_finalize<DT, PROBS, AL>(prm, ps, blockIdx.x % B, make_uint4(1u, 0u, 0u, 0u), 0, lane, true);
     } else if (PROBS) {
         for (int b = kw; b < B; b += W) ph_fold_probs<DT>(prm, ps, b, lane);
     } else {
@@ -701,7 +737,7 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
         const int before = warp_sum_i(lane < warp ? sh.scan[lane] : 0);
         if (tid < B) {
             s_base[tid] = before + inc - cnt;
-            s_lo[tid] = sel.x; s_hi[tid] = sel.y; s_last[tid] = static_cast<unsigned char>(sel.z);
+            s_lo[tid] = sel.x; s_hi[tid] = sel.y; s_last[tid] = static_cast<unsigned char>(sel.z | sel.w << 1);
             if (tid == B - 1) s_base[B] = before + inc;
         }
         __syncthreads();
@@ -714,7 +750,7 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
             int a = 0, z = B - 1;
             while (a < z) { const int m = (a + z + 1) >> 1; if (s_base[m] <= it) a = m; else z = m - 1; }
             unsigned i_lo = s_lo[a], i_hi = s_hi[a];          // this sequence's candidates after the open one
-            int i_last = s_last[a], i_c = 0, i_b = a, k_i = x0 % units, left = x1 - x0, n_i = 0;
+            int i_last = s_last[a] & 1, i_c = 0, i_b = a, k_i = x0 % units, left = x1 - x0, n_i = 0;
             for (int i = s_base[a]; i <= it; ++i) i_c = ph_pop(i_lo, i_hi, i_last, g);
             auto open = [&]() {
                 const int n = min(left, units - k_i);
@@ -742,7 +778,7 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
                 if (left > 0) {           // the next position, of this sequence or of the next one with any
                     if ((i_lo | i_hi) == 0u) {
                         do ++i_b; while (s_base[i_b + 1] == s_base[i_b]);
-                        i_lo = s_lo[i_b]; i_hi = s_hi[i_b]; i_last = s_last[i_b];
+                        i_lo = s_lo[i_b]; i_hi = s_hi[i_b]; i_last = s_last[i_b] & 1;
                     }
                     i_c = ph_pop(i_lo, i_hi, i_last, g);
                 }
@@ -840,7 +876,7 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
                     unsigned done = 0;
                     if (lane == 0) done = ph_arrive(&ps.cnt2[b], arrived, static_cast<unsigned>((s_base[b + 1] - s_base[b]) * units));
                     arrived = 0;
-                    if (__shfl_sync(0xffffffffu, done, 0)) ph_finalize<DT, PROBS, AL>(prm, ps, b, round, lane, false);
+                    if (__shfl_sync(0xffffffffu, done, 0)) ph_finalize<DT, PROBS, AL>(prm, ps, b, make_uint4(s_lo[b], s_hi[b], s_last[b] & 1u, s_last[b] >> 1), round, lane, false);
                 }
             }
             cp_async_wait<0>();
