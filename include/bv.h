@@ -306,6 +306,25 @@ int bv_draft_chain(const void* draft_table, const int32_t* first_tokens, const f
                    int32_t* out_tokens, float* out_lse, void* stream);
 
 /*
+ * The decoding loop of Algorithm 3 for models whose next-token logits depend on the last token only: target_table and
+ * draft_table [V, V] in `dtype`, DEVICE, row t = the logits after token t.  Each of `iterations` iterations drafts gamma
+ * tokens for every one of B sequences (as bv_draft_chain, from the sequence's last token, with u_draft [iterations,
+ * gamma, B]), verifies the block on the table rows along the drafted path, read where they lie (u_verify [iterations, B,
+ * gamma+2]; algo: 0 Algorithm 2 and 1 Algorithm 1 with the drafting step's normalisers, 2 and 3 the same without), and
+ * appends the emitted tokens to the sequence.  Two launches an iteration, no synchronisation; DEVICE pointers:
+ *   first_tokens [B] int32     the last token of each context
+ *   out_tokens  [B, iterations (gamma+1)] int32: the tokens generated, then -1;  out_lengths [B] int64: how many
+ *   out_tau     [iterations, B] int32 accepted drafts;  out_drafted [iterations, B, gamma] int32
+ *   out_fault   [1] int32: 1 if a sequence reported a data fault (its further tokens mean nothing)
+ *   work        B (2 gamma + 3) int32
+ * Rows must be whole 16-byte vectors on 16-byte aligned bases and B at most 768, else BV_ERR_UNSUPPORTED.
+ */
+int bv_decode_loop(const void* target_table, const void* draft_table, const int32_t* first_tokens,
+                   const float* u_draft, const float* u_verify, int iterations, int B, int gamma, int V,
+                   int dtype, float temperature, int algo, int32_t* out_tokens, int64_t* out_lengths,
+                   int32_t* out_tau, int32_t* out_drafted, int32_t* out_fault, int32_t* work, void* stream);
+
+/*
  * Waits for `stream` and reports whether a device-side wait of any call enqueued on it since the
  * last query gave up: BV_ERR_TIMEOUT (the outputs of those calls are not to be used; the library's
  * state is intact and later calls work) or BV_OK.  Every device-side wait of this library is

@@ -20,7 +20,7 @@ DTYPE_BF16 = 1
 
 # every symbol include/bv.h declares
 EXPORTS = ["bv_verify", "tv_verify", "bv_verify_ex", "tv_verify_ex", "bv_verify_host",
-           "tv_verify_host", "bv_verify_noalloc", "bv_verify_lse", "bv_verify_lse_ex", "tv_verify_lse", "tv_verify_lse_ex", "gbv_verify", "gbv_verify_ex", "bv_verify_probs", "tv_verify_probs", "bv_sample_draft", "bv_draft_chain", "bv_stream_status", "bv_set_option", "bv_release", "bv_last_launch_count", "bv_last_kernel", "bv_last_cuda_error",
+           "tv_verify_host", "bv_verify_noalloc", "bv_verify_lse", "bv_verify_lse_ex", "tv_verify_lse", "tv_verify_lse_ex", "gbv_verify", "gbv_verify_ex", "bv_verify_probs", "tv_verify_probs", "bv_sample_draft", "bv_draft_chain", "bv_decode_loop", "bv_stream_status", "bv_set_option", "bv_release", "bv_last_launch_count", "bv_last_kernel", "bv_last_cuda_error",
            "bv_status_string", "bv_version"]
 
 
@@ -56,6 +56,7 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
         getattr(lib, name).argtypes = base
     lib.bv_sample_draft.argtypes = [vp, vp, ci, ci, ci, cf, vp, vp, vp]
     lib.bv_draft_chain.argtypes = [vp, vp, vp, ci, ci, ci, ci, cf, vp, vp, vp]
+    lib.bv_decode_loop.argtypes = [vp, vp, vp, vp, vp, ci, ci, ci, ci, ci, cf, ci, vp, vp, vp, vp, vp, vp, vp]
     for name in ("bv_verify_probs", "tv_verify_probs"):
         getattr(lib, name).argtypes = [vp, vp, vp, vp, ci, ci, ci, ci, vp, vp, vp, vp, vp, vp]
     for name in ("bv_verify_lse", "tv_verify_lse"):
@@ -338,6 +339,27 @@ def bv_draft_chain(draft_table, first_tokens, uniforms, temperature: float = 1.0
                                   _dtype_code(draft_table), float(temperature), tokens.data_ptr(), lse.data_ptr(),
                                   s.cuda_stream))
     return tokens, lse
+
+
+def bv_decode_loop(target_table, draft_table, first_tokens, u_draft, u_verify, gamma: int, temperature: float, algo: int):
+    """The decoding loop for two last-token table models (see include/bv.h; contiguous CUDA tensors, algo as there): (tokens,
+    lengths, tau, drafted, fault), or None where the library has no kernel for the call."""
+    lib = load_library()
+    N, B, V = u_draft.shape[0], first_tokens.shape[0], target_table.shape[0]
+    dev = target_table.device
+    i32 = lambda *shape: torch.empty(shape, dtype=torch.int32, device=dev)
+    tokens, tau, drafted, fault = i32(B, N * (gamma + 1)), i32(N, B), i32(N, B, gamma), i32(1)
+    lengths = torch.empty((B,), dtype=torch.int64, device=dev)
+    work = i32(B * (2 * gamma + 3))
+    with torch.cuda.device(dev):
+        status = lib.bv_decode_loop(target_table.data_ptr(), draft_table.data_ptr(), first_tokens.data_ptr(), u_draft.data_ptr(),
+                                    u_verify.data_ptr(), N, B, gamma, V, _dtype_code(target_table), float(temperature), algo,
+                                    tokens.data_ptr(), lengths.data_ptr(), tau.data_ptr(), drafted.data_ptr(), fault.data_ptr(),
+                                    work.data_ptr(), torch.cuda.current_stream(dev).cuda_stream)
+    if status == -2:
+        return None
+    _check(status)
+    return tokens, lengths, tau, drafted, fault
 
 
 def bv_verify_lse(target_logits, draft_logits, draft_tokens, uniforms, draft_lse, temperature: float = 1.0,

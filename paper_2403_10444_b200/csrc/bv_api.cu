@@ -210,6 +210,7 @@ bool phase_pays(int algo, const bv::Params& prm, const Options& opt, bool vec, l
     const bool small = bv::small_fits(prm.B, prm.gamma);
     if (prm.probs) return !small || prm.B >= kPhaseProbsB;
     const int which = algo == bv::kTokenVerify ? 0 : (prm.lse_d != nullptr ? 2 : 1);
+    if (prm.first != nullptr) return !small || logit_bytes > kPhaseBytes[which][0];      // (no other kernel takes larger ones)
     const long long least = opt.small_bytes > 0 ? static_cast<long long>(opt.small_bytes) << 20 : kPhaseBytes[which][0];
     return (!small || logit_bytes > least) && (!vec || logit_bytes <= kPhaseBytes[which][1]);
 }
@@ -270,6 +271,7 @@ int run_phase(DeviceState& d, const bv::Params& prm, int dtype, bool vec, cudaSt
 struct Extra {              // what only some entry points pass
     const float* lse_d = nullptr;   // supplied draft log-normalisers (bv_verify_lse)
     int greedy = 0;                 // Algorithm 4 instead of Algorithm 2 (gbv_verify)
+    const int32_t* first = nullptr; // the rows are those of two tables (Params::first)
     int probs = 0;                  // the rows hold probabilities, not logits (bv_verify_probs, tv_verify_probs)
     float* out_p = nullptr; float* out_S = nullptr; float* out_h = nullptr;
     float* out_lse_t = nullptr; float* out_lse_d = nullptr;
@@ -298,6 +300,7 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
     prm.lse_d = ex.lse_d;
     prm.greedy = ex.greedy;
     prm.probs = ex.probs;
+    prm.first = ex.first;
     prm.B = B; prm.gamma = gamma; prm.V = V;
     const double kd = 1.4426950408889634073599246810019 / static_cast<double>(T);
     prm.kd = kd;
@@ -315,8 +318,9 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
     // Both sweeps split over all warps, with the folds between them: between the small-batch kernel's sizes and the flow
     // kernel's, and for rows at any alignment.
     const bool only_vec = prm.lse_d != nullptr || prm.greedy || prm.probs;      // (entry points without an element-wise path)
+    if (prm.first != nullptr && !vec) return BV_ERR_UNSUPPORTED;
     const bool elements = !vec && !only_vec && opt.kernel == 0 && elements_pay(algo, prm, row_bytes, d->sm_count);
-    if ((vec || !only_vec) && !elements && (opt.kernel == 5 || (opt.kernel == 0 && phase_pays(algo, prm, opt, vec, logit_bytes)))) {
+    if ((vec || !only_vec) && !elements && (opt.kernel == 5 || ((opt.kernel == 0 || prm.first != nullptr) && phase_pays(algo, prm, opt, vec, logit_bytes)))) {
         if ((rc = run_phase(*d, prm, dtype, vec, stream)) <= BV_OK) return rc;
     }
 
@@ -326,7 +330,7 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
     // (given probabilities only a few row pairs per sequence are read whatever the size of the rest: there the
     // small-batch kernel wins up to 16 sequences, 17 against 33 us for one, 33 against 38 us for sixteen)
     if ((vec || !only_vec) && !elements && bv::small_fits(B, gamma) &&
-        (opt.kernel == 4 || (opt.kernel == 0 && (prm.probs ? B <= 16 : logit_bytes <= small_limit)))) {
+        (opt.kernel == 4 || ((opt.kernel == 0 || prm.first != nullptr) && (prm.probs ? B <= 16 : logit_bytes <= small_limit)))) {
         int& nc = d->small_ctas[dtype];
         if (nc == 0) {
             nc = bv::small_max_ctas(dtype, d->sm_count);
@@ -353,6 +357,7 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
         }
     }
 
+    if (prm.first != nullptr) return BV_ERR_UNSUPPORTED;      // (the kernels below take whole tensors)
     // (only the kernels above and below serve these entry points)
     if ((prm.lse_d != nullptr || prm.greedy || prm.probs) && !flow_ok) return BV_ERR_UNSUPPORTED;
 
@@ -534,6 +539,14 @@ int note_cuda_error(cudaError_t e) {
     return BV_ERR_CUDA;
 }
 void note_launches(int n) { t_last_launches = n; }
+
+int run_tables(int algo, const void* tgt_table, const void* drf_table, const int32_t* first, const int32_t* tok, const float* uni,
+               const float* lse_d, int B, int gamma, int V, int dtype, float T, int32_t* ot, int32_t* ol, cudaStream_t stream) {
+    Extra ex;
+    ex.lse_d = lse_d;
+    ex.first = first;
+    return run_device(algo, tgt_table, drf_table, tok, uni, B, gamma, V, dtype, T, ot, ol, ex, stream);
+}
 
 int check_verify_args(const void* tgt, const void* drf, const int32_t* tok, const float* uni, int B, int gamma,
                       int V, int dtype, float T, const int32_t* ot, const int32_t* ol) {

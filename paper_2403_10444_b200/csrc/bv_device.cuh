@@ -37,7 +37,21 @@ struct Params {
     unsigned wait_limit;      // flow kernel: polls after which a bounded wait gives up (0: the built-in limits)
     int never_signal;         // flow kernel, test switch: workers never report an item as swept, so the waits run out
     int probs;                // flow kernel: tgt / drf hold probabilities, used as stored, instead of logits
+    const int32_t* first;     // small-batch and phase kernels, or null: tgt / drf are tables [V, V] whose row t holds the logits
+                              // after token t, and a sequence's rows are those of first[b], X_1, .. X_gamma
 };
+
+// The row of the tensors that row r of sequence b is (a token that is none stands for row 0: its sequence is at fault anyway).
+__device__ __forceinline__ size_t path_row(const Params& prm, int b, int r) {
+    const int t = r == 0 ? prm.first[b] : prm.tok[static_cast<size_t>(b) * prm.gamma + r - 1];
+    return t >= 0 && t < prm.V ? static_cast<size_t>(t) : 0;
+}
+__device__ __forceinline__ size_t target_row(const Params& prm, int b, int r) {
+    return prm.first ? path_row(prm, b, r) : static_cast<size_t>(b) * (prm.gamma + 1) + r;
+}
+__device__ __forceinline__ size_t draft_row(const Params& prm, int b, int r) {
+    return prm.first ? path_row(prm, b, r) : static_cast<size_t>(b) * prm.gamma + r;
+}
 
 __device__ __forceinline__ float ex2(float x) {
     float y;

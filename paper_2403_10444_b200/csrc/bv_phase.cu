@@ -293,8 +293,8 @@ __device__ __forceinline__ void ph_fetch_drafted(const Params& prm, const PhaseS
         const int x = prm.tok[static_cast<size_t>(b) * g + c];
         float2 z = make_float2(0.f, -INFINITY);
         if (x >= 0 && x < prm.V) {
-            z.x = static_cast<float>(load_logit<DT>(static_cast<const char*>(prm.tgt) + (static_cast<size_t>(b) * (g + 1) + c) * row_bytes, x));
-            z.y = static_cast<float>(load_logit<DT>(static_cast<const char*>(prm.drf) + (static_cast<size_t>(b) * g + c) * row_bytes, x));
+            z.x = static_cast<float>(load_logit<DT>(static_cast<const char*>(prm.tgt) + target_row(prm, b, c) * row_bytes, x));
+            z.y = static_cast<float>(load_logit<DT>(static_cast<const char*>(prm.drf) + draft_row(prm, b, c) * row_bytes, x));
         }
         __stcg(&ps.drafted[static_cast<size_t>(b) * g + c], z);
     }
@@ -490,8 +490,8 @@ static __device__ __noinline__ void ph_finalize(const Params& prm, const PhaseSc
         if ((ok && total > 0.0 && total < static_cast<double>(INFINITY)) || dry) unit = ph_locate(at, per, lane, mine, static_cast<double>(c < g ? u_res : u_last), rem);
         if (dry) unit = 0;
         if (unit >= 0) {
-            const char* rowP = static_cast<const char*>(prm.tgt) + ri * row_bytes;
-            const char* rowQ = c < g ? static_cast<const char*>(prm.drf) + (static_cast<size_t>(b) * g + c) * row_bytes : nullptr;
+            const char* rowP = static_cast<const char*>(prm.tgt) + target_row(prm, b, c) * row_bytes;
+            const char* rowQ = c < g ? static_cast<const char*>(prm.drf) + draft_row(prm, b, c) * row_bytes : nullptr;
             const int w0 = unit * kPhUnit;
             if (AL) {
                 found = f_rescan<DT, PROBS, 2>(rowP, rowQ, w0, min(w0 + kPhUnit, prm.V / EPV), lane, prm.kf, q.cp, q.nMP, q.nMQ, rem);
@@ -655,7 +655,7 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
             const int b = row_i / rows, j = row_i % rows;
             const bool is_t = j < g;
             PhRun& q = runs[n_i & (kPhQueue - 1)];
-            open_row(is_t ? tgt + (static_cast<size_t>(b) * (g + 1) + j) * row_bytes : drf + (static_cast<size_t>(b) * g + (j - g)) * row_bytes, k_i, n, q);
+            open_row(is_t ? tgt + target_row(prm, b, j) * row_bytes : drf + draft_row(prm, b, j - g) * row_bytes, k_i, n, q);
             if (lane == 0) { q.b = b; q.c = j; }
             if (!AL) { iAlo = is_t ? tgt : drf; iAhi = is_t ? tgt_end : drf_end; }
             __syncwarp();
@@ -758,10 +758,10 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
                 const size_t ri = static_cast<size_t>(i_b) * (g + 1) + i_c;
                 i_single = i_c == g;
                 if (!i_single && lane == 0) cp_async16_s(smem_u32(&q.pos), &ps.pos[ri]);
-                const int h = open_row(tgt + ri * row_bytes, k_i, n, q);
+                const int h = open_row(tgt + target_row(prm, i_b, i_c) * row_bytes, k_i, n, q);
                 if (!i_single) {
                     const char* baseQ; int hQ, nvQ;
-                    row_grid<DT, AL>(drf + (static_cast<size_t>(i_b) * g + i_c) * row_bytes, V, baseQ, hQ, nvQ);
+                    row_grid<DT, AL>(drf + draft_row(prm, i_b, i_c) * row_bytes, V, baseQ, hQ, nvQ);
                     int dq = 0, shift = hQ - h;
                     if (!AL && shift < 0) { shift += EPV; dq = -1; }
                     iq = k_i * kPhUnit + lane + dq;

@@ -213,10 +213,41 @@ sample_rows_kernel(const char* logits, const float* uni, int rows, int V, float 
 // 16 streaming warps, a barrier, the draw by the sampling warp, a barrier.  A token that is not in
 // [0, V) (a first token out of range, or a step whose row could not be sampled) ends the sequence's
 // chain: the remaining tokens are -1 and their normalisers NaN.
+// Before that, where the chain belongs to the decoding loop (loop.out_len), the sequence is extended by what the verification
+// of the iteration before has emitted, and the chain starts from the last of it.
+struct LoopState {
+    const int32_t* out;       // [B, gamma+1], out_len [B]: the last verification's outputs; out_len null: none yet
+    const int32_t* out_len;
+    int32_t* cur;             // [B] last token of every sequence
+    int32_t* seq;             // [B, width] tokens generated so far, lengths [B] of them
+    long long* lengths;
+    int32_t* tau;             // [B] accepted drafts of that iteration
+    int32_t* fault;           // set if a sequence reported a data fault
+    int width;
+};
+__device__ __forceinline__ void extend_sequence(const LoopState& loop, int b, int gamma, int lane) {
+    const int32_t* out = loop.out + static_cast<size_t>(b) * (gamma + 1);
+    const int len = loop.out_len[b], n = len < 1 ? 1 : len;
+    const long long pos = loop.lengths[b];
+    for (int i = lane; i < n; i += 32)
+        if (pos + i < loop.width) loop.seq[static_cast<size_t>(b) * loop.width + pos + i] = out[i];
+    __syncwarp();
+    if (lane == 0) {
+        loop.cur[b] = out[n - 1];
+        loop.lengths[b] = pos + n;
+        loop.tau[b] = len - 1;
+        if (len < 1) atomicExch(loop.fault, 1);
+    }
+}
+__global__ void extend_kernel(const LoopState loop, int B, int gamma) {
+    const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (b < B) extend_sequence(loop, b, gamma, threadIdx.x & 31);
+}
+
 template <int DT>
 __global__ void __launch_bounds__(kSAllThreads, 2)
 draft_chain_kernel(const char* table, const int32_t* first, const float* uni, int B, int gamma, int V, float kf,
-                   int32_t* tokens, float* lse) {
+                   int32_t* tokens, float* lse, const LoopState loop) {
     using R = Raw<DT>;
     constexpr int EPV = R::EPV;
     constexpr size_t ESZ = (DT == kF32) ? 4 : 2;
@@ -226,6 +257,10 @@ draft_chain_kernel(const char* table, const int32_t* first, const float* uni, in
     __shared__ float sM[kSSegs], sS[kSSegs];
     __shared__ int s_next[2];
     for (int b = blockIdx.x; b < B; b += gridDim.x) {
+        if (loop.out_len != nullptr) {
+            if (warp == 0) extend_sequence(loop, b, gamma, lane);
+            __syncthreads();
+        }
         int last = first[b];
         for (int i = 0; i < gamma; ++i) {
             const bool ok = last >= 0 && last < V;
@@ -283,6 +318,24 @@ extern "C" int bv_sample_draft(const void* logits, const float* uniforms, int ro
     return BV_OK;
 }
 
+namespace {
+// One launch of the drafting chain; the arguments have been checked.
+cudaError_t launch_chain(const void* table, const int32_t* first, const float* uni, int B, int gamma, int V, int dtype, float temperature,
+                         int32_t* tokens, float* lse, const bv::LoopState& loop, cudaStream_t st) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int grid = B < 2 * sms ? B : 2 * sms;
+    const float kf = static_cast<float>(1.4426950408889634 / static_cast<double>(temperature));
+    if (dtype == BV_DTYPE_F32)
+        bv::draft_chain_kernel<bv::kF32><<<grid, bv::kSAllThreads, 0, st>>>(static_cast<const char*>(table), first, uni, B, gamma, V, kf, tokens, lse, loop);
+    else
+        bv::draft_chain_kernel<bv::kBF16><<<grid, bv::kSAllThreads, 0, st>>>(static_cast<const char*>(table), first, uni, B, gamma, V, kf, tokens, lse, loop);
+    return cudaGetLastError();
+}
+}  // namespace
+
 extern "C" int bv_draft_chain(const void* draft_table, const int32_t* first_tokens, const float* uniforms, int B, int gamma,
                               int V, int dtype, float temperature, int32_t* out_tokens, float* out_lse, void* stream) {
     if (!draft_table || !first_tokens || !uniforms || !out_tokens) return BV_ERR_INVALID_ARG;
@@ -293,19 +346,54 @@ extern "C" int bv_draft_chain(const void* draft_table, const int32_t* first_toke
     if (row_bytes % 16 != 0 || !aligned16(draft_table)) return BV_ERR_UNSUPPORTED;
     bv::note_launches(0);
     if (B == 0) return BV_OK;
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return bv::note_cuda_error(e);
-    const int grid = B < 2 * sms ? B : 2 * sms;
-    const float kf = static_cast<float>(1.4426950408889634 / static_cast<double>(temperature));
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (dtype == BV_DTYPE_F32)
-        bv::draft_chain_kernel<bv::kF32><<<grid, bv::kSAllThreads, 0, st>>>(static_cast<const char*>(draft_table), first_tokens, uniforms, B, gamma, V, kf, out_tokens, out_lse);
-    else
-        bv::draft_chain_kernel<bv::kBF16><<<grid, bv::kSAllThreads, 0, st>>>(static_cast<const char*>(draft_table), first_tokens, uniforms, B, gamma, V, kf, out_tokens, out_lse);
-    e = cudaGetLastError();
+    const cudaError_t e = launch_chain(draft_table, first_tokens, uniforms, B, gamma, V, dtype, temperature, out_tokens, out_lse,
+                                       bv::LoopState{}, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return bv::note_cuda_error(e);
     bv::note_launches(1);
+    return BV_OK;
+}
+
+extern "C" int bv_decode_loop(const void* target_table, const void* draft_table, const int32_t* first_tokens, const float* u_draft,
+                              const float* u_verify, int iterations, int B, int gamma, int V, int dtype, float temperature, int algo,
+                              int32_t* out_tokens, int64_t* out_lengths, int32_t* out_tau, int32_t* out_drafted, int32_t* out_fault,
+                              int32_t* work, void* stream) {
+    if (!target_table || !draft_table || !first_tokens || !u_draft || !u_verify || !out_tokens || !out_lengths || !out_tau ||
+        !out_drafted || !out_fault || !work) return BV_ERR_INVALID_ARG;
+    if (iterations < 1 || B < 1 || gamma < 1 || V < 1 || algo < 0 || algo > 3) return BV_ERR_INVALID_ARG;
+    if (!(temperature > 0.f) || !std::isfinite(temperature)) return BV_ERR_INVALID_ARG;
+    if (dtype != BV_DTYPE_F32 && dtype != BV_DTYPE_BF16) return BV_ERR_INVALID_ARG;
+    const size_t row_bytes = static_cast<size_t>(V) * (dtype == BV_DTYPE_F32 ? 4 : 2);
+    if (row_bytes % 16 != 0 || !aligned16(draft_table) || !aligned16(target_table) || gamma > BV_MAX_GAMMA) return BV_ERR_UNSUPPORTED;
+    bv::note_launches(0);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const size_t b = static_cast<size_t>(B), width = static_cast<size_t>(iterations) * (gamma + 1);
+    if (width > 0x7fffffffu) return BV_ERR_UNSUPPORTED;
+    // work: last tokens, the last verification's outputs, the draft rows' normalisers
+    int32_t* cur = work;
+    int32_t* out = cur + b;
+    int32_t* out_len = out + b * (gamma + 1);
+    float* lse = reinterpret_cast<float*>(out_len + b);
+    cudaError_t e;
+    if ((e = cudaMemcpyAsync(cur, first_tokens, b * 4, cudaMemcpyDeviceToDevice, st)) != cudaSuccess ||
+        (e = cudaMemsetAsync(out_tokens, 0xff, b * width * 4, st)) != cudaSuccess ||      // (-1)
+        (e = cudaMemsetAsync(out_lengths, 0, b * 8, st)) != cudaSuccess ||
+        (e = cudaMemsetAsync(out_fault, 0, 4, st)) != cudaSuccess)
+        return bv::note_cuda_error(e);
+    bv::LoopState loop{out, nullptr, cur, out_tokens, reinterpret_cast<long long*>(out_lengths), nullptr, out_fault, static_cast<int>(width)};
+    int launches = 0;
+    for (int n = 0; n < iterations; ++n) {
+        int32_t* drafted = out_drafted + n * b * gamma;
+        if ((e = launch_chain(draft_table, cur, u_draft + n * b * gamma, B, gamma, V, dtype, temperature, drafted, lse, loop, st)) != cudaSuccess)
+            return bv::note_cuda_error(e);
+        const int rc = bv::run_tables(algo & 1 ? bv::kTokenVerify : bv::kBlockVerify, target_table, draft_table, cur, drafted, u_verify + n * b * (gamma + 2),
+                                      algo < 2 ? lse : nullptr, B, gamma, V, dtype, temperature, out, out_len, st);
+        if (rc != BV_OK) return rc;
+        loop.out_len = out_len;
+        loop.tau = out_tau + n * b;
+        launches += 2;
+    }
+    bv::extend_kernel<<<(B + 7) / 8, 256, 0, st>>>(loop, B, gamma);
+    if ((e = cudaGetLastError()) != cudaSuccess) return bv::note_cuda_error(e);
+    bv::note_launches(launches + 1);
     return BV_OK;
 }

@@ -76,8 +76,8 @@ __device__ __forceinline__ void small_seg_range(int units, int nseg, int seg, in
 // row index -> pointer: rows 0 .. gamma of a sequence are its target rows, gamma+1 .. 2 gamma its draft rows
 __device__ __forceinline__ const char* small_row(const Params& prm, size_t row_bytes, int b, int j) {
     const int g = prm.gamma;
-    return j <= g ? static_cast<const char*>(prm.tgt) + (static_cast<size_t>(b) * (g + 1) + j) * row_bytes
-                  : static_cast<const char*>(prm.drf) + (static_cast<size_t>(b) * g + (j - g - 1)) * row_bytes;
+    return j <= g ? static_cast<const char*>(prm.tgt) + target_row(prm, b, j) * row_bytes
+                  : static_cast<const char*>(prm.drf) + draft_row(prm, b, j - g - 1) * row_bytes;
 }
 
 // vector i of the nv that a row's bytes lie in, from `base` on; [lo, hi): the tensor

@@ -46,6 +46,7 @@ def run(target_table: torch.Tensor, draft_table: torch.Tensor, first_tokens: tor
     (the iteration number lives in a device counter), so with ``graph=True`` one iteration is
     captured in a CUDA graph and replayed: the launches of an iteration then cost one graph launch
     instead of one driver call each.  Data faults are looked for once, after the last iteration.
+    By default the loop runs natively (``bv_decode_loop``), two launches per iteration.
     ``chain``: the gamma drafted tokens of an iteration come from one launch of ``bv_draft_chain``
     (default) instead of gamma calls of ``bv_sample_draft`` with their look-ups and copies.
     """
@@ -59,6 +60,15 @@ def run(target_table: torch.Tensor, draft_table: torch.Tensor, first_tokens: tor
         raise ValueError("u_draft must be [N, gamma, B] and u_verify [N, B, gamma+2]")
     dev = target_table.device
     width = N * (gamma + 1)
+    if chain and not graph and _native(target_table, draft_table, first_tokens, u_draft, u_verify, gamma):
+        # (two launches an iteration, the tables' rows read where they lie)
+        res = bv.bv_decode_loop(target_table, draft_table, first_tokens.to(torch.int32).contiguous(), u_draft.contiguous(),
+                                u_verify.contiguous(), gamma, temperature, ("block_lse", "token_lse", "block", "token").index(algo))
+        if res is not None:
+            tokens, lengths, tau, drafted, fault = res
+            if int(fault.item()) != 0:
+                raise RuntimeError("a sequence reported a data fault (out_len = -1)")
+            return dict(tokens=tokens, lengths=lengths, tau=tau, drafted=drafted)
     # state of the loop, updated in place (column `width` of seq takes what is not kept)
     seq = torch.full((B, width + 1), -1, dtype=torch.int32, device=dev)
     pos = torch.zeros((B,), dtype=torch.int64, device=dev)
@@ -135,6 +145,17 @@ def run(target_table: torch.Tensor, draft_table: torch.Tensor, first_tokens: tor
     if int(fault.item()) != 0:
         raise RuntimeError("a sequence reported a data fault (out_len = -1)")
     return dict(tokens=seq[:, :width].contiguous(), lengths=pos, tau=taus, drafted=drafted)
+
+
+def _native(target_table, draft_table, first_tokens, u_draft, u_verify, gamma) -> bool:
+    """Does the library's own loop take these tensors?"""
+    dev = target_table.device
+    return (u_draft.shape[0] > 0 and 0 < first_tokens.shape[0] <= 768 and 1 <= gamma <= 64 and dev.type == "cuda"
+            and target_table.dtype == draft_table.dtype and target_table.dtype in (torch.float32, torch.bfloat16)
+            and target_table.is_contiguous() and draft_table.is_contiguous()
+            and u_draft.dtype == torch.float32 and u_verify.dtype == torch.float32
+            and first_tokens.dtype in (torch.int32, torch.int64) and first_tokens.dim() == 1
+            and all(t.device == dev for t in (draft_table, first_tokens, u_draft, u_verify)))
 
 
 def block_efficiency(result) -> float:

@@ -213,3 +213,20 @@ def test_loop_with_and_without_the_chain_kernel_generates_the_same_tokens(algo):
     b = specdec.run(tt, dt, first, ud, uv, gamma, 0.9, algo, chain=False)
     for k in ("tokens", "lengths", "tau", "drafted"):
         assert torch.equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("V,B", [(512, 5), (4096, 40)])      # the small-batch kernel; the phase kernel
+def test_a_fault_in_the_loop_is_an_exception_and_harms_nothing(V, B):
+    tt, dt = wl.markov_models(V, "bf16", 3, 2.0, 0.7, 1.1, "cuda")
+    ud, uv = wl.loop_uniforms(3, B, 3, 4, "cuda")
+    first = torch.full((B,), 2, dtype=torch.int32, device="cuda")
+    good = specdec.run(tt, dt, first, ud, uv, 3)
+    bad = dt.clone()
+    bad[2, 7] = float("nan")                # the row every chain starts from: no token can be drawn
+    for algo in specdec.ALGOS:
+        with pytest.raises(RuntimeError):
+            specdec.run(tt, bad, first, ud, uv, 3, algo=algo)
+    with pytest.raises(RuntimeError):
+        specdec.run(tt, dt, torch.full_like(first, V), ud, uv, 3)
+    again = specdec.run(tt, dt, first, ud, uv, 3)
+    assert all(torch.equal(good[k], again[k]) for k in good)
