@@ -115,6 +115,28 @@ def _check(status: int) -> None:
         raise BVError(status, text)
 
 
+class _Nothing:
+    def __enter__(self):
+        return None
+
+    def __exit__(self, *exc):
+        return False
+
+
+_NOTHING = _Nothing()
+
+
+def _on(dev: torch.device):
+    """The context in which ``dev`` is the current device (nothing to enter if it is already: entering costs 1.4 us of a
+    call that takes 9)."""
+    return _NOTHING if dev.index == torch.cuda.current_device() else torch.cuda.device(dev)
+
+
+def _raw_stream(dev: torch.device, stream) -> int:
+    """The cudaStream_t of ``stream``, or of torch's current stream on ``dev`` (without the Stream object around it: 2 us)."""
+    return stream.cuda_stream if stream is not None else torch._C._cuda_getCurrentRawStream(dev.index)
+
+
 def _dtype_code(t: torch.Tensor) -> int:
     if t.dtype == torch.float32:
         return DTYPE_F32
@@ -128,19 +150,18 @@ def _shapes(target, draft, tokens, uniforms, want_cuda: bool):
         raise ValueError("target_logits must be [B, gamma+1, V] and draft_logits [B, gamma, V]")
     B, g1, V = target.shape
     gamma = g1 - 1
-    if tuple(draft.shape) != (B, gamma, V):
+    if draft.shape != (B, gamma, V):
         raise ValueError("draft_logits must be [B, gamma, V]")
-    if tuple(tokens.shape) != (B, gamma) or tokens.dtype != torch.int32:
+    if tokens.shape != (B, gamma) or tokens.dtype != torch.int32:
         raise ValueError("draft_tokens must be int32 [B, gamma]")
-    if tuple(uniforms.shape) != (B, gamma + 2) or uniforms.dtype != torch.float32:
+    if uniforms.shape != (B, gamma + 2) or uniforms.dtype != torch.float32:
         raise ValueError("uniforms must be float32 [B, gamma+2]")
     if target.dtype != draft.dtype:
         raise TypeError("target and draft logits must share a dtype")
-    for t in (target, draft, tokens, uniforms):
-        if not t.is_contiguous():
-            raise ValueError("all tensors must be contiguous")
-        if t.is_cuda != want_cuda:
-            raise ValueError("expected %s tensors" % ("CUDA" if want_cuda else "host"))
+    if not (target.is_contiguous() and draft.is_contiguous() and tokens.is_contiguous() and uniforms.is_contiguous()):
+        raise ValueError("all tensors must be contiguous")
+    if not (target.is_cuda == draft.is_cuda == tokens.is_cuda == uniforms.is_cuda == want_cuda):
+        raise ValueError("expected %s tensors" % ("CUDA" if want_cuda else "host"))
     return B, gamma, V
 
 
@@ -149,10 +170,9 @@ def _device_call(name: str, target, draft, tokens, uniforms, temperature, diagno
     lib = load_library()
     B, gamma, V = _shapes(target, draft, tokens, uniforms, True)
     dev = target.device
-    out_tokens = torch.empty((B, gamma + 1), dtype=torch.int32, device=dev)
-    out_len = torch.empty((B,), dtype=torch.int32, device=dev)
-    with torch.cuda.device(dev):
-        s = stream if stream is not None else torch.cuda.current_stream(dev)
+    out_tokens, out_len = target.new_empty((B, gamma + 1), dtype=torch.int32), target.new_empty((B,), dtype=torch.int32)
+    with _on(dev):
+        s = _raw_stream(dev, stream)
         args = [target.data_ptr(), draft.data_ptr(), tokens.data_ptr(), uniforms.data_ptr(),
                 B, gamma, V, _dtype_code(target), float(temperature),
                 out_tokens.data_ptr(), out_len.data_ptr()]
@@ -161,7 +181,7 @@ def _device_call(name: str, target, draft, tokens, uniforms, temperature, diagno
             diag = dict(p=f(B, gamma + 1), S=f(B, gamma), h=f(B, gamma + 1),
                         lse_t=f(B, gamma + 1), lse_d=f(B, gamma))
             args += [diag[k].data_ptr() for k in ("p", "S", "h", "lse_t", "lse_d")]
-        _check(getattr(lib, name)(*args, s.cuda_stream))
+        _check(getattr(lib, name)(*args, s))
     if diagnostics:
         return out_tokens, out_len, diag
     return out_tokens, out_len
@@ -215,18 +235,17 @@ def _probs_call(name: str, target_probs, draft_probs, tokens, uniforms, diagnost
     lib = load_library()
     B, gamma, V = _shapes(target_probs, draft_probs, tokens, uniforms, True)
     dev = target_probs.device
-    out_tokens = torch.empty((B, gamma + 1), dtype=torch.int32, device=dev)
-    out_len = torch.empty((B,), dtype=torch.int32, device=dev)
+    out_tokens, out_len = target_probs.new_empty((B, gamma + 1), dtype=torch.int32), target_probs.new_empty((B,), dtype=torch.int32)
     diag, ptrs = None, [None, None, None]
     if diagnostics:
         f = lambda *shape: torch.empty(shape, dtype=torch.float32, device=dev)
         diag = dict(p=f(B, gamma + 1), S=f(B, gamma), h=f(B, gamma + 1))
         ptrs = [diag[k].data_ptr() for k in ("p", "S", "h")]
-    with torch.cuda.device(dev):
-        s = stream if stream is not None else torch.cuda.current_stream(dev)
+    with _on(dev):
+        s = _raw_stream(dev, stream)
         _check(getattr(lib, name)(target_probs.data_ptr(), draft_probs.data_ptr(), tokens.data_ptr(),
                                   uniforms.data_ptr(), B, gamma, V, _dtype_code(target_probs),
-                                  out_tokens.data_ptr(), out_len.data_ptr(), *ptrs, s.cuda_stream))
+                                  out_tokens.data_ptr(), out_len.data_ptr(), *ptrs, s))
     return (out_tokens, out_len, diag) if diagnostics else (out_tokens, out_len)
 
 
@@ -259,12 +278,12 @@ def bv_verify_noalloc(target_logits, draft_logits, draft_tokens, uniforms, out_t
     if tuple(out_len.shape) != (B,) or out_len.dtype != torch.int32 or not out_len.is_cuda:
         raise ValueError("out_len must be a CUDA int32 tensor [B]")
     dev = target_logits.device
-    with torch.cuda.device(dev):
-        s = stream if stream is not None else torch.cuda.current_stream(dev)
+    with _on(dev):
+        s = _raw_stream(dev, stream)
         _check(lib.bv_verify_noalloc(target_logits.data_ptr(), draft_logits.data_ptr(),
                                      draft_tokens.data_ptr(), uniforms.data_ptr(), B, gamma, V,
                                      _dtype_code(target_logits), float(temperature),
-                                     out_tokens.data_ptr(), out_len.data_ptr(), s.cuda_stream))
+                                     out_tokens.data_ptr(), out_len.data_ptr(), s))
 
 
 def _host_call(name: str, target, draft, tokens, uniforms, temperature, out_tokens, out_len):
@@ -307,11 +326,11 @@ def bv_sample_draft(logits, uniforms, temperature: float = 1.0, want_lse: bool =
     lib = load_library()
     tokens = torch.empty((rows,), dtype=torch.int32, device=logits.device)
     lse = torch.empty((rows,), dtype=torch.float32, device=logits.device) if want_lse else None
-    st = stream if stream is not None else torch.cuda.current_stream(logits.device)
-    with torch.cuda.device(logits.device):
+    dev = logits.device
+    with _on(dev):
         _check(lib.bv_sample_draft(logits.data_ptr(), uniforms.data_ptr(), rows, V, _dtype_code(logits),
                                    float(temperature), tokens.data_ptr(), lse.data_ptr() if want_lse else None,
-                                   st.cuda_stream))
+                                   _raw_stream(dev, stream)))
     return tokens, lse
 
 
@@ -333,11 +352,11 @@ def bv_draft_chain(draft_table, first_tokens, uniforms, temperature: float = 1.0
     dev = draft_table.device
     tokens = torch.empty((B, gamma), dtype=torch.int32, device=dev)
     lse = torch.empty((B, gamma), dtype=torch.float32, device=dev)
-    with torch.cuda.device(dev):
-        s = stream if stream is not None else torch.cuda.current_stream(dev)
+    with _on(dev):
+        s = _raw_stream(dev, stream)
         _check(lib.bv_draft_chain(draft_table.data_ptr(), first_tokens.data_ptr(), uniforms.data_ptr(), B, gamma, V,
                                   _dtype_code(draft_table), float(temperature), tokens.data_ptr(), lse.data_ptr(),
-                                  s.cuda_stream))
+                                  s))
     return tokens, lse
 
 
@@ -351,11 +370,11 @@ def bv_decode_loop(target_table, draft_table, first_tokens, u_draft, u_verify, g
     tokens, tau, drafted, fault = i32(B, N * (gamma + 1)), i32(N, B), i32(N, B, gamma), i32(1)
     lengths = torch.empty((B,), dtype=torch.int64, device=dev)
     work = i32(B * (2 * gamma + 3))
-    with torch.cuda.device(dev):
+    with _on(dev):
         status = lib.bv_decode_loop(target_table.data_ptr(), draft_table.data_ptr(), first_tokens.data_ptr(), u_draft.data_ptr(),
                                     u_verify.data_ptr(), N, B, gamma, V, _dtype_code(target_table), float(temperature), algo,
                                     tokens.data_ptr(), lengths.data_ptr(), tau.data_ptr(), drafted.data_ptr(), fault.data_ptr(),
-                                    work.data_ptr(), torch.cuda.current_stream(dev).cuda_stream)
+                                    work.data_ptr(), _raw_stream(dev, None))
     if status == -2:
         return None
     _check(status)
@@ -385,10 +404,9 @@ def _lse_call(name, target_logits, draft_logits, draft_tokens, uniforms, draft_l
             or not draft_lse.is_contiguous()):
         raise ValueError("draft_lse must be a contiguous float32 CUDA tensor of [B, gamma]")
     dev = target_logits.device
-    out_tokens = torch.empty((B, gamma + 1), dtype=torch.int32, device=dev)
-    out_len = torch.empty((B,), dtype=torch.int32, device=dev)
-    with torch.cuda.device(dev):
-        s = stream if stream is not None else torch.cuda.current_stream(dev)
+    out_tokens, out_len = target_logits.new_empty((B, gamma + 1), dtype=torch.int32), target_logits.new_empty((B,), dtype=torch.int32)
+    with _on(dev):
+        s = _raw_stream(dev, stream)
         args = [target_logits.data_ptr(), draft_logits.data_ptr(), draft_tokens.data_ptr(), uniforms.data_ptr(),
                 draft_lse.data_ptr(), B, gamma, V, _dtype_code(target_logits), float(temperature),
                 out_tokens.data_ptr(), out_len.data_ptr()]
@@ -396,7 +414,7 @@ def _lse_call(name, target_logits, draft_logits, draft_tokens, uniforms, draft_l
             f = lambda *shape: torch.empty(shape, dtype=torch.float32, device=dev)
             diag = dict(p=f(B, gamma + 1), S=f(B, gamma), h=f(B, gamma + 1), lse_t=f(B, gamma + 1), lse_d=f(B, gamma))
             args += [diag[k].data_ptr() for k in ("p", "S", "h", "lse_t", "lse_d")]
-            _check(getattr(lib, name + "_ex")(*args, s.cuda_stream))
+            _check(getattr(lib, name + "_ex")(*args, s))
             return out_tokens, out_len, diag
-        _check(getattr(lib, name)(*args, s.cuda_stream))
+        _check(getattr(lib, name)(*args, s))
     return out_tokens, out_len
