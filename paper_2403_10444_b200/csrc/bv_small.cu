@@ -102,7 +102,7 @@ __device__ __forceinline__ uint4 small_shift(const uint4& a, const uint4& b, int
 // AL: rows of whole 16-byte vectors on 16-byte aligned bases.  Otherwise a row is read as the vectors its bytes lie in
 // (row_grid), and the draft row of a pair is put on the target row's grid from two neighbouring vectors.
 template <int DT, bool PROBS, bool AL>
-__global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const Params prm, const SmallScratch sc) {
+__global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __grid_constant__ Params prm, const __grid_constant__ SmallScratch sc) {
     using R = Raw<DT>;
     constexpr int EPV = R::EPV;
     constexpr int kPairs = AL ? kSmPairsInFlight : 3;
@@ -198,16 +198,19 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const Pa
                 continue;
             }
             float M = kNoRef;
-            double z[kSmallMaxChunks];
-            float m[kSmallMaxChunks];
-#pragma unroll 4
-            for (int c = 0; c < nch; ++c) {
-                const double2 p = __ldcg(&sc.part[static_cast<size_t>(rid) * nch + c]);
-                m[c] = static_cast<float>(p.x); z[c] = p.y;
-                M = fmaxf(M, m[c]);
-            }
             double Z = 0.0;
-            for (int c = 0; c < nch; ++c) Z += z[c] * static_cast<double>(ref_scale(m[c], M));
+            for (int c0 = 0; c0 < nch; c0 += 8) {             // (eight loads in flight, nothing in local memory)
+                double2 p[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) p[j] = c0 + j < nch ? __ldcg(&sc.part[static_cast<size_t>(rid) * nch + c0 + j]) : make_double2(kNoRef, 0.0);
+                float mm = M;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) mm = fmaxf(mm, static_cast<float>(p[j].x));
+                Z *= static_cast<double>(ref_scale(M, mm));
+#pragma unroll
+                for (int j = 0; j < 8; ++j) Z += p[j].y * static_cast<double>(ref_scale(static_cast<float>(p[j].x), mm));
+                M = mm;
+            }
             sh.rowM[rid] = M;
             sh.rowZ[rid] = Z;
         }
@@ -221,6 +224,7 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const Pa
             float eta[2] = {0.f, 0.f};
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
+                if (h == 1 && g <= 32) break;
                 const int c = lane + 32 * h;
                 if (c < g) {
                     const float MP = sh.rowM[b * rpb + c], MQ = sh.rowM[b * rpb + g + 1 + c];
@@ -276,9 +280,9 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const Pa
             } else {
                 double pc = 1.0, mine[2] = {1.0, 1.0};
                 for (int c = 0; c < g; ++c) {
-                    if ((c & 31) == lane) mine[c >> 5] = pc;
-                    const double r = shfl_d(c < 32 ? rat[0] : rat[1], c & 31);
-                    const double next = pc * r;
+                    if (c == lane) mine[0] = pc;
+                    if (c == lane + 32) mine[1] = pc;
+                    const double next = pc * shfl_d(c < 32 ? rat[0] : rat[1], c & 31);
                     pc = prm.greedy ? next : fmin(next, 1.0);
                 }
                 const double p_g = pc;
@@ -377,6 +381,16 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const Pa
     // (arrivals are counted up through the launch: the second barrier of a launch on logits, the only one otherwise)
     if (alive) alive = small_grid_barrier(sc.barrier, (PROBS ? 1u : 2u) * gridDim.x, prm.status, limit,
                                           PROBS && prm.never_signal && blockIdx.x == 0);
+
+    // No CTA looks at the barrier word any more once all have come by here, whatever became of the waits: the last one puts
+    // both words back to zero.  (A warp that is not on the way to the result does it: the fence, the atomic and its answer
+    // at the end of the kernel were 1 us of the 20 that a single sequence takes.)
+    if (tid == kSmThreads - 1) {
+        if (atomicAdd(sc.barrier + 16, 1u) == gridDim.x - 1) {
+            atomicExch(sc.barrier, 0u);
+            atomicExch(sc.barrier + 16, 0u);
+        }
+    }
 
     // ---------------- phase 3: one CTA per sequence ----------------
     for (int b = blockIdx.x; alive && b < B; b += gridDim.x) {
@@ -491,16 +505,6 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const Pa
             }
         }
         __syncthreads();
-    }
-
-    // the barrier word is zero again when the last CTA leaves (whatever became of the waits)
-    __syncthreads();
-    if (tid == 0) {
-        __threadfence();
-        if (atomicAdd(sc.barrier + 16, 1u) == gridDim.x - 1) {
-            atomicExch(sc.barrier, 0u);
-            atomicExch(sc.barrier + 16, 0u);
-        }
     }
 }
 
