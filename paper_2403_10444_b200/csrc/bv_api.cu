@@ -29,7 +29,15 @@ constexpr long long kSmallBytes[2] = {160LL << 20, 90LL << 20};   // [algo]
 //   Algorithm 1, noise 0.7, B = 16 / 33 / 64 / 128: 47 / 57 / 82 / 132 us against 46 / 77 / 90 / 115 (it reads all rows, the
 //   flow kernel the ones the tests need)
 //   probabilities, noise 0.7, B = 8 / 16 / 33 / 128 / 256: 26 / 29 / 31 / 49 / 72 us against 21 / 31 / 39 / 65 / 120
-constexpr long long kPhaseBytes[3][2] = {{64LL << 20, 320LL << 20}, {64LL << 20, 1000LL << 20}, {48LL << 20, 1400LL << 20}};
+// The upper ends are lower for 32-bit logits, of which the flow kernel streams the more (half the arithmetic a byte; V = 256000,
+// gamma = 2, 312 MB: 103 us against 100; Algorithm 1, 296 MB: 81 against 73), and the one of Algorithm 1 is where a draft that
+// is hardly accepted leaves the flow kernel an eighth of the rows to read (23 sequences, noise 3, 238 MB: 53 us against 46).
+// On probabilities Algorithm 1 sweeps one row pair a sequence: 33 MB of them 1.2 times faster, 129 MB 51 us against 44;
+// Algorithm 2 at 131 MB 72 us against 120.
+constexpr long long kPhaseBytes[3][2] = {{72LL << 20, 180LL << 20}, {64LL << 20, 860LL << 20}, {48LL << 20, 1400LL << 20}};
+constexpr long long kPhaseBytesF32[3] = {120LL << 20, 280LL << 20, 280LL << 20};
+constexpr long long kPhaseProbsPairs[2] = {36LL << 20, 140LL << 20};      // [algo] bytes of one row pair of every sequence
+constexpr long long kPhaseBytesAll = 360LL << 20;
 constexpr int kPhaseProbsB = 12;
 constexpr size_t kSlotHead = 16384;   // leading bytes of a stream's workspace: status word, barrier words, the phase kernel's counters
 constexpr size_t kSlotPhase = 256;    // ... the last of these from here on
@@ -206,13 +214,17 @@ bool elements_pay(int algo, const bv::Params& prm, size_t row_bytes, int sm_coun
 }
 
 // Where the phase kernel is the default.  (Rows that are not whole 16-byte vectors: wherever the small-batch kernel is not.)
-bool phase_pays(int algo, const bv::Params& prm, const Options& opt, bool vec, long long logit_bytes) {
+bool phase_pays(int algo, const bv::Params& prm, const Options& opt, int dtype, bool vec, long long logit_bytes) {
     const bool small = bv::small_fits(prm.B, prm.gamma);
-    if (prm.probs) return !small || prm.B >= kPhaseProbsB;
+    if (prm.probs)
+        return (!small || prm.B >= kPhaseProbsB) &&
+               logit_bytes / (2 * prm.gamma + 1) * 2 <= kPhaseProbsPairs[algo == bv::kBlockVerify ? 1 : 0];
     const int which = algo == bv::kTokenVerify ? 0 : (prm.lse_d != nullptr ? 2 : 1);
     if (prm.first != nullptr) return !small || logit_bytes > kPhaseBytes[which][0];      // (no other kernel takes larger ones)
+    // (with every position swept the flow kernel's two sweeps overlap the more: 403 MB, gamma = 4, 177 us against 167)
+    if (vec && (prm.out_p || prm.out_S || prm.out_h || prm.out_lse_t || prm.out_lse_d) && logit_bytes > kPhaseBytesAll) return false;
     const long long least = opt.small_bytes > 0 ? static_cast<long long>(opt.small_bytes) << 20 : kPhaseBytes[which][0];
-    return (!small || logit_bytes > least) && (!vec || logit_bytes <= kPhaseBytes[which][1]);
+    return (!small || logit_bytes > least) && (!vec || logit_bytes <= (dtype == BV_DTYPE_F32 ? kPhaseBytesF32[which] : kPhaseBytes[which][1]));
 }
 
 // The phase kernel for the call in `prm`: BV_OK, an error, or 1 if it does not take the call.  Rows at any alignment have no
@@ -320,7 +332,7 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
     const bool only_vec = prm.lse_d != nullptr || prm.greedy || prm.probs;      // (entry points without an element-wise path)
     if (prm.first != nullptr && !vec) return BV_ERR_UNSUPPORTED;
     const bool elements = !vec && !only_vec && opt.kernel == 0 && elements_pay(algo, prm, row_bytes, d->sm_count);
-    if ((vec || !only_vec) && !elements && (opt.kernel == 5 || ((opt.kernel == 0 || prm.first != nullptr) && phase_pays(algo, prm, opt, vec, logit_bytes)))) {
+    if ((vec || !only_vec) && !elements && (opt.kernel == 5 || ((opt.kernel == 0 || prm.first != nullptr) && phase_pays(algo, prm, opt, dtype, vec, logit_bytes)))) {
         if ((rc = run_phase(*d, prm, dtype, vec, stream)) <= BV_OK) return rc;
     }
 
