@@ -245,7 +245,14 @@ int run_phase(DeviceState& d, const bv::Params& prm, int dtype, bool vec, cudaSt
     }
     if (!plan.fits) return 1;
     bv::PhaseScratch ps;
-    const size_t need = bv::phase_scratch(nullptr, nullptr, part, g, plan, &ps);
+    size_t need = bv::phase_scratch(nullptr, nullptr, part, g, plan, &ps);
+    if (prm.B % part != 0) {
+        // (the last part is planned for its own size: fewer sequences, but the warps' parts of the list are shorter too, so a
+        // row may lie in more pieces and the whole take more)
+        const int rest = prm.B % part;
+        const size_t n = bv::phase_scratch(nullptr, nullptr, rest, g, bv::phase_plan(prm.V, dtype, vec, rest, g, prm.lse_d != nullptr, nc), &ps);
+        if (n > need) need = n;
+    }
     if (!slot_can_hold(d, stream, need)) return 1;
     StreamSlot* slot = nullptr;
     const int rc = stream_slot(d, stream, need, &slot);

@@ -1,0 +1,181 @@
+// The dispatch layer (bv_api.cu) on a runtime that only keeps books, for tests without a GPU: every allocation is host
+// memory of exactly the size asked for, launches check the memory they are handed and leave in it what the kernels leave
+// (scratch: anything; counters: zero), and a captured stream records its work for replays.  Plans come from the library itself.
+#include <cuda_runtime.h>
+
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <functional>
+#include <map>
+#include <string>
+#include <vector>
+
+#include "bv_launch.h"
+
+namespace {
+
+struct Block { size_t bytes; bool live; };
+std::map<char*, Block> g_blocks;
+std::vector<std::vector<std::function<void()>>> g_graphs;
+bool g_capturing = false;
+int g_refuse_cooperative = 0;
+std::string g_errors;
+
+void complain(const std::string& what) { g_errors += what + "\n"; }
+cudaError_t give(void** p, size_t bytes) {
+    char* c = static_cast<char*>(std::malloc(bytes));
+    std::memset(c, 0xcd, bytes);
+    g_blocks[c] = Block{bytes, true};
+    *p = c;
+    return cudaSuccess;
+}
+cudaError_t take_back(void* p) {
+    auto it = g_blocks.find(static_cast<char*>(p));
+    if (it == g_blocks.end() || !it->second.live) complain("free of what is not allocated");
+    else it->second.live = false;               // (kept: what still points into it is found out, not crashed on)
+    return cudaSuccess;
+}
+bool inside(const char* what, const void* p, size_t bytes) {
+    const char* c = static_cast<const char*>(p);
+    auto it = g_blocks.upper_bound(const_cast<char*>(c));
+    if (it == g_blocks.begin()) { complain(std::string(what) + ": no allocation"); return false; }
+    --it;
+    if (c + bytes > it->first + it->second.bytes) { complain(std::string(what) + ": outside its allocation"); return false; }
+    if (!it->second.live) { complain(std::string(what) + ": memory was given back"); return false; }
+    return true;
+}
+void scratch(const char* what, void* p, size_t bytes) { if (bytes && inside(what, p, bytes)) std::memset(p, 0xab, bytes); }
+void zeros(const char* what, const void* p, size_t bytes) {
+    if (!inside(what, p, bytes)) return;
+    for (size_t i = 0; i < bytes; ++i)
+        if (static_cast<const char*>(p)[i]) { complain(std::string(what) + ": not zero at the launch"); return; }
+}
+cudaError_t enqueue(std::function<void()> f) {
+    if (g_capturing) g_graphs.back().push_back(f); else f();
+    return cudaSuccess;
+}
+
+cudaError_t fake_cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
+cudaError_t fake_cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
+    *v = a == cudaDevAttrMultiProcessorCount ? 148 : 10;
+    return cudaSuccess;
+}
+cudaError_t fake_cudaMalloc(void** p, size_t n) { return give(p, n); }
+template <class T> cudaError_t fake_cudaMalloc(T** p, size_t n) { return give(reinterpret_cast<void**>(p), n); }
+cudaError_t fake_cudaMallocAsync(void** p, size_t n, cudaStream_t) { return give(p, n); }
+cudaError_t fake_cudaFree(void* p) { return take_back(p); }
+cudaError_t fake_cudaFreeAsync(void* p, cudaStream_t) { return take_back(p); }
+cudaError_t fake_cudaMemset(void* p, int v, size_t n) { if (inside("memset", p, n)) std::memset(p, v, n); return cudaSuccess; }
+cudaError_t fake_cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t) { return enqueue([=] { fake_cudaMemset(p, v, n); }); }
+cudaError_t fake_cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) { return enqueue([=] { std::memcpy(d, s, n); }); }
+cudaError_t fake_cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) {
+    *s = g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
+cudaError_t fake_cudaGetLastError() { return cudaSuccess; }
+cudaError_t fake_cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t fake_cudaDeviceSynchronize() { return cudaSuccess; }
+cudaError_t fake_cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = reinterpret_cast<cudaStream_t>(7); return cudaSuccess; }
+cudaError_t fake_cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+
+}  // namespace
+
+namespace bv {
+
+int fake_phase_max_ctas(int, int sms) { return sms; }
+int fake_small_max_ctas(int, int sms) { return sms; }
+int fake_flow_max_ctas_per_sm(int) { return 1; }
+int fake_cluster_max_clusters(int, int, int c) { return 148 / c; }
+int fake_stream_max_clusters(int, int, bool, int c) { return 148 / c; }
+
+cudaError_t fake_launch_phase(const Params& prm, const PhaseScratch& ps, int, bool, int, cudaStream_t) {
+    if (g_refuse_cooperative) return cudaErrorCooperativeLaunchTooLarge;
+    const size_t B = prm.B, g = prm.gamma;
+    return enqueue([=] {
+        inside("status word", prm.status, 4);
+        zeros("phase counters", ps.ctr, ps.zero_words * 4);
+        scratch("phase pieces", ps.part, B * ps.rows * ps.slots * sizeof(double2));
+        scratch("drafted logits", ps.drafted, B * g * sizeof(float2));
+        scratch("positions", ps.pos, B * (g + 1) * sizeof(PhPos));
+        scratch("candidates", ps.sel, B * 3 * sizeof(uint4));
+        scratch("later candidates", ps.rest, B * sizeof(uint2));
+        scratch("unit references", ps.seg_M, B * ps.units * sizeof(float));
+        scratch("unit totals", ps.seg, B * (g + 1) * ps.units * sizeof(double));
+        zeros("phase counters beside the scratch", ps.ctr, ps.zero_words * 4);
+    });
+}
+cudaError_t fake_launch_small(const Params& prm, const SmallScratch& sc, int, bool, int, cudaStream_t) {
+    if (g_refuse_cooperative) return cudaErrorCooperativeLaunchTooLarge;
+    const size_t B = prm.B, g = prm.gamma;
+    return enqueue([=] {
+        inside("status word", prm.status, 4);
+        zeros("barrier words", sc.barrier, 17 * 4);
+        scratch("chunk pairs", sc.part, B * (2 * g + 1) * sc.nch * sizeof(double2));
+        scratch("segment totals", sc.seg, B * (g + 1) * sc.np * 16 * sizeof(double));
+        zeros("barrier words beside the scratch", sc.barrier, 17 * 4);
+    });
+}
+cudaError_t fake_launch_flow(const Params& prm, const FlowScratch& fl, int, int, cudaStream_t) {
+    const size_t B = prm.B, g = prm.gamma, rows = B * (g + 1);
+    return enqueue([=] {
+        inside("status word", prm.status, 4);
+        zeros("flow counters", fl.counters, static_cast<size_t>(fl.zero_words) * 4);
+        scratch("chunk pairs", fl.part, rows * fl.part_stride * sizeof(RowZ));
+        scratch("normalisers", fl.rowZ, rows * sizeof(RowZ));
+        scratch("prefix chain", fl.pchain, B * (g + 2) * sizeof(double));
+        scratch("scales", fl.cscale, rows * sizeof(float));
+        scratch("ratios", fl.ratio, rows * sizeof(double));
+        scratch("normaliser ratios", fl.zratio, rows * sizeof(double));
+        scratch("segment totals", fl.seg_tot, rows * fl.segs * sizeof(double));
+        scratch("residual masses", fl.S, rows * sizeof(double));
+        scratch("candidates", fl.cand, rows * sizeof(int));
+        scratch("tau", fl.tv_tau, B * sizeof(int));
+        zeros("flow counters beside the scratch", fl.counters, static_cast<size_t>(fl.zero_words) * 4);
+    });
+}
+cudaError_t fake_launch_cluster(const Params& prm, int, int, int, int, cudaStream_t) {
+    return enqueue([=] { inside("status word", prm.status, 4); });
+}
+cudaError_t fake_launch_stream(const Params& prm, int, int, bool, int, int, cudaStream_t) {
+    return enqueue([=] { inside("status word", prm.status, 4); });
+}
+
+}  // namespace bv
+
+#define cudaGetDevice fake_cudaGetDevice
+#define cudaDeviceGetAttribute fake_cudaDeviceGetAttribute
+#define cudaMalloc fake_cudaMalloc
+#define cudaMallocAsync fake_cudaMallocAsync
+#define cudaFree fake_cudaFree
+#define cudaFreeAsync fake_cudaFreeAsync
+#define cudaMemset fake_cudaMemset
+#define cudaMemsetAsync fake_cudaMemsetAsync
+#define cudaMemcpyAsync fake_cudaMemcpyAsync
+#define cudaStreamIsCapturing fake_cudaStreamIsCapturing
+#define cudaGetLastError fake_cudaGetLastError
+#define cudaStreamSynchronize fake_cudaStreamSynchronize
+#define cudaDeviceSynchronize fake_cudaDeviceSynchronize
+#define cudaStreamCreateWithFlags fake_cudaStreamCreateWithFlags
+#define cudaStreamDestroy fake_cudaStreamDestroy
+#define phase_max_ctas fake_phase_max_ctas
+#define small_max_ctas fake_small_max_ctas
+#define flow_max_ctas_per_sm fake_flow_max_ctas_per_sm
+#define cluster_max_clusters fake_cluster_max_clusters
+#define stream_max_clusters fake_stream_max_clusters
+#define launch_phase fake_launch_phase
+#define launch_small fake_launch_small
+#define launch_flow fake_launch_flow
+#define launch_cluster fake_launch_cluster
+#define launch_stream fake_launch_stream
+#include "bv_api.cu"
+
+extern "C" {
+void host_begin_capture() { g_graphs.emplace_back(); g_capturing = true; }
+int host_end_capture() { g_capturing = false; return static_cast<int>(g_graphs.size()) - 1; }
+void host_replay(int graph) { for (const auto& f : g_graphs[graph]) f(); }
+void host_refuse_cooperative(int on) { g_refuse_cooperative = on; }
+// what has gone wrong since the last question
+const char* host_errors() { static std::string out; out = g_errors; g_errors.clear(); return out.c_str(); }
+size_t host_live_bytes() { size_t n = 0; for (const auto& b : g_blocks) if (b.second.live) n += b.second.bytes; return n; }
+}

@@ -1,0 +1,76 @@
+"""The dispatch layer without a GPU: the memory it hands to the kernels, over the runtime of tests/host_runtime.cu."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+from paper_2403_10444_b200 import build as bv_build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+F32, BF16 = 0, 1
+
+
+@pytest.fixture(scope="module")
+def host_so(tmp_path_factory):
+    lib = bv_build.build()
+    out = str(tmp_path_factory.mktemp("host") / "host_runtime.so")
+    # (the plans are the library's own; names that both define bind to this file's)
+    subprocess.check_call([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17",
+                           "-Xcompiler", "-fPIC", "-shared", "-I", bv_build.CSRC, os.path.join(HERE, "host_runtime.cu"), "-o", out,
+                           "-Xlinker", "-Bsymbolic", "-Xlinker", "-rpath=" + os.path.dirname(lib), lib])
+    return ctypes.CDLL(out)
+
+
+@pytest.fixture
+def host(host_so):
+    host_so.bv_release()
+    host_so.host_errors.restype = ctypes.c_char_p
+    yield host_so
+    host_so.bv_release()
+    host_so.bv_set_option(b"kernel", 0)
+
+
+FLOAT = ctypes.c_float(1.0)
+
+
+def verify(host, B, gamma, V, dtype=BF16, fn="bv_verify", offset=0, diagnostics=False, stream=None):
+    """One call on tensors that are never touched, `offset` elements off a 16-byte boundary; (status, kernel)."""
+    p = ctypes.c_void_p
+    base = (1 << 40) + offset * (4 if dtype == F32 else 2)
+    x = p(1 << 41)
+    args = [p(base), p(base + (1 << 39)), x, x]
+    if "lse" in fn:
+        args.append(x)
+    args += [B, gamma, V, dtype]
+    if "probs" not in fn:
+        args.append(FLOAT)
+    args += [x, x]
+    if diagnostics:
+        fn = fn if "probs" in fn else fn + "_ex"
+        args += [x] * (3 if "probs" in fn else 5)
+    elif "probs" in fn:
+        args += [None] * 3
+    status = getattr(host, fn)(*args, p(stream))
+    return status, host.bv_last_kernel()
+
+
+# batches that go through the phase kernel in parts, the last of which needs more scratch a sequence than the others
+@pytest.mark.parametrize("B,gamma,V,dtype", [(1533, 2, 5089, BF16), (1533, 2, 2534, F32), (1533, 1, 10001, BF16), (1524, 1, 4601, BF16),
+                                             (2000, 2, 1003, BF16), (769, 3, 50257, BF16)])
+def test_every_part_of_a_batch_fits_the_workspace(host, B, gamma, V, dtype):
+    for fn in ("bv_verify", "tv_verify"):
+        host.bv_release()
+        assert verify(host, B, gamma, V, dtype, fn) == (0, 5)
+        assert host.host_errors() == b""
+
+
+def test_scratch_fits_over_the_range(host):
+    for B in (1, 3, 24, 33, 200, 700, 800, 1500, 1600):
+        for gamma in (1, 2, 7, 33):
+            for V in (1, 1003, 4096, 8209, 50257, 65536):
+                for fn in ("bv_verify", "tv_verify", "bv_verify_lse", "bv_verify_probs"):
+                    if V % 8 and ("lse" in fn or "probs" in fn):
+                        continue
+                    assert verify(host, B, gamma, V, fn=fn)[0] == 0
+                    assert host.host_errors() == b"", (B, gamma, V, fn)

@@ -33,7 +33,7 @@ def test_rows_around_whole_units(dtype, V, B, gamma, kernel, bv_options):
     check(inputs(B, gamma, V, dtype, V + B), (oracle.BLOCK_VERIFY, oracle.TOKEN_VERIFY), kernel)
 
 
-@pytest.mark.parametrize("V,B,gamma", [(4096, 768, 1), (64, 768, 3), (1003, 2000, 2), (16, 769, 2)])
+@pytest.mark.parametrize("V,B,gamma", [(4096, 768, 1), (64, 768, 3), (1003, 2000, 2), (16, 769, 2), (5089, 1533, 2)])
 def test_as_many_sequences_as_it_takes_and_more(V, B, gamma, bv_options):
     # 768 sequences a launch; rows at any alignment go through it in parts beyond that, others through the flow kernel
     import paper_2403_10444_b200 as bv
