@@ -26,8 +26,12 @@
  * The library keeps one workspace per stream (up to 32 streams per device, the
  * least recently used one is recycled beyond that): calls on one stream run in
  * order and share it, calls on different streams never do.  A workspace is
- * obtained and grown with cudaMallocAsync / cudaFreeAsync on that stream, so a
- * first or larger call allocates but does not synchronise the device; the
+ * obtained and grown with cudaMallocAsync on that stream, so a first or larger
+ * call allocates but does not synchronise the device.  Calls may be captured into
+ * graphs and replayed between other calls: a captured call uses the workspace of
+ * the stream it was captured on (what it needs beyond that is obtained outside the
+ * graph, on a stream of the library's, and waited for), so replays must not overlap
+ * other calls on that stream.  What is outgrown stays allocated for their sake; the
  * memory is returned by bv_release().  B = 0 is accepted and does nothing.
  *
  * Errors: every entry point returns BV_OK (0) or a negative bv_status; nothing

@@ -7,6 +7,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <vector>
 
 #include "../../include/bv.h"
 #include "bv_launch.h"
@@ -39,7 +40,7 @@ constexpr long long kPhaseBytesF32[3] = {120LL << 20, 280LL << 20, 280LL << 20};
 constexpr long long kPhaseProbsPairs[2] = {36LL << 20, 140LL << 20};      // [algo] bytes of one row pair of every sequence
 constexpr long long kPhaseBytesAll = 360LL << 20;
 constexpr int kPhaseProbsB = 12;
-constexpr size_t kSlotHead = 16384;   // leading bytes of a stream's workspace: status word, barrier words, the phase kernel's counters
+constexpr size_t kSlotHead = 16384;   // first area of a stream's workspace: status word, barrier words, the phase kernel's counters
 constexpr size_t kSlotPhase = 256;    // ... the last of these from here on
 static_assert(kSlotPhase + bv::kPhaseCounterWords * sizeof(unsigned) <= kSlotHead, "the counters fit in the head");
 constexpr int kStreamSlots = 32;  // streams per device that keep a workspace of their own
@@ -82,15 +83,23 @@ void load_env_options() {
     g_opt.flow_depth = env_int("BV_FLOW_DEPTH");
 }
 
-// The workspace a stream's calls share.  Calls on one stream run one after the other, and the flow
-// kernel leaves its counters at zero, so one area per stream serves any number of calls in flight;
-// it grows with cudaMallocAsync / cudaFreeAsync on that stream, which do not synchronise the device.
+// The workspace a stream's calls share.  Calls on one stream run one after the other, and the kernels
+// leave their counters at zero, so one set of areas per stream serves any number of calls in flight.
+// What has to be zero when a kernel starts lies apart from what kernels write as they like: a call that
+// a graph replays comes between others without the library knowing, and finds its counters at zero all
+// the same.  For the same reason an area that is outgrown stays allocated until the workspace is given
+// back (each is at least twice the size of the one before, so they add up to less than the last one).
+struct Area {
+    char* p = nullptr;
+    size_t bytes = 0;
+};
 struct StreamSlot {
     cudaStream_t stream = nullptr;
     bool used = false;
-    void* ws = nullptr;        // [head: zero between calls, but for the status word][scratch]
-    size_t bytes = 0;
-    size_t clean = 0;          // leading bytes of the scratch known to be zero between calls
+    Area head;                 // kSlotHead bytes, zero between calls but for the status word
+    Area zeros;                // the flow kernel's counters and flags, zero between calls
+    Area scratch;              // anything
+    std::vector<char*> outgrown;
     unsigned long long stamp = 0;
 };
 
@@ -110,7 +119,7 @@ struct DeviceState {
     // staging for the host-buffer entry points
     void* stage = nullptr;
     size_t stage_bytes = 0;
-    cudaStream_t stream = nullptr;
+    cudaStream_t stream = nullptr;     // theirs, and where memory is obtained while a caller's stream is captured
 };
 
 DeviceState g_dev[kMaxDevices];
@@ -145,35 +154,82 @@ int device_state(DeviceState** out) {
     return BV_OK;
 }
 
-// The workspace of `stream` with room for `need` bytes of scratch behind its head.
-// A stream seen for the first time takes a free entry, or the one used longest ago (whose area is
+int own_stream(DeviceState& d) {
+    const cudaError_t e = d.stream ? cudaSuccess : cudaStreamCreateWithFlags(&d.stream, cudaStreamNonBlocking);
+    return e == cudaSuccess ? BV_OK : cuda_fail(e);
+}
+
+// `want` bytes on `stream` (or `need`, if there are not as many), set to zero if `zero`.
+cudaError_t obtain(Area* a, size_t want, size_t need, bool zero, cudaStream_t stream) {
+    void* p = nullptr;
+    cudaError_t e = cudaMallocAsync(&p, want, stream);
+    if (e == cudaErrorMemoryAllocation && want > need) {
+        cudaGetLastError();
+        e = cudaMallocAsync(&p, want = need, stream);
+    }
+    if (e != cudaSuccess) return e;
+    if (zero && (e = cudaMemsetAsync(p, 0, want, stream)) != cudaSuccess) {
+        cudaFreeAsync(p, stream);
+        return e;
+    }
+    a->p = static_cast<char*>(p);
+    a->bytes = want;
+    return e;
+}
+// Makes room for `need` bytes in one of the areas of `s`.
+int grow(DeviceState& d, StreamSlot& s, Area* a, size_t need, bool zero) {
+    if (a->bytes >= need) return BV_OK;
+    const size_t want = need > 2 * a->bytes ? need : 2 * a->bytes;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s.stream, &cap);
+    if (e != cudaSuccess) return cuda_fail(e);
+    Area fresh;
+    if (cap == cudaStreamCaptureStatusNone) {
+        e = obtain(&fresh, want, need, zero, s.stream);
+    } else {
+        // What is allocated on a stream that is captured belongs to the graph: it is obtained on another one, and there
+        // before the graph can run.
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        if ((e = cudaThreadExchangeStreamCaptureMode(&mode)) != cudaSuccess) return cuda_fail(e);
+        const int rc = own_stream(d);
+        if (rc == BV_OK && (e = obtain(&fresh, want, need, zero, d.stream)) == cudaSuccess) e = cudaStreamSynchronize(d.stream);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (rc != BV_OK) return rc;
+    }
+    if (e != cudaSuccess) return cuda_fail(e);
+    if (a->p) s.outgrown.push_back(a->p);
+    *a = fresh;
+    return BV_OK;
+}
+
+// The workspace of `stream` with room for `zeros` bytes that are zero and `scratch` bytes that are anything.
+// A stream seen for the first time takes a free entry, or the one used longest ago (whose areas are
 // freed in its own stream's order).
-int stream_slot(DeviceState& d, cudaStream_t stream, size_t need, StreamSlot** out) {
+int stream_slot(DeviceState& d, cudaStream_t stream, size_t zeros, size_t scratch, StreamSlot** out) {
     StreamSlot* s = nullptr;
     StreamSlot* victim = nullptr;
     for (StreamSlot& c : d.slots) {
         if (c.used && c.stream == stream) { s = &c; break; }
         if (!victim || (victim->used && (!c.used || c.stamp < victim->stamp))) victim = &c;
     }
-    cudaError_t e;
     if (!s) {
         s = victim;
-        if (s->used && s->ws && (e = cudaFreeAsync(s->ws, s->stream)) != cudaSuccess) return cuda_fail(e);
-        *s = StreamSlot{};
+        if (s->used) {
+            cudaError_t e = cudaSuccess;
+            for (char* p : s->outgrown) if (e == cudaSuccess) e = cudaFreeAsync(p, s->stream);
+            for (const Area* a : {&s->head, &s->zeros, &s->scratch}) if (e == cudaSuccess && a->p) e = cudaFreeAsync(a->p, s->stream);
+            *s = StreamSlot{};
+            if (e != cudaSuccess) return cuda_fail(e);
+        }
         s->used = true;
         s->stream = stream;
     }
     s->stamp = ++d.clock;
-    const size_t total = kSlotHead + need;
-    if (s->bytes < total) {
-        if (s->ws && (e = cudaFreeAsync(s->ws, stream)) != cudaSuccess) return cuda_fail(e);
-        s->ws = nullptr; s->bytes = 0; s->clean = 0;
-        if ((e = cudaMallocAsync(&s->ws, total, stream)) != cudaSuccess) return cuda_fail(e);
-        if ((e = cudaMemsetAsync(s->ws, 0, kSlotHead, stream)) != cudaSuccess) return cuda_fail(e);
-        s->bytes = total;
-    }
+    int rc = grow(d, *s, &s->head, kSlotHead, true);
+    if (rc == BV_OK) rc = grow(d, *s, &s->zeros, zeros, true);
+    if (rc == BV_OK) rc = grow(d, *s, &s->scratch, scratch, false);
     *out = s;
-    return BV_OK;
+    return rc;
 }
 
 bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
@@ -190,16 +246,6 @@ int pick_cluster(const DeviceState& d, const Options& opt, int B, size_t row_byt
     // cheaper exchanges) win: measured 0.43 against 0.57 ms at B = 256, gamma = 8, V = 152064.
     if (c == 8 && static_cast<long long>(B) * c >= 8LL * d.sm_count) c = 4;
     return c;
-}
-
-// Is there room for `need` bytes of scratch in the stream's workspace, or may it grow now?  Not while the stream is
-// captured: what is allocated then belongs to the graph.
-bool slot_can_hold(const DeviceState& d, cudaStream_t stream, size_t need) {
-    for (const StreamSlot& c : d.slots)
-        if (c.used && c.stream == stream && c.bytes >= kSlotHead + need) return true;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) { cudaGetLastError(); return false; }
-    return cap == cudaStreamCaptureStatusNone;
 }
 
 // Where the element-wise kernel is still the default: a few short unaligned rows a sequence, one sequence an SM at most,
@@ -253,11 +299,9 @@ int run_phase(DeviceState& d, const bv::Params& prm, int dtype, bool vec, cudaSt
         const size_t n = bv::phase_scratch(nullptr, nullptr, rest, g, bv::phase_plan(prm.V, dtype, vec, rest, g, prm.lse_d != nullptr, nc), &ps);
         if (n > need) need = n;
     }
-    if (!slot_can_hold(d, stream, need)) return 1;
     StreamSlot* slot = nullptr;
-    const int rc = stream_slot(d, stream, need, &slot);
+    const int rc = stream_slot(d, stream, 0, need, &slot);
     if (rc != BV_OK) return rc;
-    slot->clean = 0;                // (the area the flow kernel expects to find zero is written here)
     const size_t row_bytes = static_cast<size_t>(prm.V) * (dtype == BV_DTYPE_F32 ? 4 : 2);
     int launches = 0;
     for (int b0 = 0; b0 < prm.B; b0 += part, ++launches) {
@@ -276,10 +320,9 @@ int run_phase(DeviceState& d, const bv::Params& prm, int dtype, bool vec, cudaSt
         if (prm.out_h) p.out_h = prm.out_h + b * (g + 1);
         if (prm.out_lse_t) p.out_lse_t = prm.out_lse_t + b * (g + 1);
         if (prm.out_lse_d) p.out_lse_d = prm.out_lse_d + b * g;
-        p.status = static_cast<int*>(slot->ws);
+        p.status = reinterpret_cast<int*>(slot->head.p);
         if (p.B != part) plan = bv::phase_plan(p.V, dtype, vec, p.B, g, p.lse_d != nullptr, nc);
-        bv::phase_scratch(static_cast<char*>(slot->ws) + kSlotHead, reinterpret_cast<unsigned*>(static_cast<char*>(slot->ws) + kSlotPhase),
-                          p.B, g, plan, &ps);
+        bv::phase_scratch(slot->scratch.p, reinterpret_cast<unsigned*>(slot->head.p + kSlotPhase), p.B, g, plan, &ps);
         const cudaError_t e = bv::launch_phase(p, ps, dtype, vec, nc, stream);
         if (e != cudaSuccess) return cuda_fail(e);
     }
@@ -358,17 +401,15 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
         // (a row that starts inside a vector lies in one more)
         const long long vecs = vec ? static_cast<long long>(row_bytes / 16) : (static_cast<long long>(row_bytes) + 30) / 16;
         const bv::SmallPlan plan = bv::small_plan(vecs, B, gamma, nc > 0 ? nc : 1);
-        if (nc > 0 && (vec || (V <= (1 << 30) && slot_can_hold(*d, stream, bv::small_scratch_bytes(B, gamma, plan))))) {
+        if (nc > 0 && (vec || V <= (1 << 30))) {
             StreamSlot* slot = nullptr;
-            if ((rc = stream_slot(*d, stream, bv::small_scratch_bytes(B, gamma, plan), &slot)) != BV_OK) return rc;
-            slot->clean = 0;                // (the area the flow kernel expects to find zero is written here)
+            if ((rc = stream_slot(*d, stream, 0, bv::small_scratch_bytes(B, gamma, plan), &slot)) != BV_OK) return rc;
             bv::SmallScratch sc;
             // the barrier words are in the head: zero since it was allocated
-            bv::small_scratch_layout(static_cast<char*>(slot->ws) + kSlotHead, reinterpret_cast<unsigned*>(static_cast<char*>(slot->ws) + 128),
-                                     B, gamma, plan, &sc);
+            bv::small_scratch_layout(slot->scratch.p, reinterpret_cast<unsigned*>(slot->head.p + 128), B, gamma, plan, &sc);
             prm.ticket = nullptr;
             prm.nclusters = 0;
-            prm.status = static_cast<int*>(slot->ws);
+            prm.status = reinterpret_cast<int*>(slot->head.p);
             cudaError_t e = bv::launch_small(prm, sc, dtype, vec, nc, stream);
             if (e != cudaSuccess) return cuda_fail(e);
             t_last_launches = 1; t_last_kernel = 4;
@@ -399,29 +440,21 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
             size_t zero_bytes = 0;
             const size_t need = bv::flow_scratch_bytes(B, gamma, plan, &zero_bytes);
             StreamSlot* slot = nullptr;
-            if ((rc = stream_slot(*d, stream, need, &slot)) != BV_OK) return rc;
-            char* scratch = static_cast<char*>(slot->ws) + kSlotHead;
+            if ((rc = stream_slot(*d, stream, zero_bytes, need, &slot)) != BV_OK) return rc;
             bv::FlowScratch fl;
-            bv::flow_scratch_layout(scratch, B, gamma, plan, &fl);
+            bv::flow_scratch_layout(slot->zeros.p, slot->scratch.p, B, gamma, plan, &fl);
             // (with every position swept the second sweeps are the larger half of the launch and never wait for one another: deeper measured better)
             if (prm.out_p || prm.out_S || prm.out_h || prm.out_lse_t || prm.out_lse_d) fl.depth = 3;
             if (opt.flow_depth >= 2 && opt.flow_depth <= 6) fl.depth = opt.flow_depth;
             fl.keep_l2 = opt.flow_keep_l2 == 1;
-            // The kernel leaves its counters and flags at zero when it ends, so they are cleared here only
-            // when the area is new or a larger problem needs more of them than the last launch left clean.
-            cudaError_t e = cudaSuccess;
-            if (slot->clean < zero_bytes) {
-                e = cudaMemsetAsync(scratch, 0, zero_bytes, stream);
-                if (e != cudaSuccess) return cuda_fail(e);
-            }
-            slot->clean = zero_bytes;
+            // (the kernel leaves its counters and flags at zero when it ends: they have been since their area was obtained)
             // (given probabilities the items are the pieces of the positions swept: at most all of them)
             long long items = prm.probs ? static_cast<long long>(B) * (gamma + 1) * fl.np : static_cast<long long>(fl.total_s1);
             if (nctas > items) nctas = items;
             prm.ticket = nullptr;
             prm.nclusters = 0;
-            prm.status = static_cast<int*>(slot->ws);
-            e = bv::launch_flow(prm, fl, dtype, static_cast<int>(nctas), stream);
+            prm.status = reinterpret_cast<int*>(slot->head.p);
+            const cudaError_t e = bv::launch_flow(prm, fl, dtype, static_cast<int>(nctas), stream);
             if (e != cudaSuccess) return cuda_fail(e);
             t_last_launches = 1; t_last_kernel = 1;
             return BV_OK;
@@ -431,8 +464,8 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
     if (prm.lse_d != nullptr || prm.greedy || prm.probs) return BV_ERR_UNSUPPORTED;   // (the flow kernel could not be launched)
 
     StreamSlot* slot = nullptr;
-    if ((rc = stream_slot(*d, stream, 0, &slot)) != BV_OK) return rc;
-    prm.status = static_cast<int*>(slot->ws);
+    if ((rc = stream_slot(*d, stream, 0, 0, &slot)) != BV_OK) return rc;
+    prm.status = reinterpret_cast<int*>(slot->head.p);
 
     int cluster = pick_cluster(*d, opt, B, row_bytes);
     if (vec && opt.kernel != 3) {
@@ -478,7 +511,7 @@ int take_stream_status(cudaStream_t stream) {
         const int rc = device_state(&d);
         if (rc != BV_OK) return rc;
         for (StreamSlot& c : d->slots)
-            if (c.used && c.stream == stream) word = static_cast<int*>(c.ws);
+            if (c.used && c.stream == stream) word = reinterpret_cast<int*>(c.head.p);
     }
     cudaError_t e;
     if (!word) {
@@ -515,8 +548,7 @@ int run_host(int algo, const void* tgt, const void* drf, const int32_t* tok, con
         DeviceState* d = nullptr;
         if ((rc = device_state(&d)) != BV_OK) return rc;
         cudaError_t e;
-        if (!d->stream && (e = cudaStreamCreateWithFlags(&d->stream, cudaStreamNonBlocking)) != cudaSuccess)
-            return cuda_fail(e);
+        if ((rc = own_stream(*d)) != BV_OK) return rc;
         // (this entry point waits for its result anyway, so its staging buffer grows with plain cudaMalloc)
         if (d->stage_bytes < total) {
             if (d->stage) cudaFree(d->stage);
@@ -716,7 +748,10 @@ int bv_release(void) {
     if ((e = cudaDeviceSynchronize()) != cudaSuccess) return cuda_fail(e);
     if (d.stage) cudaFree(d.stage);
     if (d.tickets) cudaFree(d.tickets);
-    for (StreamSlot& c : d.slots) if (c.used && c.ws) cudaFree(c.ws);
+    for (StreamSlot& c : d.slots) {
+        for (char* p : c.outgrown) cudaFree(p);
+        for (const Area* a : {&c.head, &c.zeros, &c.scratch}) if (a->p) cudaFree(a->p);
+    }
     if (d.stream) cudaStreamDestroy(d.stream);
     d = DeviceState{};
     return BV_OK;

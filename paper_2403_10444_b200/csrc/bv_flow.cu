@@ -740,7 +740,7 @@ size_t flow_scratch_bytes(int B, int gamma, const FlowPlan& plan, size_t* zero_b
         z += 2 * up256(static_cast<size_t>(B) * sizeof(unsigned));             // tv_front, tv_decided
     }
     if (zero_bytes) *zero_bytes = z;
-    size_t n = z;
+    size_t n = 0;
     n += up256(rows * plan.part_stride() * sizeof(RowZ));   // part
     n += up256(rows * sizeof(RowZ));                // rowZ
     n += up256(static_cast<size_t>(B) * (gamma + 2) * sizeof(double));   // pchain
@@ -753,10 +753,10 @@ size_t flow_scratch_bytes(int B, int gamma, const FlowPlan& plan, size_t* zero_b
     return n;
 }
 
-void flow_scratch_layout(void* base, int B, int gamma, const FlowPlan& plan, FlowScratch* fl) {
+void flow_scratch_layout(void* zeros, void* base, int B, int gamma, const FlowPlan& plan, FlowScratch* fl) {
     const size_t rows = static_cast<size_t>(B) * (gamma + 1);
     const size_t segs = flow_seg_stride(plan);
-    char* p = static_cast<char*>(base);
+    char* p = static_cast<char*>(zeros);
     auto take = [&](size_t bytes) { char* q = p; p += up256(bytes); return q; };
     fl->counters = reinterpret_cast<unsigned*>(take(kCounterWords * sizeof(unsigned)));
     fl->row_cnt = reinterpret_cast<unsigned*>(take(rows * sizeof(unsigned)));
@@ -779,6 +779,7 @@ void flow_scratch_layout(void* base, int B, int gamma, const FlowPlan& plan, Flo
         fl->tv_front = reinterpret_cast<unsigned*>(take(static_cast<size_t>(B) * sizeof(unsigned)));
         fl->tv_decided = reinterpret_cast<unsigned*>(take(static_cast<size_t>(B) * sizeof(unsigned)));
     }
+    p = static_cast<char*>(base);
     fl->part = reinterpret_cast<RowZ*>(take(rows * plan.part_stride() * sizeof(RowZ)));
     fl->rowZ = reinterpret_cast<RowZ*>(take(rows * sizeof(RowZ)));
     fl->pchain = reinterpret_cast<double*>(take(static_cast<size_t>(B) * (gamma + 2) * sizeof(double)));

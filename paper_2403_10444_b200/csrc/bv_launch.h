@@ -31,8 +31,8 @@ int cluster_max_clusters(int algo, int dtype, int cluster);
 cudaError_t launch_cluster(const Params& prm, int algo, int dtype, int cluster, int nclusters, cudaStream_t stream);
 
 // Flow kernel (Block Verification, 128-bit path): independent work items with dependency
-// counters in a scratch area of flow_scratch_bytes(); its first *zero_bytes must be zero
-// when the kernel starts, and the kernel leaves them zero when it ends.
+// counters in an area of *zero_bytes that must be zero when the kernel starts, and that the kernel
+// leaves zero when it ends; its other scratch takes flow_scratch_bytes().
 struct RowZ { double MP, ZP, MQ, ZQ; };   // row (or chunk) references and sums of 2^{z k - M}
 struct FlowScratch {
     unsigned* counters;   // ticket counter of the sweep-1 items, rows queued for their second sweep, pieces of
@@ -72,7 +72,7 @@ struct FlowScratch {
     int fine_from;        // Block Verification: rows 0 .. gamma-1 of the blocks from this one on are cut into nch_late chunks (B: none)
     int np;               // pieces per row in the second sweep (1 .. kFlowMaxChunks)
     unsigned total_s1;    // first-sweep tickets: fine_from gamma nch + (B - fine_from) gamma nch_late
-    unsigned zero_words;  // 32-bit words at the start of the scratch area (from `counters` on) that start and end at zero
+    unsigned zero_words;  // 32-bit words from `counters` on that start and end at zero
     int depth;            // flow kernel: descriptors a CTA may have handed to its workers and not yet seen swept
     int segs;             // residual totals kept per row
     int tail_mode;        // 0: a block's candidates are started all at once when the first-sweep tickets have run out;
@@ -95,7 +95,7 @@ struct FlowPlan {
 // (supplied draft normalisers); chunks / pieces > 0 force the chunk count / the piece count.
 FlowPlan flow_plan(long long units, int B, int gamma, long long nctas, bool pair_items, int chunks, int pieces, bool token_verify = false, bool probs = false);
 size_t flow_scratch_bytes(int B, int gamma, const FlowPlan& plan, size_t* zero_bytes);
-void flow_scratch_layout(void* base, int B, int gamma, const FlowPlan& plan, FlowScratch* fl);
+void flow_scratch_layout(void* zeros, void* base, int B, int gamma, const FlowPlan& plan, FlowScratch* fl);
 int flow_max_ctas_per_sm(int dtype);
 cudaError_t launch_flow(const Params& prm, const FlowScratch& fl, int dtype, int nctas, cudaStream_t stream);
 

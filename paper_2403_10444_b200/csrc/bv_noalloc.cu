@@ -79,7 +79,8 @@ extern "C" int bv_verify_noalloc(const void* tgt, const void* drf, const int32_t
     const long long units = static_cast<long long>(row_bytes / 16);
     const bv::FlowPlan plan = bv::flow_plan(units, B, gamma, static_cast<long long>(d.sm_count) * per_sm, true, 0, 0);
     size_t zero_bytes = 0;
-    const size_t need = bv::flow_scratch_bytes(B, gamma, plan, &zero_bytes) + 256;   // + the status word
+    const size_t other_bytes = bv::flow_scratch_bytes(B, gamma, plan, &zero_bytes);
+    const size_t need = zero_bytes + other_bytes + 256;   // + the status word
     if (need > kScratchBytes) return BV_ERR_TOO_LARGE;
 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -90,7 +91,7 @@ extern "C" int bv_verify_noalloc(const void* tgt, const void* drf, const int32_t
     if ((e = cudaMemsetAsync(status_word, 0, 256, s)) != cudaSuccess) return bv::note_cuda_error(e);
 
     bv::FlowScratch fl;
-    bv::flow_scratch_layout(d.scratch, B, gamma, plan, &fl);
+    bv::flow_scratch_layout(d.scratch, d.scratch + zero_bytes, B, gamma, plan, &fl);
     bv::Params prm{};
     prm.tgt = tgt; prm.drf = drf; prm.tok = tok; prm.uni = uni;
     prm.B = B; prm.gamma = gamma; prm.V = V;

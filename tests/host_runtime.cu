@@ -19,6 +19,7 @@ struct Block { size_t bytes; bool live; };
 std::map<char*, Block> g_blocks;
 std::vector<std::vector<std::function<void()>>> g_graphs;
 bool g_capturing = false;
+cudaStream_t g_captured = nullptr;       // the stream that is captured
 int g_refuse_cooperative = 0;
 std::string g_errors;
 
@@ -51,8 +52,9 @@ void zeros(const char* what, const void* p, size_t bytes) {
     for (size_t i = 0; i < bytes; ++i)
         if (static_cast<const char*>(p)[i]) { complain(std::string(what) + ": not zero at the launch"); return; }
 }
-cudaError_t enqueue(std::function<void()> f) {
-    if (g_capturing) g_graphs.back().push_back(f); else f();
+bool captured(cudaStream_t s) { return g_capturing && s == g_captured; }
+cudaError_t enqueue(cudaStream_t s, std::function<void()> f) {
+    if (captured(s)) g_graphs.back().push_back(f); else f();
     return cudaSuccess;
 }
 
@@ -63,18 +65,28 @@ cudaError_t fake_cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
 }
 cudaError_t fake_cudaMalloc(void** p, size_t n) { return give(p, n); }
 template <class T> cudaError_t fake_cudaMalloc(T** p, size_t n) { return give(reinterpret_cast<void**>(p), n); }
-cudaError_t fake_cudaMallocAsync(void** p, size_t n, cudaStream_t) { return give(p, n); }
+cudaError_t fake_cudaMallocAsync(void** p, size_t n, cudaStream_t s) {
+    if (captured(s)) complain("memory that would belong to a graph");
+    return give(p, n);
+}
 cudaError_t fake_cudaFree(void* p) { return take_back(p); }
-cudaError_t fake_cudaFreeAsync(void* p, cudaStream_t) { return take_back(p); }
+cudaError_t fake_cudaFreeAsync(void* p, cudaStream_t s) {
+    if (captured(s)) complain("memory freed by a graph");
+    return take_back(p);
+}
 cudaError_t fake_cudaMemset(void* p, int v, size_t n) { if (inside("memset", p, n)) std::memset(p, v, n); return cudaSuccess; }
-cudaError_t fake_cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t) { return enqueue([=] { fake_cudaMemset(p, v, n); }); }
-cudaError_t fake_cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) { return enqueue([=] { std::memcpy(d, s, n); }); }
-cudaError_t fake_cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) {
-    *s = g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+cudaError_t fake_cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t s) { return enqueue(s, [=] { fake_cudaMemset(p, v, n); }); }
+cudaError_t fake_cudaMemcpyAsync(void* d, const void* src, size_t n, cudaMemcpyKind, cudaStream_t s) { return enqueue(s, [=] { std::memcpy(d, src, n); }); }
+cudaError_t fake_cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode*) { return cudaSuccess; }
+cudaError_t fake_cudaStreamIsCapturing(cudaStream_t st, cudaStreamCaptureStatus* s) {
+    *s = captured(st) ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
     return cudaSuccess;
 }
 cudaError_t fake_cudaGetLastError() { return cudaSuccess; }
-cudaError_t fake_cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t fake_cudaStreamSynchronize(cudaStream_t s) {
+    if (captured(s)) complain("a captured stream is waited for");
+    return cudaSuccess;
+}
 cudaError_t fake_cudaDeviceSynchronize() { return cudaSuccess; }
 cudaError_t fake_cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = reinterpret_cast<cudaStream_t>(7); return cudaSuccess; }
 cudaError_t fake_cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
@@ -89,10 +101,10 @@ int fake_flow_max_ctas_per_sm(int) { return 1; }
 int fake_cluster_max_clusters(int, int, int c) { return 148 / c; }
 int fake_stream_max_clusters(int, int, bool, int c) { return 148 / c; }
 
-cudaError_t fake_launch_phase(const Params& prm, const PhaseScratch& ps, int, bool, int, cudaStream_t) {
+cudaError_t fake_launch_phase(const Params& prm, const PhaseScratch& ps, int, bool, int, cudaStream_t st) {
     if (g_refuse_cooperative) return cudaErrorCooperativeLaunchTooLarge;
     const size_t B = prm.B, g = prm.gamma;
-    return enqueue([=] {
+    return enqueue(st, [=] {
         inside("status word", prm.status, 4);
         zeros("phase counters", ps.ctr, ps.zero_words * 4);
         scratch("phase pieces", ps.part, B * ps.rows * ps.slots * sizeof(double2));
@@ -105,10 +117,10 @@ cudaError_t fake_launch_phase(const Params& prm, const PhaseScratch& ps, int, bo
         zeros("phase counters beside the scratch", ps.ctr, ps.zero_words * 4);
     });
 }
-cudaError_t fake_launch_small(const Params& prm, const SmallScratch& sc, int, bool, int, cudaStream_t) {
+cudaError_t fake_launch_small(const Params& prm, const SmallScratch& sc, int, bool, int, cudaStream_t st) {
     if (g_refuse_cooperative) return cudaErrorCooperativeLaunchTooLarge;
     const size_t B = prm.B, g = prm.gamma;
-    return enqueue([=] {
+    return enqueue(st, [=] {
         inside("status word", prm.status, 4);
         zeros("barrier words", sc.barrier, 17 * 4);
         scratch("chunk pairs", sc.part, B * (2 * g + 1) * sc.nch * sizeof(double2));
@@ -116,9 +128,9 @@ cudaError_t fake_launch_small(const Params& prm, const SmallScratch& sc, int, bo
         zeros("barrier words beside the scratch", sc.barrier, 17 * 4);
     });
 }
-cudaError_t fake_launch_flow(const Params& prm, const FlowScratch& fl, int, int, cudaStream_t) {
+cudaError_t fake_launch_flow(const Params& prm, const FlowScratch& fl, int, int, cudaStream_t st) {
     const size_t B = prm.B, g = prm.gamma, rows = B * (g + 1);
-    return enqueue([=] {
+    return enqueue(st, [=] {
         inside("status word", prm.status, 4);
         zeros("flow counters", fl.counters, static_cast<size_t>(fl.zero_words) * 4);
         scratch("chunk pairs", fl.part, rows * fl.part_stride * sizeof(RowZ));
@@ -134,11 +146,11 @@ cudaError_t fake_launch_flow(const Params& prm, const FlowScratch& fl, int, int,
         zeros("flow counters beside the scratch", fl.counters, static_cast<size_t>(fl.zero_words) * 4);
     });
 }
-cudaError_t fake_launch_cluster(const Params& prm, int, int, int, int, cudaStream_t) {
-    return enqueue([=] { inside("status word", prm.status, 4); });
+cudaError_t fake_launch_cluster(const Params& prm, int, int, int, int, cudaStream_t st) {
+    return enqueue(st, [=] { inside("status word", prm.status, 4); });
 }
-cudaError_t fake_launch_stream(const Params& prm, int, int, bool, int, int, cudaStream_t) {
-    return enqueue([=] { inside("status word", prm.status, 4); });
+cudaError_t fake_launch_stream(const Params& prm, int, int, bool, int, int, cudaStream_t st) {
+    return enqueue(st, [=] { inside("status word", prm.status, 4); });
 }
 
 }  // namespace bv
@@ -152,6 +164,7 @@ cudaError_t fake_launch_stream(const Params& prm, int, int, bool, int, int, cuda
 #define cudaMemset fake_cudaMemset
 #define cudaMemsetAsync fake_cudaMemsetAsync
 #define cudaMemcpyAsync fake_cudaMemcpyAsync
+#define cudaThreadExchangeStreamCaptureMode fake_cudaThreadExchangeStreamCaptureMode
 #define cudaStreamIsCapturing fake_cudaStreamIsCapturing
 #define cudaGetLastError fake_cudaGetLastError
 #define cudaStreamSynchronize fake_cudaStreamSynchronize
@@ -171,7 +184,7 @@ cudaError_t fake_launch_stream(const Params& prm, int, int, bool, int, int, cuda
 #include "bv_api.cu"
 
 extern "C" {
-void host_begin_capture() { g_graphs.emplace_back(); g_capturing = true; }
+void host_begin_capture(void* stream) { g_graphs.emplace_back(); g_capturing = true; g_captured = static_cast<cudaStream_t>(stream); }
 int host_end_capture() { g_capturing = false; return static_cast<int>(g_graphs.size()) - 1; }
 void host_replay(int graph) { for (const auto& f : g_graphs[graph]) f(); }
 void host_refuse_cooperative(int on) { g_refuse_cooperative = on; }

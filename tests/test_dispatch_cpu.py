@@ -26,6 +26,7 @@ def host_so(tmp_path_factory):
 def host(host_so):
     host_so.bv_release()
     host_so.host_errors.restype = ctypes.c_char_p
+    host_so.host_live_bytes.restype = ctypes.c_size_t
     yield host_so
     host_so.bv_release()
     host_so.bv_set_option(b"kernel", 0)
@@ -74,3 +75,51 @@ def test_scratch_fits_over_the_range(host):
                         continue
                     assert verify(host, B, gamma, V, fn=fn)[0] == 0
                     assert host.host_errors() == b"", (B, gamma, V, fn)
+
+
+# calls of every kernel and of several sizes on one stream: (entry point, B, gamma, V, with diagnostics)
+CALLS = [("bv_verify", 128, 8, 128256, False), ("bv_verify", 128, 8, 128256, True), ("bv_verify", 256, 8, 256000, False),
+         ("tv_verify", 256, 8, 152064, False), ("bv_verify_lse", 256, 8, 152064, False), ("bv_verify", 4, 4, 32768, False),
+         ("bv_verify", 700, 2, 5089, False), ("tv_verify", 24, 5, 50257, False), ("bv_verify", 2000, 16, 4096, False),
+         ("bv_verify_probs", 400, 8, 152064, False), ("bv_verify", 100, 1, 1001, False)]
+
+
+def call(host, c):
+    assert verify(host, c[1], c[2], c[3], fn=c[0], diagnostics=c[4])[0] == 0
+    return host.bv_last_kernel()
+
+
+def test_the_calls_below_reach_every_kernel_that_keeps_scratch(host):
+    assert {call(host, c) for c in CALLS} >= {1, 4, 5}
+
+
+@pytest.mark.parametrize("warm", [True, False])
+@pytest.mark.parametrize("a", CALLS)
+def test_a_graph_replayed_between_eager_calls(host, a, warm):
+    # whatever ran on the stream before or since, a replayed call finds its memory, zero where it has to be, and leaves the
+    # eager calls' memory as they expect it
+    for b in CALLS:
+        host.bv_release()
+        if warm:
+            call(host, a)
+        host.host_begin_capture(None)
+        kernel = call(host, a)
+        graph = host.host_end_capture()
+        assert host.host_errors() == b"", (a, b)
+        assert call(host, a) == kernel                    # captured or not: the same kernel
+        for step in (b, graph, b, a, graph, graph, b):
+            host.host_replay(graph) if step is graph else call(host, step)
+            assert host.host_errors() == b"", (a, b)
+
+
+def test_the_workspace_is_bounded_and_given_back(host):
+    call(host, CALLS[0])
+    for B in range(1, 600, 7):                            # grows many times
+        call(host, ("bv_verify", B, 8, 128256, False))
+    sizes = host.host_live_bytes()
+    host.bv_release()
+    for c in (("bv_verify", 595, 8, 128256, False), ("bv_verify", 130, 8, 128256, False)):
+        call(host, c)
+    assert sizes <= 5 * host.host_live_bytes()
+    host.bv_release()
+    assert host.host_live_bytes() == 0 and host.host_errors() == b""
