@@ -241,6 +241,14 @@ template <int EPV> __device__ __forceinline__ void row_mask(float (&v)[EPV], int
         if (x < 0 || x >= V) v[e] = pad;
     }
 }
+// Of the EPV elements at p, those from `first` on and below `n` lie in the tensor [lo, hi).
+template <int EPV>
+__host__ __device__ __forceinline__ void elements_inside(const char* p, const char* lo, const char* hi, int& first, int& n) {
+    constexpr int ESZ = 16 / EPV;
+    first = p < lo ? static_cast<int>((lo - p) / ESZ) : 0;
+    const long long left = (hi - p) / ESZ;                   // (up to the end of the tensor: more than an int holds)
+    n = left < EPV ? static_cast<int>(left) : EPV;
+}
 // Sixteen bytes of a row from element x0 on, elements outside [0, V) as `pad` (rows at any alignment, one at a time).
 template <int DT>
 __device__ __forceinline__ uint4 row_elements(const char* row, int x0, int V, uint32_t pad) {

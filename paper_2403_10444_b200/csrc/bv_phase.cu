@@ -536,8 +536,8 @@ __device__ __forceinline__ void ph_fetch_edge(uint32_t cell, const char* p, bool
         uint4 v = make_uint4(pad, pad, pad, pad);
         if (in) {
             constexpr int ESZ = (DT == kF32) ? 4 : 2;
-            const int first = p < lo ? static_cast<int>((lo - p) / ESZ) : 0;
-            const int n = static_cast<int>((hi - p) / ESZ);
+            int first, n;
+            elements_inside<16 / ESZ>(p, lo, hi, first, n);
             v = row_elements<DT>(p + first * ESZ, -first, n - first, pad);
         }
         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cell), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");

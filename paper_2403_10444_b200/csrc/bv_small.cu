@@ -87,8 +87,9 @@ __device__ __forceinline__ uint4 small_load(const char* base, int i, int nv, con
     if (i < 0 || i >= nv) return make_uint4(pad, pad, pad, pad);
     if (AL || (p >= lo && p + 16 <= hi)) return ld_stream_v4(p);
     constexpr int ESZ = (DT == kF32) ? 4 : 2;                // (it reaches outside the tensor: the elements inside)
-    const int first = p < lo ? static_cast<int>((lo - p) / ESZ) : 0;
-    return row_elements<DT>(p + first * ESZ, -first, static_cast<int>((hi - p) / ESZ) - first, pad);
+    int first, n;
+    elements_inside<16 / ESZ>(p, lo, hi, first, n);
+    return row_elements<DT>(p + first * ESZ, -first, n - first, pad);
 }
 // 16 bytes from byte 4 q + bits / 8 on of two neighbouring vectors
 __device__ __forceinline__ uint4 small_shift(const uint4& a, const uint4& b, int q, int bits) {

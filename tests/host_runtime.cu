@@ -11,7 +11,7 @@
 #include <string>
 #include <vector>
 
-#include "bv_launch.h"
+#include "bv_flow_common.cuh"
 
 namespace {
 
@@ -188,6 +188,11 @@ void host_begin_capture(void* stream) { g_graphs.emplace_back(); g_capturing = t
 int host_end_capture() { g_capturing = false; return static_cast<int>(g_graphs.size()) - 1; }
 void host_replay(int graph) { for (const auto& f : g_graphs[graph]) f(); }
 void host_refuse_cooperative(int on) { g_refuse_cooperative = on; }
+// which of the elements of `esz` bytes at p lie in [lo, hi)
+void host_elements_inside(unsigned long long p, unsigned long long lo, unsigned long long hi, int esz, int* first, int* n) {
+    const char *a = reinterpret_cast<const char*>(p), *b = reinterpret_cast<const char*>(lo), *c = reinterpret_cast<const char*>(hi);
+    if (esz == 4) bv::elements_inside<4>(a, b, c, *first, *n); else bv::elements_inside<8>(a, b, c, *first, *n);
+}
 // what has gone wrong since the last question
 const char* host_errors() { static std::string out; out = g_errors; g_errors.clear(); return out.c_str(); }
 size_t host_live_bytes() { size_t n = 0; for (const auto& b : g_blocks) if (b.second.live) n += b.second.bytes; return n; }

@@ -123,3 +123,17 @@ def test_the_workspace_is_bounded_and_given_back(host):
     assert sizes <= 5 * host.host_live_bytes()
     host.bv_release()
     assert host.host_live_bytes() == 0 and host.host_errors() == b""
+
+
+@pytest.mark.parametrize("esz", [2, 4])
+def test_a_vector_at_the_edge_of_a_tensor_of_any_size(host, esz):
+    # the elements of a 16-byte vector that lie in a tensor, which may hold more of them than 32 bits count
+    ull, first, n = ctypes.c_ulonglong, ctypes.c_int(), ctypes.c_int()
+    for count in (1, 3, 7, 8, 9, 1000, 2 ** 31 - 1, 2 ** 31, 2 ** 31 + 5, 2 ** 32 + 1, 2 ** 33):
+        for offset in range(0, 16, esz):
+            lo = (1 << 40) + offset
+            hi = lo + count * esz
+            for p in {lo - offset, (hi - 1) // 16 * 16}:
+                host.host_elements_inside(ull(p), ull(lo), ull(hi), esz, ctypes.byref(first), ctypes.byref(n))
+                inside = [j for j in range(16 // esz) if lo <= p + j * esz < hi]
+                assert list(range(first.value, n.value)) == inside, (count, offset, p)
