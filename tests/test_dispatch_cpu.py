@@ -137,3 +137,11 @@ def test_a_vector_at_the_edge_of_a_tensor_of_any_size(host, esz):
                 host.host_elements_inside(ull(p), ull(lo), ull(hi), esz, ctypes.byref(first), ctypes.byref(n))
                 inside = [j for j in range(16 // esz) if lo <= p + j * esz < hi]
                 assert list(range(first.value, n.value)) == inside, (count, offset, p)
+
+
+def test_smoke_expects_the_kernels_that_run(host):
+    import __graft_entry__ as entry
+    for B, option, kernel in entry.SMOKE_CALLS:
+        host.bv_set_option(b"kernel", option)
+        for fn in ("bv_verify_ex", "tv_verify_ex", "gbv_verify_ex"):
+            assert verify(host, B, 4, 32768, fn=fn[:-3], diagnostics=True) == (0, kernel), (B, option, fn)
