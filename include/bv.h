@@ -321,7 +321,8 @@ int bv_draft_chain(const void* draft_table, const int32_t* first_tokens, const f
  *   out_tau     [iterations, B] int32 accepted drafts;  out_drafted [iterations, B, gamma] int32
  *   out_fault   [1] int32: 1 if a sequence reported a data fault (its further tokens mean nothing)
  *   work        B (2 gamma + 3) int32
- * Rows must be whole 16-byte vectors on 16-byte aligned bases and B at most 768, else BV_ERR_UNSUPPORTED.
+ * Rows must be whole 16-byte vectors on 16-byte aligned bases and B at most 768, else BV_ERR_UNSUPPORTED; whether a kernel
+ * takes the call, and its workspace, is settled before anything is enqueued.
  */
 int bv_decode_loop(const void* target_table, const void* draft_table, const int32_t* first_tokens,
                    const float* u_draft, const float* u_verify, int iterations, int B, int gamma, int V,

@@ -275,7 +275,7 @@ bool phase_pays(int algo, const bv::Params& prm, const Options& opt, int dtype, 
 
 // The phase kernel for the call in `prm`: BV_OK, an error, or 1 if it does not take the call.  Rows at any alignment have no
 // other kernel of this speed, so a batch of more sequences than it takes goes through it in parts.
-int run_phase(DeviceState& d, const bv::Params& prm, int dtype, bool vec, cudaStream_t stream) {
+int run_phase(DeviceState& d, const bv::Params& prm, int dtype, bool vec, bool probe, cudaStream_t stream) {
     int& nc = d.phase_ctas[dtype];
     if (nc == 0) {
         nc = bv::phase_max_ctas(dtype, d.sm_count);
@@ -301,7 +301,7 @@ int run_phase(DeviceState& d, const bv::Params& prm, int dtype, bool vec, cudaSt
     }
     StreamSlot* slot = nullptr;
     const int rc = stream_slot(d, stream, 0, need, &slot);
-    if (rc != BV_OK) return rc;
+    if (rc != BV_OK || probe) return rc;
     const size_t row_bytes = static_cast<size_t>(prm.V) * (dtype == BV_DTYPE_F32 ? 4 : 2);
     int launches = 0;
     for (int b0 = 0; b0 < prm.B; b0 += part, ++launches) {
@@ -334,6 +334,7 @@ struct Extra {              // what only some entry points pass
     const float* lse_d = nullptr;   // supplied draft log-normalisers (bv_verify_lse)
     int greedy = 0;                 // Algorithm 4 instead of Algorithm 2 (gbv_verify)
     const int32_t* first = nullptr; // the rows are those of two tables (Params::first)
+    bool probe = false;             // find the kernel and its workspace, launch nothing
     int probs = 0;                  // the rows hold probabilities, not logits (bv_verify_probs, tv_verify_probs)
     float* out_p = nullptr; float* out_S = nullptr; float* out_h = nullptr;
     float* out_lse_t = nullptr; float* out_lse_d = nullptr;
@@ -383,7 +384,7 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
     if (prm.first != nullptr && !vec) return BV_ERR_UNSUPPORTED;
     const bool elements = !vec && !only_vec && opt.kernel == 0 && elements_pay(algo, prm, row_bytes, d->sm_count);
     if ((vec || !only_vec) && !elements && (opt.kernel == 5 || ((opt.kernel == 0 || prm.first != nullptr) && phase_pays(algo, prm, opt, dtype, vec, logit_bytes)))) {
-        if ((rc = run_phase(*d, prm, dtype, vec, stream)) <= BV_OK) return rc;
+        if ((rc = run_phase(*d, prm, dtype, vec, ex.probe, stream)) <= BV_OK) return rc;
     }
 
     // A few sequences whose logits fit in L2: the launch is a matter of latency, and the kernel with two
@@ -403,7 +404,8 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
         const bv::SmallPlan plan = bv::small_plan(vecs, B, gamma, nc > 0 ? nc : 1);
         if (nc > 0 && (vec || V <= (1 << 30))) {
             StreamSlot* slot = nullptr;
-            if ((rc = stream_slot(*d, stream, 0, bv::small_scratch_bytes(B, gamma, plan), &slot)) != BV_OK) return rc;
+            rc = stream_slot(*d, stream, 0, bv::small_scratch_bytes(B, gamma, plan), &slot);
+            if (rc != BV_OK || ex.probe) return rc;
             bv::SmallScratch sc;
             // the barrier words are in the head: zero since it was allocated
             bv::small_scratch_layout(slot->scratch.p, reinterpret_cast<unsigned*>(slot->head.p + 128), B, gamma, plan, &sc);
@@ -592,10 +594,11 @@ int note_cuda_error(cudaError_t e) {
 void note_launches(int n) { t_last_launches = n; }
 
 int run_tables(int algo, const void* tgt_table, const void* drf_table, const int32_t* first, const int32_t* tok, const float* uni,
-               const float* lse_d, int B, int gamma, int V, int dtype, float T, int32_t* ot, int32_t* ol, cudaStream_t stream) {
+               const float* lse_d, int B, int gamma, int V, int dtype, float T, int32_t* ot, int32_t* ol, bool probe, cudaStream_t stream) {
     Extra ex;
     ex.lse_d = lse_d;
     ex.first = first;
+    ex.probe = probe;
     return run_device(algo, tgt_table, drf_table, tok, uni, B, gamma, V, dtype, T, ot, ol, ex, stream);
 }
 

@@ -14,8 +14,9 @@ int check_verify_args(const void* tgt, const void* drf, const int32_t* tok, cons
 int note_cuda_error(cudaError_t e);
 void note_launches(int n);
 // One verification call on rows of two tables (Params::first): BV_OK, BV_ERR_UNSUPPORTED if no kernel takes it, or an error.
+// With `probe` only that is found out: nothing is launched.
 int run_tables(int algo, const void* tgt_table, const void* drf_table, const int32_t* first, const int32_t* tok, const float* uni,
-               const float* lse_d, int B, int gamma, int V, int dtype, float T, int32_t* ot, int32_t* ol, cudaStream_t stream);
+               const float* lse_d, int B, int gamma, int V, int dtype, float T, int32_t* ot, int32_t* ol, bool probe, cudaStream_t stream);
 
 // Most clusters of `cluster` CTAs of the streaming kernel that can be resident at once
 // on the current device (0 if that cluster size cannot be scheduled).

@@ -363,16 +363,22 @@ extern "C" int bv_decode_loop(const void* target_table, const void* draft_table,
     if (!(temperature > 0.f) || !std::isfinite(temperature)) return BV_ERR_INVALID_ARG;
     if (dtype != BV_DTYPE_F32 && dtype != BV_DTYPE_BF16) return BV_ERR_INVALID_ARG;
     const size_t row_bytes = static_cast<size_t>(V) * (dtype == BV_DTYPE_F32 ? 4 : 2);
-    if (row_bytes % 16 != 0 || !aligned16(draft_table) || !aligned16(target_table) || gamma > BV_MAX_GAMMA) return BV_ERR_UNSUPPORTED;
-    bv::note_launches(0);
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (row_bytes % 16 != 0 || !aligned16(draft_table) || !aligned16(target_table) || gamma > BV_MAX_GAMMA || B > bv::kPhaseMaxB) return BV_ERR_UNSUPPORTED;
     const size_t b = static_cast<size_t>(B), width = static_cast<size_t>(iterations) * (gamma + 1);
     if (width > 0x7fffffffu) return BV_ERR_UNSUPPORTED;
+    bv::note_launches(0);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
     // work: last tokens, the last verification's outputs, the draft rows' normalisers
     int32_t* cur = work;
     int32_t* out = cur + b;
     int32_t* out_len = out + b * (gamma + 1);
     float* lse = reinterpret_cast<float*>(out_len + b);
+    auto verify = [&](int n, bool probe) {
+        return bv::run_tables(algo & 1 ? bv::kTokenVerify : bv::kBlockVerify, target_table, draft_table, cur, out_drafted + n * b * gamma,
+                              u_verify + n * b * (gamma + 2), algo < 2 ? lse : nullptr, B, gamma, V, dtype, temperature, out, out_len, probe, st);
+    };
+    int rc = verify(0, true);
+    if (rc != BV_OK) return rc;               // (before anything is enqueued)
     cudaError_t e;
     if ((e = cudaMemcpyAsync(cur, first_tokens, b * 4, cudaMemcpyDeviceToDevice, st)) != cudaSuccess ||
         (e = cudaMemsetAsync(out_tokens, 0xff, b * width * 4, st)) != cudaSuccess ||      // (-1)
@@ -382,12 +388,9 @@ extern "C" int bv_decode_loop(const void* target_table, const void* draft_table,
     bv::LoopState loop{out, nullptr, cur, out_tokens, reinterpret_cast<long long*>(out_lengths), nullptr, out_fault, static_cast<int>(width)};
     int launches = 0;
     for (int n = 0; n < iterations; ++n) {
-        int32_t* drafted = out_drafted + n * b * gamma;
-        if ((e = launch_chain(draft_table, cur, u_draft + n * b * gamma, B, gamma, V, dtype, temperature, drafted, lse, loop, st)) != cudaSuccess)
+        if ((e = launch_chain(draft_table, cur, u_draft + n * b * gamma, B, gamma, V, dtype, temperature, out_drafted + n * b * gamma, lse, loop, st)) != cudaSuccess)
             return bv::note_cuda_error(e);
-        const int rc = bv::run_tables(algo & 1 ? bv::kTokenVerify : bv::kBlockVerify, target_table, draft_table, cur, drafted, u_verify + n * b * (gamma + 2),
-                                      algo < 2 ? lse : nullptr, B, gamma, V, dtype, temperature, out, out_len, st);
-        if (rc != BV_OK) return rc;
+        if ((rc = verify(n, false)) != BV_OK) return rc;
         loop.out_len = out_len;
         loop.tau = out_tau + n * b;
         launches += 2;

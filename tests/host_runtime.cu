@@ -21,6 +21,7 @@ std::vector<std::vector<std::function<void()>>> g_graphs;
 bool g_capturing = false;
 cudaStream_t g_captured = nullptr;       // the stream that is captured
 int g_refuse_cooperative = 0;
+int g_launches = 0;
 std::string g_errors;
 
 void complain(const std::string& what) { g_errors += what + "\n"; }
@@ -104,6 +105,7 @@ int fake_stream_max_clusters(int, int, bool, int c) { return 148 / c; }
 cudaError_t fake_launch_phase(const Params& prm, const PhaseScratch& ps, int, bool, int, cudaStream_t st) {
     if (g_refuse_cooperative) return cudaErrorCooperativeLaunchTooLarge;
     const size_t B = prm.B, g = prm.gamma;
+    ++g_launches;
     return enqueue(st, [=] {
         inside("status word", prm.status, 4);
         zeros("phase counters", ps.ctr, ps.zero_words * 4);
@@ -120,6 +122,7 @@ cudaError_t fake_launch_phase(const Params& prm, const PhaseScratch& ps, int, bo
 cudaError_t fake_launch_small(const Params& prm, const SmallScratch& sc, int, bool, int, cudaStream_t st) {
     if (g_refuse_cooperative) return cudaErrorCooperativeLaunchTooLarge;
     const size_t B = prm.B, g = prm.gamma;
+    ++g_launches;
     return enqueue(st, [=] {
         inside("status word", prm.status, 4);
         zeros("barrier words", sc.barrier, 17 * 4);
@@ -130,6 +133,7 @@ cudaError_t fake_launch_small(const Params& prm, const SmallScratch& sc, int, bo
 }
 cudaError_t fake_launch_flow(const Params& prm, const FlowScratch& fl, int, int, cudaStream_t st) {
     const size_t B = prm.B, g = prm.gamma, rows = B * (g + 1);
+    ++g_launches;
     return enqueue(st, [=] {
         inside("status word", prm.status, 4);
         zeros("flow counters", fl.counters, static_cast<size_t>(fl.zero_words) * 4);
@@ -147,9 +151,11 @@ cudaError_t fake_launch_flow(const Params& prm, const FlowScratch& fl, int, int,
     });
 }
 cudaError_t fake_launch_cluster(const Params& prm, int, int, int, int, cudaStream_t st) {
+    ++g_launches;
     return enqueue(st, [=] { inside("status word", prm.status, 4); });
 }
 cudaError_t fake_launch_stream(const Params& prm, int, int, bool, int, int, cudaStream_t st) {
+    ++g_launches;
     return enqueue(st, [=] { inside("status word", prm.status, 4); });
 }
 
@@ -188,6 +194,13 @@ void host_begin_capture(void* stream) { g_graphs.emplace_back(); g_capturing = t
 int host_end_capture() { g_capturing = false; return static_cast<int>(g_graphs.size()) - 1; }
 void host_replay(int graph) { for (const auto& f : g_graphs[graph]) f(); }
 void host_refuse_cooperative(int on) { g_refuse_cooperative = on; }
+// a verification of the decoding loop
+int host_tables(int algo, int B, int gamma, int V, int dtype, int lse, int probe) {
+    void* x = reinterpret_cast<void*>(1ull << 41);
+    return bv::run_tables(algo, x, x, static_cast<int32_t*>(x), static_cast<int32_t*>(x), static_cast<float*>(x), lse ? static_cast<float*>(x) : nullptr,
+                          B, gamma, V, dtype, 1.f, static_cast<int32_t*>(x), static_cast<int32_t*>(x), probe != 0, nullptr);
+}
+int host_launches() { return g_launches; }
 // which of the elements of `esz` bytes at p lie in [lo, hi)
 void host_elements_inside(unsigned long long p, unsigned long long lo, unsigned long long hi, int esz, int* first, int* n) {
     const char *a = reinterpret_cast<const char*>(p), *b = reinterpret_cast<const char*>(lo), *c = reinterpret_cast<const char*>(hi);

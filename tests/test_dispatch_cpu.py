@@ -145,3 +145,15 @@ def test_smoke_expects_the_kernels_that_run(host):
         host.bv_set_option(b"kernel", option)
         for fn in ("bv_verify_ex", "tv_verify_ex", "gbv_verify_ex"):
             assert verify(host, B, 4, 32768, fn=fn[:-3], diagnostics=True) == (0, kernel), (B, option, fn)
+
+
+def test_a_probe_of_the_decoding_loop_says_what_the_call_does_and_launches_nothing(host):
+    for algo in (0, 1):
+        for lse in (0, 1):
+            for B, gamma, V in ((1, 1, 8), (3, 5, 4096), (33, 8, 16384), (768, 64, 32768), (769, 2, 4096), (32, 64, 65536), (3, 2, 8209), (2, 65, 4096)):
+                before = host.host_launches()
+                status = host.host_tables(algo, B, gamma, V, BF16, lse, 1)
+                assert host.host_launches() == before and host.host_errors() == b""
+                assert status == (-2 if B > 768 or V % 8 or gamma > 64 else 0)
+                assert host.host_tables(algo, B, gamma, V, BF16, lse, 0) == status
+                assert host.host_launches() == before + (status == 0)

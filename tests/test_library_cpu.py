@@ -65,6 +65,19 @@ def test_bad_arguments_are_rejected_without_a_device(lib):
     assert lib.bv_verify_host(None, p, p, p, 1, 2, 4, 0, ctypes.c_float(1.0), p, p) == -1
 
 
+def test_the_decoding_loop_refuses_before_it_touches_a_device(lib):
+    buf = (ctypes.c_float * 64)()
+    p = ctypes.addressof(buf) + -ctypes.addressof(buf) % 16
+
+    def call(iterations=2, B=3, gamma=2, V=8, dtype=0, T=1.0, algo=0, table=p):
+        return lib.bv_decode_loop(table, p, p, p, p, iterations, B, gamma, V, dtype, ctypes.c_float(T), algo, p, p, p, p, p, p, None)
+
+    for bad in (dict(table=None), dict(iterations=0), dict(B=0), dict(gamma=0), dict(V=0), dict(dtype=5), dict(T=0.0), dict(algo=4)):
+        assert call(**bad) == -1, bad
+    for bad in (dict(B=769), dict(gamma=65), dict(V=7), dict(table=p + 4), dict(B=3, iterations=2 ** 31 - 1)):
+        assert call(**bad) == -2, bad
+
+
 def test_missing_library_fails_loudly(tmp_path):
     with pytest.raises(RuntimeError):
         bv.load_library(str(tmp_path / "nope.so"))
