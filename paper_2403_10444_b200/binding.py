@@ -361,10 +361,20 @@ def bv_draft_chain(draft_table, first_tokens, uniforms, temperature: float = 1.0
 
 
 def bv_decode_loop(target_table, draft_table, first_tokens, u_draft, u_verify, gamma: int, temperature: float, algo: int):
-    """The decoding loop for two last-token table models (see include/bv.h; contiguous CUDA tensors, algo as there): (tokens,
+    """The decoding loop for two last-token table models (see include/bv.h; contiguous CUDA tensors, all checked, algo as there): (tokens,
     lengths, tau, drafted, fault), or None where the library has no kernel for the call."""
+    V = target_table.shape[0]
+    if target_table.shape != (V, V) or draft_table.shape != (V, V) or target_table.dtype != draft_table.dtype:
+        raise ValueError("the model tables must be [V, V] of one dtype")
+    if first_tokens.dim() != 1 or first_tokens.dtype != torch.int32:
+        raise ValueError("first_tokens must be int32 [B]")
+    N, B = u_draft.shape[0], first_tokens.shape[0]
+    if u_draft.shape != (N, gamma, B) or u_verify.shape != (N, B, gamma + 2) or u_draft.dtype != torch.float32 or u_verify.dtype != torch.float32:
+        raise ValueError("u_draft must be float32 [N, gamma, B] and u_verify float32 [N, B, gamma+2]")
+    for t in (target_table, draft_table, first_tokens, u_draft, u_verify):
+        if not t.is_contiguous() or not t.is_cuda or t.device != target_table.device:
+            raise ValueError("expected contiguous CUDA tensors on one device")
     lib = load_library()
-    N, B, V = u_draft.shape[0], first_tokens.shape[0], target_table.shape[0]
     dev = target_table.device
     i32 = lambda *shape: torch.empty(shape, dtype=torch.int32, device=dev)
     tokens, tau, drafted, fault = i32(B, N * (gamma + 1)), i32(N, B), i32(N, B, gamma), i32(1)

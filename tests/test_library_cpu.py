@@ -78,6 +78,21 @@ def test_the_decoding_loop_refuses_before_it_touches_a_device(lib):
         assert call(**bad) == -2, bad
 
 
+def test_the_decoding_loop_checks_its_tensors():
+    import torch
+    from paper_2403_10444_b200 import binding
+    f, i = torch.float32, torch.int32
+    good = dict(target_table=torch.zeros(8, 8), draft_table=torch.zeros(8, 8), first_tokens=torch.zeros(3, dtype=i),
+                u_draft=torch.zeros(4, 2, 3), u_verify=torch.zeros(4, 3, 4), gamma=2, temperature=1.0, algo=0)
+    bad = [dict(target_table=torch.zeros(8, 16)), dict(draft_table=torch.zeros(16, 16)), dict(draft_table=torch.zeros(8, 8, dtype=torch.bfloat16)),
+           dict(first_tokens=torch.zeros(3, dtype=torch.int64)), dict(first_tokens=torch.zeros(3, 1, dtype=i)), dict(u_draft=torch.zeros(4, 3, 3)),
+           dict(u_draft=torch.zeros(4, 2, 3, dtype=torch.float64)), dict(u_verify=torch.zeros(3, 3, 4)), dict(u_verify=torch.zeros(4, 3, 5)),
+           dict(draft_table=torch.zeros(16, 16)[:8, :8]), dict(u_draft=torch.zeros(3, 2, 4).transpose(0, 2)), {}]      # (the last: not on a GPU)
+    for b in bad:
+        with pytest.raises((ValueError, TypeError)):
+            binding.bv_decode_loop(**dict(good, **b))
+
+
 def test_missing_library_fails_loudly(tmp_path):
     with pytest.raises(RuntimeError):
         bv.load_library(str(tmp_path / "nope.so"))
