@@ -248,6 +248,14 @@ int pick_cluster(const DeviceState& d, const Options& opt, int B, size_t row_byt
     return c;
 }
 
+// Did a kernel that needs a CTA on every SM at once find fewer (a process that is given a part of the GPU)?  The kernels
+// that need no such thing take the call.
+bool not_all_sms(cudaError_t e) {
+    if (e != cudaErrorCooperativeLaunchTooLarge) return false;
+    cudaGetLastError();
+    return true;
+}
+
 // Where the element-wise kernel is still the default: a few short unaligned rows a sequence, one sequence an SM at most,
 // whose dependent steps cost less than the phase kernel's waits for the whole batch.  Measured, V = 1001 / 2051 / 4099 bf16:
 // Algorithm 1, B = 100, gamma = 3: 24 / 26 / 30 us against 31 / 39 / 40; Algorithm 2, gamma = 2: 26 / 29 / 36 against 33 / 39 / 39
@@ -324,6 +332,7 @@ int run_phase(DeviceState& d, const bv::Params& prm, int dtype, bool vec, bool p
         if (p.B != part) plan = bv::phase_plan(p.V, dtype, vec, p.B, g, p.lse_d != nullptr, nc);
         bv::phase_scratch(slot->scratch.p, reinterpret_cast<unsigned*>(slot->head.p + kSlotPhase), p.B, g, plan, &ps);
         const cudaError_t e = bv::launch_phase(p, ps, dtype, vec, nc, stream);
+        if (launches == 0 && not_all_sms(e)) return 1;
         if (e != cudaSuccess) return cuda_fail(e);
     }
     t_last_launches = launches; t_last_kernel = 5;
@@ -412,10 +421,12 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
             prm.ticket = nullptr;
             prm.nclusters = 0;
             prm.status = reinterpret_cast<int*>(slot->head.p);
-            cudaError_t e = bv::launch_small(prm, sc, dtype, vec, nc, stream);
-            if (e != cudaSuccess) return cuda_fail(e);
-            t_last_launches = 1; t_last_kernel = 4;
-            return BV_OK;
+            const cudaError_t e = bv::launch_small(prm, sc, dtype, vec, nc, stream);
+            if (e == cudaSuccess) {
+                t_last_launches = 1; t_last_kernel = 4;
+                return BV_OK;
+            }
+            if (!not_all_sms(e)) return cuda_fail(e);
         }
     }
 

@@ -157,3 +157,19 @@ def test_a_probe_of_the_decoding_loop_says_what_the_call_does_and_launches_nothi
                 assert status == (-2 if B > 768 or V % 8 or gamma > 64 else 0)
                 assert host.host_tables(algo, B, gamma, V, BF16, lse, 0) == status
                 assert host.host_launches() == before + (status == 0)
+
+
+def test_without_room_for_a_cooperative_launch_another_kernel_takes_the_call(host):
+    # (a part of the GPU's SMs only, as under a percentage of its threads: the kernels that need one CTA on every SM are refused)
+    host.host_refuse_cooperative(1)
+    try:
+        for fn in ("bv_verify", "tv_verify", "gbv_verify", "bv_verify_lse", "bv_verify_probs"):
+            for B in (2, 12, 40, 800):
+                for V in (4096, 128256) + ((50257,) if fn in ("bv_verify", "tv_verify") else ()):
+                    assert verify(host, B, 5, V, fn=fn) == (0, 3 if V % 8 else 1), (fn, B, V)
+        assert host.host_tables(1, 40, 5, 4096, BF16, 1, 0) == -2
+        host.bv_set_option(b"kernel", 5)
+        assert verify(host, 40, 5, 4096) == (0, 2)
+    finally:
+        host.host_refuse_cooperative(0)
+    assert host.host_errors() == b"" and host.bv_last_cuda_error() == 0
