@@ -49,13 +49,44 @@ __device__ __forceinline__ void s_range(int units, int warp, int sub, int& a0, i
     a1 = min(a0 + runs * 32, u1);
 }
 
+// What a sub-segment leaves: its reference and its sum, in two parts that are added in double where the pairs are combined.
+// The vectors that are joined in fp32 decide the precision of a normaliser.  In rows of 2048 vectors and more the parts are the
+// sums of sixteen lanes each (of at most 32 vectors below 8192); in shorter ones (SHORT), of few vectors to a sub-segment, the
+// lanes are joined in double.  (All 32 lanes joined in fp32: relative error of the normaliser of rows with a flat law 5.8e-9 on
+// average at 1024 vectors, 4.1e-9 at 5000, where equal sub-segments of 8 and 39 vectors gave 2.5e-9 and 2.8e-9; like this 1.0e-9
+// and 2.7e-9.  The double costs a step of a drafting chain at 128 vectors a row 0.2 of 3.1 us, nothing from 1024 vectors on.)
+template <bool SHORT> struct alignas(16) SubSegment { float2 a, b; };                  // {sum of lanes 0 .. 15, M}, {of lanes 16 .. 31, M}
+template <> struct alignas(16) SubSegment<true> { double z; float2 b; };              // {sum}, {M, -}
+constexpr bool s_short(size_t row_bytes) { return row_bytes < static_cast<size_t>(2048) * 16; }
+// (sub-segment `sub` of warp `warp` lies where lane (8 warp + sub) / 4 of the sampling warp finds it without bank conflicts)
+__device__ __forceinline__ int s_place(int warp, int sub) { return (sub & 3) * 32 + warp * (kSSub / 4) + (sub >> 2); }
+template <bool SHORT>
+__device__ __forceinline__ void s_put(float M, float s, int lane, SubSegment<SHORT>* to) {
+    float2 v = make_float2(s, M);
+    if (SHORT) {
+        const double z = warp_sum_d(static_cast<double>(s));
+        v = lane == 0 ? make_float2(__int_as_float(__double2loint(z)), __int_as_float(__double2hiint(z))) : make_float2(M, 0.f);
+    } else {
+#pragma unroll
+        for (int off = 8; off > 0; off >>= 1) v.x += __shfl_xor_sync(0xffffffffu, v.x, off);
+    }
+    if ((lane & 15) == 0) reinterpret_cast<float2*>(to)[lane >> 4] = v;
+}
+__device__ __forceinline__ SubSegment<true> s_empty(SubSegment<true>*) { return {0.0, make_float2(kNoRef, 0.f)}; }
+__device__ __forceinline__ SubSegment<false> s_empty(SubSegment<false>*) { return {make_float2(0.f, kNoRef), make_float2(0.f, kNoRef)}; }
+template <bool SHORT>
+__device__ __forceinline__ void s_get(const SubSegment<SHORT>& from, float& M, double& z, float& za, float& zb) {
+    if constexpr (SHORT) { M = from.b.x; z = from.z; }
+    else { M = from.a.y; za = from.a.x; zb = from.b.x; }
+}
+
 // One streaming warp's pass over its sixteenth of a row: the {reference, sum} pair of each of its
-// sub-segments goes to sM / sS.  The loads of kSInFlight runs are issued together whatever sub-segments they
+// sub-segments goes to `seg`.  The loads of kSInFlight runs are issued together whatever sub-segments they
 // belong to.  (With one sub-segment's loads at a time a row of 2048 vectors, 16 to a sub-segment, waited for memory eight
 // times: a step of a drafting chain, B = 128 sequences of 16384 bf16 logits, 13 us, now 5 us; 2048 rows of 128256 logits,
 // 125 vectors to a sub-segment, 140 us, now 113 us: 4.7 TB/s.)
-template <int DT>
-__device__ __forceinline__ void s_sweep_row(const char* row, int units, float kf, int warp, int lane, float* sM, float* sS) {
+template <int DT, bool SHORT>
+__device__ __forceinline__ void s_sweep_row(const char* row, int units, float kf, int warp, int lane, SubSegment<SHORT>* seg) {
     using R = Raw<DT>;
     constexpr int EPV = R::EPV;
     // (the warp's reference carries over from one sub-segment to the next: a sub-segment's pair is
@@ -79,8 +110,7 @@ __device__ __forceinline__ void s_sweep_row(const char* row, int units, float kf
                 R::unpack(raw[j], v);
                 f_accumulate<EPV>(v, kf, M, s);
                 if (--left == 0) {                // the end of a sub-segment
-                    s = warp_sum(s);
-                    if (lane == 0) { sM[warp * kSSub + sub] = M; sS[warp * kSSub + sub] = s; }
+                    s_put<SHORT>(M, s, lane, seg + s_place(warp, sub));
                     ++sub;
                     left = runs;
                     s = 0.f;
@@ -89,29 +119,31 @@ __device__ __forceinline__ void s_sweep_row(const char* row, int units, float kf
         }
     }
     if (left < runs) {
-        s = warp_sum(s);
-        if (lane == 0) { sM[warp * kSSub + sub] = M; sS[warp * kSSub + sub] = s; }
+        s_put<SHORT>(M, s, lane, seg + s_place(warp, sub));
         ++sub;
     }
-    if (lane >= sub && lane < kSSub) { sM[warp * kSSub + lane] = kNoRef; sS[warp * kSSub + lane] = 0.f; }
+    if (lane >= sub && lane < kSSub) seg[s_place(warp, lane)] = s_empty(seg);
 }
 
 // The sampling warp's part: the row's normaliser from the 128 pairs and the token that the uniform u
 // selects (inverse CDF in index order; -1 and a NaN normaliser for a row with a NaN or +inf logit or
 // without a finite one).  release_pairs >= 0: a named barrier at which the warp arrives once it has
 // read the pairs.
-template <int DT>
-__device__ __forceinline__ int s_draw_row(const char* row, int units, float kf, const float* sM, const float* sS, float u,
+template <int DT, bool SHORT>
+__device__ __forceinline__ int s_draw_row(const char* row, int units, float kf, const SubSegment<SHORT>* seg, float u,
                                           int lane, int release_pairs, double* norm) {
     // ---- normaliser and the sampled sub-segment (fp64 prefix sums, index order) ----
-    float m[4], w[4];
+    float m[4], za[4], zb[4];
+    double w[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) { m[j] = sM[4 * lane + j]; w[j] = sS[4 * lane + j]; }
+    for (int j = 0; j < 4; ++j) s_get<SHORT>(seg[32 * j + lane], m[j], w[j], za[j], zb[j]);
     const float Mrow = warp_max(fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])));
 #pragma unroll
-    for (int j = 0; j < 4; ++j) w[j] *= ref_scale(m[j], Mrow);
-    double Z = (static_cast<double>(w[0]) + static_cast<double>(w[1])) +
-               (static_cast<double>(w[2]) + static_cast<double>(w[3]));
+    for (int j = 0; j < 4; ++j) {
+        const float to = ref_scale(m[j], Mrow);
+        w[j] = SHORT ? w[j] * static_cast<double>(to) : static_cast<double>(za[j] * to) + static_cast<double>(zb[j] * to);
+    }
+    double Z = (w[0] + w[1]) + (w[2] + w[3]);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) Z += shfl_xor_d(Z, off);
     // (the sums over sub-segments that locate the sample are formed in double: a token's cell can
@@ -134,8 +166,8 @@ __device__ __forceinline__ int s_draw_row(const char* row, int units, float kf, 
         if (lane == 0) exc = 0.0;
         const double p0 = exc, p1 = exc + l1, p2 = exc + l2, p3 = exc + l3, p4 = exc + l4;
         // first non-empty sub-segment whose inclusive prefix exceeds t, else the last non-empty one
-        const bool h1 = p1 > t && w[0] > 0.f, h2 = p2 > t && w[1] > 0.f;
-        const bool h3 = p3 > t && w[2] > 0.f, h4 = p4 > t && w[3] > 0.f;
+        const bool h1 = p1 > t && w[0] > 0.0, h2 = p2 > t && w[1] > 0.0;
+        const bool h3 = p3 > t && w[2] > 0.0, h4 = p4 > t && w[3] > 0.0;
         const unsigned hit = __ballot_sync(0xffffffffu, h1 || h2 || h3 || h4);
         const unsigned nz = __ballot_sync(0xffffffffu, l4 > 0.0);
         int e = 3; double bef = p3; int src;
@@ -145,8 +177,8 @@ __device__ __forceinline__ int s_draw_row(const char* row, int units, float kf, 
         } else {
             src = 31 - __clz(nz);
             e = 0; bef = p0;
-            if (w[3] > 0.f) { e = 3; bef = p3; } else if (w[2] > 0.f) { e = 2; bef = p2; }
-            else if (w[1] > 0.f) { e = 1; bef = p1; }
+            if (w[3] > 0.0) { e = 3; bef = p3; } else if (w[2] > 0.0) { e = 2; bef = p2; }
+            else if (w[1] > 0.0) { e = 1; bef = p1; }
         }
         const int sel = __shfl_sync(0xffffffffu, 4 * lane + e, src);
         const double before = shfl_d(bef, src);
@@ -163,7 +195,7 @@ __device__ __forceinline__ float s_lse(int found, const double* norm) {
     return found >= 0 ? static_cast<float>((norm[0] + log2(norm[1])) * 0.693147180559945309417232) : __int_as_float(0x7fc00000);
 }
 
-template <int DT>
+template <int DT, bool SHORT>
 __global__ void __launch_bounds__(kSAllThreads, 2)
 sample_rows_kernel(const char* logits, const float* uni, int rows, int V, float kf, int32_t* tokens, float* lse) {
     using R = Raw<DT>;
@@ -172,7 +204,7 @@ sample_rows_kernel(const char* logits, const float* uni, int rows, int V, float 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int units = V / EPV;
     const size_t row_bytes = static_cast<size_t>(V) * ESZ;
-    __shared__ float sM2[2][kSSegs], sS2[2][kSSegs];
+    __shared__ SubSegment<SHORT> seg[2][kSSegs];
 
     // The streaming warps sweep the CTA's rows one after the other and leave each row's pairs in one of
     // two buffers; the sampling warp follows, a row behind or so, and draws each row's token from them.
@@ -187,7 +219,7 @@ sample_rows_kernel(const char* logits, const float* uni, int rows, int V, float 
         for (int it = 0; it < nmine; ++it) {
             if (it >= 2) named_bar_sync(kBarEmpty + (it & 1), kSAllThreads);
             const int r = blockIdx.x + it * gridDim.x;
-            s_sweep_row<DT>(logits + static_cast<size_t>(r) * row_bytes, units, kf, warp, lane, sM2[it & 1], sS2[it & 1]);
+            s_sweep_row<DT, SHORT>(logits + static_cast<size_t>(r) * row_bytes, units, kf, warp, lane, seg[it & 1]);
             __threadfence_block();
             named_bar_arrive(kBarFull + (it & 1), kSAllThreads);
         }
@@ -197,7 +229,7 @@ sample_rows_kernel(const char* logits, const float* uni, int rows, int V, float 
             const int r = blockIdx.x + it * gridDim.x;
             double norm[2];
             // (row it + 2 waits for the release of this buffer; the last two rows have nobody waiting)
-            const int found = s_draw_row<DT>(logits + static_cast<size_t>(r) * row_bytes, units, kf, sM2[it & 1], sS2[it & 1], uni[r],
+            const int found = s_draw_row<DT, SHORT>(logits + static_cast<size_t>(r) * row_bytes, units, kf, seg[it & 1], uni[r],
                                              lane, it + 2 < nmine ? kBarEmpty + (it & 1) : -1, norm);
             if (lane == 0) {
                 tokens[r] = found;
@@ -244,7 +276,7 @@ __global__ void extend_kernel(const LoopState loop, int B, int gamma) {
     if (b < B) extend_sequence(loop, b, gamma, threadIdx.x & 31);
 }
 
-template <int DT>
+template <int DT, bool SHORT>
 __global__ void __launch_bounds__(kSAllThreads, 2)
 draft_chain_kernel(const char* table, const int32_t* first, const float* uni, int B, int gamma, int V, float kf,
                    int32_t* tokens, float* lse, const LoopState loop) {
@@ -254,7 +286,7 @@ draft_chain_kernel(const char* table, const int32_t* first, const float* uni, in
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int units = V / EPV;
     const size_t row_bytes = static_cast<size_t>(V) * ESZ;
-    __shared__ float sM[kSSegs], sS[kSSegs];
+    __shared__ SubSegment<SHORT> seg[kSSegs];
     __shared__ int s_next[2];
     for (int b = blockIdx.x; b < B; b += gridDim.x) {
         if (loop.out_len != nullptr) {
@@ -265,13 +297,13 @@ draft_chain_kernel(const char* table, const int32_t* first, const float* uni, in
         for (int i = 0; i < gamma; ++i) {
             const bool ok = last >= 0 && last < V;
             const char* row = table + static_cast<size_t>(ok ? last : 0) * row_bytes;
-            if (warp < kSWarps && ok) s_sweep_row<DT>(row, units, kf, warp, lane, sM, sS);
+            if (warp < kSWarps && ok) s_sweep_row<DT, SHORT>(row, units, kf, warp, lane, seg);
             const float u = uni[static_cast<size_t>(i) * B + b];
             __syncthreads();
             int found = -1;
             double norm[2] = {0.0, 0.0};
             if (warp == kSWarps) {
-                if (ok) found = s_draw_row<DT>(row, units, kf, sM, sS, u, lane, -1, norm);
+                if (ok) found = s_draw_row<DT, SHORT>(row, units, kf, seg, u, lane, -1, norm);
                 if (lane == 0) s_next[i & 1] = found;
             }
             __syncthreads();
@@ -308,10 +340,10 @@ extern "C" int bv_sample_draft(const void* logits, const float* uniforms, int ro
     const int grid = rows < 2 * sms ? rows : 2 * sms;
     const float kf = static_cast<float>(1.4426950408889634 / static_cast<double>(temperature));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (dtype == BV_DTYPE_F32)
-        bv::sample_rows_kernel<bv::kF32><<<grid, bv::kSAllThreads, 0, st>>>(static_cast<const char*>(logits), uniforms, rows, V, kf, out_tokens, out_lse);
-    else
-        bv::sample_rows_kernel<bv::kBF16><<<grid, bv::kSAllThreads, 0, st>>>(static_cast<const char*>(logits), uniforms, rows, V, kf, out_tokens, out_lse);
+    const bool f32 = dtype == BV_DTYPE_F32, brief = bv::s_short(row_bytes);
+    const auto kernel = f32 ? (brief ? bv::sample_rows_kernel<bv::kF32, true> : bv::sample_rows_kernel<bv::kF32, false>)
+                            : (brief ? bv::sample_rows_kernel<bv::kBF16, true> : bv::sample_rows_kernel<bv::kBF16, false>);
+    kernel<<<grid, bv::kSAllThreads, 0, st>>>(static_cast<const char*>(logits), uniforms, rows, V, kf, out_tokens, out_lse);
     e = cudaGetLastError();
     if (e != cudaSuccess) return bv::note_cuda_error(e);
     bv::note_launches(1);
@@ -328,10 +360,10 @@ cudaError_t launch_chain(const void* table, const int32_t* first, const float* u
     if (e != cudaSuccess) return e;
     const int grid = B < 2 * sms ? B : 2 * sms;
     const float kf = static_cast<float>(1.4426950408889634 / static_cast<double>(temperature));
-    if (dtype == BV_DTYPE_F32)
-        bv::draft_chain_kernel<bv::kF32><<<grid, bv::kSAllThreads, 0, st>>>(static_cast<const char*>(table), first, uni, B, gamma, V, kf, tokens, lse, loop);
-    else
-        bv::draft_chain_kernel<bv::kBF16><<<grid, bv::kSAllThreads, 0, st>>>(static_cast<const char*>(table), first, uni, B, gamma, V, kf, tokens, lse, loop);
+    const bool f32 = dtype == BV_DTYPE_F32, brief = bv::s_short(static_cast<size_t>(V) * (f32 ? 4 : 2));
+    const auto kernel = f32 ? (brief ? bv::draft_chain_kernel<bv::kF32, true> : bv::draft_chain_kernel<bv::kF32, false>)
+                            : (brief ? bv::draft_chain_kernel<bv::kBF16, true> : bv::draft_chain_kernel<bv::kBF16, false>);
+    kernel<<<grid, bv::kSAllThreads, 0, st>>>(static_cast<const char*>(table), first, uni, B, gamma, V, kf, tokens, lse, loop);
     return cudaGetLastError();
 }
 }  // namespace

@@ -82,3 +82,26 @@ def test_sampler_domain_errors_and_refusals():
         bv.bv_sample_draft(torch.zeros((2, 5)).cuda(), u[:2].cuda(), 1.0)
     with pytest.raises(bv.BVError):
         bv.bv_sample_draft(z.cuda(), u.cuda(), 0.0)
+
+
+@pytest.mark.parametrize("V,large", [(1024, lambda i: i % 8 == 0), (4096, lambda i: i % 8 == 0), (16384, lambda i: i % 32 < 16)])
+def test_vectors_of_a_short_row_are_joined_in_double(V, large):
+    # Weights that are powers of two: the sum of the large vectors is 1, the others' sum is less than half an fp32 ulp of what
+    # it would have to be added to if more than one vector (long rows: sixteen) were summed in fp32.  A scale log2(e) / T that
+    # rounds to 1 keeps every weight and every sum exact, so the normaliser is ln(1 + tiny), known to fp32.
+    import paper_2403_10444_b200 as bv
+    T = float(np.float32(1.4426950408889634))
+    i = np.arange(V // 8)
+    big = np.array([large(int(x)) for x in i])
+    shift = -int(np.log2(8 * big.sum()))
+    assert 2.0 ** -shift == 8 * big.sum()
+    z = np.repeat(np.where(big, shift, shift - 26), 8).astype(np.float32)
+    tiny = float(np.sum(np.exp2(z.astype(np.float64))) - 1.0)
+    assert 1e-9 < tiny < 2.0 ** -22
+    row = torch.from_numpy(z).bfloat16().cuda()
+    _, lse = bv.bv_sample_draft(row.expand(3, V).contiguous(), torch.full((3,), 0.5, device="cuda"), T)
+    assert np.abs(lse.cpu().numpy().astype(np.float64) / np.log1p(tiny) - 1.0).max() < 1e-4
+    if V <= 4096:
+        first = torch.zeros((2,), dtype=torch.int32, device="cuda")
+        _, lse = bv.bv_draft_chain(row.expand(V, V).contiguous(), first, torch.full((3, 2), 0.5, device="cuda"), T)
+        assert np.abs(lse.cpu().numpy().astype(np.float64) / np.log1p(tiny) - 1.0).max() < 1e-4
