@@ -371,9 +371,10 @@ def bv_decode_loop(target_table, draft_table, first_tokens, u_draft, u_verify, g
     N, B = u_draft.shape[0], first_tokens.shape[0]
     if u_draft.shape != (N, gamma, B) or u_verify.shape != (N, B, gamma + 2) or u_draft.dtype != torch.float32 or u_verify.dtype != torch.float32:
         raise ValueError("u_draft must be float32 [N, gamma, B] and u_verify float32 [N, B, gamma+2]")
-    for t in (target_table, draft_table, first_tokens, u_draft, u_verify):
-        if not t.is_contiguous() or not t.is_cuda or t.device != target_table.device:
-            raise ValueError("expected contiguous CUDA tensors on one device")
+    if not (target_table.is_contiguous() and draft_table.is_contiguous() and first_tokens.is_contiguous() and u_draft.is_contiguous() and u_verify.is_contiguous()):
+        raise ValueError("all tensors must be contiguous")
+    if not (0 <= target_table.get_device() == draft_table.get_device() == first_tokens.get_device() == u_draft.get_device() == u_verify.get_device()):
+        raise ValueError("expected CUDA tensors on one device")
     lib = load_library()
     dev = target_table.device
     i32 = lambda *shape: torch.empty(shape, dtype=torch.int32, device=dev)

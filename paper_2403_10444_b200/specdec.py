@@ -154,8 +154,7 @@ def _native(target_table, draft_table, first_tokens, u_draft, u_verify, gamma) -
             and target_table.dtype == draft_table.dtype and target_table.dtype in (torch.float32, torch.bfloat16)
             and target_table.is_contiguous() and draft_table.is_contiguous()
             and u_draft.dtype == torch.float32 and u_verify.dtype == torch.float32
-            and first_tokens.dtype in (torch.int32, torch.int64) and first_tokens.dim() == 1
-            and all(t.device == dev for t in (draft_table, first_tokens, u_draft, u_verify)))
+            and first_tokens.dtype in (torch.int32, torch.int64) and first_tokens.dim() == 1)
 
 
 def block_efficiency(result) -> float:
