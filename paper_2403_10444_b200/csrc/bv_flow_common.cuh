@@ -139,13 +139,42 @@ struct FlowCtx {
     double kd;
 };
 
-// One warp walks vectors [w0, w1) of a row pair in index order and returns the first element
+// Of the EPV elements at p, those from `first` on and below `n` lie in the tensor [lo, hi).
+template <int EPV>
+__host__ __device__ __forceinline__ void elements_inside(const char* p, const char* lo, const char* hi, int& first, int& n) {
+    constexpr int ESZ = 16 / EPV;
+    first = p < lo ? static_cast<int>((lo - p) / ESZ) : 0;
+    const long long left = (hi - p) / ESZ;                   // (up to the end of the tensor: more than an int holds)
+    n = left < EPV ? static_cast<int>(left) : EPV;
+}
+// Sixteen bytes of a row from element x0 on, elements outside [0, V) as `pad` (rows at any alignment, one at a time).
+template <int DT>
+__device__ __forceinline__ uint4 row_elements(const char* row, int x0, int V, uint32_t pad) {
+    uint32_t w[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (DT == kF32) {
+            const int x = x0 + j;
+            w[j] = x >= 0 && x < V ? __ldg(reinterpret_cast<const unsigned*>(row) + x) : pad;
+        } else {
+            const int x = x0 + 2 * j;
+            const uint32_t l = x >= 0 && x < V ? __ldg(reinterpret_cast<const unsigned short*>(row) + x) : (pad & 0xffffu);
+            const uint32_t h = x + 1 >= 0 && x + 1 < V ? __ldg(reinterpret_cast<const unsigned short*>(row) + x + 1) : (pad & 0xffffu);
+            w[j] = l | (h << 16);
+        }
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+// One warp walks segment [w0, w1) of a row pair in index order and returns the first element
 // whose running residual mass exceeds tw (else the last element with positive mass, else -1).
-// load(i, in, rp, rq): vector i of both rows, or what weighs nothing if it is not `in` the range.
-template <int DT, bool PROBS, int kAhead, class LoadFn>    // kAhead: runs of 32 vectors whose loads are in flight together
-__device__ __forceinline__ int f_rescan_with(LoadFn load, bool have_q, int w0, int w1, int lane, float kf, float cp,
-                                             float nMP, float nMQ, double tw) {
+// (AL: rows of whole 16-byte vectors.  Otherwise the rows hold V elements, vector 0 begins h elements before them, and the
+// elements count from there.  The choice is made where the vectors are loaded and nowhere else: with the loads handed in as a
+// function object the flow kernel spilled 4 bytes more and 256 sequences of V = 256000 took 0.6 % longer.)
+template <int DT, bool PROBS = false, int kAhead = 4, bool AL = true>      // kAhead: runs of 32 vectors whose loads are in flight together
+__device__ int f_rescan(const char* rowP, const char* rowQ, int w0, int w1, int lane, float kf, float cp,
+                        float nMP, float nMQ, double tw, int V = 0, int h = 0) {
     constexpr int EPV = Raw<DT>::EPV;
+    constexpr uint32_t kPad = PROBS ? 0u : Raw<DT>::kNegInf;   // an element beyond the segment weighs nothing
     // The terms are the fp32 values of the sweeps; their running sum, which decides the token, is
     // kept in fp64 (a cell of the distribution can be far narrower than fp32 resolves next to the
     // mass before it).
@@ -158,7 +187,14 @@ __device__ __forceinline__ int f_rescan_with(LoadFn load, bool have_q, int w0, i
 #pragma unroll
         for (int a = 0; a < kAhead; ++a) {
             const int i = base0 + 32 * a + lane;
-            load(i, i < w1, rp[a], rq[a]);
+            const bool ok = i < w1;
+            if (AL) {
+                rp[a] = ok ? ld_stream_v4(rowP + static_cast<size_t>(i) * 16) : make_uint4(kPad, kPad, kPad, kPad);
+                rq[a] = (ok && rowQ) ? ld_stream_v4(rowQ + static_cast<size_t>(i) * 16) : make_uint4(kPad, kPad, kPad, kPad);
+            } else {
+                rp[a] = ok ? row_elements<DT>(rowP, i * EPV - h, V, kPad) : make_uint4(kPad, kPad, kPad, kPad);
+                rq[a] = (ok && rowQ) ? row_elements<DT>(rowQ, i * EPV - h, V, kPad) : make_uint4(kPad, kPad, kPad, kPad);
+            }
         }
 #pragma unroll
         for (int a = 0; a < kAhead; ++a) {
@@ -168,7 +204,7 @@ __device__ __forceinline__ int f_rescan_with(LoadFn load, bool have_q, int w0, i
             float vp[EPV], vq[EPV], tt[EPV];
             Raw<DT>::unpack(rp[a], vp);
             Raw<DT>::unpack(rq[a], vq);
-            if (have_q) f_pair_sum<EPV, true, PROBS>(vp, vq, kf, cp, nMP, nMQ, tt);
+            if (rowQ) f_pair_sum<EPV, true, PROBS>(vp, vq, kf, cp, nMP, nMQ, tt);
             else f_pair_sum<EPV, false, PROBS>(vp, vq, kf, cp, nMP, nMQ, tt);
             double ls = 0.0;
 #pragma unroll
@@ -210,17 +246,6 @@ __device__ __forceinline__ int f_rescan_with(LoadFn load, bool have_q, int w0, i
     return found;
 }
 
-// ... of rows of whole 16-byte vectors
-template <int DT, bool PROBS = false, int kAhead = 4>
-__device__ int f_rescan(const char* rowP, const char* rowQ, int w0, int w1, int lane, float kf, float cp,
-                        float nMP, float nMQ, double tw) {
-    constexpr uint32_t kPad = PROBS ? 0u : Raw<DT>::kNegInf;   // an element beyond the segment weighs nothing
-    return f_rescan_with<DT, PROBS, kAhead>([&](int i, bool in, uint4& rp, uint4& rq) {
-        rp = in ? ld_stream_v4(rowP + static_cast<size_t>(i) * 16) : make_uint4(kPad, kPad, kPad, kPad);
-        rq = (in && rowQ) ? ld_stream_v4(rowQ + static_cast<size_t>(i) * 16) : make_uint4(kPad, kPad, kPad, kPad);
-    }, rowQ != nullptr, w0, w1, lane, kf, cp, nMP, nMQ, tw);
-}
-
 // ---- rows at any alignment: a row is read as the aligned vectors that its bytes lie in; what of the first and the last
 // of them belongs to its neighbours weighs nothing ----
 // row start -> first 16-byte vector, elements of it that belong to the row before, vectors
@@ -241,44 +266,13 @@ template <int EPV> __device__ __forceinline__ void row_mask(float (&v)[EPV], int
         if (x < 0 || x >= V) v[e] = pad;
     }
 }
-// Of the EPV elements at p, those from `first` on and below `n` lie in the tensor [lo, hi).
-template <int EPV>
-__host__ __device__ __forceinline__ void elements_inside(const char* p, const char* lo, const char* hi, int& first, int& n) {
-    constexpr int ESZ = 16 / EPV;
-    first = p < lo ? static_cast<int>((lo - p) / ESZ) : 0;
-    const long long left = (hi - p) / ESZ;                   // (up to the end of the tensor: more than an int holds)
-    n = left < EPV ? static_cast<int>(left) : EPV;
-}
-// Sixteen bytes of a row from element x0 on, elements outside [0, V) as `pad` (rows at any alignment, one at a time).
-template <int DT>
-__device__ __forceinline__ uint4 row_elements(const char* row, int x0, int V, uint32_t pad) {
-    uint32_t w[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        if (DT == kF32) {
-            const int x = x0 + j;
-            w[j] = x >= 0 && x < V ? __ldg(reinterpret_cast<const unsigned*>(row) + x) : pad;
-        } else {
-            const int x = x0 + 2 * j;
-            const uint32_t l = x >= 0 && x < V ? __ldg(reinterpret_cast<const unsigned short*>(row) + x) : (pad & 0xffffu);
-            const uint32_t h = x + 1 >= 0 && x + 1 < V ? __ldg(reinterpret_cast<const unsigned short*>(row) + x + 1) : (pad & 0xffffu);
-            w[j] = l | (h << 16);
-        }
-    }
-    return make_uint4(w[0], w[1], w[2], w[3]);
-}
 // ... the rescan: vectors [w0, w1) on the target row's grid
 template <int DT, bool PROBS, int kAhead>
 __device__ int f_rescan_any(const char* rowP, const char* rowQ, int V, int w0, int w1, int lane, float kf, float cp,
                             float nMP, float nMQ, double tw) {
-    constexpr uint32_t kPad = PROBS ? 0u : Raw<DT>::kNegInf;
-    constexpr int EPV = Raw<DT>::EPV;
     const char* base; int h, nv;
     row_grid<DT, false>(rowP, V, base, h, nv);
-    const int found = f_rescan_with<DT, PROBS, kAhead>([&](int i, bool in, uint4& rp, uint4& rq) {
-        rp = in ? row_elements<DT>(rowP, i * EPV - h, V, kPad) : make_uint4(kPad, kPad, kPad, kPad);
-        rq = in && rowQ ? row_elements<DT>(rowQ, i * EPV - h, V, kPad) : make_uint4(kPad, kPad, kPad, kPad);
-    }, rowQ != nullptr, w0, w1 < nv ? w1 : nv, lane, kf, cp, nMP, nMQ, tw);
+    const int found = f_rescan<DT, PROBS, kAhead, false>(rowP, rowQ, w0, w1 < nv ? w1 : nv, lane, kf, cp, nMP, nMQ, tw, V, h);
     return found >= 0 ? found - h : found;
 }
 
