@@ -18,7 +18,8 @@ constexpr int kMaxDevices = 64;
 constexpr int kTicketSlots = 64;  // concurrent calls of the cluster kernels on one device each need their own slot
 // Logit bytes up to which the small-batch kernel is the default (measured against the flow kernel at
 // V = 152064, B <= 32: Algorithm 2 gains up to about 90 MB at low and high acceptance alike, Algorithm 1,
-// whose one residual sweep per sequence is cheap, up to about 160 MB)
+// whose one residual sweep per sequence is cheap, up to about 160 MB).  The phase kernel takes over below that, but for few
+// sequences or many positions swept (phase_pays).
 constexpr long long kSmallBytes[2] = {160LL << 20, 90LL << 20};   // [algo]
 // Logit bytes between which the phase kernel is the default for rows of 16-byte vectors ({Algorithm 1, Algorithms 2 and 4,
 // Algorithm 2 with supplied normalisers}), and the sequences from which it is on probabilities.  Measured at V = 128256 bf16,
@@ -37,9 +38,29 @@ constexpr long long kSmallBytes[2] = {160LL << 20, 90LL << 20};   // [algo]
 // Algorithm 2 at 131 MB 72 us against 120.
 constexpr long long kPhaseBytes[3][2] = {{72LL << 20, 180LL << 20}, {64LL << 20, 860LL << 20}, {48LL << 20, 1400LL << 20}};
 constexpr long long kPhaseBytesF32[3] = {120LL << 20, 280LL << 20, 280LL << 20};
-constexpr long long kPhaseProbsPairs[2] = {36LL << 20, 140LL << 20};      // [algo] bytes of one row pair of every sequence
-constexpr long long kPhaseBytesAll = 360LL << 20;
-constexpr int kPhaseProbsB = 12;
+constexpr long long kPhaseProbsPairs[2] = {36LL << 20, 140LL << 20}, kPhaseProbsPairsF32[2] = {24LL << 20, 110LL << 20};   // [algo] bytes of one row pair of every sequence
+// (Fewer sequences than this: small-batch kernel, gamma = 1 / 4, V = 8192, B = 12: 14 us against 20 / 24; V = 152064 18 / 21 against 24 / 28.)
+constexpr int kPhaseProbsB = 17;
+// On probabilities, Algorithm 1 on more sequences than SMs: 256 of V = 32768 (34 MB of pairs) takes 1.09 times as long as in the
+// flow kernel, 250 of V = 8192 in 32 bits (16 MB) 1.19, 256 of V = 8192 in 16 (8 MB) as long.  Algorithm 2 with many positions:
+// gamma = 16, noise 0.1 / 1, B = 17 of V = 8192: 34 against 30 / 25 against 27 us (flow); of V = 32768: even / 1.29 times faster;
+// gamma = 64, B = 40 of V = 8192: 71 against 49.
+constexpr long long kPhaseProbsMany = 12LL << 20, kPhaseProbsRow = 60000;
+// Fewer sequences than this leave the phase kernel with rows in many pieces: B = 6, V = 152064, gamma = 8, 32-bit logits with
+// supplied normalisers (62 MB) 52 / 55 / 45 us against 48 / 42 / 38 in the small-batch kernel; B = 10 (bf16, 52 MB) 51 / 48 / 43 against 57 / 50 / 45;
+// beyond its sizes V = 256000, 32-bit, gamma = 16, B = 3 (101 MB) 93 / 83 us (noise 0.1 / 1) against 75 / 66 (flow).  Algorithm 1, whose tests
+// the small-batch kernel makes as fast for any outcome: gamma = 8, 32-bit, V = 152064, B = 10 51 / 48 / 47 us against 41 / 43 / 43; gamma = 12
+// (bf16) 42 / 39 / 40 against 44 / 45 / 44.
+constexpr int kPhaseFew = 8, kPhaseFewTv = 12;
+constexpr long long kPhaseFewRow = 700000;
+// With every position swept (diagnostic outputs): bytes of logits, for gamma below 12 and from there on, and bytes of one
+// sequence's target rows, [32-bit logits].  bf16, against the flow kernel: V = 256000 gamma = 8, B = 40 (348 MB) 166 against 148 us;
+// gamma = 4, B = 24 85 against 89; V = 152064 gamma = 16, B = 24 (241 MB) 141 against 125; V = 65536 gamma = 16, B = 64 1.05 times
+// faster.  32-bit: V = 152064 gamma = 4, B = 24 (131 MB) 0.88 times as fast; V = 32768 gamma = 4, B = 128 (151 MB) 1.07, gamma = 8 0.93
+// (285 MB); gamma = 12, V = 8192, B = 128 (105 MB) 0.95, B = 64 1.11.  Against the small-batch kernel: V = 152064 gamma = 8, B = 16
+// (bf16, 83 MB) 80 against 71 us; gamma = 4, B = 32 71 against 77.
+constexpr long long kPhaseAllBytes[2] = {360LL << 20, 144LL << 20}, kPhaseAllBytesLong[2] = {360LL << 20, 60LL << 20};
+constexpr long long kPhaseAllRows[2] = {2500000, 2200000}, kPhaseAllSmall = 1300000;
 constexpr size_t kSlotHead = 16384;   // first area of a stream's workspace: status word, barrier words, the phase kernel's counters
 constexpr size_t kSlotPhase = 256;    // ... the last of these from here on
 static_assert(kSlotPhase + bv::kPhaseCounterWords * sizeof(unsigned) <= kSlotHead, "the counters fit in the head");
@@ -256,29 +277,58 @@ bool not_all_sms(cudaError_t e) {
     return true;
 }
 
-// Where the element-wise kernel is still the default: a few short unaligned rows a sequence, one sequence an SM at most,
-// whose dependent steps cost less than the phase kernel's waits for the whole batch.  Measured, V = 1001 / 2051 / 4099 bf16:
-// Algorithm 1, B = 100, gamma = 3: 24 / 26 / 30 us against 31 / 39 / 40; Algorithm 2, gamma = 2: 26 / 29 / 36 against 33 / 39 / 39
-// (gamma = 3: 32 / 36 / 46 against 34 / 41 / 40).  Where the small-batch kernel fits: Algorithm 1, B = 32, gamma = 2: 20 / 22 / 25
-// against 22 / 23 / 24 us; Algorithm 2: never by more than the runs differ.
-bool elements_pay(int algo, const bv::Params& prm, size_t row_bytes, int sm_count) {
-    if (prm.B > sm_count) return false;
-    if (algo == bv::kTokenVerify) return bv::small_fits(prm.B, prm.gamma) ? prm.gamma <= 2 && row_bytes <= 4200 : prm.gamma <= 3 && row_bytes <= 8200;
-    return !bv::small_fits(prm.B, prm.gamma) && prm.gamma <= 2 && row_bytes <= 8200;
+// Where the element-wise kernel is the default for rows that are not whole 16-byte vectors: a few short ones a sequence, whose
+// dependent steps cost less than the phase kernel's waits for the whole batch.  What a step costs it depends on the part of a
+// row, in elements, that one CTA of a sequence's cluster goes through, and on whether all sequences are at work at once.
+// Measured, bf16, time over the phase kernel's:
+//   Algorithm 1, drafts of noise 0.3 / 1 / 3, all at once, 1000 to 4100 a CTA: gamma = 1 (B = 33 .. 148) 0.50 / 0.49 / 0.48 to 0.67,
+//   3: 0.68 to 0.82, 5: 0.96 / 1.01 / 0.78, 6: 1.10 / 1.09 / 0.83; 8200 (B = 148): gamma = 1 0.70, 3: 0.99 / 0.97 / 0.93,
+//   4: 1.12 / 1.11 / 1.03; two rounds of sequences (B = 200): gamma = 1 0.84 / 0.82 / 0.79, 2: 1.03 / 0.91 / 0.85
+//   Algorithm 2, all at once: gamma = 1 0.55 to 0.70 (1000 to 4100), 0.92 (8200); 2: 0.74 to 0.93 (1000 to 4100); 3: 0.90 to 0.99
+//   (1000 to 2050), 1.11 (4100); two rounds: 0.90 to 1.15
+// and 32-bit logits, B = 148, 8200 elements a CTA, Algorithm 1: gamma = 1 0.69, 2: 0.86, 3: 0.98 / - / 0.92; Algorithm 2: gamma = 1 0.90.
+// Drafts that are hardly accepted at all, which Algorithm 1 leaves after a row, are up to a third faster here at any gamma, the
+// others up to seven times slower: the lines lie where the three noises together are even.  Against the small-batch kernel:
+//   Algorithm 1, B = 32: V = 1003 gamma = 1 0.88, 2: 0.92 / 0.90 / 0.84; V = 4099 1.07; V = 16421 0.90 / 0.85 / 0.81, 0.97 / 0.93 / 0.88
+bool elements_pay(int algo, const bv::Params& prm, const DeviceState& d, const Options& opt, int dtype, size_t row_bytes) {
+    const int g = prm.gamma;
+    if (bv::small_fits(prm.B, g)) return algo == bv::kTokenVerify && g <= 2 && (row_bytes <= 4200 || (dtype == BV_DTYPE_BF16 && prm.B >= 24 && prm.V > 8250 && prm.V <= 16500));
+    const int cluster = pick_cluster(d, opt, prm.B, row_bytes);
+    const int part = prm.V / cluster;
+    const long long ctas = static_cast<long long>(prm.B) * cluster;
+    if (algo == bv::kTokenVerify) {
+        if (ctas <= d.sm_count) return g <= (part <= 4250 ? 5 : part <= 8250 ? 3 : 0);
+        return g == 1 && ctas <= 2LL * d.sm_count && part <= 4250 && prm.V <= 16500;
+    }
+    return ctas <= d.sm_count && g <= (part <= 2100 ? 3 : part <= 4250 ? 2 : part <= 8250 ? 1 : 0);
 }
 
-// Where the phase kernel is the default.  (Rows that are not whole 16-byte vectors: wherever the small-batch kernel is not.)
-bool phase_pays(int algo, const bv::Params& prm, const Options& opt, int dtype, bool vec, long long logit_bytes) {
-    const bool small = bv::small_fits(prm.B, prm.gamma);
-    if (prm.probs)
-        return (!small || prm.B >= kPhaseProbsB) &&
-               logit_bytes / (2 * prm.gamma + 1) * 2 <= kPhaseProbsPairs[algo == bv::kBlockVerify ? 1 : 0];
-    const int which = algo == bv::kTokenVerify ? 0 : (prm.lse_d != nullptr ? 2 : 1);
+// Where the phase kernel is the default.  (Rows that are not whole 16-byte vectors: wherever the kernels above and below are not.)
+bool phase_pays(int algo, const bv::Params& prm, const Options& opt, const DeviceState& d, int dtype, bool vec, long long logit_bytes) {
+    const bool small = bv::small_fits(prm.B, prm.gamma), f32 = dtype == BV_DTYPE_F32;
+    const int a = algo == bv::kBlockVerify ? 1 : 0;
+    const long long one_row = logit_bytes / (2 * prm.gamma + 1);      // of every sequence
+    if (prm.probs) {
+        if (small && prm.B < kPhaseProbsB) return false;
+        if (a == 0) return 2 * one_row <= (prm.B > d.sm_count ? kPhaseProbsMany : f32 ? kPhaseProbsPairsF32[a] : kPhaseProbsPairs[a]);
+        // (few short rows with many candidates each: the ends of sequences, one candidate after the other)
+        if (prm.gamma >= 14 && prm.B < 48 && one_row < prm.gamma * kPhaseProbsRow) return false;
+        return 2 * one_row <= (f32 ? kPhaseProbsPairsF32[a] : kPhaseProbsPairs[a]);
+    }
+    const int which = a == 0 ? 0 : (prm.lse_d != nullptr ? 2 : 1);
     if (prm.first != nullptr) return !small || logit_bytes > kPhaseBytes[which][0];      // (no other kernel takes larger ones)
-    // (with every position swept the flow kernel's two sweeps overlap the more: 403 MB, gamma = 4, 177 us against 167)
-    if (vec && (prm.out_p || prm.out_S || prm.out_h || prm.out_lse_t || prm.out_lse_d) && logit_bytes > kPhaseBytesAll) return false;
-    const long long least = opt.small_bytes > 0 ? static_cast<long long>(opt.small_bytes) << 20 : kPhaseBytes[which][0];
-    return (!small || logit_bytes > least) && (!vec || logit_bytes <= (dtype == BV_DTYPE_F32 ? kPhaseBytesF32[which] : kPhaseBytes[which][1]));
+    const long long small_limit = opt.small_bytes > 0 ? static_cast<long long>(opt.small_bytes) << 20 : kSmallBytes[a];
+    if (small && prm.B < kPhaseFew && logit_bytes <= small_limit) return false;
+    if (vec && f32 && prm.B < kPhaseFew && one_row / prm.B > kPhaseFewRow) return false;
+    if (small && a == 0 && prm.B < kPhaseFewTv && prm.gamma <= 8 && logit_bytes <= small_limit) return false;
+    if (vec && (prm.out_p || prm.out_S || prm.out_h || prm.out_lse_t || prm.out_lse_d)) {
+        // (every position is swept, and the flow kernel overlaps its two sweeps)
+        const long long positions = one_row / prm.B * prm.gamma;                          // bytes of a sequence's target rows
+        if (positions > (small && logit_bytes <= small_limit ? kPhaseAllSmall : kPhaseAllRows[f32]) ||
+            logit_bytes > (prm.gamma < 12 ? kPhaseAllBytes[f32] : kPhaseAllBytesLong[f32])) return false;
+    }
+    const long long least = opt.small_bytes > 0 ? small_limit : kPhaseBytes[which][0];
+    return (!small || logit_bytes > least) && (!vec || logit_bytes <= (f32 ? kPhaseBytesF32[which] : kPhaseBytes[which][1]));
 }
 
 // The phase kernel for the call in `prm`: BV_OK, an error, or 1 if it does not take the call.  Rows at any alignment have no
@@ -391,8 +441,8 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
     // kernel's, and for rows at any alignment.
     const bool only_vec = prm.lse_d != nullptr || prm.greedy || prm.probs;      // (entry points without an element-wise path)
     if (prm.first != nullptr && !vec) return BV_ERR_UNSUPPORTED;
-    const bool elements = !vec && !only_vec && opt.kernel == 0 && elements_pay(algo, prm, row_bytes, d->sm_count);
-    if ((vec || !only_vec) && !elements && (opt.kernel == 5 || ((opt.kernel == 0 || prm.first != nullptr) && phase_pays(algo, prm, opt, dtype, vec, logit_bytes)))) {
+    const bool elements = !vec && !only_vec && opt.kernel == 0 && elements_pay(algo, prm, *d, opt, dtype, row_bytes);
+    if ((vec || !only_vec) && !elements && (opt.kernel == 5 || ((opt.kernel == 0 || prm.first != nullptr) && phase_pays(algo, prm, opt, *d, dtype, vec, logit_bytes)))) {
         if ((rc = run_phase(*d, prm, dtype, vec, ex.probe, stream)) <= BV_OK) return rc;
     }
 

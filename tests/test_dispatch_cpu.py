@@ -173,3 +173,41 @@ def test_without_room_for_a_cooperative_launch_another_kernel_takes_the_call(hos
     finally:
         host.host_refuse_cooperative(0)
     assert host.host_errors() == b"" and host.bv_last_cuda_error() == 0
+
+
+# calls on both sides of the lines between the kernels: (entry point, B, gamma, V, dtype, diagnostics), kernel
+ROUTES = [
+    # rows that are not whole vectors: the element-wise kernel for a few short ones a sequence, if all sequences are at work at once
+    (("tv_verify", 148, 5, 4099, BF16, False), 3), (("tv_verify", 148, 6, 4099, BF16, False), 5), (("tv_verify", 149, 5, 4099, BF16, False), 5),
+    (("tv_verify", 148, 3, 8209, BF16, False), 3), (("tv_verify", 148, 4, 8209, BF16, False), 5), (("tv_verify", 148, 3, 8209, F32, False), 3),
+    (("tv_verify", 148, 1, 16421, BF16, False), 5), (("tv_verify", 296, 1, 4099, BF16, False), 3), (("tv_verify", 297, 1, 4099, BF16, False), 5),
+    (("tv_verify", 64, 1, 16421, BF16, False), 3), (("tv_verify", 33, 1, 32771, BF16, False), 5), (("tv_verify", 32, 2, 2051, BF16, False), 3),
+    (("tv_verify", 32, 2, 4099, BF16, False), 4), (("tv_verify", 32, 2, 16421, BF16, False), 3), (("tv_verify", 16, 2, 16421, BF16, False), 4),
+    (("bv_verify", 148, 2, 4099, BF16, False), 3), (("bv_verify", 148, 3, 4099, BF16, False), 5), (("bv_verify", 148, 3, 2051, BF16, False), 3),
+    (("bv_verify", 148, 1, 8209, F32, False), 3), (("bv_verify", 148, 2, 8209, BF16, False), 5), (("bv_verify", 149, 1, 1003, BF16, False), 5),
+    (("bv_verify", 32, 1, 1003, BF16, False), 4), (("bv_verify", 24, 5, 50257, BF16, False), 4), (("bv_verify", 150, 8, 50257, BF16, True), 5),
+    # probabilities
+    (("bv_verify_probs", 16, 4, 152064, BF16, False), 4), (("bv_verify_probs", 17, 4, 152064, BF16, False), 5), (("bv_verify_probs", 64, 8, 128256, BF16, False), 5),
+    (("bv_verify_probs", 24, 16, 8192, BF16, False), 1), (("bv_verify_probs", 24, 13, 8192, BF16, False), 5), (("bv_verify_probs", 48, 16, 8192, BF16, False), 5),
+    (("tv_verify_probs", 148, 8, 32768, BF16, False), 5), (("tv_verify_probs", 256, 8, 32768, BF16, False), 1), (("tv_verify_probs", 24, 8, 152064, F32, False), 1),
+    (("bv_verify_probs", 100, 1, 152064, F32, False), 1), (("bv_verify_probs", 100, 1, 152064, BF16, False), 5),
+    # every position swept
+    (("bv_verify", 40, 8, 256000, BF16, True), 1), (("bv_verify", 40, 4, 256000, BF16, True), 5), (("bv_verify", 24, 16, 152064, BF16, True), 1),
+    (("bv_verify", 64, 16, 65536, BF16, True), 5), (("bv_verify", 128, 8, 32768, F32, True), 1), (("bv_verify", 128, 4, 32768, F32, True), 5),
+    (("bv_verify", 64, 12, 8192, F32, True), 5), (("bv_verify", 128, 12, 8192, F32, True), 1), (("bv_verify", 16, 8, 152064, BF16, True), 4),
+    (("bv_verify", 32, 4, 152064, BF16, True), 5),
+    # few sequences of long rows
+    (("bv_verify_lse", 6, 8, 152064, F32, False), 4), (("bv_verify_lse", 10, 8, 152064, F32, False), 5), (("tv_verify_lse", 10, 8, 152064, F32, False), 4),
+    (("tv_verify_lse", 10, 12, 152064, BF16, False), 5), (("bv_verify", 3, 16, 256000, F32, False), 1), (("bv_verify", 9, 16, 256000, F32, False), 1),
+    (("bv_verify", 7, 16, 256000, BF16, False), 5), (("bv_verify", 7, 16, 128000, F32, False), 5),
+    # the ordinary batches
+    (("bv_verify", 1, 8, 152064, BF16, False), 4), (("bv_verify", 8, 8, 32000, F32, False), 4), (("bv_verify", 64, 8, 128256, BF16, False), 5),
+    (("bv_verify", 96, 12, 152064, BF16, False), 5), (("bv_verify", 256, 8, 256000, BF16, False), 1), (("tv_verify", 256, 8, 152064, BF16, False), 1),
+    (("bv_verify_lse", 64, 8, 128256, BF16, False), 5), (("gbv_verify", 64, 8, 128256, BF16, False), 5),
+]
+
+
+def test_which_kernel_takes_a_call(host):
+    for (fn, B, gamma, V, dtype, diagnostics), kernel in ROUTES:
+        assert verify(host, B, gamma, V, dtype, fn, diagnostics=diagnostics) == (0, kernel), (fn, B, gamma, V, dtype, diagnostics)
+    assert host.host_errors() == b""
