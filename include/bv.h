@@ -356,8 +356,8 @@ int bv_stream_status(void* stream);
  *                   chunks that last target rows get, so that the launch ends on short items (default 0:
  *                   none; it helped only where most drafted tokens are accepted)
  *   "wait_limit"    polls after which a bounded device-side wait gives up (tests)
- *   "never_signal"  tests: the kernels' workers never report what they have swept, so the waits
- *                   run out and the call ends with BV_ERR_TIMEOUT
+ *   "never_signal"  tests: 1: the kernels' workers never report what they have swept, so the waits
+ *                   run out and the call ends with BV_ERR_TIMEOUT (2: only the phase kernel's second sweeps are not reported)
  * Their first values come from the environment variables BV_KERNEL (flow / cluster / stream / small / phase),
  * BV_CLUSTER, BV_MAX_CLUSTERS, BV_FLOW_CHUNKS, BV_FLOW_PIECES, BV_FLOW_CTAS, BV_FLOW_DEPTH, read once.
  * Returns BV_ERR_INVALID_ARG for an unknown name.

@@ -76,7 +76,7 @@ struct Options {
     int flow_fine = 0;     // > 0: this many blocks at the end of the batch have their rows cut into the finer chunks
     int flow_keep_l2 = 0;  // 1: the lines of a first sweep stay in L2 at normal priority; 0: every load streams past L2
     int wait_limit = 0;    // polls after which a bounded device-side wait gives up; 0: the built-in limits
-    int never_signal = 0;  // test switch: the flow kernel's workers never report an item as swept
+    int never_signal = 0;  // test switch: 1 the kernels' workers never report what they have swept; 2 only the phase kernel's second sweeps
 };
 Options g_opt;
 std::once_flag g_opt_once;

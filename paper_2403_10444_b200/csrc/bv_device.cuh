@@ -35,7 +35,7 @@ struct Params {
     int greedy;               // flow kernel: Greedy Block Verification (Algorithm 4) instead of Algorithm 2
     int algo;                 // flow kernel: kBlockVerify (Algorithms 2, 4) or kTokenVerify (Algorithm 1)
     unsigned wait_limit;      // flow kernel: polls after which a bounded wait gives up (0: the built-in limits)
-    int never_signal;         // flow kernel, test switch: workers never report an item as swept, so the waits run out
+    int never_signal;         // test switch, 1: nobody reports what is swept, so the waits run out; 2: phase kernel, only the second sweeps are not
     int probs;                // flow kernel: tgt / drf hold probabilities, used as stored, instead of logits
     const int32_t* first;     // small-batch and phase kernels, or null: tgt / drf are tables [V, V] whose row t holds the logits
                               // after token t, and a sequence's rows are those of first[b], X_1, .. X_gamma

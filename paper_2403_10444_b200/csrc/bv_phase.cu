@@ -634,7 +634,7 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
         __threadfence();
         __syncwarp();
         unsigned last = 0;
-        if (lane == 0 && !prm.never_signal) last = ph_arrive(&ps.cnt1[b], 1u, static_cast<unsigned>(ps.rows * units) + 1u);
+        if (lane == 0 && prm.never_signal != 1) last = ph_arrive(&ps.cnt1[b], 1u, static_cast<unsigned>(ps.rows * units) + 1u);
         if (__shfl_sync(0xffffffffu, last, 0)) ph_fold(prm, ps, b, lane, false);
     };
 
@@ -705,7 +705,7 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
             todo -= n;
             if (todo <= 0 || (j + 1 == rows && k + n == units)) {      // the end of this warp's part, or of the sequence
                 unsigned last = 0;
-                if (lane == 0 && !prm.never_signal) last = ph_arrive(&ps.cnt1[b], arrived, static_cast<unsigned>(rows * units) + 1u);
+                if (lane == 0 && prm.never_signal != 1) last = ph_arrive(&ps.cnt1[b], arrived, static_cast<unsigned>(rows * units) + 1u);
                 arrived = 0;
                 if (__shfl_sync(0xffffffffu, last, 0)) ph_fold(prm, ps, b, lane, false);
             }
@@ -874,7 +874,7 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
                 // (the next run is open already unless this was the last: the issue side runs ahead)
                 if (todo <= 0 || runs[(n_c + 1) & (kPhQueue - 1)].b != b) {
                     unsigned done = 0;
-                    if (lane == 0) done = ph_arrive(&ps.cnt2[b], arrived, static_cast<unsigned>((s_base[b + 1] - s_base[b]) * units));
+                    if (lane == 0 && !prm.never_signal) done = ph_arrive(&ps.cnt2[b], arrived, static_cast<unsigned>((s_base[b + 1] - s_base[b]) * units));
                     arrived = 0;
                     if (__shfl_sync(0xffffffffu, done, 0)) ph_finalize<DT, PROBS, AL>(prm, ps, b, make_uint4(s_lo[b], s_hi[b], s_last[b] & 1u, s_last[b] >> 1), round, lane, false);
                 }

@@ -13,7 +13,7 @@ from parity import run_oracle, run_cuda, compare, assert_parity, record
 pytestmark = pytest.mark.gpu
 
 ALGOS = [oracle.BLOCK_VERIFY, oracle.TOKEN_VERIFY]
-KERNELS = {"flow": 1, "cluster": 2, "stream": 3, "small": 4}     # values of the library's "kernel" option
+KERNELS = {"flow": 1, "cluster": 2, "stream": 3, "small": 4, "phase": 5}     # values of the library's "kernel" option
 
 
 def parity_case(inp, algo, check_diag=True):
@@ -57,7 +57,7 @@ def test_full_size_configs(name, algo):
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("V", [1, 2, 3, 8, 17, 1000, 1027, 4104, 20000])
 def test_ragged_vocabularies(V, dtype, algo):
-    # V = 1..17 and odd V take the element-wise path; multiples of 16 bytes the 128-bit path
+    # odd V: rows at every alignment (the small-batch and the phase kernel, the element-wise one for short rows of a few positions)
     for gamma, B in ((1, 5), (2, 37), (5, 9)):
         parity_case(random_inputs(B, gamma, V, dtype, seed=V * 7 + gamma), algo)
 
@@ -72,7 +72,7 @@ def test_every_cluster_width(cluster, algo, bv_options):
 
 
 @pytest.mark.parametrize("algo", ALGOS)
-@pytest.mark.parametrize("kernel", ["flow", "cluster", "stream", "small"])
+@pytest.mark.parametrize("kernel", ["flow", "cluster", "stream", "small", "phase"])
 def test_every_kernel(kernel, algo, bv_options):
     # the library has several kernels for each algorithm; each must match the oracle
     bv_options("kernel", KERNELS[kernel])
@@ -101,14 +101,14 @@ def test_flow_finer_chunks_for_the_last_sequences(fine, bv_options):
 
 
 @pytest.mark.parametrize("algo", ALGOS)
-@pytest.mark.parametrize("kernel", ["flow", "small", "default"])
+@pytest.mark.parametrize("kernel", ["flow", "small", "phase", "default"])
 @pytest.mark.parametrize("dtype,V", [("f32", 1 << 21), ("bf16", (1 << 21) + 8), ("bf16", (1 << 21) + 1)])
 def test_very_large_vocabularies(dtype, V, kernel, algo, bv_options):
-    # two million logits a row: chunk, piece and segment ranges far beyond the benchmark's sizes; the odd V
-    # takes the element-wise path
+    # two million logits a row: chunk, piece and segment ranges far beyond the benchmark's sizes, and
+    # rows at odd alignments
     if kernel != "default":
-        if V % 8:
-            pytest.skip("the flow and small-batch kernels take rows of whole 16-byte vectors")
+        if V % 8 and kernel == "flow":
+            pytest.skip("the flow kernel takes rows of whole 16-byte vectors")
         bv_options("kernel", KERNELS[kernel])
     parity_case(random_inputs(3, 2, V, dtype, seed=V % 97, T=0.9), algo)
 
@@ -126,7 +126,7 @@ def test_more_sequences_than_resident_clusters(algo):
     parity_case(random_inputs(700, 3, 512, "f32", seed=3), algo)
 
 
-@pytest.mark.parametrize("kernel", ["flow", "small"])
+@pytest.mark.parametrize("kernel", ["flow", "small", "phase"])
 @pytest.mark.parametrize("algo", ALGOS)
 @pytest.mark.parametrize("gamma", [1, 16, 64])
 def test_block_lengths(gamma, algo, kernel, bv_options):
@@ -134,7 +134,7 @@ def test_block_lengths(gamma, algo, kernel, bv_options):
     parity_case(random_inputs(6, gamma, 2048, "bf16", seed=gamma, sigma_d=0.3), algo)
 
 
-@pytest.mark.parametrize("kernel", ["flow", "small"])
+@pytest.mark.parametrize("kernel", ["flow", "small", "phase"])
 @pytest.mark.parametrize("T", [0.2, 0.6, 1.0, 2.5])
 def test_temperatures(T, kernel, bv_options):
     bv_options("kernel", KERNELS[kernel])
@@ -161,7 +161,7 @@ def test_gamma1_block_equals_token_bitwise():
     assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
 
 
-@pytest.mark.parametrize("kernel", ["flow", "small"])
+@pytest.mark.parametrize("kernel", ["flow", "small", "phase"])
 def test_draft_equals_target(kernel, bv_options):
     bv_options("kernel", KERNELS[kernel])
     inp = random_inputs(16, 6, 4096, "bf16", seed=22)
@@ -175,7 +175,7 @@ def test_draft_equals_target(kernel, bv_options):
     assert torch.all(diag["S"] == 0) and torch.all(diag["p"] == 1)
 
 
-@pytest.mark.parametrize("kernel", ["flow", "small"])
+@pytest.mark.parametrize("kernel", ["flow", "small", "phase"])
 def test_masked_logits_and_domain_errors(kernel, bv_options):
     bv_options("kernel", KERNELS[kernel])
     inp = random_inputs(8, 3, 640, "f32", seed=23)
@@ -259,7 +259,7 @@ def test_skipped_second_sweeps_change_nothing(sigma_d):
 
 def test_calls_on_several_streams_at_once():
     # every stream has a workspace of its own: calls in flight together on different streams, of shapes
-    # that the flow kernel and the small-batch kernel serve, give what the same calls give one by one
+    # that the phase kernel and the small-batch kernel serve, give what the same calls give one by one
     import paper_2403_10444_b200 as bv
     shapes = [(48, 5, 16384, "bf16"), (6, 4, 8192, "f32"), (80, 3, 4096, "bf16"), (2, 8, 32000, "bf16")]
     cases = []

@@ -102,6 +102,36 @@ def test_faults_are_per_sequence(V, kernel, bv_options):
     assert (ol.cpu().numpy() == ref.out_len).all() and (ot.cpu().numpy() == ref.out_tokens).all()
 
 
+@pytest.mark.parametrize("dtype,V", [("bf16", 8), ("bf16", 504), ("bf16", 520), ("bf16", 8200), ("f32", 4), ("f32", 260), ("f32", 20000)])
+@pytest.mark.parametrize("B,gamma", [(1, 1), (7, 34), (50, 5)])
+def test_the_other_entry_points_around_whole_units(dtype, V, B, gamma, bv_options):
+    # Algorithm 4, supplied normalisers and probabilities, forced onto the phase kernel
+    import paper_2403_10444_b200 as bv
+    import test_gpu_lse
+    import test_gpu_probs
+    bv_options("kernel", 5)
+    inp = inputs(B, gamma, V, dtype, V + B)
+    check(inp, (oracle.GREEDY_BLOCK_VERIFY,))
+    for algo in (oracle.BLOCK_VERIFY, oracle.TOKEN_VERIFY):
+        test_gpu_lse.run_case(inp, test_gpu_lse.own_lse(inp), algo)
+        assert bv.bv_last_kernel() == 5 and bv.bv_stream_status() == 0
+    pin = test_gpu_probs.probs_inputs(wl.Workload("ph", B, gamma, V, dtype, 0.9, V + B, 2.0, 0.0, 0, 0.0, 0.5))
+    for algo in ("block", "token"):
+        test_gpu_probs.run_case(algo, pin, "phase kernel probs V=%d B=%d gamma=%d %s %s" % (V, B, gamma, dtype, algo))
+        assert bv.bv_last_kernel() == 5 and bv.bv_stream_status() == 0
+
+
+@pytest.mark.parametrize("algo", [oracle.BLOCK_VERIFY, oracle.TOKEN_VERIFY])
+def test_supplied_normalisers_that_are_not_finite(algo, bv_options):
+    import test_gpu_lse
+    bv_options("kernel", 5)
+    inp = inputs(12, 4, 4096, "bf16", 8)
+    lse = test_gpu_lse.own_lse(inp)
+    lse[2, 0], lse[3, 0], lse[4, 0], lse[5, 3] = float("nan"), float("inf"), -float("inf"), float("nan")
+    ref = test_gpu_lse.run_case(inp, lse, algo)
+    assert (ref.out_len[2:5] == -1).all() and (ref.out_len[[0, 1, 6]] > 0).all()
+
+
 @pytest.mark.parametrize("V", [4096, 4099])
 def test_a_wait_that_runs_out_is_reported_and_the_next_call_works(V, bv_options):
     import paper_2403_10444_b200 as bv
@@ -116,5 +146,31 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_call_works(V, bv_options)
     bv_options("never_signal", 0)
     bv_options("wait_limit", 0)
     got = bv.bv_verify(*a)
+    assert bv.bv_stream_status() == 0
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+@pytest.mark.parametrize("probs", [False, True])
+@pytest.mark.parametrize("V", [4096, 4099])
+def test_the_wait_for_the_second_sweeps_runs_out_too(V, probs, bv_options):
+    # never_signal: 1 on probabilities, which have no first sweep, and 2 leave only the second sweeps unreported
+    import paper_2403_10444_b200 as bv
+    if probs and V % 8:
+        pytest.skip("probabilities come in rows of whole 16-byte vectors")
+    bv_options("kernel", 5)
+    inp = inputs(3, 2, V, "bf16", 1)
+    a = [inp[k].cuda() for k in ("target_logits", "draft_logits", "draft_tokens", "uniforms")]
+    if probs:
+        a[0], a[1] = a[0].float().softmax(-1).bfloat16(), a[1].float().softmax(-1).bfloat16()
+    call = (lambda: bv.bv_verify_probs(*a)) if probs else (lambda: bv.bv_verify(*a, inp["temperature"]))
+    want = call()
+    assert bv.bv_stream_status() == 0
+    bv_options("wait_limit", 2000)
+    bv_options("never_signal", 1 if probs else 2)
+    call()
+    assert bv.bv_stream_status() == -4
+    bv_options("never_signal", 0)
+    bv_options("wait_limit", 0)
+    got = call()
     assert bv.bv_stream_status() == 0
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])

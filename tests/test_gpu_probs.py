@@ -53,7 +53,7 @@ def test_probabilities_match_the_oracle(algo, name, B, gamma):
     run_case(algo, probs_inputs(w), "probs %s B=%d gamma=%d %s" % (name, B, gamma, algo))
 
 
-@pytest.mark.parametrize("kernel", [1, 4])         # the flow kernel, the small-batch kernel
+@pytest.mark.parametrize("kernel", [1, 4, 5])         # the flow, the small-batch and the phase kernel
 @pytest.mark.parametrize("algo", ["block", "token"])
 @pytest.mark.parametrize("V", [8, 24, 1000, 4104, 33000, (1 << 21) + 8])
 def test_ragged_vocabularies(algo, V, kernel, bv_options):
@@ -71,7 +71,7 @@ def test_high_acceptance_reaches_the_last_row(algo):
     assert (ref.out_len == 7).sum() > 5
 
 
-@pytest.mark.parametrize("kernel", [1, 4])
+@pytest.mark.parametrize("kernel", [1, 4, 5])
 @pytest.mark.parametrize("algo", ["block", "token"])
 def test_faults_are_per_sequence_and_rows_are_used_as_stored(algo, kernel, bv_options):
     bv_options("kernel", kernel)
@@ -97,7 +97,7 @@ def test_rows_that_are_not_whole_vectors_are_refused():
     assert e.value.status == -2
 
 
-@pytest.mark.parametrize("kernel", [1, 4])
+@pytest.mark.parametrize("kernel", [1, 4, 5])
 def test_only_the_needed_rows_are_read(kernel, bv_options):
     bv_options("kernel", kernel)
     # rows that neither algorithm reads may hold anything: here NaN everywhere except the entries of

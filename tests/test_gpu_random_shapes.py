@@ -12,7 +12,7 @@ from parity import run_oracle, run_cuda, compare, assert_parity, record
 
 pytestmark = pytest.mark.gpu
 
-KERNELS = {"default": 0, "flow": 1, "small": 4}
+KERNELS = {"default": 0, "flow": 1, "small": 4, "phase": 5}
 
 
 def draw(rnd):
@@ -47,6 +47,29 @@ def test_random_shapes(seed, bv_options):
                     record(rep, "random shape B=%d gamma=%d V=%d %s T=%g sigma=%g algo %d kernel %s %s" % (
                         w.B, w.gamma, w.V, w.dtype, w.temperature, w.draft_sigma, algo, name, "diagnostics" if diag else "plain"))
                     assert_parity(rep, diag), (w, algo, name, diag)
+                    assert bv.bv_stream_status() == 0
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_random_odd_vocabularies(seed, bv_options):
+    """Rows that are not whole 16-byte vectors, through the kernels that take them."""
+    import paper_2403_10444_b200 as bv
+    rnd = random.Random(3000 + seed)
+    for _ in range(8):
+        w = draw(rnd)
+        V = w.V + rnd.randrange(1, 8)
+        w = wl.scaled(w, V=V + (V % (4 if w.dtype == "f32" else 8) == 0))
+        inp = wl.make_inputs(w, "cpu")
+        fits_small = w.B <= 32 and w.B * (2 * w.gamma + 1) <= 1056 and w.B * (w.gamma + 1) <= 560
+        for algo in (oracle.BLOCK_VERIFY, oracle.TOKEN_VERIFY):
+            ref = run_oracle(algo, inp)
+            for code in (0, 3, 5) + ((4,) if fits_small else ()):
+                bv_options("kernel", code)
+                for diag in (True, False):
+                    out = run_cuda(algo, inp, diagnostics=diag)
+                    assert code in (0, bv.bv_last_kernel()) and bv.bv_last_kernel() in (3, 4, 5)
+                    rep = compare(algo, ref, out[0], out[1], out[2] if diag else None, inp)
+                    assert_parity(rep, diag), (w, algo, code, diag)
                     assert bv.bv_stream_status() == 0
 
 
