@@ -283,22 +283,24 @@ bool not_all_sms(cudaError_t e) {
 // Measured, bf16, time over the phase kernel's:
 //   Algorithm 1, drafts of noise 0.3 / 1 / 3, all at once, 1000 to 4100 a CTA: gamma = 1 (B = 33 .. 148) 0.50 / 0.49 / 0.48 to 0.67,
 //   3: 0.68 to 0.82, 5: 0.96 / 1.01 / 0.78, 6: 1.10 / 1.09 / 0.83; 8200 (B = 148): gamma = 1 0.70, 3: 0.99 / 0.97 / 0.93,
-//   4: 1.12 / 1.11 / 1.03; two rounds of sequences (B = 200): gamma = 1 0.84 / 0.82 / 0.79, 2: 1.03 / 0.91 / 0.85
+//   4: 1.12 / 1.11 / 1.03; two rounds of sequences (B = 200): gamma = 1 0.84 / 0.82 / 0.79, 2: 0.91 / 0.80 / 0.76 (2050), 1.07 / 0.93 / 0.87 (4100)
 //   Algorithm 2, all at once: gamma = 1 0.55 to 0.70 (1000 to 4100), 0.92 (8200); 2: 0.74 to 0.93 (1000 to 4100); 3: 0.90 to 0.99
 //   (1000 to 2050), 1.11 (4100); two rounds: 0.90 to 1.15
-// and 32-bit logits, B = 148, 8200 elements a CTA, Algorithm 1: gamma = 1 0.69, 2: 0.86, 3: 0.98 / - / 0.92; Algorithm 2: gamma = 1 0.90.
+// and 32-bit logits, B = 148, 8200 elements a CTA, Algorithm 1: gamma = 1 0.69, 2: 0.86, 3: 0.98 / - / 0.92; two rounds (B = 40, 2050) 2: 0.89 /
+// 0.80 / 0.81; Algorithm 2: gamma = 1 0.90.
 // Drafts that are hardly accepted at all, which Algorithm 1 leaves after a row, are up to a third faster here at any gamma, the
 // others up to seven times slower: the lines lie where the three noises together are even.  Against the small-batch kernel:
-//   Algorithm 1, B = 32: V = 1003 gamma = 1 0.88, 2: 0.92 / 0.90 / 0.84; V = 4099 1.07; V = 16421 0.90 / 0.85 / 0.81, 0.97 / 0.93 / 0.88
-bool elements_pay(int algo, const bv::Params& prm, const DeviceState& d, const Options& opt, int dtype, size_t row_bytes) {
+//   Algorithm 1, B = 32: V = 1003 gamma = 1 0.88, 2: 0.92 / 0.90 / 0.84; V = 4099 1.07; V = 16421 0.90 / 0.85 / 0.81, 0.97 / 0.93 / 0.88;
+//   V = 8209 in 32 bits 0.86, 0.87 / 0.85 / 0.81
+bool elements_pay(int algo, const bv::Params& prm, const DeviceState& d, const Options& opt, size_t row_bytes) {
     const int g = prm.gamma;
-    if (bv::small_fits(prm.B, g)) return algo == bv::kTokenVerify && g <= 2 && (row_bytes <= 4200 || (dtype == BV_DTYPE_BF16 && prm.B >= 24 && prm.V > 8250 && prm.V <= 16500));
+    if (bv::small_fits(prm.B, g)) return algo == bv::kTokenVerify && g <= 2 && (row_bytes <= 4200 || (prm.B >= 24 && row_bytes > 16500 && row_bytes <= 33000));
     const int cluster = pick_cluster(d, opt, prm.B, row_bytes);
     const int part = prm.V / cluster;
     const long long ctas = static_cast<long long>(prm.B) * cluster;
     if (algo == bv::kTokenVerify) {
         if (ctas <= d.sm_count) return g <= (part <= 4250 ? 5 : part <= 8250 ? 3 : 0);
-        return g == 1 && ctas <= 2LL * d.sm_count && part <= 4250 && prm.V <= 16500;
+        return ctas <= 2LL * d.sm_count && prm.V <= 16500 && g <= (part <= 2100 ? 2 : part <= 4250 ? 1 : 0);
     }
     return ctas <= d.sm_count && g <= (part <= 2100 ? 3 : part <= 4250 ? 2 : part <= 8250 ? 1 : 0);
 }
@@ -441,7 +443,7 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
     // kernel's, and for rows at any alignment.
     const bool only_vec = prm.lse_d != nullptr || prm.greedy || prm.probs;      // (entry points without an element-wise path)
     if (prm.first != nullptr && !vec) return BV_ERR_UNSUPPORTED;
-    const bool elements = !vec && !only_vec && opt.kernel == 0 && elements_pay(algo, prm, *d, opt, dtype, row_bytes);
+    const bool elements = !vec && !only_vec && opt.kernel == 0 && elements_pay(algo, prm, *d, opt, row_bytes);
     if ((vec || !only_vec) && !elements && (opt.kernel == 5 || ((opt.kernel == 0 || prm.first != nullptr) && phase_pays(algo, prm, opt, *d, dtype, vec, logit_bytes)))) {
         if ((rc = run_phase(*d, prm, dtype, vec, ex.probe, stream)) <= BV_OK) return rc;
     }

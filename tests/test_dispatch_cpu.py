@@ -181,7 +181,8 @@ ROUTES = [
     (("tv_verify", 148, 5, 4099, BF16, False), 3), (("tv_verify", 148, 6, 4099, BF16, False), 5), (("tv_verify", 149, 5, 4099, BF16, False), 5),
     (("tv_verify", 148, 3, 8209, BF16, False), 3), (("tv_verify", 148, 4, 8209, BF16, False), 5), (("tv_verify", 148, 3, 8209, F32, False), 3),
     (("tv_verify", 148, 1, 16421, BF16, False), 5), (("tv_verify", 296, 1, 4099, BF16, False), 3), (("tv_verify", 297, 1, 4099, BF16, False), 5),
-    (("tv_verify", 64, 1, 16421, BF16, False), 3), (("tv_verify", 33, 1, 32771, BF16, False), 5), (("tv_verify", 32, 2, 2051, BF16, False), 3),
+    (("tv_verify", 40, 2, 8209, F32, False), 3), (("tv_verify", 40, 3, 8209, F32, False), 5), (("tv_verify", 200, 2, 2051, BF16, False), 3),
+    (("tv_verify", 200, 2, 4099, BF16, False), 5), (("tv_verify", 32, 2, 8209, F32, False), 3), (("tv_verify", 64, 1, 16421, BF16, False), 3), (("tv_verify", 33, 1, 32771, BF16, False), 5), (("tv_verify", 32, 2, 2051, BF16, False), 3),
     (("tv_verify", 32, 2, 4099, BF16, False), 4), (("tv_verify", 32, 2, 16421, BF16, False), 3), (("tv_verify", 16, 2, 16421, BF16, False), 4),
     (("bv_verify", 148, 2, 4099, BF16, False), 3), (("bv_verify", 148, 3, 4099, BF16, False), 5), (("bv_verify", 148, 3, 2051, BF16, False), 3),
     (("bv_verify", 148, 1, 8209, F32, False), 3), (("bv_verify", 148, 2, 8209, BF16, False), 5), (("bv_verify", 149, 1, 1003, BF16, False), 5),
