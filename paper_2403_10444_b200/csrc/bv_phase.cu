@@ -236,48 +236,37 @@ static __device__ __forceinline__ void ph_reduce_rows(const PhaseScratch& ps, in
         }
         return;
     }
-    // (few long rows, in many pieces: the lanes share a row)
-    int L = 1;
-    while (L < slots && L < 32) L <<= 1;  // lanes that look at one row
-    const int rp = 32 / L, sub = lane / L, k = lane % L;
-    for (int r0 = 0; r0 < rows; r0 += 4 * rp) {
+    // (few long rows, in more pieces than that: all lanes on one row, four rows asked for at a time)
+    for (int r0 = 0; r0 < rows; r0 += 4) {
         double2 v[4];
         int np[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int r = r0 + q * rp + sub;
-            // (the pieces of a row: one for each warp whose part of the list holds some of it)
+            const int r = r0 + q;
             const unsigned x = static_cast<unsigned>((b * rows + r) * ps.units);
             np[q] = r < rows ? static_cast<int>((x + ps.units - 1) / ps.per1 - x / ps.per1) + 1 : 0;
-            v[q] = k < np[q] ? __ldcg(&ps.part[(static_cast<size_t>(b) * rows + r) * slots + k]) : make_double2(kNoRef, 0.0);
+            v[q] = lane < np[q] ? __ldcg(&ps.part[(static_cast<size_t>(b) * rows + r) * slots + lane]) : make_double2(kNoRef, 0.0);
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            if (r0 + q * rp >= rows) break;
+            const int r = r0 + q;
+            if (r >= rows) break;
             float m = static_cast<float>(v[q].x);
             double s = v[q].y;
-            for (int p = k + L; p < np[q]; p += L) {          // (only where the rows are few)
-                const double2 w = __ldcg(&ps.part[(static_cast<size_t>(b) * rows + r0 + q * rp + sub) * slots + p]);
+            for (int p = lane + 32; p < np[q]; p += 32) {
+                const double2 w = __ldcg(&ps.part[(static_cast<size_t>(b) * rows + r) * slots + p]);
                 const float wm = static_cast<float>(w.x), mm = fmaxf(m, wm);
                 s = s * static_cast<double>(ref_scale(m, mm)) + w.y * static_cast<double>(ref_scale(wm, mm));
                 m = mm;
             }
-            float mr = m;
-            for (int off = L >> 1; off > 0; off >>= 1) mr = fmaxf(mr, __shfl_xor_sync(0xffffffffu, mr, off));
-            s *= static_cast<double>(ref_scale(m, mr));
-            for (int off = L >> 1; off > 0; off >>= 1) s += shfl_xor_d(s, off);
+            const float mr = warp_max(m);
+            s = warp_sum_d(s * static_cast<double>(ref_scale(m, mr)));
+            const int c = r < g ? r : r - g;                  // target row c or draft row c
 #pragma unroll
-            for (int h = 0; h < 4; ++h) {                     // target rows c and c + 32, draft rows c and c + 32
-                if ((h & 1) && g <= 32) continue;
-                if (h >= 2 && rows == g) continue;
-                const int c = lane + 32 * (h & 1), idx = c + (h < 2 ? 0 : g) - (r0 + q * rp);
-                const bool here = c < g && idx >= 0 && idx < rp;
-                const float mm = __shfl_sync(0xffffffffu, mr, here ? idx * L : 0);
-                const double zz = shfl_d(s, here ? idx * L : 0);
-                if (here) {
-                    if (h < 2) { MP[h & 1] = mm; ZP[h & 1] = zz; }
-                    else { MQ[h & 1] = mm; ZQ[h & 1] = zz; }
-                }
+            for (int h = 0; h < 2; ++h) {
+                if (c != lane + 32 * h) continue;
+                if (r < g) { MP[h] = mr; ZP[h] = s; }
+                else { MQ[h] = mr; ZQ[h] = s; }
             }
         }
     }

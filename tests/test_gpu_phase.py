@@ -33,6 +33,17 @@ def test_rows_around_whole_units(dtype, V, B, gamma, kernel, bv_options):
     check(inputs(B, gamma, V, dtype, V + B), (oracle.BLOCK_VERIFY, oracle.TOKEN_VERIFY), kernel)
 
 
+@pytest.mark.parametrize("dtype,V,gamma", [("bf16", 152065, 1), ("f32", 152064, 33), ("f32", 152065, 20)])
+def test_rows_in_more_than_32_pieces(dtype, V, gamma, bv_options):
+    # (a fold in which all lanes of a warp look at one row)
+    import test_gpu_lse
+    bv_options("kernel", 5)
+    inp = inputs(1, gamma, V, dtype, gamma)
+    check(inp, (oracle.BLOCK_VERIFY, oracle.TOKEN_VERIFY))
+    if V % 4 == 0:
+        test_gpu_lse.run_case(inp, test_gpu_lse.own_lse(inp))
+
+
 @pytest.mark.parametrize("V,B,gamma", [(4096, 768, 1), (64, 768, 3), (1003, 2000, 2), (16, 769, 2), (5089, 1533, 2)])
 def test_as_many_sequences_as_it_takes_and_more(V, B, gamma, bv_options):
     # 768 sequences a launch; rows at any alignment go through it in parts beyond that, others through the flow kernel
