@@ -31,7 +31,8 @@
  * graphs and replayed between other calls: a captured call uses the workspace of
  * the stream it was captured on (what it needs beyond that is obtained outside the
  * graph, on a stream of the library's, and waited for), so replays must not overlap
- * other calls on that stream.  What is outgrown stays allocated for their sake; the
+ * other calls on that stream; the first call on a device sets the library up there
+ * and must not be a captured one.  What is outgrown stays allocated for their sake; the
  * memory is returned by bv_release().  B = 0 is accepted and does nothing.
  *
  * Errors: every entry point returns BV_OK (0) or a negative bv_status; nothing
@@ -80,12 +81,15 @@ enum { BV_NOALLOC_SCRATCH_BYTES = 8 * 1024 * 1024 };
  *   out_tokens    [B, gamma+1] int32: X_1..X_tau, Y, then -1
  *   out_len       [B] int32: tau + 1, or -1 for a sequence with a data fault
  *   stream        a cudaStream_t (NULL = the default stream)
- * Rows of any V >= 1 at any alignment are read 16 bytes at a time.
- * Since S_i <= p_i, h_i <= p_i: S_i is evaluated only for
- * positions with eta_i <= p_i that can still be the highest one to pass
- * eta_i <= h_i; tau and Y are those of the full evaluation (bv_verify_ex does the
- * full evaluation).  The cost of a call therefore depends on how many drafted
- * tokens are accepted.
+ * Rows of any V >= 1 at any alignment are taken, and read 16 bytes at a time but
+ * for a few short ones a sequence that are not whole 16-byte vectors, and unaligned
+ * ones of more than 2^30 elements: those go through an element-wise kernel, which
+ * evaluates every S_i.  Elsewhere, since S_i <= p_i and so h_i <= p_i, S_i is
+ * evaluated only for positions with eta_i <= p_i that can still be the highest one
+ * to pass eta_i <= h_i; tau and Y are those of the full evaluation (bv_verify_ex
+ * does it), up to the rounding of the sums where the two calls take different
+ * kernels.  The cost of a call therefore depends on how many drafted tokens are
+ * accepted.
  */
 int bv_verify(const void* target_logits, const void* draft_logits,
               const int32_t* draft_tokens, const float* uniforms,
@@ -96,8 +100,9 @@ int bv_verify(const void* target_logits, const void* draft_logits,
  * Token Verification: Algorithm 1 with Eq. "accept_probability"
  * (h_i = min(P_{i-1}(X_i)/Q_{i-1}(X_i), 1)); tau = length of the initial run of
  * i with h_i > 0 and eta_i <= h_i; Y from Eq. "pres-token" at position tau, or
- * from P_gamma when tau = gamma.  Only rows 0..tau are read.  Arguments as for
- * bv_verify.
+ * from P_gamma when tau = gamma.  The outcome depends on rows 0..tau only (the
+ * kernels for middling batches and unaligned rows read the others too; a data
+ * fault there does not count).  Arguments as for bv_verify.
  */
 int tv_verify(const void* target_logits, const void* draft_logits,
               const int32_t* draft_tokens, const float* uniforms,
@@ -343,7 +348,9 @@ int bv_stream_status(void* stream);
  *   "kernel"        1 flow, 2 cluster, 3 element-wise streaming kernel, 4 small-batch kernel, 5 phase kernel (for
  *                   the shapes each admits; the default picks the small-batch kernel for up to 32 sequences
  *                   whose logits are few enough to make the launch a matter of latency, the phase kernel for
- *                   middling batches and for rows that are not whole 16-byte vectors, else the flow kernel)
+ *                   middling batches and for rows that are not whole 16-byte vectors, the element-wise kernel for
+ *                   a few short ones of these a sequence, else the flow kernel; where fewer SMs than the GPU has can
+ *                   be had at once, the flow or the element-wise kernel)
  *   "small_bytes"   logit megabytes up to which the small-batch kernel is the default
  *   "cluster"       cluster width of the cluster / streaming kernels (1, 2, 4, 8)
  *   "max_clusters"  cap on the clusters those kernels launch

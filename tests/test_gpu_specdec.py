@@ -127,7 +127,7 @@ def test_block_verification_generates_more_per_iteration():
     assert be["block"] > be["token"] and be["block_lse"] > be["token"]
 
 
-@pytest.mark.parametrize("B", [48, 12])        # the flow kernel; the small-batch kernel (a cooperative launch) for block / token
+@pytest.mark.parametrize("B", [48, 12])        # the phase kernel; the small-batch kernel (both cooperative launches)
 @pytest.mark.parametrize("algo", ["block_lse", "block", "token"])
 def test_graph_replay_generates_the_same_tokens(algo, B):
     V, N, gamma = 4096, 9, 5
