@@ -114,6 +114,12 @@ __device__ __forceinline__ float pow2_nonpos(float d) {
     return __int_as_float((n + 127) << 23);
 }
 
+// "No reference yet": finite, so that -inf logits still give 2^-inf = 0 and any logit that counts overflows to +inf, which
+// exceeds the raise bound and installs a real reference.  A scaled logit below it never becomes a reference and weighs nothing: a
+// type's lowest value, as masks put it (-3.4e38), divided by a temperature that leaves it finite, would be its own reference only
+// to within its last bit, 1e31, and 2 to the power of that difference spoils the sum.
+constexpr float kNoRef = -1.0e30f;
+
 // Running sum of 2^{z*k - M} over the elements a thread has seen, where the
 // reference M is an INTEGER (the rounded scaled maximum so far).  An integer
 // reference is exact in fp32, so z*k - M costs one fused multiply-add with a
@@ -127,7 +133,7 @@ struct MaxSum {
 #pragma unroll
         for (int e = 1; e < N; ++e) vm = fmaxf(vm, v[e]);
         const float y = rintf(vm * kf);
-        if (y > M) { s = (s != s) ? s : s * pow2_nonpos(M - y); M = y; }
+        if (y > M && y > kNoRef) { s = (s != s) ? s : s * pow2_nonpos(M - y); M = y; }
         if (M > -INFINITY) {
             const float nM = -M;
 #pragma unroll
@@ -366,9 +372,6 @@ __device__ __forceinline__ uint4 lds128(uint32_t saddr) {
     return v;
 }
 
-// "No reference yet": finite, so that -inf logits still give 2^-inf = 0 and any finite
-// logit overflows to +inf, which exceeds the raise bound and installs a real reference.
-constexpr float kNoRef = -3.0e38f;
 // A vector of 8 terms all at the reference sums to at most 8 * 2^0.5 = 11.3; a sum above
 // this bound therefore means some term exceeds 2^0.5, i.e. its logit lies above the reference.
 // Without a raise every term is below 12, so its exponent is below 4 and is rounded to 1.2e-7.

@@ -204,6 +204,30 @@ def test_masked_logits_and_domain_errors(kernel, bv_options):
     assert np.array_equal(ot.cpu().numpy(), ref.out_tokens)
 
 
+@pytest.mark.parametrize("T", [0.7, 1.0, 2.0])
+@pytest.mark.parametrize("dtype,V", [("bf16", 4096), ("f32", 4096), ("bf16", 4099)])
+@pytest.mark.parametrize("kernel", ["flow", "cluster", "stream", "small", "phase"])
+def test_masks_of_the_lowest_value(kernel, dtype, V, T, bv_options):
+    # all but a few tokens of every row at the type's lowest finite value, which temperatures above log2(e) leave finite:
+    # whole steps of a sweep see nothing else, and it must weigh nothing
+    if V % 8 and kernel in ("flow", "cluster"):
+        pytest.skip("these kernels take rows of whole 16-byte vectors")
+    bv_options("kernel", KERNELS[kernel])
+    inp = random_inputs(12, 3, V, dtype, seed=V, T=T, sigma_d=0.5)
+    t, d, tok = inp["target_logits"], inp["draft_logits"], inp["draft_tokens"]
+    keep = torch.rand((V,), generator=torch.Generator().manual_seed(1)) < 0.01
+    t[:, :, ~keep] = torch.finfo(t.dtype).min
+    d[:, :, ~keep] = torch.finfo(d.dtype).min
+    kept = torch.nonzero(keep).flatten()
+    tok[:] = kept[torch.randint(0, len(kept), tok.shape, generator=torch.Generator().manual_seed(2))].to(torch.int32)
+    for algo in ALGOS:
+        ref = run_oracle(algo, inp)
+        assert (ref.out_len > 0).all()
+        for diag in (True, False):
+            out = run_cuda(algo, inp, diagnostics=diag)
+            assert_parity(compare(algo, ref, out[0], out[1], out[2] if diag else None, inp), diag)
+
+
 def test_deterministic_bits():
     inp = wl.make_inputs(wl.scaled(wl.CONFIGS["c3"], B=8), "cuda")
     a = run_cuda(oracle.BLOCK_VERIFY, inp)

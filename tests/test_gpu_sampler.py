@@ -105,3 +105,13 @@ def test_vectors_of_a_short_row_are_joined_in_double(V, large):
         first = torch.zeros((2,), dtype=torch.int32, device="cuda")
         _, lse = bv.bv_draft_chain(row.expand(V, V).contiguous(), first, torch.full((3, 2), 0.5, device="cuda"), T)
         assert np.abs(lse.cpu().numpy().astype(np.float64) / np.log1p(tiny) - 1.0).max() < 1e-4
+
+
+@pytest.mark.parametrize("dtype,T", [("bf16", 2.0), ("f32", 2.0), ("bf16", 1.0)])
+def test_masks_of_the_lowest_value(dtype, T):
+    g = torch.Generator().manual_seed(5)
+    z = torch.randn((40, 8192), generator=g) * 2.0
+    z = z.bfloat16() if dtype == "bf16" else z
+    z[torch.rand(z.shape, generator=g) > 0.004] = torch.finfo(z.dtype).min
+    z[:, 77] = 1.0
+    check(z, torch.rand((40,), generator=g), T)
