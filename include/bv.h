@@ -320,7 +320,8 @@ int bv_draft_chain(const void* draft_table, const int32_t* first_tokens, const f
  * tokens for every one of B sequences (as bv_draft_chain, from the sequence's last token, with u_draft [iterations,
  * gamma, B]), verifies the block on the table rows along the drafted path, read where they lie (u_verify [iterations, B,
  * gamma+2]; algo: 0 Algorithm 2 and 1 Algorithm 1 with the drafting step's normalisers, 2 and 3 the same without), and
- * appends the emitted tokens to the sequence.  Two launches an iteration, no synchronisation; DEVICE pointers:
+ * appends the emitted tokens to the sequence.  One launch for all of it where two rows fit in an SM's shared memory (up to
+ * 106496 bytes a row), else two an iteration; no synchronisation; DEVICE pointers:
  *   first_tokens [B] int32     the last token of each context
  *   out_tokens  [B, iterations (gamma+1)] int32: the tokens generated, then -1;  out_lengths [B] int64: how many
  *   out_tau     [iterations, B] int32 accepted drafts;  out_drafted [iterations, B, gamma] int32

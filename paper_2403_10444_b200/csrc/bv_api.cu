@@ -655,6 +655,11 @@ int note_cuda_error(cudaError_t e) {
     return BV_ERR_CUDA;
 }
 void note_launches(int n) { t_last_launches = n; }
+int kernel_option() {
+    std::call_once(g_opt_once, load_env_options);
+    std::lock_guard<std::mutex> lock(g_mu);
+    return g_opt.kernel;
+}
 
 int run_tables(int algo, const void* tgt_table, const void* drf_table, const int32_t* first, const int32_t* tok, const float* uni,
                const float* lse_d, int B, int gamma, int V, int dtype, float T, int32_t* ot, int32_t* ol, bool probe, cudaStream_t stream) {

@@ -18,6 +18,30 @@ void note_launches(int n);
 int run_tables(int algo, const void* tgt_table, const void* drf_table, const int32_t* first, const int32_t* tok, const float* uni,
                const float* lse_d, int B, int gamma, int V, int dtype, float T, int32_t* ot, int32_t* ol, bool probe, cudaStream_t stream);
 
+// The option "kernel" (0: chosen by shape).
+int kernel_option();
+
+// The decoding loop in one kernel (bv_loop.cu), a CTA per sequence, for rows of which two fit in shared memory.
+struct LoopArgs {
+    const void* tgt;          // tables [V, V]
+    const void* drf;
+    const int32_t* first;     // [B]
+    const float* u_draft;     // [iterations, gamma, B]
+    const float* u_verify;    // [iterations, B, gamma+2]
+    int iterations, B, gamma, V, width;
+    float kf;
+    double kd;
+    int token;                // Algorithm 1 instead of Algorithm 2
+    int lse;                  // the verification takes the draft rows' normalisers as the drafting step rounds them to 32 bits
+    int32_t* seq;             // [B, width]
+    long long* lengths;       // [B]
+    int32_t* tau;             // [iterations, B]
+    int32_t* drafted;         // [iterations, B, gamma]
+    int32_t* fault;           // set if a sequence reports a data fault
+};
+bool loop_fits(int V, int dtype);
+cudaError_t launch_loop(const LoopArgs& args, int dtype, cudaStream_t stream);
+
 // Most clusters of `cluster` CTAs of the streaming kernel that can be resident at once
 // on the current device (0 if that cluster size cannot be scheduled).
 int stream_max_clusters(int algo, int dtype, bool vec, int cluster);

@@ -46,7 +46,7 @@ def run(target_table: torch.Tensor, draft_table: torch.Tensor, first_tokens: tor
     (the iteration number lives in a device counter), so with ``graph=True`` one iteration is
     captured in a CUDA graph and replayed: the launches of an iteration then cost one graph launch
     instead of one driver call each.  Data faults are looked for once, after the last iteration.
-    By default the loop runs natively (``bv_decode_loop``), two launches per iteration.
+    By default the loop runs natively (``bv_decode_loop``): one launch, or two per iteration for rows above 104 KB.
     ``chain``: the gamma drafted tokens of an iteration come from one launch of ``bv_draft_chain``
     (default) instead of gamma calls of ``bv_sample_draft`` with their look-ups and copies.
     """
@@ -61,7 +61,7 @@ def run(target_table: torch.Tensor, draft_table: torch.Tensor, first_tokens: tor
     dev = target_table.device
     width = N * (gamma + 1)
     if chain and not graph and _native(target_table, draft_table, first_tokens, u_draft, u_verify, gamma):
-        # (two launches an iteration, the tables' rows read where they lie)
+        # (the tables' rows read where they lie)
         res = bv.bv_decode_loop(target_table, draft_table, first_tokens.to(torch.int32).contiguous(), u_draft.contiguous(),
                                 u_verify.contiguous(), gamma, temperature, ("block_lse", "token_lse", "block", "token").index(algo))
         if res is not None:
