@@ -10,7 +10,7 @@
 // (Eq. "pacc_block"), whose rows come from L2 once more.
 //
 // Bound: latency, gamma dependent rows and one or two dependent sweeps an iteration; bytes B (2 gamma + 1) rows an iteration.
-// 128 sequences of gamma = 5 over V = 16384 in bf16, 8 iterations: 318 us, 40 an iteration (two launches an iteration, the
+// 128 sequences of gamma = 5 over V = 16384 in bf16, 8 iterations: 283 us, 35 an iteration (two launches an iteration, the
 // chain and a verification by all SMs together with its waits for the whole batch: 606 us; the bytes take 56).
 #include "bv_sample_row.cuh"
 
@@ -40,27 +40,92 @@ __device__ __forceinline__ void l_fetch(uint32_t image, const char* row, int uni
 __device__ __forceinline__ uint4 l_cell(uint32_t image, int i, int u1, uint32_t pad) {
     return i < u1 ? lds128(image + static_cast<uint32_t>(i) * 16u) : make_uint4(pad, pad, pad, pad);
 }
-constexpr int kLoopRuns = 4;                      // runs of 32 vectors whose cells are read together
+constexpr int kLoopRuns = 4;                      // runs of 32 vectors that a warp goes through together
+// A step waits for each of these sweeps, and a warp has few runs of its row: what costs is the chain of dependent instructions,
+// not their number.  So kLoopRuns runs share one reference, the rounded maximum of all their logits, found before the first
+// exponential (a run at a time, each testing whether its sum shows a logit above the reference: 1.65 us for a row of 2048
+// vectors; like this 0.8), and their sums cross the lanes side by side.
+
+// the larger of the elements of two vectors, pair by pair (a NaN loses: it shows in the sum)
+template <int DT> __device__ __forceinline__ uint4 l_max(const uint4& x, const uint4& y);
+template <> __device__ __forceinline__ uint4 l_max<kBF16>(const uint4& x, const uint4& y) {
+    uint4 m;
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(m.x) : "r"(x.x), "r"(y.x));
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(m.y) : "r"(x.y), "r"(y.y));
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(m.z) : "r"(x.z), "r"(y.z));
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(m.w) : "r"(x.w), "r"(y.w));
+    return m;
+}
+template <> __device__ __forceinline__ uint4 l_max<kF32>(const uint4& x, const uint4& y) {
+    auto m = [](uint32_t p, uint32_t q) { return __float_as_uint(fmaxf(__uint_as_float(p), __uint_as_float(q))); };
+    return make_uint4(m(x.x, y.x), m(x.y, y.y), m(x.z, y.z), m(x.w, y.w));
+}
+// kLoopRuns runs of a row from vector `base` on: the reference raised to their maximum, by how much 2^-that is returned, and
+// each run's sum of this lane's terms
+template <int DT>
+__device__ __forceinline__ float l_group(uint32_t image, int base, int u1, int lane, float kf, float& M, float (&vs)[kLoopRuns]) {
+    using R = Raw<DT>;
+    constexpr int EPV = R::EPV;
+    uint4 raw[kLoopRuns];
+#pragma unroll
+    for (int j = 0; j < kLoopRuns; ++j) raw[j] = l_cell(image, base + 32 * j + lane, u1, R::kNegInf);
+    uint4 top = raw[0];
+#pragma unroll
+    for (int j = 1; j < kLoopRuns; ++j) top = l_max<DT>(top, raw[j]);
+    float v[EPV];
+    R::unpack(top, v);
+    const float y = fmaxf(M, rintf(warp_max(vec_max<EPV>(v)) * kf)), scale = ref_scale(M, y);
+    M = y;
+#pragma unroll
+    for (int j = 0; j < kLoopRuns; ++j) {
+        R::unpack(raw[j], v);
+        vs[j] = f_exp_sum<EPV>(v, kf, -M);
+    }
+    return scale;
+}
 
 // s_sweep_row on the row's image
 template <int DT, bool SHORT>
 __device__ __forceinline__ void l_sweep_draft(uint32_t image, int units, float kf, int warp, int lane, SubSegment<SHORT>* seg) {
-    using R = Raw<DT>;
-    constexpr int EPV = R::EPV;
     float M = kNoRef, s = 0.f;
     int u0, u1, runs;
     s_part(units, warp, u0, u1, runs);
     int sub = 0, left = runs;
     for (int base = u0; base < u1; base += 32 * kLoopRuns) {
-        uint4 raw[kLoopRuns];
+        float vs[kLoopRuns];
+        s *= l_group<DT>(image, base, u1, lane, kf, M, vs);
+        const int n = min((u1 - base + 31) / 32, kLoopRuns);
+        if (runs == 1) {                          // (a sub-segment a run; a group of fewer has empty ones behind it)
+            if (SHORT) {
+                double z[kLoopRuns];
 #pragma unroll
-        for (int j = 0; j < kLoopRuns; ++j) raw[j] = l_cell(image, base + 32 * j + lane, u1, R::kNegInf);
+                for (int j = 0; j < kLoopRuns; ++j) z[j] = static_cast<double>(vs[j]);
 #pragma unroll
-        for (int j = 0; j < kLoopRuns; ++j) {
-            if (base + 32 * j < u1) {
-                float v[EPV];
-                R::unpack(raw[j], v);
-                f_accumulate<EPV>(v, kf, M, s);
+                for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+                    for (int j = 0; j < kLoopRuns; ++j) z[j] += shfl_xor_d(z[j], off);
+                }
+#pragma unroll
+                for (int j = 0; j < kLoopRuns; ++j)
+                    if (j < n && (lane & 15) == 0)
+                        reinterpret_cast<float2*>(seg + s_place(warp, sub + j))[lane >> 4] =
+                            lane == 0 ? make_float2(__int_as_float(__double2loint(z[j])), __int_as_float(__double2hiint(z[j]))) : make_float2(M, 0.f);
+            } else {
+#pragma unroll
+                for (int off = 8; off > 0; off >>= 1) {
+#pragma unroll
+                    for (int j = 0; j < kLoopRuns; ++j) vs[j] += __shfl_xor_sync(0xffffffffu, vs[j], off);
+                }
+#pragma unroll
+                for (int j = 0; j < kLoopRuns; ++j)
+                    if (j < n && (lane & 15) == 0) reinterpret_cast<float2*>(seg + s_place(warp, sub + j))[lane >> 4] = make_float2(vs[j], M);
+            }
+            sub += n;
+        } else {
+#pragma unroll
+            for (int j = 0; j < kLoopRuns; ++j) {
+                if (j >= n) break;
+                s += vs[j];
                 if (--left == 0) {
                     s_put<SHORT>(M, s, lane, seg + s_place(warp, sub));
                     ++sub;
@@ -79,23 +144,13 @@ __device__ __forceinline__ void l_sweep_draft(uint32_t image, int units, float k
 // a warp's share {reference, sum} of a target row: fp32 over a lane's vectors (13 at most), joined in double
 template <int DT>
 __device__ __forceinline__ void l_sweep_target(uint32_t image, int units, float kf, int warp, int lane, LoopShared& sh) {
-    using R = Raw<DT>;
-    constexpr int EPV = R::EPV;
     float M = kNoRef, s = 0.f;
     int u0, u1, runs;
     s_part(units, warp, u0, u1, runs);
     for (int base = u0; base < u1; base += 32 * kLoopRuns) {
-        uint4 raw[kLoopRuns];
-#pragma unroll
-        for (int j = 0; j < kLoopRuns; ++j) raw[j] = l_cell(image, base + 32 * j + lane, u1, R::kNegInf);
-#pragma unroll
-        for (int j = 0; j < kLoopRuns; ++j) {
-            if (base + 32 * j < u1) {
-                float v[EPV];
-                R::unpack(raw[j], v);
-                f_accumulate<EPV>(v, kf, M, s);
-            }
-        }
+        float vs[kLoopRuns];
+        s *= l_group<DT>(image, base, u1, lane, kf, M, vs);
+        s += (vs[0] + vs[1]) + (vs[2] + vs[3]);
     }
     const double z = warp_sum_d(static_cast<double>(s));
     if (lane == 0) { sh.wM[warp] = static_cast<double>(M); sh.wZ[warp] = z; }
@@ -110,17 +165,30 @@ __device__ __forceinline__ void l_sweep_pair(uint32_t imageP, uint32_t imageQ, i
     s_part(units, warp, u0, u1, runs);
     double acc = 0.0;
     int sub = 0, left = runs;
-    for (int base = u0; base < u1; base += 32) {
-        float vp[EPV], vq[EPV], t[EPV];
-        R::unpack(l_cell(imageP, base + lane, u1, R::kNegInf), vp);
-        R::unpack(l_cell(imageQ, base + lane, u1, R::kNegInf), vq);
-        acc += static_cast<double>(f_pair_sum<EPV, true>(vp, vq, kf, cp, nMP, nMQ, t));
-        if (--left == 0 || base + 32 >= u1) {
-            const double z = warp_sum_d(acc);
-            if (lane == 0) res[warp * kSSub + sub] = z;
-            ++sub;
-            left = runs;
-            acc = 0.0;
+    for (int base = u0; base < u1; base += 32 * kLoopRuns) {
+        double z[kLoopRuns];
+#pragma unroll
+        for (int j = 0; j < kLoopRuns; ++j) {
+            float vp[EPV], vq[EPV], t[EPV];
+            R::unpack(l_cell(imageP, base + 32 * j + lane, u1, R::kNegInf), vp);
+            R::unpack(l_cell(imageQ, base + 32 * j + lane, u1, R::kNegInf), vq);
+            z[j] = static_cast<double>(f_pair_sum<EPV, true>(vp, vq, kf, cp, nMP, nMQ, t));
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+            for (int j = 0; j < kLoopRuns; ++j) z[j] += shfl_xor_d(z[j], off);
+        }
+#pragma unroll
+        for (int j = 0; j < kLoopRuns; ++j) {
+            if (base + 32 * j >= u1) break;
+            acc += z[j];
+            if (--left == 0 || base + 32 * (j + 1) >= u1) {
+                if (lane == 0) res[warp * kSSub + sub] = acc;
+                ++sub;
+                left = runs;
+                acc = 0.0;
+            }
         }
     }
     if (lane >= sub && lane < kSSub) res[warp * kSSub + lane] = 0.0;
@@ -141,12 +209,14 @@ __device__ __forceinline__ int l_rescan(uint32_t imageP, uint32_t imageQ, int un
         R::unpack(l_cell(imageP, i, w1, R::kNegInf), vp);
         if (HAVEQ) R::unpack(l_cell(imageQ, i, w1, R::kNegInf), vq);
         f_pair_sum<EPV, HAVEQ>(vp, vq, kf, cp, nMP, nMQ, t);
-        double ls = 0.0;
+        // (a lane's own prefix sums beside the sums over the lanes, so that the lane that is found has only to compare)
+        double own[EPV];
 #pragma unroll
         for (int e = 0; e < EPV; ++e) {
-            ls += static_cast<double>(t[e]);
+            own[e] = (e > 0 ? own[e > 0 ? e - 1 : 0] : 0.0) + static_cast<double>(t[e]);
             if (t[e] > 0.f) last_pos = i * EPV + e;
         }
+        const double ls = own[EPV - 1];
         double inc = ls;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -155,20 +225,15 @@ __device__ __forceinline__ int l_rescan(uint32_t imageP, uint32_t imageQ, int un
         }
         const unsigned bal = __ballot_sync(0xffffffffu, run + inc > tw && ls > 0.0);
         if (bal) {
-            const int src = __ffs(bal) - 1;
-            int f = -1;
-            if (lane == src) {
-                double cum = run + inc - ls;
-                int lp = -1;
+            const double before = run + inc - ls;
+            int f = -1, lp = -1;
 #pragma unroll
-                for (int e = 0; e < EPV; ++e) {
-                    cum += static_cast<double>(t[e]);
-                    if (t[e] > 0.f) lp = i * EPV + e;
-                    if (f < 0 && cum > tw && t[e] > 0.f) f = i * EPV + e;
-                }
-                if (f < 0) f = lp;
+            for (int e = EPV - 1; e >= 0; --e) {
+                if (t[e] > 0.f && lp < 0) lp = i * EPV + e;
+                if (t[e] > 0.f && before + own[e] > tw) f = i * EPV + e;
             }
-            found = __shfl_sync(0xffffffffu, f, src);
+            if (f < 0) f = lp;
+            found = __shfl_sync(0xffffffffu, f, __ffs(bal) - 1);
         }
         run += shfl_d(inc, 31);
     }
