@@ -137,14 +137,17 @@ struct DeviceState {
     int flow_ctas_per_sm[2] = {};
     int small_ctas[2] = {};            // small-batch kernel: CTAs of a launch per dtype (0: not asked yet)
     int phase_ctas[2] = {};            // the phase kernel's
-    // staging for the host-buffer entry points
+    // staging for the host-buffer entry points, on the device and, for what is small, in pinned host memory
     void* stage = nullptr;
     size_t stage_bytes = 0;
+    char* pinned = nullptr;
+    size_t pinned_bytes = 0;
     cudaStream_t stream = nullptr;     // theirs, and where memory is obtained while a caller's stream is captured
 };
 
 DeviceState g_dev[kMaxDevices];
 std::mutex g_mu;
+std::mutex g_host_mu;               // held for the whole of a call on host buffers: they share the staging areas
 
 thread_local int t_last_launches = 0;
 thread_local int t_last_kernel = 0;     // which kernel the last verification call on this thread launched (the "kernel" option's codes)
@@ -380,7 +383,7 @@ int run_phase(DeviceState& d, const bv::Params& prm, int dtype, bool vec, bool p
         if (prm.out_h) p.out_h = prm.out_h + b * (g + 1);
         if (prm.out_lse_t) p.out_lse_t = prm.out_lse_t + b * (g + 1);
         if (prm.out_lse_d) p.out_lse_d = prm.out_lse_d + b * g;
-        p.status = reinterpret_cast<int*>(slot->head.p);
+        if (p.status == nullptr) p.status = reinterpret_cast<int*>(slot->head.p);
         if (p.B != part) plan = bv::phase_plan(p.V, dtype, vec, p.B, g, p.lse_d != nullptr, nc);
         bv::phase_scratch(slot->scratch.p, reinterpret_cast<unsigned*>(slot->head.p + kSlotPhase), p.B, g, plan, &ps);
         const cudaError_t e = bv::launch_phase(p, ps, dtype, vec, nc, stream);
@@ -395,6 +398,7 @@ struct Extra {              // what only some entry points pass
     const float* lse_d = nullptr;   // supplied draft log-normalisers (bv_verify_lse)
     int greedy = 0;                 // Algorithm 4 instead of Algorithm 2 (gbv_verify)
     const int32_t* first = nullptr; // the rows are those of two tables (Params::first)
+    int* status = nullptr;          // where a wait that gives up is recorded (null: the stream's status word)
     bool probe = false;             // find the kernel and its workspace, launch nothing
     int probs = 0;                  // the rows hold probabilities, not logits (bv_verify_probs, tv_verify_probs)
     float* out_p = nullptr; float* out_S = nullptr; float* out_h = nullptr;
@@ -434,6 +438,7 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
     prm.out_lse_t = ex.out_lse_t; prm.out_lse_d = ex.out_lse_d;
     prm.wait_limit = opt.wait_limit > 0 ? static_cast<unsigned>(opt.wait_limit) : 0u;
     prm.never_signal = opt.never_signal;
+    prm.status = ex.status;
 
     prm.algo = algo;
     const long long logit_bytes = static_cast<long long>(B) * (2 * gamma + 1) * static_cast<long long>(row_bytes);
@@ -472,7 +477,7 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
             bv::small_scratch_layout(slot->scratch.p, reinterpret_cast<unsigned*>(slot->head.p + 128), B, gamma, plan, &sc);
             prm.ticket = nullptr;
             prm.nclusters = 0;
-            prm.status = reinterpret_cast<int*>(slot->head.p);
+            prm.status = ex.status ? ex.status : reinterpret_cast<int*>(slot->head.p);
             const cudaError_t e = bv::launch_small(prm, sc, dtype, vec, nc, stream);
             if (e == cudaSuccess) {
                 t_last_launches = 1; t_last_kernel = 4;
@@ -518,7 +523,7 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
             if (nctas > items) nctas = items;
             prm.ticket = nullptr;
             prm.nclusters = 0;
-            prm.status = reinterpret_cast<int*>(slot->head.p);
+            prm.status = ex.status ? ex.status : reinterpret_cast<int*>(slot->head.p);
             const cudaError_t e = bv::launch_flow(prm, fl, dtype, static_cast<int>(nctas), stream);
             if (e != cudaSuccess) return cuda_fail(e);
             t_last_launches = 1; t_last_kernel = 1;
@@ -530,7 +535,7 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
 
     StreamSlot* slot = nullptr;
     if ((rc = stream_slot(*d, stream, 0, 0, &slot)) != BV_OK) return rc;
-    prm.status = reinterpret_cast<int*>(slot->head.p);
+    prm.status = ex.status ? ex.status : reinterpret_cast<int*>(slot->head.p);
 
     int cluster = pick_cluster(*d, opt, B, row_bytes);
     if (vec && opt.kernel != 3) {
@@ -602,19 +607,24 @@ int run_host(int algo, const void* tgt, const void* drf, const int32_t* tok, con
     const size_t n_d = static_cast<size_t>(B) * gamma * V * esz;
     const size_t n_tok = static_cast<size_t>(B) * gamma * 4, n_uni = static_cast<size_t>(B) * (gamma + 2) * 4;
     const size_t n_ot = static_cast<size_t>(B) * (gamma + 1) * 4, n_ol = static_cast<size_t>(B) * 4;
-    const size_t o_t = 0, o_d = align_up(o_t + n_t, 256), o_tok = align_up(o_d + n_d, 256);
-    const size_t o_uni = align_up(o_tok + n_tok, 256), o_ot = align_up(o_uni + n_uni, 256);
-    const size_t o_ol = align_up(o_ot + n_ot, 256), total = align_up(o_ol + n_ol, 256);
+    // The small arrays travel together, in with the status word behind them and out with it in front: one copy each way beside
+    // the two of the logits.  (A copy more costs some 5 us in the stream's order: 8 sequences of gamma = 8, V = 32000 in 32 bits,
+    // 17 MB, with seven copies and a memset 391 us a call, 311 of them the logits' on the link.)
+    const size_t o_t = 0, o_d = align_up(o_t + n_t, 256), o_in = align_up(o_d + n_d, 256);
+    const size_t i_uni = align_up(n_tok, 16), i_status = align_up(i_uni + n_uni, 16), i_ot = i_status + 16, i_ol = align_up(i_ot + n_ot, 16);
+    const size_t n_in = i_ot, n_small = i_ol + n_ol, total = o_in + n_small;
 
+    std::lock_guard<std::mutex> host_lock(g_host_mu);
     char* base = nullptr;
+    char* pin = nullptr;
     cudaStream_t s = nullptr;
+    cudaError_t e;
     {
         std::lock_guard<std::mutex> lock(g_mu);
         DeviceState* d = nullptr;
         if ((rc = device_state(&d)) != BV_OK) return rc;
-        cudaError_t e;
         if ((rc = own_stream(*d)) != BV_OK) return rc;
-        // (this entry point waits for its result anyway, so its staging buffer grows with plain cudaMalloc)
+        // (this entry point waits for its result anyway, so its staging buffers grow with plain cudaMalloc)
         if (d->stage_bytes < total) {
             if (d->stage) cudaFree(d->stage);
             d->stage = nullptr;
@@ -622,21 +632,43 @@ int run_host(int algo, const void* tgt, const void* drf, const int32_t* tok, con
             if ((e = cudaMalloc(&d->stage, total)) != cudaSuccess) return cuda_fail(e);
             d->stage_bytes = total;
         }
+        if (d->pinned_bytes < n_small) {
+            if (d->pinned) cudaFreeHost(d->pinned);
+            d->pinned = nullptr;
+            d->pinned_bytes = 0;
+            if ((e = cudaHostAlloc(reinterpret_cast<void**>(&d->pinned), n_small, cudaHostAllocPortable)) != cudaSuccess) return cuda_fail(e);
+            d->pinned_bytes = n_small;
+        }
         base = static_cast<char*>(d->stage);
+        pin = d->pinned;
         s = d->stream;
     }
-    cudaError_t e;
-    if ((e = cudaMemcpyAsync(base + o_t, tgt, n_t, cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail(e);
-    if ((e = cudaMemcpyAsync(base + o_d, drf, n_d, cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail(e);
-    if ((e = cudaMemcpyAsync(base + o_tok, tok, n_tok, cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail(e);
-    if ((e = cudaMemcpyAsync(base + o_uni, uni, n_uni, cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail(e);
-    rc = run_device(algo, base + o_t, base + o_d, reinterpret_cast<const int32_t*>(base + o_tok),
-                    reinterpret_cast<const float*>(base + o_uni), B, gamma, V, dtype, T,
-                    reinterpret_cast<int32_t*>(base + o_ot), reinterpret_cast<int32_t*>(base + o_ol), Extra{}, s);
+    char* const in = base + o_in;
+    std::memcpy(pin, tok, n_tok);
+    std::memcpy(pin + i_uni, uni, n_uni);
+    std::memset(pin + i_status, 0, 16);
+    // (whatever fails below, nothing of this call is under way any more when the buffers are let go)
+    auto enqueue = [&]() -> int {
+        if ((e = cudaMemcpyAsync(in, pin, n_in, cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail(e);
+        if ((e = cudaMemcpyAsync(base + o_t, tgt, n_t, cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail(e);
+        if ((e = cudaMemcpyAsync(base + o_d, drf, n_d, cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail(e);
+        Extra ex;
+        ex.status = reinterpret_cast<int*>(in + i_status);
+        const int done = run_device(algo, base + o_t, base + o_d, reinterpret_cast<const int32_t*>(in), reinterpret_cast<const float*>(in + i_uni),
+                                    B, gamma, V, dtype, T, reinterpret_cast<int32_t*>(in + i_ot), reinterpret_cast<int32_t*>(in + i_ol), ex, s);
+        if (done != BV_OK) return done;
+        if ((e = cudaMemcpyAsync(pin + i_status, in + i_status, n_small - i_status, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return cuda_fail(e);
+        return BV_OK;
+    };
+    rc = enqueue();
+    e = cudaStreamSynchronize(s);
     if (rc != BV_OK) return rc;
-    if ((e = cudaMemcpyAsync(ot, base + o_ot, n_ot, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return cuda_fail(e);
-    if ((e = cudaMemcpyAsync(ol, base + o_ol, n_ol, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return cuda_fail(e);
-    return take_stream_status(s);
+    if (e != cudaSuccess) return cuda_fail(e);
+    std::memcpy(ot, pin + i_ot, n_ot);
+    std::memcpy(ol, pin + i_ol, n_ol);
+    int status = 0;
+    std::memcpy(&status, pin + i_status, sizeof(int));
+    return status ? BV_ERR_TIMEOUT : BV_OK;
 }
 
 Extra diagnostics(float* out_p, float* out_S, float* out_h, float* out_lse_t, float* out_lse_d) {
@@ -810,6 +842,7 @@ int bv_set_option(const char* name, int value) {
 }
 
 int bv_release(void) {
+    std::lock_guard<std::mutex> host_lock(g_host_mu);
     std::lock_guard<std::mutex> lock(g_mu);
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -818,6 +851,7 @@ int bv_release(void) {
     DeviceState& d = g_dev[dev];
     if ((e = cudaDeviceSynchronize()) != cudaSuccess) return cuda_fail(e);
     if (d.stage) cudaFree(d.stage);
+    if (d.pinned) cudaFreeHost(d.pinned);
     if (d.tickets) cudaFree(d.tickets);
     for (StreamSlot& c : d.slots) {
         for (char* p : c.outgrown) cudaFree(p);
