@@ -62,8 +62,8 @@ constexpr long long kPhaseFewRow = 700000;
 constexpr long long kPhaseAllBytes[2] = {360LL << 20, 144LL << 20}, kPhaseAllBytesLong[2] = {360LL << 20, 60LL << 20};
 constexpr long long kPhaseAllRows[2] = {2500000, 2200000}, kPhaseAllSmall = 1300000;
 constexpr size_t kSlotHead = 16384;   // first area of a stream's workspace: status word, barrier words, the phase kernel's counters
-constexpr size_t kSlotPhase = 256;    // ... the last of these from here on
-static_assert(kSlotPhase + bv::kPhaseCounterWords * sizeof(unsigned) <= kSlotHead, "the counters fit in the head");
+constexpr size_t kSlotPhase = 256, kSlotSmall = 8192;    // ... the phase kernel's from here on, the small-batch kernel's counters of its sequences
+static_assert(kSlotPhase + bv::kPhaseCounterWords * sizeof(unsigned) <= kSlotSmall && kSlotSmall + bv::kSmallMaxB * sizeof(unsigned) <= kSlotHead, "the counters fit in the head");
 constexpr int kStreamSlots = 32;  // streams per device that keep a workspace of their own
 
 // Tuning and test options (bv_set_option); their first values come from the environment, read once.
@@ -474,7 +474,8 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
             if (rc != BV_OK || ex.probe) return rc;
             bv::SmallScratch sc;
             // the barrier words are in the head: zero since it was allocated
-            bv::small_scratch_layout(slot->scratch.p, reinterpret_cast<unsigned*>(slot->head.p + 128), B, gamma, plan, &sc);
+            bv::small_scratch_layout(slot->scratch.p, reinterpret_cast<unsigned*>(slot->head.p + 128), reinterpret_cast<unsigned*>(slot->head.p + kSlotSmall),
+                                     B, gamma, plan, &sc);
             prm.ticket = nullptr;
             prm.nclusters = 0;
             prm.status = ex.status ? ex.status : reinterpret_cast<int*>(slot->head.p);

@@ -288,6 +288,16 @@ template <> struct Raw<kF32> {
     }
 };
 
+// the larger of the elements of two vectors, element by element (a NaN loses)
+template <int DT> __device__ __forceinline__ uint4 vec_max(const uint4& x, const uint4& y) {
+    auto m = [](uint32_t p, uint32_t q) {
+        if (DT == kF32) return __float_as_uint(fmaxf(__uint_as_float(p), __uint_as_float(q)));
+        uint32_t r;
+        asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(p), "r"(q));
+        return r;
+    };
+    return make_uint4(m(x.x, y.x), m(x.y, y.y), m(x.z, y.z), m(x.w, y.w));
+}
 template <int EPV> __device__ __forceinline__ float vec_max(const float (&v)[EPV]) {
     float vm = v[0];
 #pragma unroll

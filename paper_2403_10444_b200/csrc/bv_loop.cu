@@ -44,22 +44,8 @@ constexpr int kLoopRuns = 4;                      // runs of 32 vectors that a w
 // A step waits for each of these sweeps, and a warp has few runs of its row: what costs is the chain of dependent instructions,
 // not their number.  So kLoopRuns runs share one reference, the rounded maximum of all their logits, found before the first
 // exponential (a run at a time, each testing whether its sum shows a logit above the reference: 1.65 us for a row of 2048
-// vectors; like this 0.8), and their sums cross the lanes side by side.
+// vectors; like this 1.2), and their sums cross the lanes side by side.
 
-// the larger of the elements of two vectors, pair by pair (a NaN loses: it shows in the sum)
-template <int DT> __device__ __forceinline__ uint4 l_max(const uint4& x, const uint4& y);
-template <> __device__ __forceinline__ uint4 l_max<kBF16>(const uint4& x, const uint4& y) {
-    uint4 m;
-    asm("max.bf16x2 %0, %1, %2;" : "=r"(m.x) : "r"(x.x), "r"(y.x));
-    asm("max.bf16x2 %0, %1, %2;" : "=r"(m.y) : "r"(x.y), "r"(y.y));
-    asm("max.bf16x2 %0, %1, %2;" : "=r"(m.z) : "r"(x.z), "r"(y.z));
-    asm("max.bf16x2 %0, %1, %2;" : "=r"(m.w) : "r"(x.w), "r"(y.w));
-    return m;
-}
-template <> __device__ __forceinline__ uint4 l_max<kF32>(const uint4& x, const uint4& y) {
-    auto m = [](uint32_t p, uint32_t q) { return __float_as_uint(fmaxf(__uint_as_float(p), __uint_as_float(q))); };
-    return make_uint4(m(x.x, y.x), m(x.y, y.y), m(x.z, y.z), m(x.w, y.w));
-}
 // kLoopRuns runs of a row from vector `base` on: the reference raised to their maximum, by how much 2^-that is returned, and
 // each run's sum of this lane's terms
 template <int DT>
@@ -71,7 +57,7 @@ __device__ __forceinline__ float l_group(uint32_t image, int base, int u1, int l
     for (int j = 0; j < kLoopRuns; ++j) raw[j] = l_cell(image, base + 32 * j + lane, u1, R::kNegInf);
     uint4 top = raw[0];
 #pragma unroll
-    for (int j = 1; j < kLoopRuns; ++j) top = l_max<DT>(top, raw[j]);
+    for (int j = 1; j < kLoopRuns; ++j) top = vec_max<DT>(top, raw[j]);
     float v[EPV];
     R::unpack(top, v);
     const float y = fmaxf(M, rintf(warp_max(vec_max<EPV>(v)) * kf)), scale = ref_scale(M, y);

@@ -4,7 +4,7 @@
 //
 // The flow kernel hands work from CTA to CTA through queues and counters in global memory, and a
 // sequence goes through a dozen such hand-overs of a microsecond or more each.  Here all CTAs of a
-// cooperative launch walk through three phases separated by two grid-wide barriers:
+// cooperative launch walk through three phases, a grid-wide barrier between the first two:
 //   1. every row (all 2 gamma + 1 of every sequence, whether the algorithm will want them or not:
 //      the bytes are few) is cut into chunks and every CTA reduces its chunks to {reference, sum};
 //   2. every CTA combines all chunks (fp64) and runs the scalar part for every sequence itself -
@@ -12,8 +12,11 @@
 //      Algorithm 1, and which positions can be the selected one - so that all CTAs know the same
 //      list of (position, piece) items without talking to each other; each takes its share and
 //      leaves per-segment sums of the residual terms max(p_i P_i - Q_i, 0) (rows now come from L2);
-//   3. one CTA per sequence: S_i and h_i (Eq. "pacc_block") of the candidates from the top down, tau,
-//      and the token by inverse CDF over the segment sums and a rescan of one segment.
+//   3. the CTA whose item is the last of a sequence ends it, a warp per candidate: S_i and h_i (Eq. "pacc_block") and, if the
+//      position passes, its token by inverse CDF over the segment sums and a rescan of one segment; then tau and the output.
+//      (A second barrier, the sums of all candidates, and only then the chosen one's token were two trips to L2 more.)
+// Bound: latency, a trip to L2 or memory for each of some eight dependent steps.  B = 1, gamma = 8, V = 152064 bf16 19.1 us a call
+// (19.8 with two barriers and pieces fixed on the host), B = 8, V = 32000 in 32 bits 19.8 (22.6), B = 24, gamma = 5, V = 50257 45 (45).
 // Arithmetic, sampling convention and outputs are those of the flow kernel.
 #include <cooperative_groups.h>
 
@@ -27,7 +30,7 @@ constexpr int kSmAllThreads = kSmThreads + 32;
 constexpr int kSmMaxRows = 1056;      // rows B (2 gamma + 1) whose normalisers a CTA keeps in shared memory
 constexpr int kSmMaxPos = 560;        // positions B (gamma + 1)
 constexpr int kSmInFlight = 8;        // 16-byte loads a thread has in flight in the first phase
-constexpr int kSmPairsInFlight = 5;   // pairs of them in the second (unaligned rows: three of one and two)
+constexpr int kSmPairsInFlight = 5;   // pairs of them in the second (unaligned rows: one less, the registers)
 constexpr int kSmMaxUni = kSmMaxPos + kSmallMaxB;   // uniforms B (gamma + 2)
 
 struct SmallShared {
@@ -43,7 +46,11 @@ struct SmallShared {
     int item0[kSmallMaxB + 1];        // first item of every sequence in the second phase
     float wM[kSmWarps];
     float wS[kSmWarps];
-    double cS[kSmMaxPos];             // third phase: S_i of this CTA's sequence
+    double cS[kMaxGamma];             // third phase: S_i of this CTA's sequence, the positions' tokens, which of them pass
+    int found[kMaxGamma + 1];
+    unsigned char pass[kMaxGamma + 1];
+    int np;                           // pieces a position is cut into in the second phase
+    unsigned ends;                    // sequences whose last item was this CTA's
     // fetched by the extra warp during the first phase: the logits of the drafted tokens, the uniforms
     float zp[kSmMaxPos], zq[kSmMaxPos];
     unsigned char xok[kSmMaxPos];
@@ -80,16 +87,22 @@ __device__ __forceinline__ const char* small_row(const Params& prm, size_t row_b
                   : static_cast<const char*>(prm.drf) + draft_row(prm, b, j - g - 1) * row_bytes;
 }
 
-// vector i of the nv that a row's bytes lie in, from `base` on; [lo, hi): the tensor
-template <int DT, bool AL>
-__device__ __forceinline__ uint4 small_load(const char* base, int i, int nv, const char* lo, const char* hi, uint32_t pad) {
-    const char* p = base + static_cast<long long>(i) * 16;
+// Vector i of a row if it is one of i0 .. i1-1, which lie in the tensor as a whole.
+__device__ __forceinline__ uint4 small_load(const char* base, int i, int i0, int i1, uint32_t pad) {
+    if (i < i0 || i >= i1) return make_uint4(pad, pad, pad, pad);
+    return ld_stream_v4(base + static_cast<long long>(i) * 16);
+}
+// The first and the last of the nv vectors that a row of V elements lies in, h elements into the first (rows at any alignment):
+// the row's own elements, the others as `pad`.
+template <int DT>
+__device__ __forceinline__ uint4 small_edge(const char* row, int i, int h, int V, uint32_t pad) {
+    return row_elements<DT>(row, i * Raw<DT>::EPV - h, V, pad);
+}
+// ... any of the nv, those between them as they lie in memory
+template <int DT>
+__device__ __forceinline__ uint4 small_any(const char* base, int i, int nv, const char* row, int h, int V, uint32_t pad) {
     if (i < 0 || i >= nv) return make_uint4(pad, pad, pad, pad);
-    if (AL || (p >= lo && p + 16 <= hi)) return ld_stream_v4(p);
-    constexpr int ESZ = (DT == kF32) ? 4 : 2;                // (it reaches outside the tensor: the elements inside)
-    int first, n;
-    elements_inside<16 / ESZ>(p, lo, hi, first, n);
-    return row_elements<DT>(p + first * ESZ, -first, n - first, pad);
+    return i > 0 && i < nv - 1 ? ld_stream_v4(base + static_cast<long long>(i) * 16) : small_edge<DT>(row, i, h, V, pad);
 }
 // 16 bytes from byte 4 q + bits / 8 on of two neighbouring vectors
 __device__ __forceinline__ uint4 small_shift(const uint4& a, const uint4& b, int q, int bits) {
@@ -106,18 +119,13 @@ template <int DT, bool PROBS, bool AL>
 __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __grid_constant__ Params prm, const __grid_constant__ SmallScratch sc) {
     using R = Raw<DT>;
     constexpr int EPV = R::EPV;
-    constexpr int kPairs = AL ? kSmPairsInFlight : 3;
-    const float kPadF = PROBS ? 0.f : -INFINITY;
+    constexpr int kPairs = AL ? kSmPairsInFlight : kSmPairsInFlight - 1;
     constexpr uint32_t kPad = PROBS ? 0u : R::kNegInf;       // what a lane beyond the end of a segment finds: no weight
     constexpr size_t ESZ = (DT == kF32) ? 4 : 2;
     __shared__ SmallShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int g = prm.gamma, B = prm.B, V = prm.V;
     const size_t row_bytes = static_cast<size_t>(prm.V) * ESZ;
-    const char* const tgt = static_cast<const char*>(prm.tgt);
-    const char* const drf = static_cast<const char*>(prm.drf);
-    const char* const tgt_end = tgt + static_cast<size_t>(B) * (g + 1) * row_bytes;
-    const char* const drf_end = drf + static_cast<size_t>(B) * g * row_bytes;
     const float kf = prm.kf;
     const int rpb = 2 * g + 1, nrows = B * rpb;
     const unsigned limit = prm.wait_limit ? prm.wait_limit : (1u << 22);
@@ -146,29 +154,46 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __
         const char* row = small_row(prm, row_bytes, rid / rpb, rid % rpb);
         const char* base16; int h, nv, u0, u1;
         row_grid<DT, AL>(row, V, base16, h, nv);
-        const char* const lo = rid % rpb <= g ? tgt : drf;
-        const char* const hi = rid % rpb <= g ? tgt_end : drf_end;
         small_seg_range(nv, nch, ch, u0, u1);
+        // (a row that is not whole vectors: its outer two are put together from elements, one each by two lanes of a warp that
+        // has a vector less to stream than others, and between them nothing tells one vector from another)
+        const int i0 = AL ? u0 : max(u0, 1), i1 = AL ? u1 : min(u1, nv - 1);
+        uint4 outer = make_uint4(R::kNegInf, R::kNegInf, R::kNegInf, R::kNegInf);
+        if (!AL && warp == kSmWarps - 1) {
+            if (lane == 0 && u0 == 0) outer = small_edge<DT>(row, 0, h, V, R::kNegInf);
+            if (lane == 1 && u1 == nv && nv > 1) outer = small_edge<DT>(row, nv - 1, h, V, R::kNegInf);
+        }
         float M = kNoRef, s = 0.f;
-        for (int base = u0; warp < kSmWarps && base < u1; base += kSmThreads * kSmInFlight) {
+        for (int base = i0; warp < kSmWarps && base < i1; base += kSmThreads * kSmInFlight) {
             uint4 raw[kSmInFlight];
 #pragma unroll
-            for (int j = 0; j < kSmInFlight; ++j) {
-                const int i = base + j * kSmThreads + tid;
-                raw[j] = small_load<DT, AL>(base16, i, u1, lo, hi, R::kNegInf);
+            for (int j = 0; j < kSmInFlight; ++j) raw[j] = small_load(base16, base + j * kSmThreads + tid, i0, i1, R::kNegInf);
+            // One reference for all of them, the rounded maximum of their logits: a test of every vector's sum before the next
+            // one's exponentials (f_accumulate) is a chain that sixteen warps do not hide (B = 1: 3.7 us until the last row is in,
+            // like this 3.2).
+            uint4 top = raw[0];
+#pragma unroll
+            for (int j = 1; j < kSmInFlight; ++j) top = vec_max<DT>(top, raw[j]);
+            {
+                float v[EPV];
+                R::unpack(top, v);
+                const float y = fmaxf(M, rintf(warp_max(vec_max<EPV>(v)) * kf));
+                s *= ref_scale(M, y);
+                M = y;
             }
 #pragma unroll
             for (int j = 0; j < kSmInFlight; ++j) {
-                if (base + j * kSmThreads + (warp << 5) < u1) {          // (warp-uniform)
+                if (base + j * kSmThreads + (warp << 5) < i1) {          // (warp-uniform)
                     float v[EPV];
                     R::unpack(raw[j], v);
-                    if (!AL) {
-                        const int i = base + j * kSmThreads + tid;
-                        if (i == 0 || i == nv - 1) row_mask<EPV>(v, i, h, V, kPadF);
-                    }
-                    f_accumulate<EPV>(v, kf, M, s);
+                    s += f_exp_sum<EPV>(v, kf, -M);
                 }
             }
+        }
+        if (!AL && warp == kSmWarps - 1) {
+            float v[EPV];
+            R::unpack(outer, v);
+            f_accumulate<EPV>(v, kf, M, s);
         }
         s = warp_sum(s);
         if (lane == 0 && warp < kSmWarps) { sh.wM[warp] = M; sh.wS[warp] = s; }
@@ -279,12 +304,22 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __
                     if (c < g) sh.csc[b * (g + 1) + c] = static_cast<float>(sh.rowZ[b * rpb + g + 1 + c] / sh.rowZ[b * rpb + c]);
                 }
             } else {
+                // (every lane walks the chain, the ratios read together beforehand from where they have just been left)
+                __syncwarp();
                 double pc = 1.0, mine[2] = {1.0, 1.0};
-                for (int c = 0; c < g; ++c) {
-                    if (c == lane) mine[0] = pc;
-                    if (c == lane + 32) mine[1] = pc;
-                    const double next = pc * shfl_d(c < 32 ? rat[0] : rat[1], c & 31);
-                    pc = prm.greedy ? next : fmin(next, 1.0);
+                for (int c0 = 0; c0 < g; c0 += 8) {
+                    double r[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) r[j] = c0 + j < g ? sh.ratio[b * (g + 1) + c0 + j] : 1.0;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const int c = c0 + j;
+                        if (c >= g) break;
+                        if (c == lane) mine[0] = pc;
+                        if (c == lane + 32) mine[1] = pc;
+                        const double next = pc * r[j];
+                        pc = prm.greedy ? next : fmin(next, 1.0);
+                    }
                 }
                 const double p_g = pc;
                 bool need[2] = {false, false};
@@ -313,169 +348,104 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __
         }
     }
     __syncthreads();
-    const int np = sc.np, nseg = np * kSmWarps;
-    if (tid == 0) {
-        int acc = 0;
-        for (int b = 0; b < B; ++b) {
-            sh.item0[b] = acc;
-            acc += (__popc(sh.mask_lo[b]) + __popc(sh.mask_hi[b]) + sh.last_wanted[b]) * np;
+    if (warp == 0) {
+        const int n = alive && lane < B ? __popc(sh.mask_lo[lane]) + __popc(sh.mask_hi[lane]) + sh.last_wanted[lane] : 0;
+        int acc = n;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, acc, off);
+            if (lane >= off) acc += o;
         }
-        sh.item0[B] = acc;
+        // Pieces a position: a CTA goes through its items one after the other, each its share of the row and what ends it (as
+        // long as streaming some 1200 vectors), so the count is the one with the least rounds x (vectors + 1200).
+        const int all = __shfl_sync(0xffffffffu, acc, 31), k = (lane & 7) + 1, units = V / EPV;
+        const unsigned rounds = static_cast<unsigned>((all * k + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x));
+        const unsigned cost = k == 1 || (k <= sc.np && units / k >= 512) ? min(rounds * static_cast<unsigned>(units / k + 1200), 0x0fffffffu) : 0x0fffffffu;
+        const unsigned least = __reduce_min_sync(0xffffffffu, cost);
+        const int np = ((__ffs(__ballot_sync(0xffffffffu, cost == least)) - 1) & 7) + 1;
+        if (lane < B) sh.item0[lane] = (acc - n) * np;
+        if (lane == B - 1) { sh.item0[B] = acc * np; sh.np = np; }
     }
     __syncthreads();
 
-    // ---------------- phase 2b: per-segment sums of the residual terms of every candidate position ----------------
-    if (alive) {
-        const int total = sh.item0[B];
-        for (int item = blockIdx.x; item < total; item += gridDim.x) {
-            int b = 0;
-            while (item >= sh.item0[b + 1]) ++b;
-            const int k = (item - sh.item0[b]) / np, piece = (item - sh.item0[b]) % np;
-            // the k-th candidate of the sequence, from position 0 up; position gamma last
-            const int n_lo = __popc(sh.mask_lo[b]), n_hi = __popc(sh.mask_hi[b]);
-            int i;
-            if (k < n_lo) i = __fns(sh.mask_lo[b], 0, k + 1);
-            else if (k < n_lo + n_hi) i = 32 + __fns(sh.mask_hi[b], 0, k - n_lo + 1);
-            else i = g;
-            const bool have_q = i < g;
-            const char* rowP = small_row(prm, row_bytes, b, i);
-            const char* rowQ = have_q ? small_row(prm, row_bytes, b, g + 1 + i) : nullptr;
-            const float cp = sh.csc[b * (g + 1) + i];
-            const float nMP = -sh.rowM[b * rpb + i], nMQ = have_q ? -sh.rowM[b * rpb + g + 1 + i] : 0.f;
-            int s0, s1, hP, nvP, hQ = 0, nvQ = 0;
-            const char* baseP;
-            const char* baseQ = nullptr;
-            row_grid<DT, AL>(rowP, V, baseP, hP, nvP);
-            if (have_q) row_grid<DT, AL>(rowQ, V, baseQ, hQ, nvQ);
-            int shift = hQ - hP, dq = 0;                      // the draft row's elements against the target row's grid
-            if (!AL && shift < 0) { shift += EPV; dq = -1; }
-            const int sq = shift * static_cast<int>(ESZ) >> 2, sbits = (shift * static_cast<int>(ESZ) & 3) * 8;
-            small_seg_range(nvP, nseg, piece * kSmWarps + (warp < kSmWarps ? warp : 0), s0, s1);
-            double acc = 0.0;
-            for (int base = s0; warp < kSmWarps && base < s1; base += 32 * kPairs) {
-                uint4 rp[kPairs], rq[kPairs], rx[AL ? 1 : kPairs];
-#pragma unroll
-                for (int j = 0; j < kPairs; ++j) {
-                    const int v = base + 32 * j + lane;
-                    rp[j] = small_load<DT, AL>(baseP, v, s1, tgt, tgt_end, kPad);
-                    const int lim = v < s1 ? (AL ? s1 : nvQ) : 0;
-                    rq[j] = small_load<DT, AL>(baseQ, v + dq, have_q ? lim : 0, drf, drf_end, kPad);
-                    if (!AL) rx[AL ? 0 : j] = small_load<DT, AL>(baseQ, v + dq + 1, have_q ? lim : 0, drf, drf_end, kPad);
-                }
-#pragma unroll
-                for (int j = 0; j < kPairs; ++j) {
-                    float vp[EPV], vq[EPV], t[EPV];
-                    R::unpack(rp[j], vp);
-                    R::unpack(AL ? rq[j] : small_shift(rq[j], rx[AL ? 0 : j], sq, sbits), vq);
-                    if (!AL) {
-                        const int v = base + 32 * j + lane;
-                        if (v == 0 || v >= nvP - 1) { row_mask<EPV>(vp, v, hP, V, kPadF); row_mask<EPV>(vq, v, hP, V, kPadF); }
-                    }
-                    if (have_q) acc += static_cast<double>(f_pair_sum<EPV, true, PROBS>(vp, vq, kf, cp, nMP, nMQ, t));
-                    else acc += static_cast<double>(f_pair_sum<EPV, false, PROBS>(vp, vq, kf, cp, nMP, nMQ, t));
-                }
-            }
-            acc = warp_sum_d(acc);
-            if (lane == 0 && warp < kSmWarps) sc.seg[(static_cast<size_t>(b) * (g + 1) + i) * nseg + piece * kSmWarps + warp] = acc;
-        }
-    }
-    // (arrivals are counted up through the launch: the second barrier of a launch on logits, the only one otherwise)
-    if (alive) alive = small_grid_barrier(sc.barrier, (PROBS ? 1u : 2u) * gridDim.x, prm.status, limit,
-                                          PROBS && prm.never_signal && blockIdx.x == 0);
+    const int np = sh.np, nseg = np * kSmWarps;
 
-    // No CTA looks at the barrier word any more once all have come by here, whatever became of the waits: the last one puts
-    // both words back to zero.  (A warp that is not on the way to the result does it: the fence, the atomic and its answer
-    // at the end of the kernel were 1 us of the 20 that a single sequence takes.)
-    if (tid == kSmThreads - 1) {
-        if (atomicAdd(sc.barrier + 16, 1u) == gridDim.x - 1) {
-            atomicExch(sc.barrier, 0u);
-            atomicExch(sc.barrier + 16, 0u);
-        }
-    }
-
-    // ---------------- phase 3: one CTA per sequence ----------------
-    for (int b = blockIdx.x; alive && b < B; b += gridDim.x) {
-        // S_i of every candidate (a warp per position at a time)
+    // ---------------- phase 3: the end of sequence b (all warps of a CTA) ----------------
+    auto finish = [&](int b) {
         const unsigned m_lo = sh.mask_lo[b], m_hi = sh.mask_hi[b];
-        for (int i = warp; i < g; i += kSmAllThreads / 32) {
-            const bool cand = (i < 32 ? m_lo >> i : m_hi >> (i - 32)) & 1u;
-            double tot = 0.0;
+        const float* u = sh.u + b * (g + 2);
+        for (int i = warp; i <= g; i += kSmAllThreads / 32) {
+            const bool have_q = i < g, cand = have_q ? ((i < 32 ? m_lo >> i : m_hi >> (i - 32)) & 1u) != 0u : sh.last_wanted[b] != 0;
+            double S = 0.0;
+            int y = -1;
+            bool pass = false;
             if (cand) {
-                const double* segs = sc.seg + (static_cast<size_t>(b) * (g + 1) + i) * nseg;
-                for (int s = lane; s < nseg; s += 32) tot += __ldcg(&segs[s]);
-                tot = warp_sum_d(tot) / sh.rowZ[b * rpb + g + 1 + i];
+                // S_i, and by fp64 sums of the segment totals in index order the segment that holds the sample
+                const double* segs = sc.seg + (static_cast<size_t>(b) * (g + 1) + i) * (sc.np * kSmWarps);
+                double w[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) w[j] = 4 * lane + j < nseg ? __ldcg(&segs[4 * lane + j]) : 0.0;
+                const double d1 = w[0], d2 = d1 + w[1], d3 = d2 + w[2], d4 = d3 + w[3];
+                double inc = d4;
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const double o = shfl_up_d(inc, off);
+                    if (lane >= off) inc += o;
+                }
+                const double total = shfl_d(inc, 31);
+                // h_gamma = p_gamma, h_i = S_i / (S_i + 1 - p_i); position 0 is what remains when no other passes
+                if (have_q) S = total / sh.rowZ[b * rpb + g + 1 + i];
+                if (tv || i == 0) {
+                    pass = true;
+                } else {
+                    const double p = sh.pch[b * (g + 1) + i], hw = have_q ? f_weight(p, S) : p;
+                    pass = hw > 0.0 && static_cast<double>(u[i - 1]) <= hw;
+                }
+                if (pass && total > 0.0 && total < static_cast<double>(INFINITY)) {
+                    const double t = static_cast<double>(u[have_q ? g : g + 1]) * total;
+                    double exc = shfl_up_d(inc, 1);
+                    if (lane == 0) exc = 0.0;
+                    const double p0 = exc, p1 = exc + d1, p2 = exc + d2, p3 = exc + d3, p4 = exc + d4;
+                    const bool h1 = p1 > t && w[0] > 0.0, h2 = p2 > t && w[1] > 0.0;
+                    const bool h3 = p3 > t && w[2] > 0.0, h4 = p4 > t && w[3] > 0.0;
+                    const unsigned hit = __ballot_sync(0xffffffffu, h1 || h2 || h3 || h4);
+                    const unsigned nz = __ballot_sync(0xffffffffu, d4 > 0.0);
+                    int e = 3, src;
+                    double bef = p3;
+                    if (hit) {
+                        src = __ffs(hit) - 1;
+                        if (h1) { e = 0; bef = p0; } else if (h2) { e = 1; bef = p1; } else if (h3) { e = 2; bef = p2; }
+                    } else {
+                        src = 31 - __clz(nz);
+                        e = 0; bef = p0;
+                        if (w[3] > 0.0) { e = 3; bef = p3; } else if (w[2] > 0.0) { e = 2; bef = p2; }
+                        else if (w[1] > 0.0) { e = 1; bef = p1; }
+                    }
+                    const int sel = __shfl_sync(0xffffffffu, 4 * lane + e, src);
+                    const double before = shfl_d(bef, src);
+                    const char* rowP = small_row(prm, row_bytes, b, i);
+                    const char* rowQ = have_q ? small_row(prm, row_bytes, b, g + 1 + i) : nullptr;
+                    const float cp = sh.csc[b * (g + 1) + i], nMP = -sh.rowM[b * rpb + i], nMQ = have_q ? -sh.rowM[b * rpb + g + 1 + i] : 0.f;
+                    const char* baseP; int h, nv, s0, s1;
+                    row_grid<DT, AL>(rowP, V, baseP, h, nv);
+                    small_seg_range(nv, nseg, sel, s0, s1);
+                    y = AL ? f_rescan<DT, PROBS, 5>(rowP, rowQ, s0, s1, lane, kf, cp, nMP, nMQ, t - before)
+                           : f_rescan_any<DT, PROBS, 2>(rowP, rowQ, V, s0, s1, lane, kf, cp, nMP, nMQ, t - before);
+                }
             }
-            if (lane == 0) sh.cS[i] = tot;
+            if (lane == 0) { if (have_q) sh.cS[i] = S; sh.found[i] = y; sh.pass[i] = pass; }
         }
         __syncthreads();
         if (warp == 0) {
-            const float* u = sh.u + b * (g + 2);
-            int tau;
-            if (tv) {
-                tau = sh.tv_tau[b];
-            } else {
-                // tau = max{i >= 1 : h_i > 0 and eta_i <= h_i}, else 0; h_gamma = p_gamma, h_i = S_i / (S_i + 1 - p_i)
-                bool pass[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int i = lane + 32 * h;
-                    const bool cand = i >= 1 && i < g && ((i < 32 ? m_lo >> i : m_hi >> (i - 32)) & 1u);
-                    const double hw = cand ? f_weight(sh.pch[b * (g + 1) + i], sh.cS[i]) : 0.0;
-                    pass[h] = cand && hw > 0.0 && static_cast<double>(u[i - 1]) <= hw;
-                }
-                const unsigned p_lo = __ballot_sync(0xffffffffu, pass[0]), p_hi = __ballot_sync(0xffffffffu, pass[1]);
-                const double p_g = sh.pch[b * (g + 1) + g];
-                tau = 0;
-                if (sh.last_wanted[b] && p_g > 0.0 && static_cast<double>(u[g - 1]) <= p_g) tau = g;
+            // tau = max{i >= 1 : h_i > 0 and eta_i <= h_i}, else 0
+            int tau = tv ? sh.tv_tau[b] : 0;
+            if (!tv) {
+                const unsigned p_lo = __ballot_sync(0xffffffffu, lane < g && sh.pass[lane < g ? lane : 0] != 0), p_hi = __ballot_sync(0xffffffffu, lane + 32 < g && sh.pass[lane + 32 < g ? lane + 32 : 0] != 0);
+                if (sh.pass[g]) tau = g;
                 else if (p_hi) tau = 32 + 31 - __clz(p_hi);
                 else if (p_lo) tau = 31 - __clz(p_lo);
             }
-            // Y by inverse CDF in index order over the segment sums of position tau, then within one segment
-            const bool have_q = tau < g;
-            const double* segs = sc.seg + (static_cast<size_t>(b) * (g + 1) + tau) * nseg;
-            double w[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) w[j] = 4 * lane + j < nseg ? __ldcg(&segs[4 * lane + j]) : 0.0;
-            const double d1 = w[0], d2 = d1 + w[1], d3 = d2 + w[2], d4 = d3 + w[3];
-            double inc = d4;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const double o = shfl_up_d(inc, off);
-                if (lane >= off) inc += o;
-            }
-            const double total = shfl_d(inc, 31);
-            int found = -1;
-            if (total > 0.0 && total < static_cast<double>(INFINITY)) {
-                const double t = static_cast<double>(u[have_q ? g : g + 1]) * total;
-                double exc = shfl_up_d(inc, 1);
-                if (lane == 0) exc = 0.0;
-                const double p0 = exc, p1 = exc + d1, p2 = exc + d2, p3 = exc + d3, p4 = exc + d4;
-                const bool h1 = p1 > t && w[0] > 0.0, h2 = p2 > t && w[1] > 0.0;
-                const bool h3 = p3 > t && w[2] > 0.0, h4 = p4 > t && w[3] > 0.0;
-                const unsigned hit = __ballot_sync(0xffffffffu, h1 || h2 || h3 || h4);
-                const unsigned nz = __ballot_sync(0xffffffffu, d4 > 0.0);
-                int e = 3, src;
-                double bef = p3;
-                if (hit) {
-                    src = __ffs(hit) - 1;
-                    if (h1) { e = 0; bef = p0; } else if (h2) { e = 1; bef = p1; } else if (h3) { e = 2; bef = p2; }
-                } else {
-                    src = 31 - __clz(nz);
-                    e = 0; bef = p0;
-                    if (w[3] > 0.0) { e = 3; bef = p3; } else if (w[2] > 0.0) { e = 2; bef = p2; }
-                    else if (w[1] > 0.0) { e = 1; bef = p1; }
-                }
-                const int sel = __shfl_sync(0xffffffffu, 4 * lane + e, src);
-                const double before = shfl_d(bef, src);
-                const char* rowP = small_row(prm, row_bytes, b, tau);
-                const char* rowQ = have_q ? small_row(prm, row_bytes, b, g + 1 + tau) : nullptr;
-                const float cp = sh.csc[b * (g + 1) + tau], nMP = -sh.rowM[b * rpb + tau], nMQ = have_q ? -sh.rowM[b * rpb + g + 1 + tau] : 0.f;
-                const char* baseP; int h, nv, s0, s1;
-                row_grid<DT, AL>(rowP, V, baseP, h, nv);
-                small_seg_range(nv, nseg, sel, s0, s1);
-                found = AL ? f_rescan<DT, PROBS, 5>(rowP, rowQ, s0, s1, lane, kf, cp, nMP, nMQ, t - before)
-                           : f_rescan_any<DT, PROBS, 2>(rowP, rowQ, V, s0, s1, lane, kf, cp, nMP, nMQ, t - before);
-            }
+            const int found = sh.found[tau];
             const bool bad = sh.bad[b] != 0 || found < 0;      // (an empty residual where the algorithm must sample: a domain error)
             int32_t* ot = prm.out_tokens + static_cast<size_t>(b) * (g + 1);
             const int32_t* X = prm.tok + static_cast<size_t>(b) * g;
@@ -506,7 +476,122 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __
             }
         }
         __syncthreads();
+    };
+
+    // ---------------- phase 2b: per-segment sums of the residual terms of every candidate position ----------------
+    unsigned ends = 0;                    // sequences whose last item was this CTA's
+    if (alive) {
+        const int total = sh.item0[B];
+        for (int item = blockIdx.x; item < total; item += gridDim.x) {
+            const int b = __popc(__ballot_sync(0xffffffffu, lane < B && item >= sh.item0[lane < B ? lane + 1 : 0]));
+            const int k = (item - sh.item0[b]) / np, piece = (item - sh.item0[b]) % np;
+            // the k-th candidate of the sequence, from position 0 up; position gamma last
+            const unsigned c_lo = sh.mask_lo[b], c_hi = sh.mask_hi[b], below = (1u << lane) - 1u;
+            const unsigned in_lo = __ballot_sync(0xffffffffu, (c_lo >> lane & 1u) && __popc(c_lo & below) == k);
+            const unsigned in_hi = __ballot_sync(0xffffffffu, (c_hi >> lane & 1u) && __popc(c_lo) + __popc(c_hi & below) == k);
+            const int i = in_lo ? __ffs(in_lo) - 1 : in_hi ? 31 + __ffs(in_hi) : g;
+            const bool have_q = i < g;
+            const char* rowP = small_row(prm, row_bytes, b, i);
+            const char* rowQ = have_q ? small_row(prm, row_bytes, b, g + 1 + i) : nullptr;
+            const float cp = sh.csc[b * (g + 1) + i];
+            const float nMP = -sh.rowM[b * rpb + i], nMQ = have_q ? -sh.rowM[b * rpb + g + 1 + i] : 0.f;
+            int s0, s1, hP, nvP, hQ = 0, nvQ = 0;
+            const char* baseP;
+            const char* baseQ = nullptr;
+            row_grid<DT, AL>(rowP, V, baseP, hP, nvP);
+            if (have_q) row_grid<DT, AL>(rowQ, V, baseQ, hQ, nvQ);
+            int shift = hQ - hP, dq = 0;                      // the draft row's elements against the target row's grid
+            if (!AL && shift < 0) { shift += EPV; dq = -1; }
+            const int sq = shift * static_cast<int>(ESZ) >> 2, sbits = (shift * static_cast<int>(ESZ) & 3) * 8;
+            small_seg_range(nvP, nseg, piece * kSmWarps + (warp < kSmWarps ? warp : 0), s0, s1);
+            // (AL: all of a segment's vectors; otherwise the target row's outer two are put together from elements, and so are
+            // the draft row's elements under them)
+            const int i0 = AL ? s0 : max(s0, 1), i1 = AL ? s1 : min(s1, nvP - 1);
+            double acc = 0.0;
+            uint4 edge_p = make_uint4(kPad, kPad, kPad, kPad), edge_q = edge_p;
+            const bool edges = !AL && warp < kSmWarps && (s0 == 0 || s1 == nvP) && s0 < s1;      // (warp-uniform)
+            if (edges) {
+                const int i = lane == 0 && s0 == 0 ? 0 : (lane == 1 && s1 == nvP && nvP > 1 ? nvP - 1 : -1);
+                if (i >= 0) {
+                    edge_p = small_edge<DT>(rowP, i, hP, V, kPad);
+                    if (have_q) edge_q = small_edge<DT>(rowQ, i, hP, V, kPad);
+                }
+            }
+            // a draft vector that holds a whole target vector's elements, or some of them, lies in the draft row's tensor: all but
+            // its outer two do, and the neighbour of one that is shifted is the next lane's
+            for (int base = i0; warp < kSmWarps && base < i1; base += 32 * kPairs) {
+                uint4 rp[kPairs], rq[kPairs], rx[AL ? 1 : kPairs];
+#pragma unroll
+                for (int j = 0; j < kPairs; ++j) {
+                    const int v = base + 32 * j + lane;
+                    rp[j] = small_load(baseP, v, i0, i1, kPad);
+                    if (AL) {
+                        rq[j] = small_load(baseQ, v, i0, have_q ? i1 : 0, kPad);
+                    } else {
+                        const int q1 = have_q && v < i1 ? nvQ : 0;
+                        rq[j] = small_any<DT>(baseQ, v + dq, q1, rowQ, hQ, V, kPad);
+                        // (the last lane has nobody to ask, and neither has the one before the end)
+                        rx[AL ? 0 : j] = lane == 31 || v + 1 >= i1 ? small_any<DT>(baseQ, v + dq + 1, q1, rowQ, hQ, V, kPad) : make_uint4(0u, 0u, 0u, 0u);
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < kPairs; ++j) {
+                    const int v = base + 32 * j + lane;
+                    float vp[EPV], vq[EPV], t[EPV];
+                    R::unpack(rp[j], vp);
+                    if (AL) {
+                        R::unpack(rq[j], vq);
+                    } else {
+                        const uint4 n = make_uint4(__shfl_down_sync(0xffffffffu, rq[j].x, 1), __shfl_down_sync(0xffffffffu, rq[j].y, 1),
+                                                   __shfl_down_sync(0xffffffffu, rq[j].z, 1), __shfl_down_sync(0xffffffffu, rq[j].w, 1));
+                        R::unpack(small_shift(rq[j], lane == 31 || v + 1 >= i1 ? rx[AL ? 0 : j] : n, sq, sbits), vq);
+                    }
+                    if (have_q) acc += static_cast<double>(f_pair_sum<EPV, true, PROBS>(vp, vq, kf, cp, nMP, nMQ, t));
+                    else acc += static_cast<double>(f_pair_sum<EPV, false, PROBS>(vp, vq, kf, cp, nMP, nMQ, t));
+                }
+            }
+            if (edges) {
+                float vp[EPV], vq[EPV], t[EPV];
+                R::unpack(edge_p, vp);
+                R::unpack(edge_q, vq);
+                if (have_q) acc += static_cast<double>(f_pair_sum<EPV, true, PROBS>(vp, vq, kf, cp, nMP, nMQ, t));
+                else acc += static_cast<double>(f_pair_sum<EPV, false, PROBS>(vp, vq, kf, cp, nMP, nMQ, t));
+            }
+            acc = warp_sum_d(acc);
+            if (lane == 0 && warp < kSmWarps) __stcg(&sc.seg[(static_cast<size_t>(b) * (g + 1) + i) * (sc.np * kSmWarps) + piece * kSmWarps + warp], acc);
+        }
+        // This CTA's items are in: said of all of them together, so that none waits for another's answer.
+        __syncthreads();
+        if (warp == 0) {
+            __threadfence();
+            for (int item = blockIdx.x + lane * static_cast<int>(gridDim.x); __any_sync(0xffffffffu, item < total); item += 32 * static_cast<int>(gridDim.x)) {
+                unsigned mine = 0;
+                if (item < total) {
+                    int b = 0;
+                    while (item >= sh.item0[b + 1]) ++b;
+                    if (atomicAdd(&sc.seq[b], 1u) + 1u == static_cast<unsigned>(sh.item0[b + 1] - sh.item0[b])) mine = 1u << b;
+                }
+                ends |= __reduce_or_sync(0xffffffffu, mine);
+            }
+            __threadfence();
+            if (lane == 0) sh.ends = ends;
+        }
+        __syncthreads();
+        ends = sh.ends;
     }
+
+    // No CTA looks at the barrier word or a sequence's counter any more once all have come by here, whatever became of the wait:
+    // the last one puts them back to zero.  (A warp that is not on the way to the result does it: the fence, the atomic and its
+    // answer at the end of the kernel were 1 us of the 20 that a single sequence takes.)
+    if (warp == kSmWarps - 1) {
+        unsigned gone = 0;
+        if (lane == 0) gone = atomicAdd(sc.barrier + 16, 1u);
+        if (__shfl_sync(0xffffffffu, gone, 0) == gridDim.x - 1) {
+            if (lane < B) atomicExch(&sc.seq[lane], 0u);
+            if (lane == 0) { atomicExch(sc.barrier, 0u); atomicExch(sc.barrier + 16, 0u); }
+        }
+    }
+    for (; ends != 0u; ends &= ends - 1u) finish(__ffs(ends) - 1);
 }
 
 // ---------------------------------------------------------------------------
@@ -519,7 +604,7 @@ bool small_fits(int B, int gamma) {
            static_cast<long long>(B) * (gamma + 1) <= kSmMaxPos;
 }
 
-// Chunks per row in the first phase and pieces per position in the second.  A CTA goes through its
+// Chunks per row in the first phase.  A CTA goes through its
 // items one after the other, each costing its share of the row plus a fixed part (the reduction
 // across the CTA and its barriers: about as long as streaming 2500 vectors), so the count is the
 // one that minimises rounds x (vectors per item + 2500); no chunk below 512 vectors.
@@ -537,8 +622,7 @@ static int small_best_split(long long units, long long rows, int nctas, int most
 SmallPlan small_plan(long long units, int B, int gamma, int nctas) {
     SmallPlan pl{};
     pl.nch = small_best_split(units, static_cast<long long>(B) * (2 * gamma + 1), nctas, kSmallMaxChunks);
-    // (about two candidate positions per sequence and the odd last target row: 5 rows for every 2 sequences)
-    pl.np = small_best_split(units, (5LL * B + 1) / 2, nctas, 8);
+    pl.np = 8;           // (the most: the kernel knows how many positions there are)
     return pl;
 }
 
@@ -547,11 +631,12 @@ size_t small_scratch_bytes(int B, int gamma, const SmallPlan& pl) {
     return up256s(rows * pl.nch * sizeof(double2)) + up256s(pos * pl.np * kSmWarps * sizeof(double));
 }
 
-// barrier: two words 64 bytes apart that are zero between launches (the kernel leaves them so)
-void small_scratch_layout(void* base, unsigned* barrier, int B, int gamma, const SmallPlan& pl, SmallScratch* sc) {
+// barrier: two words 64 bytes apart; seq: a word a sequence; all zero between launches (the kernel leaves them so)
+void small_scratch_layout(void* base, unsigned* barrier, unsigned* seq, int B, int gamma, const SmallPlan& pl, SmallScratch* sc) {
     char* p = static_cast<char*>(base);
     const size_t rows = static_cast<size_t>(B) * (2 * gamma + 1);
     sc->barrier = barrier;
+    sc->seq = seq;
     sc->part = reinterpret_cast<double2*>(p);
     sc->seg = reinterpret_cast<double*>(p + up256s(rows * pl.nch * sizeof(double2)));
     sc->nch = pl.nch;
