@@ -93,12 +93,23 @@ __device__ __forceinline__ void s_sweep_row(const char* row, int units, float kf
             const int i = base + 32 * j + lane;
             raw[j] = i < u1 ? ld_stream_v4(row + static_cast<size_t>(i) * 16) : ninf;
         }
+        // (One reference for all of them, the rounded maximum of their logits: a test of every vector's sum before the next one's
+        // exponentials was a chain of dependent steps.  256 rows of 128256 bf16 logits 22.5 -> 21.9 us, 300 of 65536 18.4 -> 16.4,
+        // 1000 of 32768 27.3 -> 24.6, 2048 of 256000 as before; a normaliser's error before it is rounded to 32 bits as before or
+        // 1 to 3 % less: no exponent is above 1/2.)
+        uint4 top = raw[0];
+#pragma unroll
+        for (int j = 1; j < kSInFlight; ++j) top = vec_max<DT>(top, raw[j]);
+        float v[EPV];
+        R::unpack(top, v);
+        const float y = fmaxf(M, rintf(warp_max(vec_max<EPV>(v)) * kf));
+        s *= ref_scale(M, y);
+        M = y;
 #pragma unroll
         for (int j = 0; j < kSInFlight; ++j) {
             if (base + 32 * j < u1) {
-                float v[EPV];
                 R::unpack(raw[j], v);
-                f_accumulate<EPV>(v, kf, M, s);
+                s += f_exp_sum<EPV>(v, kf, -M);
                 if (--left == 0) {                // the end of a sub-segment
                     s_put<SHORT>(M, s, lane, seg + s_place(warp, sub));
                     ++sub;
