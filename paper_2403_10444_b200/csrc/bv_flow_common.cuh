@@ -165,6 +165,32 @@ __device__ __forceinline__ uint4 row_elements(const char* row, int x0, int V, ui
     }
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
+// ---- rows at any alignment: a row is read as the aligned vectors that its bytes lie in ----
+// row start -> first 16-byte vector, elements of it that belong to the row before, vectors
+// (AL: rows of whole 16-byte vectors on 16-byte aligned bases)
+template <int DT, bool AL>
+__device__ __forceinline__ void row_grid(const char* row, int V, const char*& base, int& h, int& nv) {
+    constexpr int EPV = Raw<DT>::EPV;
+    constexpr int ESZ = (DT == kF32) ? 4 : 2;
+    if (AL) { base = row; h = 0; nv = V / EPV; return; }
+    const unsigned off = static_cast<unsigned>(reinterpret_cast<uintptr_t>(row) & 15u);
+    base = row - off; h = static_cast<int>(off) / ESZ; nv = (h + V + EPV - 1) / EPV;
+}
+// Vector i of the nv that a row of V elements lies in, h elements into the first: those between the first and the last as they
+// lie in memory, these two put together from the row's own elements (the others as `pad`: they are a neighbour's, or nobody's).
+template <int DT>
+__device__ __forceinline__ uint4 row_vector(const char* base, int i, int nv, const char* row, int h, int V, uint32_t pad) {
+    if (i < 0 || i >= nv) return make_uint4(pad, pad, pad, pad);
+    if (i > 0 && i < nv - 1) return ld_stream_v4(base + static_cast<long long>(i) * 16);
+    return row_elements<DT>(row, i * Raw<DT>::EPV - h, V, pad);
+}
+// 16 bytes from byte 4 q + bits / 8 on of two neighbouring vectors
+__device__ __forceinline__ uint4 vector_shift(const uint4& a, const uint4& b, int q, int bits) {
+    uint32_t w0 = a.x, w1 = a.y, w2 = a.z, w3 = a.w, w4 = b.x, w5 = b.y, w6 = b.z, w7 = b.w;
+    if (q & 2) { w0 = w2; w1 = w3; w2 = w4; w3 = w5; w4 = w6; w5 = w7; }
+    if (q & 1) { w0 = w1; w1 = w2; w2 = w3; w3 = w4; w4 = w5; }
+    return make_uint4(__funnelshift_r(w0, w1, bits), __funnelshift_r(w1, w2, bits), __funnelshift_r(w2, w3, bits), __funnelshift_r(w3, w4, bits));
+}
 // One warp walks segment [w0, w1) of a row pair in index order and returns the first element
 // whose running residual mass exceeds tw (else the last element with positive mass, else -1).
 // (AL: rows of whole 16-byte vectors.  Otherwise the rows hold V elements, vector 0 begins h elements before them, and the
@@ -172,7 +198,7 @@ __device__ __forceinline__ uint4 row_elements(const char* row, int x0, int V, ui
 // function object the flow kernel spilled 4 bytes more and 256 sequences of V = 256000 took 0.6 % longer.)
 template <int DT, bool PROBS = false, int kAhead = 4, bool AL = true>      // kAhead: runs of 32 vectors whose loads are in flight together
 __device__ int f_rescan(const char* rowP, const char* rowQ, int w0, int w1, int lane, float kf, float cp,
-                        float nMP, float nMQ, double tw, int V = 0, int h = 0) {
+                        float nMP, float nMQ, double tw, int V = 0) {
     constexpr int EPV = Raw<DT>::EPV;
     constexpr uint32_t kPad = PROBS ? 0u : Raw<DT>::kNegInf;   // an element beyond the segment weighs nothing
     // The terms are the fp32 values of the sweeps; their running sum, which decides the token, is
@@ -180,6 +206,15 @@ __device__ int f_rescan(const char* rowP, const char* rowQ, int w0, int w1, int 
     // mass before it).
     double run = 0.0;
     int found = -1, last_pos = -1;
+    const char *gridP = nullptr, *gridQ = nullptr;
+    int hP = 0, nvP = 0, hQ = 0, nvQ = 0, shift = 0, dq = 0;
+    if (!AL) {
+        row_grid<DT, false>(rowP, V, gridP, hP, nvP);
+        if (rowQ) row_grid<DT, false>(rowQ, V, gridQ, hQ, nvQ);
+        shift = rowQ ? hQ - hP : 0;           // the draft row's elements against the target row's grid
+        if (shift < 0) { shift += EPV; dq = -1; }
+    }
+    const int sq = shift * (16 / EPV) >> 2, sbits = (shift * (16 / EPV) & 3) * 8;
     for (int base0 = w0; base0 < w1 && found < 0; base0 += 32 * kAhead) {
         // the loads of kAhead runs are issued before the first is looked at: the walk is a chain of
         // dependent steps, and a load's latency is what each step would otherwise wait for
@@ -192,8 +227,15 @@ __device__ int f_rescan(const char* rowP, const char* rowQ, int w0, int w1, int 
                 rp[a] = ok ? ld_stream_v4(rowP + static_cast<size_t>(i) * 16) : make_uint4(kPad, kPad, kPad, kPad);
                 rq[a] = (ok && rowQ) ? ld_stream_v4(rowQ + static_cast<size_t>(i) * 16) : make_uint4(kPad, kPad, kPad, kPad);
             } else {
-                rp[a] = ok ? row_elements<DT>(rowP, i * EPV - h, V, kPad) : make_uint4(kPad, kPad, kPad, kPad);
-                rq[a] = (ok && rowQ) ? row_elements<DT>(rowQ, i * EPV - h, V, kPad) : make_uint4(kPad, kPad, kPad, kPad);
+                // (a vector's elements one by one, eight loads a lane and row, until this: 24 sequences of gamma = 5, V = 50257 1.5 % longer.)
+                // (a draft vector's elements under a target vector's lie in two of its own; where the target row has no element,
+                // in its outer vectors, its term is zero whatever the draft row's holds)
+                rp[a] = row_vector<DT>(gridP, ok ? i : -1, nvP, rowP, hP, V, kPad);
+                rq[a] = make_uint4(kPad, kPad, kPad, kPad);
+                if (rowQ) {
+                    const uint4 q0 = row_vector<DT>(gridQ, ok ? i + dq : -1, nvQ, rowQ, hQ, V, kPad), q1 = row_vector<DT>(gridQ, ok && shift ? i + dq + 1 : -1, nvQ, rowQ, hQ, V, kPad);
+                    rq[a] = vector_shift(q0, q1, sq, sbits);
+                }
             }
         }
 #pragma unroll
@@ -248,16 +290,6 @@ __device__ int f_rescan(const char* rowP, const char* rowQ, int w0, int w1, int 
 
 // ---- rows at any alignment: a row is read as the aligned vectors that its bytes lie in; what of the first and the last
 // of them belongs to its neighbours weighs nothing ----
-// row start -> first 16-byte vector, elements of it that belong to the row before, vectors
-// (AL: rows of whole 16-byte vectors on 16-byte aligned bases)
-template <int DT, bool AL>
-__device__ __forceinline__ void row_grid(const char* row, int V, const char*& base, int& h, int& nv) {
-    constexpr int EPV = Raw<DT>::EPV;
-    constexpr int ESZ = (DT == kF32) ? 4 : 2;
-    if (AL) { base = row; h = 0; nv = V / EPV; return; }
-    const unsigned off = static_cast<unsigned>(reinterpret_cast<uintptr_t>(row) & 15u);
-    base = row - off; h = static_cast<int>(off) / ESZ; nv = (h + V + EPV - 1) / EPV;
-}
 // elements of vector i (on the row's 16-byte grid, h elements into the vector before) outside [0, V) weigh nothing
 template <int EPV> __device__ __forceinline__ void row_mask(float (&v)[EPV], int i, int h, int V, float pad) {
 #pragma unroll
@@ -272,7 +304,7 @@ __device__ int f_rescan_any(const char* rowP, const char* rowQ, int V, int w0, i
                             float nMP, float nMQ, double tw) {
     const char* base; int h, nv;
     row_grid<DT, false>(rowP, V, base, h, nv);
-    const int found = f_rescan<DT, PROBS, kAhead, false>(rowP, rowQ, w0, w1 < nv ? w1 : nv, lane, kf, cp, nMP, nMQ, tw, V, h);
+    const int found = f_rescan<DT, PROBS, kAhead, false>(rowP, rowQ, w0, w1 < nv ? w1 : nv, lane, kf, cp, nMP, nMQ, tw, V);
     return found >= 0 ? found - h : found;
 }
 

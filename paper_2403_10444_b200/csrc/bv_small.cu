@@ -98,20 +98,6 @@ template <int DT>
 __device__ __forceinline__ uint4 small_edge(const char* row, int i, int h, int V, uint32_t pad) {
     return row_elements<DT>(row, i * Raw<DT>::EPV - h, V, pad);
 }
-// ... any of the nv, those between them as they lie in memory
-template <int DT>
-__device__ __forceinline__ uint4 small_any(const char* base, int i, int nv, const char* row, int h, int V, uint32_t pad) {
-    if (i < 0 || i >= nv) return make_uint4(pad, pad, pad, pad);
-    return i > 0 && i < nv - 1 ? ld_stream_v4(base + static_cast<long long>(i) * 16) : small_edge<DT>(row, i, h, V, pad);
-}
-// 16 bytes from byte 4 q + bits / 8 on of two neighbouring vectors
-__device__ __forceinline__ uint4 small_shift(const uint4& a, const uint4& b, int q, int bits) {
-    uint32_t w0 = a.x, w1 = a.y, w2 = a.z, w3 = a.w, w4 = b.x, w5 = b.y, w6 = b.z, w7 = b.w;
-    if (q & 2) { w0 = w2; w1 = w3; w2 = w4; w3 = w5; w4 = w6; w5 = w7; }
-    if (q & 1) { w0 = w1; w1 = w2; w2 = w3; w3 = w4; w4 = w5; }
-    return make_uint4(__funnelshift_r(w0, w1, bits), __funnelshift_r(w1, w2, bits), __funnelshift_r(w2, w3, bits), __funnelshift_r(w3, w4, bits));
-}
-
 // PROBS: the rows hold probabilities, used as stored: there is no first phase (and no first barrier).
 // AL: rows of whole 16-byte vectors on 16-byte aligned bases.  Otherwise a row is read as the vectors its bytes lie in
 // (row_grid), and the draft row of a pair is put on the target row's grid from two neighbouring vectors.
@@ -430,7 +416,7 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __
                     row_grid<DT, AL>(rowP, V, baseP, h, nv);
                     small_seg_range(nv, nseg, sel, s0, s1);
                     y = AL ? f_rescan<DT, PROBS, 5>(rowP, rowQ, s0, s1, lane, kf, cp, nMP, nMQ, t - before)
-                           : f_rescan_any<DT, PROBS, 2>(rowP, rowQ, V, s0, s1, lane, kf, cp, nMP, nMQ, t - before);
+                           : f_rescan_any<DT, PROBS, 3>(rowP, rowQ, V, s0, s1, lane, kf, cp, nMP, nMQ, t - before);
                 }
             }
             if (lane == 0) { if (have_q) sh.cS[i] = S; sh.found[i] = y; sh.pass[i] = pass; }
@@ -529,9 +515,9 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __
                         rq[j] = small_load(baseQ, v, i0, have_q ? i1 : 0, kPad);
                     } else {
                         const int q1 = have_q && v < i1 ? nvQ : 0;
-                        rq[j] = small_any<DT>(baseQ, v + dq, q1, rowQ, hQ, V, kPad);
+                        rq[j] = row_vector<DT>(baseQ, v + dq, q1, rowQ, hQ, V, kPad);
                         // (the last lane has nobody to ask, and neither has the one before the end)
-                        rx[AL ? 0 : j] = lane == 31 || v + 1 >= i1 ? small_any<DT>(baseQ, v + dq + 1, q1, rowQ, hQ, V, kPad) : make_uint4(0u, 0u, 0u, 0u);
+                        rx[AL ? 0 : j] = lane == 31 || v + 1 >= i1 ? row_vector<DT>(baseQ, v + dq + 1, q1, rowQ, hQ, V, kPad) : make_uint4(0u, 0u, 0u, 0u);
                     }
                 }
 #pragma unroll
@@ -544,7 +530,7 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __
                     } else {
                         const uint4 n = make_uint4(__shfl_down_sync(0xffffffffu, rq[j].x, 1), __shfl_down_sync(0xffffffffu, rq[j].y, 1),
                                                    __shfl_down_sync(0xffffffffu, rq[j].z, 1), __shfl_down_sync(0xffffffffu, rq[j].w, 1));
-                        R::unpack(small_shift(rq[j], lane == 31 || v + 1 >= i1 ? rx[AL ? 0 : j] : n, sq, sbits), vq);
+                        R::unpack(vector_shift(rq[j], lane == 31 || v + 1 >= i1 ? rx[AL ? 0 : j] : n, sq, sbits), vq);
                     }
                     if (have_q) acc += static_cast<double>(f_pair_sum<EPV, true, PROBS>(vp, vq, kf, cp, nMP, nMQ, t));
                     else acc += static_cast<double>(f_pair_sum<EPV, false, PROBS>(vp, vq, kf, cp, nMP, nMQ, t));
