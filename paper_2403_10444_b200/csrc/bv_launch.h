@@ -133,8 +133,9 @@ struct SmallScratch {
     double2* part;        // [B (2 gamma + 1)][nch] {reference, sum} of every chunk
     double* seg;          // [B (gamma + 1)][np * 16] per-segment sums of the residual terms
     int nch, np;          // chunks of a row, the most pieces of a position
+    int ahead;            // the first phase's loads run ahead of its arithmetic through shared memory
 };
-struct SmallPlan { int nch, np; };
+struct SmallPlan { int nch, np, ahead; };
 bool small_fits(int B, int gamma);
 SmallPlan small_plan(long long units, int B, int gamma, int nctas);
 size_t small_scratch_bytes(int B, int gamma, const SmallPlan& pl);

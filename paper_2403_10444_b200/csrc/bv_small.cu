@@ -16,7 +16,7 @@
 //      position passes, its token by inverse CDF over the segment sums and a rescan of one segment; then tau and the output.
 //      (A second barrier, the sums of all candidates, and only then the chosen one's token were two trips to L2 more.)
 // Bound: latency, a trip to L2 or memory for each of some eight dependent steps.  B = 1, gamma = 8, V = 152064 bf16 19.1 us a call
-// (19.8 with two barriers and pieces fixed on the host), B = 8, V = 32000 in 32 bits 19.8 (22.6), B = 24, gamma = 5, V = 50257 45 (45).
+// (19.8 with two barriers and pieces fixed on the host), B = 8, V = 32000 in 32 bits 19.8 (22.6), B = 24, gamma = 5, V = 50257 42 (45).
 // Arithmetic, sampling convention and outputs are those of the flow kernel.
 #include <cooperative_groups.h>
 
@@ -29,6 +29,9 @@ constexpr int kSmWarps = kSmThreads / 32;
 constexpr int kSmAllThreads = kSmThreads + 32;
 constexpr int kSmMaxRows = 1056;      // rows B (2 gamma + 1) whose normalisers a CTA keeps in shared memory
 constexpr int kSmMaxPos = 560;        // positions B (gamma + 1)
+constexpr int kSmGroup = 4;           // vectors of a thread that the first phase goes through together where its loads run ahead
+constexpr int kSmAhead = 3;           // ... groups of them in flight
+constexpr int kSmRingBytes = kSmAhead * kSmGroup * kSmThreads * 16;
 constexpr int kSmInFlight = 8;        // 16-byte loads a thread has in flight in the first phase
 constexpr int kSmPairsInFlight = 5;   // pairs of them in the second (unaligned rows: one less, the registers)
 constexpr int kSmMaxUni = kSmMaxPos + kSmallMaxB;   // uniforms B (gamma + 2)
@@ -44,8 +47,8 @@ struct SmallShared {
     int bad[kSmallMaxB];
     int tv_tau[kSmallMaxB];
     int item0[kSmallMaxB + 1];        // first item of every sequence in the second phase
-    float wM[kSmWarps];
-    float wS[kSmWarps];
+    float wM[2][kSmWarps];
+    float wS[2][kSmWarps];
     double cS[kMaxGamma];             // third phase: S_i of this CTA's sequence, the positions' tokens, which of them pass
     int found[kMaxGamma + 1];
     unsigned char pass[kMaxGamma + 1];
@@ -134,65 +137,166 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __
         }
         for (int i = lane; i < B * (g + 2); i += 32) sh.u[i] = prm.uni[i];
     }
-    for (int item = blockIdx.x; !PROBS && item < nrows * nch; item += gridDim.x) {
-        const int rid = item / nch, ch = item % nch;
-        if (prm.lse_d != nullptr && rid % rpb > g) continue;      // (a draft row whose normaliser is supplied: nothing to learn)
-        const char* row = small_row(prm, row_bytes, rid / rpb, rid % rpb);
-        const char* base16; int h, nv, u0, u1;
-        row_grid<DT, AL>(row, V, base16, h, nv);
-        small_seg_range(nv, nch, ch, u0, u1);
-        // (a row that is not whole vectors: its outer two are put together from elements, one each by two lanes of a warp that
-        // has a vector less to stream than others, and between them nothing tells one vector from another)
-        const int i0 = AL ? u0 : max(u0, 1), i1 = AL ? u1 : min(u1, nv - 1);
-        uint4 outer = make_uint4(R::kNegInf, R::kNegInf, R::kNegInf, R::kNegInf);
-        if (!AL && warp == kSmWarps - 1) {
-            if (lane == 0 && u0 == 0) outer = small_edge<DT>(row, 0, h, V, R::kNegInf);
-            if (lane == 1 && u1 == nv && nv > 1) outer = small_edge<DT>(row, nv - 1, h, V, R::kNegInf);
+    const int items = PROBS ? 0 : nrows * nch;
+    // With loads ahead (small_plan) every thread's vectors go through a ring of its own in shared memory, kSmAhead groups ahead of the
+    // arithmetic and on into the next item: a CTA has as many warps as one item can use, and with the loads of eight vectors waited for
+    // together and then their exponentials, neither memory nor the exponential pipe is busy for more than half of the time.
+    if (sc.ahead) {
+        extern __shared__ __align__(16) unsigned char cells[];
+        const uint32_t ring = smem_u32(cells) + static_cast<uint32_t>(tid) * 16u;
+        struct Part { const char* base; int h, nv, u0, u1, i0, i1; } pt;      // chunk of a row: its vectors, and those between the row's outer two
+        auto part_of = [&](int item) {
+            const int rid = item / nch;
+            row_grid<DT, AL>(small_row(prm, row_bytes, rid / rpb, rid % rpb), V, pt.base, pt.h, pt.nv);
+            small_seg_range(pt.nv, nch, item % nch, pt.u0, pt.u1);
+            pt.i0 = AL ? pt.u0 : max(pt.u0, 1);
+            pt.i1 = AL ? pt.u1 : min(pt.u1, pt.nv - 1);
+        };
+        auto wanted = [&](int item) { return prm.lse_d == nullptr || item / nch % rpb <= g; };      // (a draft row whose normaliser is supplied: nothing to learn)
+        int item_i = static_cast<int>(blockIdx.x), i_at = 0, i_end = 0;       // issue side: item, the next of its vectors, their end
+        const char* i_base = nullptr;
+        auto open = [&]() {
+            for (; item_i < items; item_i += gridDim.x) {
+                if (!wanted(item_i)) continue;
+                part_of(item_i);
+                i_base = pt.base; i_at = pt.i0 + tid; i_end = pt.i1;
+                if (pt.i0 < pt.i1) break;
+            }
+        };
+        auto issue = [&](uint32_t cell) {
+            if (item_i < items) {
+#pragma unroll
+                for (int j = 0; j < kSmGroup; ++j)
+                    ring_fetch_s(cell + j * kSmThreads * 16, i_base + static_cast<long long>(i_at + j * kSmThreads) * 16, i_at + j * kSmThreads < i_end, R::kNegInf);
+                i_at += kSmGroup * kSmThreads;
+                if (i_at - tid >= i_end) { item_i += gridDim.x; open(); }
+            }
+            cp_async_commit();
+        };
+        if (warp < kSmWarps) {
+            open();
+#pragma unroll 1
+            for (int a = 0; a < kSmAhead; ++a) issue(ring + a * kSmGroup * kSmThreads * 16);
         }
-        float M = kNoRef, s = 0.f;
-        for (int base = i0; warp < kSmWarps && base < i1; base += kSmThreads * kSmInFlight) {
-            uint4 raw[kSmInFlight];
+        uint32_t rp = ring;
+        int turn = 0;
+        for (int item = blockIdx.x; item < items; item += gridDim.x) {
+            if (!wanted(item)) continue;
+            const int rid = item / nch;
+            part_of(item);
+            // (a row that is not whole vectors: its outer two are put together from elements, one each by two lanes of a warp)
+            uint4 outer = make_uint4(R::kNegInf, R::kNegInf, R::kNegInf, R::kNegInf);
+            if (!AL && warp == kSmWarps - 1) {
+                const char* row = small_row(prm, row_bytes, rid / rpb, rid % rpb);
+                if (lane == 0 && pt.u0 == 0) outer = small_edge<DT>(row, 0, pt.h, V, R::kNegInf);
+                if (lane == 1 && pt.u1 == pt.nv && pt.nv > 1) outer = small_edge<DT>(row, pt.nv - 1, pt.h, V, R::kNegInf);
+            }
+            const int i1 = pt.i1;
+            float M = kNoRef, s = 0.f;
+            for (int base = pt.i0; warp < kSmWarps && base < i1; base += kSmThreads * kSmGroup) {
+                cp_async_wait<kSmAhead - 1>();
+                uint4 raw[kSmGroup];
 #pragma unroll
-            for (int j = 0; j < kSmInFlight; ++j) raw[j] = small_load(base16, base + j * kSmThreads + tid, i0, i1, R::kNegInf);
-            // One reference for all of them, the rounded maximum of their logits: a test of every vector's sum before the next
-            // one's exponentials (f_accumulate) is a chain that sixteen warps do not hide (B = 1: 3.7 us until the last row is in,
-            // like this 3.2).
-            uint4 top = raw[0];
+                for (int j = 0; j < kSmGroup; ++j) raw[j] = lds128(rp + j * kSmThreads * 16);
+                // one reference for all of them, the rounded maximum of their logits (a test of every vector's sum before the next
+                // one's exponentials is a chain that a few warps do not hide)
+                uint4 top = raw[0];
 #pragma unroll
-            for (int j = 1; j < kSmInFlight; ++j) top = vec_max<DT>(top, raw[j]);
-            {
+                for (int j = 1; j < kSmGroup; ++j) top = vec_max<DT>(top, raw[j]);
                 float v[EPV];
                 R::unpack(top, v);
                 const float y = fmaxf(M, rintf(warp_max(vec_max<EPV>(v)) * kf));
                 s *= ref_scale(M, y);
                 M = y;
-            }
 #pragma unroll
-            for (int j = 0; j < kSmInFlight; ++j) {
-                if (base + j * kSmThreads + (warp << 5) < i1) {          // (warp-uniform)
+                for (int j = 0; j < kSmGroup; ++j) {
+                    if (base + j * kSmThreads + (warp << 5) < i1) {          // (warp-uniform)
+                        R::unpack(raw[j], v);
+                        s += f_exp_sum<EPV>(v, kf, -M);
+                    }
+                }
+                issue(rp);
+                rp += kSmGroup * kSmThreads * 16;
+                if (rp == ring + kSmAhead * kSmGroup * kSmThreads * 16) rp = ring;
+            }
+            if (!AL && warp == kSmWarps - 1) {
+                float v[EPV];
+                R::unpack(outer, v);
+                f_accumulate<EPV>(v, kf, M, s);
+            }
+            s = warp_sum(s);
+            if (lane == 0 && warp < kSmWarps) { sh.wM[turn][warp] = M; sh.wS[turn][warp] = s; }
+            __syncthreads();
+            if (warp == 0) {                  // (the next item's shares go to the other half, and the barrier after it is behind this)
+                const float m = lane < kSmWarps ? sh.wM[turn][lane] : kNoRef;
+                const float Mc = warp_max(m);
+                double z = lane < kSmWarps ? static_cast<double>(sh.wS[turn][lane]) * static_cast<double>(ref_scale(m, Mc)) : 0.0;
+                z = warp_sum_d(z);
+                if (lane == 0) __stcg(&sc.part[static_cast<size_t>(rid) * nch + item % nch], make_double2(static_cast<double>(Mc), z));
+            }
+            turn ^= 1;
+        }
+} else {
+        for (int item = blockIdx.x; item < items; item += gridDim.x) {
+            const int rid = item / nch, ch = item % nch;
+            if (prm.lse_d != nullptr && rid % rpb > g) continue;      // (a draft row whose normaliser is supplied: nothing to learn)
+            const char* row = small_row(prm, row_bytes, rid / rpb, rid % rpb);
+            const char* base16; int h, nv, u0, u1;
+            row_grid<DT, AL>(row, V, base16, h, nv);
+            small_seg_range(nv, nch, ch, u0, u1);
+            // (a row that is not whole vectors: its outer two are put together from elements, one each by two lanes of a warp that
+            // has a vector less to stream than others, and between them nothing tells one vector from another)
+            const int i0 = AL ? u0 : max(u0, 1), i1 = AL ? u1 : min(u1, nv - 1);
+            uint4 outer = make_uint4(R::kNegInf, R::kNegInf, R::kNegInf, R::kNegInf);
+            if (!AL && warp == kSmWarps - 1) {
+                if (lane == 0 && u0 == 0) outer = small_edge<DT>(row, 0, h, V, R::kNegInf);
+                if (lane == 1 && u1 == nv && nv > 1) outer = small_edge<DT>(row, nv - 1, h, V, R::kNegInf);
+            }
+            float M = kNoRef, s = 0.f;
+            for (int base = i0; warp < kSmWarps && base < i1; base += kSmThreads * kSmInFlight) {
+                uint4 raw[kSmInFlight];
+#pragma unroll
+                for (int j = 0; j < kSmInFlight; ++j) raw[j] = small_load(base16, base + j * kSmThreads + tid, i0, i1, R::kNegInf);
+                // One reference for all of them, the rounded maximum of their logits: a test of every vector's sum before the next
+                // one's exponentials (f_accumulate) is a chain that sixteen warps do not hide (B = 1: 3.7 us until the last row is in,
+                // like this 3.2).
+                uint4 top = raw[0];
+#pragma unroll
+                for (int j = 1; j < kSmInFlight; ++j) top = vec_max<DT>(top, raw[j]);
+                {
                     float v[EPV];
-                    R::unpack(raw[j], v);
-                    s += f_exp_sum<EPV>(v, kf, -M);
+                    R::unpack(top, v);
+                    const float y = fmaxf(M, rintf(warp_max(vec_max<EPV>(v)) * kf));
+                    s *= ref_scale(M, y);
+                    M = y;
+                }
+#pragma unroll
+                for (int j = 0; j < kSmInFlight; ++j) {
+                    if (base + j * kSmThreads + (warp << 5) < i1) {          // (warp-uniform)
+                        float v[EPV];
+                        R::unpack(raw[j], v);
+                        s += f_exp_sum<EPV>(v, kf, -M);
+                    }
                 }
             }
+            if (!AL && warp == kSmWarps - 1) {
+                float v[EPV];
+                R::unpack(outer, v);
+                f_accumulate<EPV>(v, kf, M, s);
+            }
+            s = warp_sum(s);
+            if (lane == 0 && warp < kSmWarps) { sh.wM[0][warp] = M; sh.wS[0][warp] = s; }
+            __syncthreads();
+            if (warp == 0) {
+                const float m = lane < kSmWarps ? sh.wM[0][lane] : kNoRef;
+                const float Mc = warp_max(m);
+                double z = lane < kSmWarps ? static_cast<double>(sh.wS[0][lane]) * static_cast<double>(ref_scale(m, Mc)) : 0.0;
+                z = warp_sum_d(z);
+                if (lane == 0) sc.part[static_cast<size_t>(rid) * nch + ch] = make_double2(static_cast<double>(Mc), z);
+            }
+            __syncthreads();
         }
-        if (!AL && warp == kSmWarps - 1) {
-            float v[EPV];
-            R::unpack(outer, v);
-            f_accumulate<EPV>(v, kf, M, s);
-        }
-        s = warp_sum(s);
-        if (lane == 0 && warp < kSmWarps) { sh.wM[warp] = M; sh.wS[warp] = s; }
-        __syncthreads();
-        if (warp == 0) {
-            const float m = lane < kSmWarps ? sh.wM[lane] : kNoRef;
-            const float Mc = warp_max(m);
-            double z = lane < kSmWarps ? static_cast<double>(sh.wS[lane]) * static_cast<double>(ref_scale(m, Mc)) : 0.0;
-            z = warp_sum_d(z);
-            if (lane == 0) sc.part[static_cast<size_t>(rid) * nch + ch] = make_double2(static_cast<double>(Mc), z);
-        }
-        __syncthreads();
-    }
+}
     if (PROBS) __syncthreads();
     else alive = small_grid_barrier(sc.barrier, gridDim.x, prm.status, limit, prm.never_signal && blockIdx.x == 0);
 
@@ -608,6 +712,10 @@ static int small_best_split(long long units, long long rows, int nctas, int most
 SmallPlan small_plan(long long units, int B, int gamma, int nctas) {
     SmallPlan pl{};
     pl.nch = small_best_split(units, static_cast<long long>(B) * (2 * gamma + 1), nctas, kSmallMaxChunks);
+    // Loads ahead of the arithmetic: where a CTA has more than one item, or one of more than 16 vectors a thread (B = 24, gamma = 5, V = 50257 46.5 us
+    // without, 42.3 with; B = 20, gamma = 6, V = 65536, Algorithm 1, 30.7 / 28.6).  A single item of fewer waits for memory once or twice either way, and the
+    // ring only costs: B = 1, gamma = 8, V = 152064 19.1 / 20.5, B = 3, gamma = 3, V = 256000 24.7 / 25.2, B = 8, V = 32000 in 32 bits 19.2 / 19.5.
+    pl.ahead = static_cast<long long>(B) * (2 * gamma + 1) * pl.nch > nctas || units / pl.nch > 16 * kSmThreads;
     pl.np = 8;           // (the most: the kernel knows how many positions there are)
     return pl;
 }
@@ -626,6 +734,7 @@ void small_scratch_layout(void* base, unsigned* barrier, unsigned* seq, int B, i
     sc->part = reinterpret_cast<double2*>(p);
     sc->seg = reinterpret_cast<double*>(p + up256s(rows * pl.nch * sizeof(double2)));
     sc->nch = pl.nch;
+    sc->ahead = pl.ahead;
     sc->np = pl.np;
 }
 
@@ -639,7 +748,8 @@ static SKernelFn pick_small(int dtype, bool probs, bool aligned) {
 int small_max_ctas(int dtype, int sm_count) {
     for (int v = 0; v < 3; ++v) {
         int n = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pick_small(dtype, v == 2, v != 1), kSmAllThreads, 0) != cudaSuccess || n < 1) {
+        if (cudaFuncSetAttribute(reinterpret_cast<const void*>(pick_small(dtype, v == 2, v != 1)), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmRingBytes) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pick_small(dtype, v == 2, v != 1), kSmAllThreads, kSmRingBytes) != cudaSuccess || n < 1) {
             cudaGetLastError();
             return 0;
         }
@@ -650,8 +760,10 @@ int small_max_ctas(int dtype, int sm_count) {
 cudaError_t launch_small(const Params& prm, const SmallScratch& sc, int dtype, bool aligned, int nctas, cudaStream_t stream) {
     Params p = prm;
     SmallScratch s = sc;
+    if (prm.probs) s.ahead = 0;
     void* args[] = {&p, &s};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(pick_small(dtype, prm.probs != 0, aligned)), dim3(nctas), dim3(kSmAllThreads), args, 0, stream);
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(pick_small(dtype, prm.probs != 0, aligned)), dim3(nctas), dim3(kSmAllThreads), args,
+                                       s.ahead ? kSmRingBytes : 0, stream);
 }
 
 }  // namespace bv
