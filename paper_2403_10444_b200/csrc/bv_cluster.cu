@@ -60,7 +60,7 @@ template <int EPV> __device__ __forceinline__ void accumulate(const float (&v)[E
     float vs = exp_sum<EPV>(v, kf, -M);
     if (__any_sync(0xffffffffu, vs > kRaiseBound)) {      // some logit lies above the reference
         const float y = rintf(warp_max(vec_max<EPV>(v)) * kf);
-        if (y > M) { s *= ref_scale(M, y); M = y; }
+        if (y > M) { s = ref_sum(s, M, y); M = y; }
         vs = exp_sum<EPV>(v, kf, -M);
     }
     s += vs;
@@ -242,10 +242,10 @@ __global__ void __launch_bounds__(kCThreads, 2) verify_cluster_kernel(const Para
                 const float4 e2 = sh.x_ms[4 * lane + 2], e3 = sh.x_ms[4 * lane + 3];
                 const float MPr = warp_max(fmaxf(fmaxf(e0.x, e1.x), fmaxf(e2.x, e3.x)));
                 const float MQr = warp_max(fmaxf(fmaxf(e0.z, e1.z), fmaxf(e2.z, e3.z)));
-                double ZP = static_cast<double>(e0.y) * ref_scale(e0.x, MPr) + static_cast<double>(e1.y) * ref_scale(e1.x, MPr) +
-                            static_cast<double>(e2.y) * ref_scale(e2.x, MPr) + static_cast<double>(e3.y) * ref_scale(e3.x, MPr);
-                double ZQ = static_cast<double>(e0.w) * ref_scale(e0.z, MQr) + static_cast<double>(e1.w) * ref_scale(e1.z, MQr) +
-                            static_cast<double>(e2.w) * ref_scale(e2.z, MQr) + static_cast<double>(e3.w) * ref_scale(e3.z, MQr);
+                double ZP = ref_sum(static_cast<double>(e0.y), e0.x, MPr) + ref_sum(static_cast<double>(e1.y), e1.x, MPr) +
+                            ref_sum(static_cast<double>(e2.y), e2.x, MPr) + ref_sum(static_cast<double>(e3.y), e3.x, MPr);
+                double ZQ = ref_sum(static_cast<double>(e0.w), e0.z, MQr) + ref_sum(static_cast<double>(e1.w), e1.z, MQr) +
+                            ref_sum(static_cast<double>(e2.w), e2.z, MQr) + ref_sum(static_cast<double>(e3.w), e3.z, MQr);
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) { ZP += shfl_xor_d(ZP, off); ZQ += shfl_xor_d(ZQ, off); }
                 if (lane == 0) {

@@ -116,7 +116,7 @@ __device__ void f_draw_from_sweep1(const Params& prm, const FlowScratch& fl, con
     }
     const float Mrow = warp_max(fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])));
 #pragma unroll
-    for (int j = 0; j < 4; ++j) w[j] *= static_cast<double>(ref_scale(m[j], Mrow));
+    for (int j = 0; j < 4; ++j) w[j] = ref_sum(w[j], m[j], Mrow);
     // (fp64 sums of the segment totals, as for the residual samples)
     const double d1 = w[0], d2 = d1 + w[1], d3 = d2 + w[2], d4 = d3 + w[3];
     double inc = d4;
@@ -172,8 +172,8 @@ __device__ void f_store_sweep1(const Params& prm, const FlowScratch& fl, const F
     const float mP = lane < kFWarps ? sh.stage_M[j][0][lane] : kNoRef;
     const float mQ = lane < kFWarps ? sh.stage_M[j][1][lane] : kNoRef;
     const float MPc = warp_max(mP), MQc = warp_max(mQ);
-    double zP = lane < kFWarps ? sh.stage_d[j][lane] * ref_scale(mP, MPc) : 0.0;
-    double zQ = lane < kFWarps ? static_cast<double>(sh.stage_s[j][lane]) * ref_scale(mQ, MQc) : 0.0;
+    double zP = lane < kFWarps ? ref_sum(sh.stage_d[j][lane], mP, MPc) : 0.0;
+    double zQ = lane < kFWarps ? ref_sum(static_cast<double>(sh.stage_s[j][lane]), mQ, MQc) : 0.0;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) { zP += shfl_xor_d(zP, off); zQ += shfl_xor_d(zQ, off); }
     // A last target row is swept for one purpose only: the sample from P_gamma.  Its warps' pairs
@@ -254,12 +254,12 @@ __device__ __forceinline__ void f_step_sweep1_pair(const float (&vp)[EPV], const
     if (__any_sync(0xffffffffu, fmaxf(vsP, vsQ) > kRaiseBound)) {   // a logit above a reference
         if (__any_sync(0xffffffffu, vsP > kRaiseBound)) {
             const float y = rintf(warp_max(vec_max<EPV>(vp)) * kf);
-            if (y > MPw) { sP *= ref_scale(MPw, y); MPw = y; }
+            if (y > MPw) { sP = ref_sum(sP, MPw, y); MPw = y; }
             vsP = f_exp_sum<EPV>(vp, kf, -MPw);
         }
         if (__any_sync(0xffffffffu, vsQ > kRaiseBound)) {
             const float y = rintf(warp_max(vec_max<EPV>(vq)) * kf);
-            if (y > MQw) { sQ *= ref_scale(MQw, y); MQw = y; }
+            if (y > MQw) { sQ = ref_sum(sQ, MQw, y); MQw = y; }
             vsQ = f_exp_sum<EPV>(vq, kf, -MQw);
         }
     }

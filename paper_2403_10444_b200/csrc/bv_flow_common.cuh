@@ -54,7 +54,7 @@ template <int EPV> __device__ __forceinline__ void f_accumulate(const float (&v)
     float vs = f_exp_sum<EPV>(v, kf, -M);
     if (__any_sync(0xffffffffu, vs > kRaiseBound)) {      // some logit lies above the reference
         const float y = rintf(warp_max(vec_max<EPV>(v)) * kf);
-        if (y > M) { s *= ref_scale(M, y); M = y; }
+        if (y > M) { s = ref_sum(s, M, y); M = y; }
         vs = f_exp_sum<EPV>(v, kf, -M);
     }
     s += vs;
@@ -96,7 +96,7 @@ __device__ __forceinline__ void f_step_sweep1_single(const float (&va)[EPV], con
     float vsB = f_exp_sum<EPV>(vb, kf, -MPw);
     if (__any_sync(0xffffffffu, fmaxf(vsA, vsB) > kRaiseBound)) {
         const float y = rintf(warp_max(fmaxf(vec_max<EPV>(va), vec_max<EPV>(vb))) * kf);
-        if (y > MPw) { sP *= static_cast<Sum>(ref_scale(MPw, y)); MPw = y; }
+        if (y > MPw) { sP = ref_sum(sP, MPw, y); MPw = y; }
         vsA = f_exp_sum<EPV>(va, kf, -MPw);
         vsB = f_exp_sum<EPV>(vb, kf, -MPw);
     }
@@ -725,8 +725,8 @@ __device__ void f_row_complete(const Params& prm, const FlowScratch& fl, const F
     if (xok && lane < 2) zl = load_logit<DT>(lane == 0 ? rowP : rowQ, x);
     // row reference = max of the chunk references (integers, exact as floats), then the scaled sums
     const float MPf = warp_max(static_cast<float>(z.MP)), MQf = warp_max(static_cast<float>(z.MQ));
-    double ZP = z.ZP * static_cast<double>(ref_scale(static_cast<float>(z.MP), MPf));
-    double ZQ = z.ZQ * static_cast<double>(ref_scale(static_cast<float>(z.MQ), MQf));
+    double ZP = ref_sum(z.ZP, static_cast<float>(z.MP), MPf);
+    double ZQ = ref_sum(z.ZQ, static_cast<float>(z.MQ), MQf);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) { ZP += shfl_xor_d(ZP, off); ZQ += shfl_xor_d(ZQ, off); }
     const double zp = shfl_d(zl, 0), zq = shfl_d(zl, 1);

@@ -46,10 +46,10 @@ constexpr int kLoopRuns = 4;                      // runs of 32 vectors that a w
 // exponential (a run at a time, each testing whether its sum shows a logit above the reference: 1.65 us for a row of 2048
 // vectors; like this 1.2), and their sums cross the lanes side by side.
 
-// kLoopRuns runs of a row from vector `base` on: the reference raised to their maximum, by how much 2^-that is returned, and
-// each run's sum of this lane's terms
+// kLoopRuns runs of a row from vector `base` on: the reference raised to their maximum, the sum so far against it, and each
+// run's sum of this lane's terms
 template <int DT>
-__device__ __forceinline__ float l_group(uint32_t image, int base, int u1, int lane, float kf, float& M, float (&vs)[kLoopRuns]) {
+__device__ __forceinline__ void l_group(uint32_t image, int base, int u1, int lane, float kf, float& M, float& s, float (&vs)[kLoopRuns]) {
     using R = Raw<DT>;
     constexpr int EPV = R::EPV;
     uint4 raw[kLoopRuns];
@@ -60,14 +60,14 @@ __device__ __forceinline__ float l_group(uint32_t image, int base, int u1, int l
     for (int j = 1; j < kLoopRuns; ++j) top = vec_max<DT>(top, raw[j]);
     float v[EPV];
     R::unpack(top, v);
-    const float y = fmaxf(M, rintf(warp_max(vec_max<EPV>(v)) * kf)), scale = ref_scale(M, y);
+    const float y = fmaxf(M, rintf(warp_max(vec_max<EPV>(v)) * kf));
+    s = ref_sum(s, M, y);
     M = y;
 #pragma unroll
     for (int j = 0; j < kLoopRuns; ++j) {
         R::unpack(raw[j], v);
         vs[j] = f_exp_sum<EPV>(v, kf, -M);
     }
-    return scale;
 }
 
 // s_sweep_row on the row's image
@@ -79,7 +79,7 @@ __device__ __forceinline__ void l_sweep_draft(uint32_t image, int units, float k
     int sub = 0, left = runs;
     for (int base = u0; base < u1; base += 32 * kLoopRuns) {
         float vs[kLoopRuns];
-        s *= l_group<DT>(image, base, u1, lane, kf, M, vs);
+        l_group<DT>(image, base, u1, lane, kf, M, s, vs);
         const int n = min((u1 - base + 31) / 32, kLoopRuns);
         if (runs == 1) {                          // (a sub-segment a run; a group of fewer has empty ones behind it)
             if (SHORT) {
@@ -135,7 +135,7 @@ __device__ __forceinline__ void l_sweep_target(uint32_t image, int units, float 
     s_part(units, warp, u0, u1, runs);
     for (int base = u0; base < u1; base += 32 * kLoopRuns) {
         float vs[kLoopRuns];
-        s *= l_group<DT>(image, base, u1, lane, kf, M, vs);
+        l_group<DT>(image, base, u1, lane, kf, M, s, vs);
         s += (vs[0] + vs[1]) + (vs[2] + vs[3]);
     }
     const double z = warp_sum_d(static_cast<double>(s));
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(kSAllThreads, 2) decode_loop_kernel(const __gr
             if (sampling) {
                 // behind the streaming warps' next loads: what the verification wants to know of this row
                 const float m = lane < kSWarps && ok ? static_cast<float>(sh.wM[lane]) : kNoRef, mr = warp_max(m);
-                const double z = warp_sum_d(lane < kSWarps && ok ? sh.wZ[lane] * static_cast<double>(ref_scale(m, mr)) : 0.0);
+                const double z = warp_sum_d(lane < kSWarps && ok ? ref_sum(sh.wZ[lane], m, mr) : 0.0);
                 float zl = 0.f;           // the drafted token's logits
                 if (found >= 0 && lane < 2) zl = logit((lane == 0 ? tgt : drf) + at, found);
                 const float zq = __shfl_sync(0xffffffffu, zl, 1);

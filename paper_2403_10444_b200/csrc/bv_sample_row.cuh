@@ -103,7 +103,7 @@ __device__ __forceinline__ void s_sweep_row(const char* row, int units, float kf
         float v[EPV];
         R::unpack(top, v);
         const float y = fmaxf(M, rintf(warp_max(vec_max<EPV>(v)) * kf));
-        s *= ref_scale(M, y);
+        s = ref_sum(s, M, y);
         M = y;
 #pragma unroll
         for (int j = 0; j < kSInFlight; ++j) {
@@ -164,8 +164,7 @@ __device__ __forceinline__ int s_locate(const SubSegment<SHORT>* seg, float u, i
     const float Mrow = warp_max(fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])));
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const float to = ref_scale(m[j], Mrow);
-        w[j] = SHORT ? w[j] * static_cast<double>(to) : static_cast<double>(za[j] * to) + static_cast<double>(zb[j] * to);
+        w[j] = SHORT ? ref_sum(w[j], m[j], Mrow) : static_cast<double>(ref_sum(za[j], m[j], Mrow)) + static_cast<double>(ref_sum(zb[j], m[j], Mrow));
     }
     double Z = (w[0] + w[1]) + (w[2] + w[3]);
 #pragma unroll
