@@ -252,8 +252,8 @@ __global__ void __launch_bounds__(kCThreads, 2) verify_cluster_kernel(const Para
                     int bad = sh.bad;
                     // the row's maximum is finite iff its reference is; Z is NaN / inf iff the row
                     // holds a NaN / the sum overflowed
-                    if (!(MPr > kNoRef && MPr < INFINITY) || !(ZP < INFINITY)) bad = 1;
-                    if (have_q && (!(MQr > kNoRef && MQr < INFINITY) || !(ZQ < INFINITY))) bad = 1;
+                    if (!(MPr > kNoRef && MPr < INFINITY) || !row_sum_ok(ZP)) bad = 1;
+                    if (have_q && (!(MQr > kNoRef && MQr < INFINITY) || !row_sum_ok(ZQ))) bad = 1;
                     double ratio = 0.0;
                     if (have_q) {
                         if (!x_ok || zq_x == -INFINITY) bad = 1;

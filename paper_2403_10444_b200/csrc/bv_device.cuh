@@ -399,5 +399,8 @@ constexpr float kRaiseBound = 12.f;
 template <class Sum> __device__ __forceinline__ Sum ref_sum(Sum s, float own, float row) {
     return ref_moved(s, own > kNoRef ? own - row : -INFINITY);
 }
+// Is Z, the sum of a row with a finite maximum, a normaliser?  NaN: the row holds one.  Zero or infinite: its largest scaled logit is
+// beyond 2^31 either way, the reference lies further off it than an exponent reaches, and nothing is known of the row.
+__device__ __forceinline__ bool row_sum_ok(double Z) { return Z > 0.0 && Z < static_cast<double>(INFINITY); }
 
 }  // namespace bv

@@ -744,9 +744,9 @@ __device__ void f_row_complete(const Params& prm, const FlowScratch& fl, const F
         RowZ out; out.MP = MP; out.ZP = ZP; out.MQ = MQ; out.ZQ = ZQ;
         fl.rowZ[rowi] = out;
         // the row's maximum is finite iff its reference is; Z is NaN / inf iff the row holds a NaN / overflowed
-        bool bad = !(MP > kNoRef && MP < INFINITY) || !(ZP < INFINITY);
+        bool bad = !(MP > kNoRef && MP < INFINITY) || !row_sum_ok(ZP);
         if (have_q) {
-            bad = bad || !(MQ > kNoRef && MQ < INFINITY) || !(ZQ < INFINITY) || !xok || zq == -INFINITY;
+            bad = bad || !(MQ > kNoRef && MQ < INFINITY) || !row_sum_ok(ZQ) || !xok || zq == -INFINITY;
             // ratio = P_r(X_{r+1}) / Q_r(X_{r+1}) from the two logits of the drafted token
             fl.ratio[rowi] = bad ? 0.0 : exp2((zp - zq) * cx.kd - (MP - MQ)) * (ZQ / ZP);
             fl.zratio[rowi] = ZQ / ZP;

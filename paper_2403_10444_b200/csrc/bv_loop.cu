@@ -250,7 +250,7 @@ __device__ __forceinline__ int l_decide(const LoopArgs& a, LoopShared& sh, int l
         if (c >= g) continue;
         const double MP = sh.MP[c], ZP = sh.ZP[c], MQ = sh.MQ[c], ZQ = sh.ZQ[c], zp = sh.zp[c], zq = sh.zq[c];
         const double none = static_cast<double>(kNoRef), inf = static_cast<double>(INFINITY);
-        badrow[h] = !(MP > none && MP < inf) || !(ZP < inf) || !(MQ > none && MQ < inf) || !(ZQ < inf) || sh.tok[c] < 0 || zq == -inf;
+        badrow[h] = !(MP > none && MP < inf) || !row_sum_ok(ZP) || !(MQ > none && MQ < inf) || !row_sum_ok(ZQ) || sh.tok[c] < 0 || zq == -inf;
         zr[h] = ZQ / ZP;
         rat[h] = badrow[h] ? 0.0 : exp2((zp - zq) * a.kd - (MP - MQ)) * zr[h];
     }

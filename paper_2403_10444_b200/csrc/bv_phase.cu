@@ -324,8 +324,8 @@ static __device__ __noinline__ void ph_fold(const Params& prm, const PhaseScratc
         if (h == 1 && g <= 32) break;
         if (lane + 32 * h < g) {
             // the row's maximum is finite iff its reference is; Z is NaN / inf iff the row holds a NaN / overflowed
-            badrow[h] = !(MP[h] > kNoRef && MP[h] < INFINITY) || !(ZP[h] < static_cast<double>(INFINITY)) ||
-                        !(MQ[h] > kNoRef && MQ[h] < INFINITY) || !(ZQ[h] < static_cast<double>(INFINITY)) || zq[h] == -INFINITY;
+            badrow[h] = !(MP[h] > kNoRef && MP[h] < INFINITY) || !row_sum_ok(ZP[h]) ||
+                        !(MQ[h] > kNoRef && MQ[h] < INFINITY) || !row_sum_ok(ZQ[h]) || zq[h] == -INFINITY;
             rat[h] = badrow[h] ? 0.0 : exp2((zp[h] - zq[h]) * prm.kd - (static_cast<double>(MP[h]) - static_cast<double>(MQ[h]))) * (ZQ[h] / ZP[h]);
         }
     }
@@ -460,7 +460,7 @@ static __device__ __noinline__ void ph_finalize(const Params& prm, const PhaseSc
         const double mine = ph_lane_sum(at, per, lane), total = warp_sum_d(mine);
         bool pass;
         if (c == g) {
-            if (!ok || !(total < static_cast<double>(INFINITY))) bad = true;      // (a fault in a last target row that is read is the sequence's)
+            if (!ok || !(PROBS ? total < static_cast<double>(INFINITY) : row_sum_ok(total))) bad = true;      // (a fault in a last target row that is read is the sequence's)
             pass = tv || (p_g > 0.0 && static_cast<double>(eta_g) <= p_g);
             if (all && prm.out_h && !tv && lane == 0) prm.out_h[ri] = static_cast<float>(p_g);
             if (all && prm.out_lse_t && lane == 0) prm.out_lse_t[ri] = static_cast<float>((static_cast<double>(Mr) + log2(total)) * ln2);

@@ -353,8 +353,8 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __
                         bad = !xok || !(zq > 0.0 && zq < static_cast<double>(INFINITY)) || !(zp >= 0.0 && zp < static_cast<double>(INFINITY));
                         rat[h] = bad ? 0.0 : zp / zq;
                     } else {
-                        bad = !(MP > kNoRef && MP < INFINITY) || !(ZP < static_cast<double>(INFINITY)) ||
-                              !(MQ > kNoRef && MQ < INFINITY) || !(ZQ < static_cast<double>(INFINITY)) || !xok || zq == -INFINITY;
+                        bad = !(MP > kNoRef && MP < INFINITY) || !row_sum_ok(ZP) ||
+                              !(MQ > kNoRef && MQ < INFINITY) || !row_sum_ok(ZQ) || !xok || zq == -INFINITY;
                         rat[h] = bad ? 0.0 : exp2((zp - zq) * prm.kd - (static_cast<double>(MP) - static_cast<double>(MQ))) * (ZQ / ZP);
                     }
                     badrow[h] = bad;
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __
             }
             const float MPg = sh.rowM[b * rpb + g];
             const double ZPg = sh.rowZ[b * rpb + g];
-            const bool bad_last = !PROBS && (!(MPg > kNoRef && MPg < INFINITY) || !(ZPg < static_cast<double>(INFINITY)));
+            const bool bad_last = !PROBS && (!(MPg > kNoRef && MPg < INFINITY) || !row_sum_ok(ZPg));
             const unsigned bad_lo = __ballot_sync(0xffffffffu, badrow[0]), bad_hi = __ballot_sync(0xffffffffu, badrow[1]);
             unsigned m_lo = 0, m_hi = 0;
             int lastw = 0, bad = 0, tau_tv = 0;

@@ -338,8 +338,8 @@ __global__ void __launch_bounds__(kThreads, 1) verify_stream_kernel(const Params
                     const double ln2 = 0.693147180559945309417232;
                     int bad = sh.bad;
                     // M is finite iff the row's maximum is; Z is NaN iff the row holds a NaN
-                    if (!(fabsf(MP) < INFINITY) || !(ZP == ZP)) bad = 1;
-                    if (have_q && (!(fabsf(MQ) < INFINITY) || !(ZQ == ZQ))) bad = 1;
+                    if (!(fabsf(MP) < INFINITY) || !row_sum_ok(ZP)) bad = 1;
+                    if (have_q && (!(fabsf(MQ) < INFINITY) || !row_sum_ok(ZQ))) bad = 1;
                     const double lse2P = static_cast<double>(MP) + log2(ZP);
                     const double lse2Q = static_cast<double>(MQ) + log2(ZQ);
                     sh.lse_t[r] = lse2P * ln2;

@@ -69,3 +69,22 @@ def test_decoding_loop(dtype, V, value):
         got = [out["tokens"][b, : out["lengths"][b]].tolist() for b in range(B)]
         # (a draw within 1e-6 of the edge of its cell, 200 of them, sends a sequence its own way; none does here)
         assert got == want, algo
+
+
+# (the scaled value and the integer that a float has for it lie 312, -328, 512 and 328 apart)
+@pytest.mark.parametrize("value,T", [(-1e10, 1.3), (-1e10, 1.0), (-3e10, 1.3), (1e10, 1.0)])
+@pytest.mark.parametrize("V", [4096, 4099])
+@pytest.mark.parametrize("kernel", [1, 2, 3, 4, 5])
+def test_a_row_without_a_normaliser_is_a_data_fault(kernel, V, value, T, bv_options):
+    if V % 8 and kernel in (1, 2):
+        pytest.skip("these kernels take rows of whole 16-byte vectors")
+    bv_options("kernel", kernel)
+    inp = wl.make_inputs(wl.Workload("m", 8, 3, V, "bf16", T, V, 2.0, 0.0, 0, 0.0, 0.5), "cpu")
+    for b in range(8):
+        (inp["target_logits"] if b < 4 else inp["draft_logits"])[b, b % 3] = value        # (flat)
+    for algo in (oracle.BLOCK_VERIFY, oracle.TOKEN_VERIFY):
+        out = run_cuda(algo, inp, diagnostics=False)
+        ref = run_oracle(algo, inp)
+        for b in range(8):
+            # (Algorithm 1 may end before it gets to the row)
+            assert out[1][b] == -1 or (algo == oracle.TOKEN_VERIFY and out[1][b] == ref.out_len[b] <= b % 3), (algo, b)
