@@ -40,7 +40,7 @@
  * NaN or +inf logit in a row the algorithm reads, a row of all -inf, a drafted
  * token outside [0, V) or whose draft logit is -inf give out_len[b] = -1 and
  * out_tokens[b, :] = -1; other sequences are unaffected.  Masks may be -inf or finite
- * (-1e9, -1e20, the type's lowest value): they weigh nothing beside smaller logits.  A row
+ * (-1e9, -1e20, the type's lowest value): they weigh nothing beside ordinary logits.  A row
  * whose LARGEST logit times log2(e) / T is beyond 2^31 in magnitude, which fp32 arithmetic
  * does not resolve, may count as one that cannot be read.
  */

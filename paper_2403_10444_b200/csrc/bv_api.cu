@@ -147,7 +147,9 @@ struct DeviceState {
 
 DeviceState g_dev[kMaxDevices];
 std::mutex g_mu;
-std::mutex g_host_mu;               // held for the whole of a call on host buffers: they share the staging areas
+// Held for the whole of a call on host buffers: a device's calls share its staging areas and stream.  (One each, taken before g_mu:
+// calls on different devices run side by side.)
+std::mutex g_host_mu[kMaxDevices];
 
 thread_local int t_last_launches = 0;
 thread_local int t_last_kernel = 0;     // which kernel the last verification call on this thread launched (the "kernel" option's codes)
@@ -615,11 +617,14 @@ int run_host(int algo, const void* tgt, const void* drf, const int32_t* tok, con
     const size_t i_uni = align_up(n_tok, 16), i_status = align_up(i_uni + n_uni, 16), i_ot = i_status + 16, i_ol = align_up(i_ot + n_ot, 16);
     const size_t n_in = i_ot, n_small = i_ol + n_ol, total = o_in + n_small;
 
-    std::lock_guard<std::mutex> host_lock(g_host_mu);
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return cuda_fail(e);
+    if (dev < 0 || dev >= kMaxDevices) return BV_ERR_UNSUPPORTED;
+    std::lock_guard<std::mutex> host_lock(g_host_mu[dev]);
     char* base = nullptr;
     char* pin = nullptr;
     cudaStream_t s = nullptr;
-    cudaError_t e;
     {
         std::lock_guard<std::mutex> lock(g_mu);
         DeviceState* d = nullptr;
@@ -843,12 +848,12 @@ int bv_set_option(const char* name, int value) {
 }
 
 int bv_release(void) {
-    std::lock_guard<std::mutex> host_lock(g_host_mu);
-    std::lock_guard<std::mutex> lock(g_mu);
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e);
     if (dev < 0 || dev >= kMaxDevices) return BV_ERR_UNSUPPORTED;
+    std::lock_guard<std::mutex> host_lock(g_host_mu[dev]);
+    std::lock_guard<std::mutex> lock(g_mu);
     DeviceState& d = g_dev[dev];
     if ((e = cudaDeviceSynchronize()) != cudaSuccess) return cuda_fail(e);
     if (d.stage) cudaFree(d.stage);

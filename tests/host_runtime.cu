@@ -3,11 +3,14 @@
 // (scratch: anything; counters: zero), and a captured stream records its work for replays.  Plans come from the library itself.
 #include <cuda_runtime.h>
 
+#include <chrono>
+#include <condition_variable>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
 #include <functional>
 #include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -59,7 +62,8 @@ cudaError_t enqueue(cudaStream_t s, std::function<void()> f) {
     return cudaSuccess;
 }
 
-cudaError_t fake_cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
+thread_local int t_device = 0;
+cudaError_t fake_cudaGetDevice(int* d) { *d = t_device; return cudaSuccess; }
 cudaError_t fake_cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
     *v = a == cudaDevAttrMultiProcessorCount ? 148 : 10;
     return cudaSuccess;
@@ -84,10 +88,22 @@ cudaError_t fake_cudaStreamIsCapturing(cudaStream_t st, cudaStreamCaptureStatus*
     return cudaSuccess;
 }
 cudaError_t fake_cudaGetLastError() { return cudaSuccess; }
+// threads that wait for a stream at the same time: each waits for as many as are asked for, or for a while
+std::mutex g_meet_mu;
+std::condition_variable g_meet_cv;
+int g_meet_want = 0, g_meet_now = 0, g_meet_most = 0;
 cudaError_t fake_cudaStreamSynchronize(cudaStream_t s) {
     if (captured(s)) complain("a captured stream is waited for");
+    std::unique_lock<std::mutex> lock(g_meet_mu);
+    if (g_meet_want > 0) {
+        if (++g_meet_now > g_meet_most) { g_meet_most = g_meet_now; g_meet_cv.notify_all(); }
+        g_meet_cv.wait_for(lock, std::chrono::milliseconds(500), [] { return g_meet_most >= g_meet_want; });
+        --g_meet_now;
+    }
     return cudaSuccess;
 }
+cudaError_t fake_cudaHostAlloc(void** p, size_t n, unsigned) { return give(p, n); }
+cudaError_t fake_cudaFreeHost(void* p) { return take_back(p); }
 cudaError_t fake_cudaDeviceSynchronize() { return cudaSuccess; }
 cudaError_t fake_cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = reinterpret_cast<cudaStream_t>(7); return cudaSuccess; }
 cudaError_t fake_cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
@@ -174,6 +190,8 @@ cudaError_t fake_launch_stream(const Params& prm, int, int, bool, int, int, cuda
 #define cudaStreamIsCapturing fake_cudaStreamIsCapturing
 #define cudaGetLastError fake_cudaGetLastError
 #define cudaStreamSynchronize fake_cudaStreamSynchronize
+#define cudaHostAlloc fake_cudaHostAlloc
+#define cudaFreeHost fake_cudaFreeHost
 #define cudaDeviceSynchronize fake_cudaDeviceSynchronize
 #define cudaStreamCreateWithFlags fake_cudaStreamCreateWithFlags
 #define cudaStreamDestroy fake_cudaStreamDestroy
@@ -193,6 +211,10 @@ extern "C" {
 void host_begin_capture(void* stream) { g_graphs.emplace_back(); g_capturing = true; g_captured = static_cast<cudaStream_t>(stream); }
 int host_end_capture() { g_capturing = false; return static_cast<int>(g_graphs.size()) - 1; }
 void host_replay(int graph) { for (const auto& f : g_graphs[graph]) f(); }
+void host_set_device(int device) { t_device = device; }
+// from now on: how many threads wait for a stream together, at most
+void host_meet(int want) { g_meet_want = want; g_meet_most = 0; }
+int host_met() { return g_meet_most; }
 void host_refuse_cooperative(int on) { g_refuse_cooperative = on; }
 // a verification of the decoding loop
 int host_tables(int algo, int B, int gamma, int V, int dtype, int lse, int probe) {

@@ -2,7 +2,9 @@
 import ctypes
 import os
 import subprocess
+import threading
 
+import numpy as np
 import pytest
 
 from paper_2403_10444_b200 import build as bv_build
@@ -212,3 +214,36 @@ def test_which_kernel_takes_a_call(host):
     for (fn, B, gamma, V, dtype, diagnostics), kernel in ROUTES:
         assert verify(host, B, gamma, V, dtype, fn, diagnostics=diagnostics) == (0, kernel), (fn, B, gamma, V, dtype, diagnostics)
     assert host.host_errors() == b""
+
+
+@pytest.mark.parametrize("devices,together", [((0, 1), 2), ((0, 0), 1)])
+def test_host_buffers_are_shared_by_a_device_s_calls_and_by_no_others(host, devices, together):
+    # two threads' calls of different sizes: on two devices both are under way at once, on one device one after the other
+    status = []
+
+    def call(device, B):
+        host.host_set_device(device)
+        gamma, V = 2, 64
+        a = [np.zeros(n, np.float32) for n in (B * (gamma + 1) * V, B * gamma * V, B * gamma, B * (gamma + 2), B * (gamma + 1), B)]
+        p = [ctypes.c_void_p(x.ctypes.data) for x in a]
+        status.append(host.bv_verify_host(*p[:4], B, gamma, V, F32, FLOAT, *p[4:]))
+
+    for d in set(devices):
+        warm = threading.Thread(target=call, args=(d, 1))
+        warm.start()
+        warm.join()
+    host.host_meet(2)
+    try:
+        threads = [threading.Thread(target=call, args=(d, B)) for d, B in zip(devices, (3, 40))]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+    finally:
+        met = host.host_met()
+        host.host_meet(0)
+    assert met == together and status == [0] * len(status) and host.host_errors() == b""
+    for d in set(devices):
+        release = threading.Thread(target=lambda: (host.host_set_device(d), host.bv_release()))
+        release.start()
+        release.join()

@@ -255,6 +255,27 @@ def test_host_buffer_entry_matches_device_entry():
         assert torch.equal(ot, dt.cpu()) and torch.equal(ol, dl.cpu())
 
 
+def test_host_calls_of_different_sizes_from_two_threads():
+    import threading
+    import paper_2403_10444_b200 as bv
+    calls = [random_inputs(33, 4, 3000, "bf16", seed=31), random_inputs(5, 2, 40000, "f32", seed=32)]
+    want = [run_cuda(oracle.BLOCK_VERIFY, inp, diagnostics=False) for inp in calls]
+    bad = []
+
+    def work(i):
+        for _ in range(30):
+            ot, ol = bv.bv_verify_host(*(calls[i][k] for k in ("target_logits", "draft_logits", "draft_tokens", "uniforms", "temperature")))
+            if not (torch.equal(ot, want[i][0].cpu()) and torch.equal(ol, want[i][1].cpu())):
+                bad.append(i)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
+
+
 def test_launch_count_and_nonblocking_stream():
     import paper_2403_10444_b200 as bv
     inp = {k: (v.cuda() if torch.is_tensor(v) else v) for k, v in random_inputs(5, 2, 1024, "f32", 1).items()}
