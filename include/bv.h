@@ -328,7 +328,9 @@ int bv_draft_chain(const void* draft_table, const int32_t* first_tokens, const f
  *   first_tokens [B] int32     the last token of each context
  *   out_tokens  [B, iterations (gamma+1)] int32: the tokens generated, then -1;  out_lengths [B] int64: how many
  *   out_tau     [iterations, B] int32 accepted drafts;  out_drafted [iterations, B, gamma] int32
- *   out_fault   [1] int32: 1 if a sequence reported a data fault (its further tokens mean nothing)
+ *   out_fault   [1] int32: 1 if a sequence reported a data fault (its further tokens mean nothing).  Of Algorithm 2's rows the
+ *               last target row counts, where position gamma is not selected, only in batches that are small enough for the
+ *               small-batch kernel (up to 32 sequences)
  *   work        B (2 gamma + 3) int32
  * Rows must be whole 16-byte vectors on 16-byte aligned bases and B at most 768, else BV_ERR_UNSUPPORTED; whether a kernel
  * takes the call, and its workspace, is settled before anything is enqueued.

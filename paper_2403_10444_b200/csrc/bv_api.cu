@@ -323,7 +323,7 @@ bool phase_pays(int algo, const bv::Params& prm, const Options& opt, const Devic
         return 2 * one_row <= (f32 ? kPhaseProbsPairsF32[a] : kPhaseProbsPairs[a]);
     }
     const int which = a == 0 ? 0 : (prm.lse_d != nullptr ? 2 : 1);
-    if (prm.first != nullptr) return !small || logit_bytes > kPhaseBytes[which][0];      // (no other kernel takes larger ones)
+    if (prm.first != nullptr) return !bv::small_takes_tables(algo, prm.lse_d != nullptr, prm.B, prm.gamma, static_cast<size_t>(one_row / prm.B));      // (no other kernel takes larger ones)
     const long long small_limit = opt.small_bytes > 0 ? static_cast<long long>(opt.small_bytes) << 20 : kSmallBytes[a];
     if (small && prm.B < kPhaseFew && logit_bytes <= small_limit) return false;
     if (vec && f32 && prm.B < kPhaseFew && one_row / prm.B > kPhaseFewRow) return false;
@@ -693,6 +693,10 @@ int note_cuda_error(cudaError_t e) {
     return BV_ERR_CUDA;
 }
 void note_launches(int n) { t_last_launches = n; }
+bool small_takes_tables(int algo, bool lse, int B, int gamma, size_t row_bytes) {
+    return small_fits(B, gamma) &&
+           static_cast<long long>(B) * (2 * gamma + 1) * static_cast<long long>(row_bytes) <= kPhaseBytes[algo != kBlockVerify ? 0 : lse ? 2 : 1][0];
+}
 int kernel_option() {
     std::call_once(g_opt_once, load_env_options);
     std::lock_guard<std::mutex> lock(g_mu);

@@ -18,6 +18,9 @@ void note_launches(int n);
 int run_tables(int algo, const void* tgt_table, const void* drf_table, const int32_t* first, const int32_t* tok, const float* uni,
                const float* lse_d, int B, int gamma, int V, int dtype, float T, int32_t* ot, int32_t* ol, bool probe, cudaStream_t stream);
 
+// Does the small-batch kernel take these (else the phase kernel does)?
+bool small_takes_tables(int algo, bool lse, int B, int gamma, size_t row_bytes);
+
 // The option "kernel" (0: chosen by shape).
 int kernel_option();
 
@@ -32,6 +35,7 @@ struct LoopArgs {
     float kf;
     double kd;
     int token;                // Algorithm 1 instead of Algorithm 2
+    int last_counts;          // a last target row that cannot be read is a fault even where position gamma is not selected
     int lse;                  // the verification takes the draft rows' normalisers as the drafting step rounds them to 32 bits
     int32_t* seq;             // [B, width]
     long long* lengths;       // [B]

@@ -396,11 +396,11 @@ __global__ void __launch_bounds__(kSAllThreads, 2) decode_loop_kernel(const __gr
         __syncthreads();
         int tau = -1, found = -1;
         if (sampling && !bad && have_last) {
-            // (a fault in the last target row is the sequence's, for Algorithm 1 if it is the row to sample from)
+            // (a fault in the last target row is the sequence's if it is the row to sample from, or if it counts in any case)
             double norm[2], rem = 0.0;
             const int sel = s_locate<true>(segL, sh.u[g + 1], lane, -1, norm, rem);
             if (sh.last) { tau = g; if (sel >= 0) found = l_rescan<DT, false>(imageP, 0u, units, sel, lane, kf, 1.f, -static_cast<float>(norm[0]), 0.f, rem); }
-            else if (sel < 0 && !a.token) bad = 1;
+            else if (sel < 0 && a.last_counts) bad = 1;
         }
         unsigned lo = sh.lo, hi = sh.hi;
         bool over = sh.last != 0 || sh.over != 0;

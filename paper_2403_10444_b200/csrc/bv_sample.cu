@@ -224,8 +224,11 @@ extern "C" int bv_decode_loop(const void* target_table, const void* draft_table,
     cudaError_t e;
     if (bv::loop_fits(V, dtype) && bv::kernel_option() == 0) {
         const double kd = 1.4426950408889634073599246810019 / static_cast<double>(temperature);
+        // (a last target row that is not wanted: the small-batch kernel sweeps every row and faults the sequence, the phase kernel does
+        // not look; of a loop's calls, which of them takes it decides)
+        const int last_counts = !(algo & 1) && bv::small_takes_tables(bv::kBlockVerify, algo < 2, B, gamma, row_bytes);
         const bv::LoopArgs args{target_table, draft_table, first_tokens, u_draft, u_verify, iterations, B, gamma, V, static_cast<int>(width),
-                                static_cast<float>(kd), kd, algo & 1, algo < 2, out_tokens, reinterpret_cast<long long*>(out_lengths),
+                                static_cast<float>(kd), kd, algo & 1, last_counts, algo < 2, out_tokens, reinterpret_cast<long long*>(out_lengths),
                                 out_tau, out_drafted, out_fault};
         if ((e = cudaMemsetAsync(out_fault, 0, 4, st)) != cudaSuccess || (e = bv::launch_loop(args, dtype, st)) != cudaSuccess) return bv::note_cuda_error(e);
         bv::note_launches(1);

@@ -44,3 +44,41 @@ def test_rows_that_cannot_be_read(algo):
     bad[2, 7] = float("nan")
     with pytest.raises(RuntimeError):
         specdec.run(bad, dt, first, ud, uv, 3, algo=algo)
+
+
+# (32 sequences and fewer: whatever is selected, the last target row counts; more: where it is read)
+@pytest.mark.parametrize("B,kernel", [(24, 4), (80, 5)])
+@pytest.mark.parametrize("algo", range(4))
+@pytest.mark.parametrize("gamma", [1, 4])
+def test_faults_end_the_sequences_that_meet_them_and_no_others(B, kernel, algo, gamma, bv_options):
+    # the draft goes from token t to t + 1, so that sequence b meets bad rows at position 40 - b and so on, or stops before it
+    from paper_2403_10444_b200 import binding as bv
+    V, N = 128, 2
+    gen = torch.Generator().manual_seed(gamma)
+    t = torch.randn((V, V), generator=gen)
+    d = torch.full((V, V), -8.0)
+    nxt = (torch.arange(V) + 1) % V
+    t[torch.arange(V), nxt] += 4.0
+    d[torch.arange(V), nxt] = 8.0
+    t[40, 3], t[60, 5], d[50, 9], d[70] = float("nan"), float("inf"), float("nan"), float("-inf")
+    tt, dt = t.cuda(), d.cuda()
+    first = (36 + 2 * torch.arange(B) % 41).to(torch.int32)
+    first[5], first[11] = V, -1
+    ud, uv = wl.loop_uniforms(N, B, gamma, 7, "cuda")
+
+    def run():
+        return [x.cpu() for x in bv.bv_decode_loop(tt, dt, first.cuda(), ud, uv, gamma, 1.0, algo)]
+
+    one = run()
+    assert bv.bv_last_launch_count() == 1
+    bv_options("kernel", kernel)
+    two = run()
+    assert bv.bv_last_launch_count() == 2 * N + 1 and bv.bv_last_kernel() == kernel
+    for a, b in zip(one, two):
+        assert torch.equal(a, b)
+    tau = one[2]
+    assert one[4][0] == 1 and (tau == -2).any() and (tau[0] >= 0).sum() >= B // 3
+    if B > 32 and algo % 2 == 0:
+        # the sequence that starts gamma before a target row that cannot be read is at fault only where that row is read
+        last = [b for b in range(B) if first[b] + gamma in (40, 60)]
+        assert last and all(tau[0, b] == -2 or tau[0, b] < gamma for b in last) and any(tau[0, b] >= 0 for b in last)
