@@ -12,6 +12,8 @@
 // Bound: latency, gamma dependent rows and one or two dependent sweeps an iteration; bytes B (2 gamma + 1) rows an iteration.
 // 128 sequences of gamma = 5 over V = 16384 in bf16, 8 iterations: 283 us, 35 an iteration (two launches an iteration, the
 // chain and a verification by all SMs together with its waits for the whole batch: 606 us; the bytes take 56).
+#include <type_traits>
+
 #include "bv_sample_row.cuh"
 
 namespace bv {
@@ -48,8 +50,8 @@ constexpr int kLoopRuns = 4;                      // runs of 32 vectors that a w
 
 // kLoopRuns runs of a row from vector `base` on: the reference raised to their maximum, the sum so far against it, and each
 // run's sum of this lane's terms
-template <int DT>
-__device__ __forceinline__ void l_group(uint32_t image, int base, int u1, int lane, float kf, float& M, float& s, float (&vs)[kLoopRuns]) {
+template <int DT, class Sum>
+__device__ __forceinline__ void l_group(uint32_t image, int base, int u1, int lane, float kf, float& M, Sum& s, float (&vs)[kLoopRuns]) {
     using R = Raw<DT>;
     constexpr int EPV = R::EPV;
     uint4 raw[kLoopRuns];
@@ -70,10 +72,14 @@ __device__ __forceinline__ void l_group(uint32_t image, int base, int u1, int la
     }
 }
 
-// s_sweep_row on the row's image
+// s_sweep_row on the row's image.  (Sub-segments of the last target row, from which a token of the output is drawn, hold doubles
+// (SHORT) whatever the row's length: a lane's vectors are added in double as well, where there are several to a sub-segment, from 4096
+// vectors a row on.  In fp32 the sum of a flat row of 6656 vectors was off by 4.5e-10 on average, like this by 3.0e-10, as in the verification kernels.)
 template <int DT, bool SHORT>
 __device__ __forceinline__ void l_sweep_draft(uint32_t image, int units, float kf, int warp, int lane, SubSegment<SHORT>* seg) {
-    float M = kNoRef, s = 0.f;
+    using Sum = std::conditional_t<SHORT, double, float>;
+    float M = kNoRef;
+    Sum s = 0;
     int u0, u1, runs;
     s_part(units, warp, u0, u1, runs);
     int sub = 0, left = runs;
@@ -111,12 +117,12 @@ __device__ __forceinline__ void l_sweep_draft(uint32_t image, int units, float k
 #pragma unroll
             for (int j = 0; j < kLoopRuns; ++j) {
                 if (j >= n) break;
-                s += vs[j];
+                s += static_cast<Sum>(vs[j]);
                 if (--left == 0) {
                     s_put<SHORT>(M, s, lane, seg + s_place(warp, sub));
                     ++sub;
                     left = runs;
-                    s = 0.f;
+                    s = 0;
                 }
             }
         }

@@ -50,9 +50,9 @@ template <> struct alignas(16) SubSegment<true> { double z; float2 b; };        
 constexpr bool s_short(size_t row_bytes) { return row_bytes < static_cast<size_t>(2048) * 16; }
 // (sub-segment `sub` of warp `warp` lies where lane (8 warp + sub) / 4 of the sampling warp finds it without bank conflicts)
 __device__ __forceinline__ int s_place(int warp, int sub) { return (sub & 3) * 32 + warp * (kSSub / 4) + (sub >> 2); }
-template <bool SHORT>
-__device__ __forceinline__ void s_put(float M, float s, int lane, SubSegment<SHORT>* to) {
-    float2 v = make_float2(s, M);
+template <bool SHORT, class Sum>
+__device__ __forceinline__ void s_put(float M, Sum s, int lane, SubSegment<SHORT>* to) {
+    float2 v = make_float2(static_cast<float>(s), M);
     if (SHORT) {
         const double z = warp_sum_d(static_cast<double>(s));
         v = lane == 0 ? make_float2(__int_as_float(__double2loint(z)), __int_as_float(__double2hiint(z))) : make_float2(M, 0.f);

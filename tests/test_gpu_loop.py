@@ -82,3 +82,24 @@ def test_faults_end_the_sequences_that_meet_them_and_no_others(B, kernel, algo, 
         # the sequence that starts gamma before a target row that cannot be read is at fault only where that row is read
         last = [b for b in range(B) if first[b] + gamma in (40, 60)]
         assert last and all(tau[0, b] == -2 or tau[0, b] < gamma for b in last) and any(tau[0, b] >= 0 for b in last)
+
+
+@pytest.mark.parametrize("algo", range(4))
+def test_a_token_drawn_from_the_last_target_row_sees_every_vector(algo):
+    # row 7 holds 2560 ones and, behind each of the first half of them, a 1.5e-8 that a 32-bit sum of two vectors loses: half of the
+    # row's mass ends within the first half, 1e-5 before the place where it would end without them
+    from paper_2403_10444_b200 import binding as bv
+    V, gone = 20480, float("-inf")
+    row = torch.full((V // 128, 32, 4), gone)                   # (runs of 32 vectors, two to a sub-segment)
+    row[0::2, :, 0] = 0.0
+    row[1:V // 256:2, :, 0] = -18.0
+    tt = torch.full((V, V), gone, device="cuda")
+    tt[0, 7] = 0.0
+    tt[7] = row.flatten().cuda()
+    dt = torch.full((V, V), gone, device="cuda")
+    dt[0, 7] = 0.0
+    first = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    u = torch.full((1, 1, 3), 0.5, device="cuda")
+    tokens = bv.bv_decode_loop(tt, dt, first, u[:, :, :1].contiguous(), u, 1, 1.0, algo)[0]
+    assert bv.bv_last_launch_count() == 1
+    assert tokens[0].tolist() == [7, V // 2 - 132]
