@@ -323,15 +323,16 @@ int bv_draft_chain(const void* draft_table, const int32_t* first_tokens, const f
  * tokens for every one of B sequences (as bv_draft_chain, from the sequence's last token, with u_draft [iterations,
  * gamma, B]), verifies the block on the table rows along the drafted path, read where they lie (u_verify [iterations, B,
  * gamma+2]; algo: 0 Algorithm 2 and 1 Algorithm 1 with the drafting step's normalisers, 2 and 3 the same without), and
- * appends the emitted tokens to the sequence.  One launch for all of it where two rows fit in an SM's shared memory (up to
- * 106496 bytes a row), else two an iteration; no synchronisation; DEVICE pointers:
+ * appends the emitted tokens to the sequence.  One launch for all of it where that was measured faster (two rows in an SM's
+ * shared memory, up to 106496 bytes each, and not too many sequences and drafted tokens for them), else two an iteration; no
+ * synchronisation; DEVICE pointers:
  *   first_tokens [B] int32     the last token of each context
  *   out_tokens  [B, iterations (gamma+1)] int32: the tokens generated, then -1;  out_lengths [B] int64: how many
  *   out_tau     [iterations, B] int32 accepted drafts;  out_drafted [iterations, B, gamma] int32
  *   out_fault   [1] int32: 1 if a sequence reported a data fault (its further tokens mean nothing).  Of Algorithm 2's rows the
  *               last target row counts, where position gamma is not selected, only in batches that are small enough for the
  *               small-batch kernel (up to 32 sequences)
- *   work        B (2 gamma + 3) int32
+ *   work        B (2 gamma + 3) int32 (of no use to a call that is one launch, but not null)
  * Rows must be whole 16-byte vectors on 16-byte aligned bases and B at most 768, else BV_ERR_UNSUPPORTED; whether a kernel
  * takes the call, and its workspace, is settled before anything is enqueued.
  */
@@ -357,6 +358,8 @@ int bv_stream_status(void* stream);
  *                   middling batches and for rows that are not whole 16-byte vectors, the element-wise kernel for
  *                   a few short ones of these a sequence, else the flow kernel; where fewer SMs than the GPU has can
  *                   be had at once, the flow or the element-wise kernel)
+ *   "loop"          bv_decode_loop: 1 in one launch wherever two rows fit in shared memory, 2 in two launches an iteration (the
+ *                   default where "kernel" is set, which chooses among the kernels of those)
  *   "small_bytes"   logit megabytes up to which the small-batch kernel is the default
  *   "cluster"       cluster width of the cluster / streaming kernels (1, 2, 4, 8)
  *   "max_clusters"  cap on the clusters those kernels launch

@@ -69,6 +69,7 @@ constexpr int kStreamSlots = 32;  // streams per device that keep a workspace of
 // Tuning and test options (bv_set_option); their first values come from the environment, read once.
 struct Options {
     int kernel = 0;        // 0: chosen by shape; 1 flow, 2 cluster, 3 stream, 4 small-batch, 5 phase
+    int loop = 0;          // the decoding loop: 0 by shape, 1 in one kernel wherever two rows fit in shared memory, 2 in two launches an iteration
     int small_bytes = 0;   // logit bytes (in MB) up to which the small-batch kernel is chosen; 0: the built-in limit
     int cluster = 0;       // cluster width of the cluster / stream kernels (1, 2, 4, 8); 0: chosen by shape
     int max_clusters = 0;  // cap on the clusters launched; 0: none
@@ -697,10 +698,10 @@ bool small_takes_tables(int algo, bool lse, int B, int gamma, size_t row_bytes) 
     return small_fits(B, gamma) &&
            static_cast<long long>(B) * (2 * gamma + 1) * static_cast<long long>(row_bytes) <= kPhaseBytes[algo != kBlockVerify ? 0 : lse ? 2 : 1][0];
 }
-int kernel_option() {
+int loop_option() {
     std::call_once(g_opt_once, load_env_options);
     std::lock_guard<std::mutex> lock(g_mu);
-    return g_opt.kernel;
+    return g_opt.loop ? g_opt.loop : g_opt.kernel ? 2 : 0;
 }
 
 int run_tables(int algo, const void* tgt_table, const void* drf_table, const int32_t* first, const int32_t* tok, const float* uni,
@@ -836,6 +837,7 @@ int bv_set_option(const char* name, int value) {
     std::call_once(g_opt_once, load_env_options);
     std::lock_guard<std::mutex> lock(g_mu);
     if (!std::strcmp(name, "kernel")) g_opt.kernel = value;
+    else if (!std::strcmp(name, "loop")) g_opt.loop = value;
     else if (!std::strcmp(name, "small_bytes")) g_opt.small_bytes = value;
     else if (!std::strcmp(name, "cluster")) g_opt.cluster = value;
     else if (!std::strcmp(name, "max_clusters")) g_opt.max_clusters = value;

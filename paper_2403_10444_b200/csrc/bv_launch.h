@@ -21,8 +21,9 @@ int run_tables(int algo, const void* tgt_table, const void* drf_table, const int
 // Does the small-batch kernel take these (else the phase kernel does)?
 bool small_takes_tables(int algo, bool lse, int B, int gamma, size_t row_bytes);
 
-// The option "kernel" (0: chosen by shape).
-int kernel_option();
+// How the decoding loop runs: 0 by shape, 1 in one kernel wherever that fits, 2 in two launches an iteration (as where the option
+// "kernel" names one of theirs).
+int loop_option();
 
 // The decoding loop in one kernel (bv_loop.cu), a CTA per sequence, for rows of which two fit in shared memory.
 struct LoopArgs {
@@ -44,6 +45,7 @@ struct LoopArgs {
     int32_t* fault;           // set if a sequence reports a data fault
 };
 bool loop_fits(int V, int dtype);
+bool loop_pays(int V, int dtype, int B, int gamma, bool token, int sms);
 cudaError_t launch_loop(const LoopArgs& args, int dtype, cudaStream_t stream);
 
 // Most clusters of `cluster` CTAs of the streaming kernel that can be resident at once

@@ -222,7 +222,12 @@ extern "C" int bv_decode_loop(const void* target_table, const void* draft_table,
     bv::note_launches(0);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e;
-    if (bv::loop_fits(V, dtype) && bv::kernel_option() == 0) {
+    int dev = 0, sms = 0;
+    const int how = bv::loop_option();
+    if (how == 0 && ((e = cudaGetDevice(&dev)) != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess))
+        return bv::note_cuda_error(e);
+    const bool fits = bv::loop_fits(V, dtype);
+    auto one_kernel = [&]() -> int {
         const double kd = 1.4426950408889634073599246810019 / static_cast<double>(temperature);
         // (a last target row that is not wanted: the small-batch kernel sweeps every row and faults the sequence, the phase kernel does
         // not look; of a loop's calls, which of them takes it decides)
@@ -233,7 +238,8 @@ extern "C" int bv_decode_loop(const void* target_table, const void* draft_table,
         if ((e = cudaMemsetAsync(out_fault, 0, 4, st)) != cudaSuccess || (e = bv::launch_loop(args, dtype, st)) != cudaSuccess) return bv::note_cuda_error(e);
         bv::note_launches(1);
         return BV_OK;
-    }
+    };
+    if (fits && (how == 1 || (how == 0 && bv::loop_pays(V, dtype, B, gamma, algo & 1, sms)))) return one_kernel();
     // work: last tokens, the last verification's outputs, the draft rows' normalisers
     int32_t* cur = work;
     int32_t* out = cur + b;
@@ -244,6 +250,8 @@ extern "C" int bv_decode_loop(const void* target_table, const void* draft_table,
                               u_verify + n * b * (gamma + 2), algo < 2 ? lse : nullptr, B, gamma, V, dtype, temperature, out, out_len, probe, st);
     };
     int rc = verify(0, true);
+    const bool other = fits && how == 0;      // (where too few SMs can be had for the verification's kernels, the one kernel needs none at once)
+    if (rc == BV_ERR_UNSUPPORTED && other) return one_kernel();
     if (rc != BV_OK) return rc;               // (before anything is enqueued)
     if ((e = cudaMemcpyAsync(cur, first_tokens, b * 4, cudaMemcpyDeviceToDevice, st)) != cudaSuccess ||
         (e = cudaMemsetAsync(out_tokens, 0xff, b * width * 4, st)) != cudaSuccess ||      // (-1)
@@ -255,7 +263,9 @@ extern "C" int bv_decode_loop(const void* target_table, const void* draft_table,
     for (int n = 0; n < iterations; ++n) {
         if ((e = launch_chain(draft_table, cur, u_draft + n * b * gamma, B, gamma, V, dtype, temperature, out_drafted + n * b * gamma, lse, loop, st)) != cudaSuccess)
             return bv::note_cuda_error(e);
-        if ((rc = verify(n, false)) != BV_OK) return rc;
+        rc = verify(n, false);
+        if (rc == BV_ERR_UNSUPPORTED && other && n == 0) return one_kernel();      // (it writes all outputs anew)
+        if (rc != BV_OK) return rc;
         loop.out_len = out_len;
         loop.tau = out_tau + n * b;
         launches += 2;

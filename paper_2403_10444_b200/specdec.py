@@ -46,7 +46,7 @@ def run(target_table: torch.Tensor, draft_table: torch.Tensor, first_tokens: tor
     (the iteration number lives in a device counter), so with ``graph=True`` one iteration is
     captured in a CUDA graph and replayed: the launches of an iteration then cost one graph launch
     instead of one driver call each.  Data faults are looked for once, after the last iteration.
-    By default the loop runs natively (``bv_decode_loop``): one launch, or two per iteration for rows above 104 KB.
+    By default the loop runs natively (``bv_decode_loop``): one launch, or two per iteration where that is faster.
     ``chain``: the gamma drafted tokens of an iteration come from one launch of ``bv_draft_chain``
     (default) instead of gamma calls of ``bv_sample_draft`` with their look-ups and copies.
     """

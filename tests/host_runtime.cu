@@ -223,6 +223,7 @@ int host_tables(int algo, int B, int gamma, int V, int dtype, int lse, int probe
                           B, gamma, V, dtype, 1.f, static_cast<int32_t*>(x), static_cast<int32_t*>(x), probe != 0, nullptr);
 }
 int host_launches() { return g_launches; }
+int host_loop_pays(int V, int dtype, int B, int gamma, int token) { return bv::loop_pays(V, dtype, B, gamma, token != 0, 148); }
 // which of the elements of `esz` bytes at p lie in [lo, hi)
 void host_elements_inside(unsigned long long p, unsigned long long lo, unsigned long long hi, int esz, int* first, int* n) {
     const char *a = reinterpret_cast<const char*>(p), *b = reinterpret_cast<const char*>(lo), *c = reinterpret_cast<const char*>(hi);

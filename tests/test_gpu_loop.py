@@ -13,8 +13,9 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("dtype,V,B,gamma,N", [("bf16", 8, 5, 1, 6), ("bf16", 40, 9, 3, 5), ("f32", 2052, 7, 5, 4), ("bf16", 4104, 33, 4, 4), ("bf16", 16376, 8, 2, 3),
                                                ("bf16", 16384, 150, 3, 3), ("f32", 8192, 6, 34, 2), ("bf16", 1024, 3, 64, 3), ("f32", 26624, 3, 2, 2), ("f32", 26628, 3, 2, 2)])
 @pytest.mark.parametrize("sigma_d", [0.2, 1.0])
-def test_one_kernel_generates_what_the_steps_generate(dtype, V, B, gamma, N, sigma_d):
+def test_one_kernel_generates_what_the_steps_generate(dtype, V, B, gamma, N, sigma_d, bv_options):
     import paper_2403_10444_b200 as bv
+    bv_options("loop", 1)
     tt, dt = wl.markov_models(V, dtype, V + gamma, 2.0, sigma_d, 1.1 if V > 8 else 0.0, "cuda")
     ud, uv = wl.loop_uniforms(N, B, gamma, V, "cuda")
     first = torch.arange(B, dtype=torch.int32, device="cuda") % V
