@@ -120,13 +120,16 @@ __device__ __forceinline__ float pow2_nonpos(float d) {
 // to within its last bit, 1e31, and 2 to the power of that difference spoils the sum.
 constexpr float kNoRef = -1.0e30f;
 
-// A sum taken against one reference, against another one that lies d below (d <= 0).  From 2^31 on a float reference is an integer
-// only to within 128 and more, so the sum of logits of that size, as masks of -1e10 or -1e20 are, may have overflowed; against
-// a reference that leaves nothing of it it is zero all the same (not inf x 0), and only a NaN stays one.
-template <class Sum> __device__ __forceinline__ Sum ref_moved(Sum s, float d) {
-    const float to = pow2_nonpos(d);
-    return to > 0.f || s != s ? s * static_cast<Sum>(to) : Sum(0);
+// From 2^31 on a float reference is an integer only to within 128 and more, so the sum of logits of that size, as masks of -1e10 or
+// -1e20 are, may overflow.  Against a reference that leaves nothing of it, it has to be zero all the same, and inf x 0 is not: such a sum is
+// held at kTooLarge, beyond any that row_sum_ok takes for a normaliser.  A NaN stays one.
+constexpr float kTooLarge = 0x1.8p127f;
+__device__ __forceinline__ float ref_keep(float s) {
+    float r;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(s), "f"(kTooLarge));
+    return r;
 }
+__device__ __forceinline__ double ref_keep(double s) { return s > static_cast<double>(kTooLarge) ? static_cast<double>(kTooLarge) : s; }
 
 // Running sum of 2^{z*k - M} over the elements a thread has seen, where the
 // reference M is an INTEGER (the rounded scaled maximum so far).  An integer
@@ -141,7 +144,7 @@ struct MaxSum {
 #pragma unroll
         for (int e = 1; e < N; ++e) vm = fmaxf(vm, v[e]);
         const float y = rintf(vm * kf);
-        if (y > M && y > kNoRef) { s = ref_moved(s, M - y); M = y; }
+        if (y > M && y > kNoRef) { s = ref_keep(s) * pow2_nonpos(M - y); M = y; }
         if (M > -INFINITY) {
             const float nM = -M;
 #pragma unroll
@@ -158,7 +161,7 @@ __device__ __forceinline__ void warp_combine(float& M, float& s) {
     float Mw = M;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) Mw = fmaxf(Mw, __shfl_xor_sync(0xffffffffu, Mw, off));
-    s = ref_moved(s, M - Mw);
+    s = ref_keep(s) * pow2_nonpos(M - Mw);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
     M = Mw;
@@ -395,12 +398,16 @@ __device__ __forceinline__ uint4 lds128(uint32_t saddr) {
 // Without a raise every term is below 12, so its exponent is below 4 and is rounded to 1.2e-7.
 constexpr float kRaiseBound = 12.f;
 
-// s 2^{own - row}: a sum against its own reference, against the row's, which is no lower (no own reference: nothing but a NaN is left)
-template <class Sum> __device__ __forceinline__ Sum ref_sum(Sum s, float own, float row) {
-    return ref_moved(s, own > kNoRef ? own - row : -INFINITY);
+// 2^d for d = (own reference) - (row reference) <= 0, or 0 when there is no own reference
+__device__ __forceinline__ float ref_scale(float own, float row) {
+    return own > kNoRef ? pow2_nonpos(own - row) : 0.f;
 }
-// Is Z, the sum of a row with a finite maximum, a normaliser?  NaN: the row holds one.  Zero or infinite: its largest scaled logit is
+// a sum against its own reference, against the row's
+__device__ __forceinline__ float ref_sum(float s, float own, float row) { return ref_keep(s) * ref_scale(own, row); }
+__device__ __forceinline__ double ref_sum(double s, float own, float row) { return ref_keep(s) * static_cast<double>(ref_scale(own, row)); }
+// Is Z, the sum of a row with a finite maximum, a normaliser?  NaN: the row holds one.  Zero or overflowed: its largest scaled logit is
 // beyond 2^31 either way, the reference lies further off it than an exponent reaches, and nothing is known of the row.
-__device__ __forceinline__ bool row_sum_ok(double Z) { return Z > 0.0 && Z < static_cast<double>(INFINITY); }
+// (Between 0 and 2^127 by the high word alone, one integer comparison on the small-batch kernel's serial way.)
+__device__ __forceinline__ bool row_sum_ok(double Z) { return static_cast<unsigned>(__double2hiint(Z)) - 1u < 0x47dfffffu; }
 
 }  // namespace bv

@@ -215,9 +215,9 @@ static __device__ __forceinline__ void ph_reduce_rows(const PhaseScratch& ps, in
                 float mm = m;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) mm = fmaxf(mm, static_cast<float>(v[j].x));
-                s = ref_sum(s, m, mm);
+                s *= static_cast<double>(ref_scale(m, mm));
 #pragma unroll
-                for (int j = 0; j < 8; ++j) s += ref_sum(v[j].y, static_cast<float>(v[j].x), mm);
+                for (int j = 0; j < 8; ++j) s += v[j].y * static_cast<double>(ref_scale(static_cast<float>(v[j].x), mm));
                 m = mm;
             }
 #pragma unroll
@@ -256,11 +256,11 @@ static __device__ __forceinline__ void ph_reduce_rows(const PhaseScratch& ps, in
             for (int p = lane + 32; p < np[q]; p += 32) {
                 const double2 w = __ldcg(&ps.part[(static_cast<size_t>(b) * rows + r) * slots + p]);
                 const float wm = static_cast<float>(w.x), mm = fmaxf(m, wm);
-                s = ref_sum(s, m, mm) + ref_sum(w.y, wm, mm);
+                s = s * static_cast<double>(ref_scale(m, mm)) + w.y * static_cast<double>(ref_scale(wm, mm));
                 m = mm;
             }
             const float mr = warp_max(m);
-            s = warp_sum_d(ref_sum(s, m, mr));
+            s = warp_sum_d(s * static_cast<double>(ref_scale(m, mr)));
             const int c = r < g ? r : r - g;                  // target row c or draft row c
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -455,7 +455,7 @@ static __device__ __noinline__ void ph_finalize(const Params& prm, const PhaseSc
         auto at = [&](int i) -> double {
             if (i >= units) return 0.0;
             const double w = __ldcg(&seg[i]);
-            return c == g && !PROBS ? ref_sum(w, __ldcg(&seg_M[i]), Mr) : w;
+            return c == g && !PROBS ? w * static_cast<double>(ref_scale(__ldcg(&seg_M[i]), Mr)) : w;
         };
         const double mine = ph_lane_sum(at, per, lane), total = warp_sum_d(mine);
         bool pass;
@@ -681,13 +681,13 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
                 if (st == 0) M = fmaxf(rintf(warp_max(fmaxf(vec_max<EPV>(va), vec_max<EPV>(vb))) * kf), kNoRef);
                 const float was = M;
                 f_step_sweep1_single<EPV>(va, vb, kf, M, s);
-                if (M != was) sd = ref_sum(sd, was, M);
-                if ((st & 15) == 15) { sd += static_cast<double>(s); s = 0.f; }       // (32-bit sums stay short)
+                if (M != was) sd *= static_cast<double>(ref_scale(was, M));
+                if ((st & 15) == 15) { sd += static_cast<double>(ref_keep(s)); s = 0.f; }       // (32-bit sums stay short)
                 advance(rp);
                 rp += kPhSlotBytes;
                 if (rp == ring_end) rp = ring;
             }
-            sd = warp_sum_d(sd + static_cast<double>(s));
+            sd = warp_sum_d(sd + static_cast<double>(ref_keep(s)));       // (so it is not infinite where it is scaled)
             const int slot = kw - (b * rows + j) * units / ps.per1;
             if (lane == 0) __stcg(&ps.part[(static_cast<size_t>(b) * rows + j) * ps.slots + slot], make_double2(static_cast<double>(M), sd));
             arrived += static_cast<unsigned>(n);
@@ -809,7 +809,7 @@ __global__ void __launch_bounds__(kPhThreads, 1) verify_phase_kernel(const __gri
                         }
                         acc = warp_sum_d(acc);
                         if (lane == 0) {
-                            __stcg(&seg[v / kPhUnit], acc);
+                            __stcg(&seg[v / kPhUnit], PROBS ? acc : ref_keep(acc));
                             if (!PROBS) __stcg(&seg_M[v / kPhUnit], M);
                         }
                         advance(rp);

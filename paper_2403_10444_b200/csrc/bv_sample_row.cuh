@@ -180,7 +180,7 @@ __device__ __forceinline__ int s_locate(const SubSegment<SHORT>* seg, float u, i
     }
     const double total = shfl_d(inc, 31);
     // a row with a NaN or +inf logit has a NaN / infinite sum or reference; one without a finite logit has none
-    const bool ok = Mrow > kNoRef && Mrow < INFINITY && Z > 0.0 && Z < INFINITY && total > 0.0 && total < static_cast<double>(INFINITY);
+    const bool ok = Mrow > kNoRef && Mrow < INFINITY && row_sum_ok(Z) && row_sum_ok(total);
     if (release_pairs >= 0) named_bar_arrive(release_pairs, kSAllThreads);   // (the pairs are in registers: their buffer may be written again)
     norm[0] = Mrow;
     norm[1] = Z;

@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __
             if (warp == 0) {                  // (the next item's shares go to the other half, and the barrier after it is behind this)
                 const float m = lane < kSmWarps ? sh.wM[turn][lane] : kNoRef;
                 const float Mc = warp_max(m);
-                double z = lane < kSmWarps ? ref_sum(static_cast<double>(sh.wS[turn][lane]), m, Mc) : 0.0;
+                double z = lane < kSmWarps ? static_cast<double>(ref_keep(sh.wS[turn][lane])) * static_cast<double>(ref_scale(m, Mc)) : 0.0;
                 z = warp_sum_d(z);
                 if (lane == 0) __stcg(&sc.part[static_cast<size_t>(rid) * nch + item % nch], make_double2(static_cast<double>(Mc), z));
             }
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __
             if (warp == 0) {
                 const float m = lane < kSmWarps ? sh.wM[0][lane] : kNoRef;
                 const float Mc = warp_max(m);
-                double z = lane < kSmWarps ? ref_sum(static_cast<double>(sh.wS[0][lane]), m, Mc) : 0.0;
+                double z = lane < kSmWarps ? static_cast<double>(ref_keep(sh.wS[0][lane])) * static_cast<double>(ref_scale(m, Mc)) : 0.0;
                 z = warp_sum_d(z);
                 if (lane == 0) sc.part[static_cast<size_t>(rid) * nch + ch] = make_double2(static_cast<double>(Mc), z);
             }
@@ -322,9 +322,9 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __
                 float mm = M;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) mm = fmaxf(mm, static_cast<float>(p[j].x));
-                Z = ref_sum(Z, M, mm);
+                Z *= static_cast<double>(ref_scale(M, mm));
 #pragma unroll
-                for (int j = 0; j < 8; ++j) Z += ref_sum(p[j].y, static_cast<float>(p[j].x), mm);
+                for (int j = 0; j < 8; ++j) Z += p[j].y * static_cast<double>(ref_scale(static_cast<float>(p[j].x), mm));
                 M = mm;
             }
             sh.rowM[rid] = M;

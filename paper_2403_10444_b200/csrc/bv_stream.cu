@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(kThreads, 1) verify_stream_kernel(const Params
                     float Mc = M;
 #pragma unroll
                     for (int off = 16; off > 0; off >>= 1) Mc = fmaxf(Mc, __shfl_xor_sync(0xffffffffu, Mc, off));
-                    s = ref_moved(s, M - Mc);
+                    s = ref_keep(s) * static_cast<double>(pow2_nonpos(M - Mc));
 #pragma unroll
                     for (int off = 16; off > 0; off >>= 1) s += shfl_xor_d(s, off);
                     if (lane < C) {
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(kThreads, 1) verify_stream_kernel(const Params
                 float Mr = M;
 #pragma unroll
                 for (int off = 4; off > 0; off >>= 1) Mr = fmaxf(Mr, __shfl_xor_sync(0xffffffffu, Mr, off));
-                s = ref_moved(s, M - Mr);
+                s = ref_keep(s) * static_cast<double>(pow2_nonpos(M - Mr));
 #pragma unroll
                 for (int off = 4; off > 0; off >>= 1) s += shfl_xor_d(s, off);
                 const float MQ = __shfl_sync(0xffffffffu, Mr, 8);

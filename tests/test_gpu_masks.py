@@ -88,3 +88,14 @@ def test_a_row_without_a_normaliser_is_a_data_fault(kernel, V, value, T, bv_opti
         for b in range(8):
             # (Algorithm 1 may end before it gets to the row)
             assert out[1][b] == -1 or (algo == oracle.TOKEN_VERIFY and out[1][b] == ref.out_len[b] <= b % 3), (algo, b)
+
+
+@pytest.mark.parametrize("value,T", [(-1e10, 1.3), (-1e10, 1.0), (-3e10, 1.3), (1e10, 1.0)])
+@pytest.mark.parametrize("V", [1024, 65536])
+def test_nothing_is_drawn_from_a_row_without_a_normaliser(V, value, T):
+    import paper_2403_10444_b200 as bv
+    z = torch.randn((6, V), generator=torch.Generator().manual_seed(1)).bfloat16()
+    z[1::2] = value
+    tok, lse = bv.bv_sample_draft(z.cuda(), torch.full((6,), 0.3, device="cuda"), T)
+    assert (tok[1::2] == -1).all() and torch.isnan(lse[1::2]).all()
+    assert (tok[0::2] >= 0).all() and torch.isfinite(lse[0::2]).all()
