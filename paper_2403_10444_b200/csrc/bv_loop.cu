@@ -479,28 +479,28 @@ bool loop_fits(int V, int dtype) { return 2 * static_cast<size_t>(V) * (dtype ==
 
 // Where one kernel is the faster loop.  A CTA here sweeps its sequence's rows alone and its candidates one after the other; the two
 // launches of an iteration share the batch's candidates over all SMs, but wait for the whole batch twice.  So it is a matter of the
-// sequences to an SM (at work at once: 2 with rows of up to 51200 bytes, else 1), of the steps that a sweep takes (kLoopRuns runs of
+// sequences to an SM (at work at once: 2 with rows of up to 53200 bytes, else 1), of the steps that a sweep takes (kLoopRuns runs of
 // 16 warps: 2048 vectors each) and of gamma, with which the candidates grow.  Per length of a row, and for up to 8 sequences, 24, one to an
-// SM, 2, 3, 4 and more: the largest gamma at which this kernel was measured faster (Algorithm 2).  Measured over 7300 calls of 38
+// SM, 2, 3, 4 and more: the largest gamma at which this kernel was measured faster (Algorithm 2).  Measured over 8400 calls of 40
 // lengths from 1024 to 53248, drafts of noise 0.1 to 3, against the faster of the two launches as they are and as they were when this
 // kernel came; time over theirs, bf16, noise 0.2 / 0.4 / 0.7:
 //   V = 16384 gamma = 8: B = 1 0.74 / 0.70 / 0.81, 148 0.57 / 0.55 / 0.53, 296 0.70 / 0.66 / 0.66, 768 0.77 / 0.78 / 0.80
 //   V = 2048 gamma = 8: B = 148 0.67, 297 0.81 / 0.89 / 0.91, 450 1.02 / 1.05 / 1.06, 768 1.15;  gamma = 3: 768 0.89 / 0.94 / 0.96
 //   V = 24576 gamma = 8: B = 4 1.03 / 1.12 / 1.00, 148 0.82 / 0.74 / 0.69, 768 0.98 / 1.01 / 1.02;  gamma = 16: B = 4 1.12 / 1.24 / 1.15, 148 0.97 / 0.89 / 0.87
 //   V = 32768 (one CTA to an SM) gamma = 3: B = 149 0.67, 297 0.74, 768 1.00 / 1.02 / 1.06;  gamma = 12: B = 64 0.89 / 0.94 / 0.81, 149 1.09 / 1.10 / 1.13
-//   V = 51200 gamma = 5, noise 1: B = 1 1.22, 32 0.95, 128 0.86, 150 1.18, 768 1.39
+//   V = 51200 gamma = 5, noise 1: B = 1 1.22, 32 0.95, 128 0.86, 150 1.18, 768 1.39;  gamma = 1, noise 0.2 / 0.7: B = 1 0.58 / 0.59, 444 0.80 / 0.88, 768 1.04 / 1.11
 // Within the lines 2 of 4400 calls were 3 % or more slower than the loop that this kernel replaced (3 and 6 %).  Algorithm 1, which has
 // one candidate, gains up to half as much gamma again (V = 17000: gamma = 6 / 10, B = 4 0.83 / 1.01, B = 149 0.84 / 1.01), and up to
 // twice where every sequence has an SM (V = 36864, B = 148: gamma = 16 0.84).
 bool loop_pays(int V, int dtype, int B, int gamma, bool token, int sms) {
     struct Line { int V; unsigned char gamma[7]; };
     static constexpr Line kBf16[] = {{3072, {12, 16, 16, 8, 8, 4, 3}},      {6144, {12, 32, 32, 12, 8, 8, 5}}, {10240, {16, 32, 32, 16, 16, 16, 12}},
-                                     {16384, {16, 32, 32, 32, 32, 32, 32}}, {20000, {5, 6, 16, 8, 6, 4, 3}},   {25600, {5, 6, 16, 8, 8, 6, 5}},
-                                     {32768, {5, 16, 32, 5, 3, 0, 0}},      {34816, {2, 2, 6, 2, 0, 0, 0}},    {49152, {2, 3, 8, 2, 0, 0, 0}},
-                                     {53248, {0, 0, 5, 0, 0, 0, 0}},        {INT_MAX, {}}};
+                                     {16384, {16, 32, 32, 32, 32, 32, 32}}, {20000, {5, 6, 16, 8, 6, 4, 3}},   {26600, {5, 6, 16, 8, 8, 6, 5}},
+                                     {32768, {5, 16, 32, 5, 4, 2, 1}},      {34816, {2, 3, 6, 2, 2, 1, 1}},    {49152, {2, 3, 8, 3, 2, 1, 1}},
+                                     {53248, {2, 3, 5, 2, 1, 1, 0}},        {INT_MAX, {}}};
     static constexpr Line kF32s[] = {{1536, {16, 32, 32, 24, 16, 12, 8}},   {3072, {32, 32, 32, 32, 16, 16, 12}}, {6144, {32, 32, 32, 32, 16, 16, 16}},
-                                     {8192, {64, 64, 64, 64, 64, 64, 64}},  {12800, {8, 16, 32, 32, 32, 32, 32}}, {16384, {8, 16, 24, 10, 8, 6, 3}},
-                                     {24576, {5, 6, 16, 5, 5, 3, 0}},       {26624, {2, 2, 8, 2, 2, 2, 0}},          {INT_MAX, {}}};
+                                     {8192, {64, 64, 64, 64, 64, 64, 64}},  {13300, {8, 16, 32, 32, 32, 32, 32}}, {16384, {8, 16, 24, 10, 8, 6, 3}},
+                                     {24576, {5, 6, 16, 5, 5, 3, 2}},       {26624, {2, 2, 8, 3, 3, 2, 1}},       {INT_MAX, {}}};
     const int load = B <= 8 ? 0 : B <= 24 ? 1 : B > 4 * sms ? 6 : 2 + (B - 1) / sms;
     const Line* line = dtype == kF32 ? kF32s : kBf16;
     while (V > line->V) ++line;
