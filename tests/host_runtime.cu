@@ -142,9 +142,11 @@ cudaError_t fake_launch_small(const Params& prm, const SmallScratch& sc, int, bo
     return enqueue(st, [=] {
         inside("status word", prm.status, 4);
         zeros("barrier words", sc.barrier, 17 * 4);
+        zeros("counters of the sequences", sc.seq, kSmallMaxB * 4);
         scratch("chunk pairs", sc.part, B * (2 * g + 1) * sc.nch * sizeof(double2));
         scratch("segment totals", sc.seg, B * (g + 1) * sc.np * 16 * sizeof(double));
         zeros("barrier words beside the scratch", sc.barrier, 17 * 4);
+        zeros("counters of the sequences beside the scratch", sc.seq, kSmallMaxB * 4);
     });
 }
 cudaError_t fake_launch_flow(const Params& prm, const FlowScratch& fl, int, int, cudaStream_t st) {
