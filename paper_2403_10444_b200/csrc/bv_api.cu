@@ -16,21 +16,24 @@ namespace {
 
 constexpr int kMaxDevices = 64;
 constexpr int kTicketSlots = 64;  // concurrent calls of the cluster kernels on one device each need their own slot
-// Logit bytes up to which the small-batch kernel is the default (measured against the flow kernel at
-// V = 152064, B <= 32: Algorithm 2 gains up to about 90 MB at low and high acceptance alike, Algorithm 1,
-// whose one residual sweep per sequence is cheap, up to about 160 MB).  The phase kernel takes over below that, but for few
-// sequences or many positions swept (phase_pays).
+// Logit bytes up to which the small-batch kernel is the default (against the flow kernel, drafts of noise 0.1 / 0.7: Algorithm 2,
+// V = 256000, gamma = 16, B = 5 (81 MB) 72 / 55 us against 72 / 66, 6 (97 MB) 84 / 52 against 73 / 67; Algorithm 1, gamma = 8, noise
+// 0.1 / 0.7 / 3, B = 18 (149 MB) 73 / 74 / 74 against 85 / 77 / 51, 22 (183 MB) 73 / 74 / 74 against 87 / 81 / 66).  The phase kernel
+// takes over below that, but for few sequences or many positions swept (phase_pays).
 constexpr long long kSmallBytes[2] = {160LL << 20, 90LL << 20};   // [algo]
 // Logit bytes between which the phase kernel is the default for rows of 16-byte vectors ({Algorithm 1, Algorithms 2 and 4,
 // Algorithm 2 with supplied normalisers}), and the sequences from which it is on probabilities.  Measured at V = 128256 bf16,
-// gamma = 8, drafts of noise 0.1 / 0.7 / 1.5, against the kernel that ran there before:
-//   Algorithm 2, B = 8 (35 MB): 50 / 52 / 47 us against 39 / 34 / 31 (small-batch); 16: 53 / 53 / 50 against 62 / 55 / 48;
+// gamma = 8, drafts of noise 0.1 / 0.7 / 1.5, against the small-batch kernel (as it is) and the flow kernel:
+//   Algorithm 2, B = 8 (35 MB): 42 / 41 / 39 us against 38 / 31 / 27 (small-batch); 12: 44 / 44 / 42 against 58 / 45 / 38; 14: 45 / 46 / 43
+//   against 60 / 47 / 40; 16: 49 / 48 / 45 against 60 / 48 / 40; in 32 bits 8 (70 MB): 50 / 48 / 46 against 46 / 35 / 32, 10: 57 / 51 / 49
+//   against 67 / 51 / 45 (the line was drawn for 16 bits and for a small-batch kernel with two barriers: it could lie 15 MB lower there, and higher here);
 //   33: 65 / 62 / 60 against 86 / 80 / 77 (flow); 128: 144 / 145 / 136 against 168 / 154 / 140; 200 (874 MB): 202 / 208 / 194
 //   against 230 / 218 / 195; the 2.2 GB of B = 256, V = 256000: 432 against 416 (the flow kernel overlaps the two sweeps)
-//   supplied normalisers, noise 0.7, B = 8 / 16 / 33 / 128 / 256: 46 / 48 / 52 / 101 / 164 us against 33 / 55 / 67 / 121 / 184
-//   Algorithm 1, noise 0.7, B = 16 / 33 / 64 / 128: 47 / 57 / 82 / 132 us against 46 / 77 / 90 / 115 (it reads all rows, the
-//   flow kernel the ones the tests need)
-//   probabilities, noise 0.7, B = 8 / 16 / 33 / 128 / 256: 26 / 29 / 31 / 49 / 72 us against 21 / 31 / 39 / 65 / 120
+//   supplied normalisers, noise 0.7, B = 8 / 10 / 12 / 16 (small-batch): 43 / 44 / 43 / 46 us against 31 / 44 / 41 / 50, 0.1: 44 / 47 / 43 / 46
+//   against 40 / 58 / 54 / 63; 33 / 128 / 256 (flow): 52 / 101 / 164 against 67 / 121 / 184
+//   Algorithm 1, noise 0.7, B = 12 / 16 / 18 / 24 (small-batch): 40 / 42 / 44 / 49 us against 35 / 35 / 49 / 53; 33 / 64 / 128 (flow): 57 / 82 / 132
+//   against 77 / 90 / 115 (it reads all rows, the flow kernel the ones the tests need)
+//   probabilities, noise 0.7, B = 33 / 128 / 256 (flow): 31 / 49 / 72 us against 39 / 65 / 120
 // The upper ends are lower for 32-bit logits, of which the flow kernel streams the more (half the arithmetic a byte; V = 256000,
 // gamma = 2, 312 MB: 103 us against 100; Algorithm 1, 296 MB: 81 against 73), and the one of Algorithm 1 is where a draft that
 // is hardly accepted leaves the flow kernel an eighth of the rows to read (23 sequences, noise 3, 238 MB: 53 us against 46).
@@ -39,18 +42,22 @@ constexpr long long kSmallBytes[2] = {160LL << 20, 90LL << 20};   // [algo]
 constexpr long long kPhaseBytes[3][2] = {{72LL << 20, 180LL << 20}, {64LL << 20, 860LL << 20}, {48LL << 20, 1400LL << 20}};
 constexpr long long kPhaseBytesF32[3] = {120LL << 20, 280LL << 20, 280LL << 20};
 constexpr long long kPhaseProbsPairs[2] = {36LL << 20, 140LL << 20}, kPhaseProbsPairsF32[2] = {24LL << 20, 110LL << 20};   // [algo] bytes of one row pair of every sequence
-// (Fewer sequences than this: small-batch kernel, gamma = 1 / 4, V = 8192, B = 12: 14 us against 20 / 24; V = 152064 18 / 21 against 24 / 28.)
+// (Fewer sequences than this: small-batch kernel.  One line for rows of any length and any gamma, noise 0.1 / 0.7, us against the phase
+// kernel's: V = 8192, gamma = 4, B = 12 15 / 14 against 23 / 22, 32 20 / 19 against 23 / 23; gamma = 8, 16 17 / 17 against 25 / 23, 24 27 / 21 against 25 / 24;
+// V = 32768, gamma = 8, 16 23 / 19 against 27 / 24, 24 36 / 27 against 28 / 26; V = 128256, gamma = 8, 12 37 / 26 against 26 / 27, 16 40 / 29 against 30 / 29, 24 63 / 40
+// against 32 / 29; Algorithm 1, gamma = 8, V = 128256, 16 17 / 19 against 23 / 23, 32 24 / 26 against 25 / 25.)
 constexpr int kPhaseProbsB = 17;
 // On probabilities, Algorithm 1 on more sequences than SMs: 256 of V = 32768 (34 MB of pairs) takes 1.09 times as long as in the
 // flow kernel, 250 of V = 8192 in 32 bits (16 MB) 1.19, 256 of V = 8192 in 16 (8 MB) as long.  Algorithm 2 with many positions:
 // gamma = 16, noise 0.1 / 1, B = 17 of V = 8192: 34 against 30 / 25 against 27 us (flow); of V = 32768: even / 1.29 times faster;
 // gamma = 64, B = 40 of V = 8192: 71 against 49.
 constexpr long long kPhaseProbsMany = 12LL << 20, kPhaseProbsRow = 60000;
-// Fewer sequences than this leave the phase kernel with rows in many pieces: B = 6, V = 152064, gamma = 8, 32-bit logits with
-// supplied normalisers (62 MB) 52 / 55 / 45 us against 48 / 42 / 38 in the small-batch kernel; B = 10 (bf16, 52 MB) 51 / 48 / 43 against 57 / 50 / 45;
+// Fewer sequences than this leave the phase kernel with rows in many pieces: V = 152064, gamma = 8, 32-bit logits with supplied
+// normalisers, B = 6 (62 MB) 53 / 50 / 46 us against 47 / 38 / 35 in the small-batch kernel, 7 50 / 50 / 47 against 54 / 39 / 36, without 52 / 52 / 49 against 51 / 37 / 34;
+// B = 10 (bf16, V = 128256, 44 MB) 47 / 44 / 42 against 58 / 44 / 39;
 // beyond its sizes V = 256000, 32-bit, gamma = 16, B = 3 (101 MB) 93 / 83 us (noise 0.1 / 1) against 75 / 66 (flow).  Algorithm 1, whose tests
-// the small-batch kernel makes as fast for any outcome: gamma = 8, 32-bit, V = 152064, B = 10 51 / 48 / 47 us against 41 / 43 / 43; gamma = 12
-// (bf16) 42 / 39 / 40 against 44 / 45 / 44.
+// the small-batch kernel makes as fast for any outcome: V = 256000, gamma = 8 (bf16), B = 10 (87 MB) 50 / 47 / 47 us (noise 0.1 / 0.7 / 3) against
+// 49 / 49 / 50; V = 152064, gamma = 12, B = 10 44 / 42 / 42 against 38 / 39 / 39, 12 47 / 45 / 45 against 52 / 52 / 52.
 constexpr int kPhaseFew = 8, kPhaseFewTv = 12;
 constexpr long long kPhaseFewRow = 700000;
 // With every position swept (diagnostic outputs): bytes of logits, for gamma below 12 and from there on, and bytes of one
@@ -58,7 +65,7 @@ constexpr long long kPhaseFewRow = 700000;
 // gamma = 4, B = 24 85 against 89; V = 152064 gamma = 16, B = 24 (241 MB) 141 against 125; V = 65536 gamma = 16, B = 64 1.05 times
 // faster.  32-bit: V = 152064 gamma = 4, B = 24 (131 MB) 0.88 times as fast; V = 32768 gamma = 4, B = 128 (151 MB) 1.07, gamma = 8 0.93
 // (285 MB); gamma = 12, V = 8192, B = 128 (105 MB) 0.95, B = 64 1.11.  Against the small-batch kernel: V = 152064 gamma = 8, B = 16
-// (bf16, 83 MB) 80 against 71 us; gamma = 4, B = 32 71 against 77.
+// (bf16, 83 MB) 76 against 68 us; gamma = 4, B = 24 64 against 67, 32 69 against 88.
 constexpr long long kPhaseAllBytes[2] = {360LL << 20, 144LL << 20}, kPhaseAllBytesLong[2] = {360LL << 20, 60LL << 20};
 constexpr long long kPhaseAllRows[2] = {2500000, 2200000}, kPhaseAllSmall = 1300000;
 constexpr size_t kSlotHead = 16384;   // first area of a stream's workspace: status word, barrier words, the phase kernel's counters
@@ -296,8 +303,8 @@ bool not_all_sms(cudaError_t e) {
 // 0.80 / 0.81; Algorithm 2: gamma = 1 0.90.
 // Drafts that are hardly accepted at all, which Algorithm 1 leaves after a row, are up to a third faster here at any gamma, the
 // others up to seven times slower: the lines lie where the three noises together are even.  Against the small-batch kernel:
-//   Algorithm 1, B = 32: V = 1003 gamma = 1 0.88, 2: 0.92 / 0.90 / 0.84; V = 4099 1.07; V = 16421 0.90 / 0.85 / 0.81, 0.97 / 0.93 / 0.88;
-//   V = 8209 in 32 bits 0.86, 0.87 / 0.85 / 0.81
+//   Algorithm 1, B = 32: V = 1003 gamma = 1 0.85 / 0.82 / 0.76, 2: 0.82 / 0.82 / 0.78; V = 4099 0.95 / 0.93 / 0.91, 1.02 / 1.01 / 0.96; V = 16421
+//   0.99 / 0.98 / 0.92, 0.99 / 0.96 / 0.85; V = 8209 in 32 bits, gamma = 1, 0.93 / 0.91 / 0.90;  B = 24: V = 16421 0.97 / 0.96 / 0.91, 1.18 / 1.14 / 1.01
 bool elements_pay(int algo, const bv::Params& prm, const DeviceState& d, const Options& opt, size_t row_bytes) {
     const int g = prm.gamma;
     if (bv::small_fits(prm.B, g)) return algo == bv::kTokenVerify && g <= 2 && (row_bytes <= 4200 || (prm.B >= 24 && row_bytes > 16500 && row_bytes <= 33000));
@@ -456,11 +463,10 @@ int run_device(int algo, const void* tgt, const void* drf, const int32_t* tok, c
         if ((rc = run_phase(*d, prm, dtype, vec, ex.probe, stream)) <= BV_OK) return rc;
     }
 
-    // A few sequences whose logits fit in L2: the launch is a matter of latency, and the kernel with two
-    // grid-wide barriers instead of queues takes half the time of the flow kernel or less.
+    // A few sequences whose logits fit in L2: the launch is a matter of latency, and the kernel with one grid-wide
+    // barrier (none on probabilities) instead of queues takes half the time of the flow kernel or less.
     const long long small_limit = opt.small_bytes > 0 ? static_cast<long long>(opt.small_bytes) << 20 : kSmallBytes[algo == bv::kBlockVerify ? 1 : 0];
-    // (given probabilities only a few row pairs per sequence are read whatever the size of the rest: there the
-    // small-batch kernel wins up to 16 sequences, 17 against 33 us for one, 33 against 38 us for sixteen)
+    // (given probabilities only a few row pairs per sequence are read whatever the size of the rest: kPhaseProbsB)
     if ((vec || !only_vec) && !elements && bv::small_fits(B, gamma) &&
         (opt.kernel == 4 || ((opt.kernel == 0 || prm.first != nullptr) && (prm.probs ? B <= 16 : logit_bytes <= small_limit)))) {
         int& nc = d->small_ctas[dtype];

@@ -2,8 +2,11 @@
 // in every step of it (Algorithms 1 and 2 look at one block), so a CTA takes a sequence through all iterations and nothing is
 // ever exchanged between CTAs, nor left in memory between steps but the rows themselves.
 //
-// A drafting step is the sweep of the draft row of the last token by 16 streaming warps and the draw by one more (the
-// sampler's device functions: the same arithmetic and the same tokens as bv_draft_chain).  Both models' rows of a step are
+// A drafting step is the sweep of the draft row of the last token by 16 streaming warps and the draw by one more, by the sampler's
+// cut of a row and its choice of a sub-segment.  (Its sums in rows of up to 2048 vectors too, bit for bit; in longer ones the reference is
+// raised every four runs here and every eight in bv_draft_chain, so a uniform within rounding of a cell's edge may fall to the neighbour.)
+// Without supplied normalisers the verification still takes the one that the drafting step has formed, before it is rounded to
+// 32 bits: sixteen lanes of it are joined in fp32 from 2048 vectors on, as there.  Both models' rows of a step are
 // copied into shared memory at once; while the sampling warp draws, the streaming warps sweep the target row, so that when
 // the block is drafted all normalisers of its verification are known.  What is left of the verification is the recursion
 // of Eq. "def_as" or the tests of Algorithm 1 and, position after position from the top, the residual sums of the candidates

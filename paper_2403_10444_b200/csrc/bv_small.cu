@@ -15,8 +15,9 @@
 //   3. the CTA whose item is the last of a sequence ends it, a warp per candidate: S_i and h_i (Eq. "pacc_block") and, if the
 //      position passes, its token by inverse CDF over the segment sums and a rescan of one segment; then tau and the output.
 //      (A second barrier, the sums of all candidates, and only then the chosen one's token were two trips to L2 more.)
-// Bound: latency, a trip to L2 or memory for each of some eight dependent steps.  B = 1, gamma = 8, V = 152064 bf16 19.1 us a call
-// (19.8 with two barriers and pieces fixed on the host), B = 8, V = 32000 in 32 bits 19.8 (22.6), B = 24, gamma = 5, V = 50257 40 to 46 (43 to 47).
+// Bound: latency, a trip to L2 or memory for each of some eight dependent steps.  Us a call, in brackets with two barriers and pieces
+// fixed on the host, in turn on one box: B = 1, gamma = 8, V = 152064 bf16 18.9 (19.1; no more than two runs differ by, and 18.9 to 20.4 by box),
+// B = 8, V = 32000 in 32 bits 19.5 (22.6), B = 24, gamma = 5, V = 50257 45.2 (47.3; 42 to 46 by box).
 // Arithmetic, sampling convention and outputs are those of the flow kernel.
 #include <cooperative_groups.h>
 
@@ -236,7 +237,7 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __
             }
             turn ^= 1;
         }
-} else {
+    } else {
         for (int item = blockIdx.x; item < items; item += gridDim.x) {
             const int rid = item / nch, ch = item % nch;
             if (prm.lse_d != nullptr && rid % rpb > g) continue;      // (a draft row whose normaliser is supplied: nothing to learn)
@@ -296,7 +297,7 @@ __global__ void __launch_bounds__(kSmAllThreads, 1) verify_small_kernel(const __
             }
             __syncthreads();
         }
-}
+    }
     if (PROBS) __syncthreads();
     else alive = small_grid_barrier(sc.barrier, gridDim.x, prm.status, limit, prm.never_signal && blockIdx.x == 0);
 
@@ -712,9 +713,10 @@ static int small_best_split(long long units, long long rows, int nctas, int most
 SmallPlan small_plan(long long units, int B, int gamma, int nctas) {
     SmallPlan pl{};
     pl.nch = small_best_split(units, static_cast<long long>(B) * (2 * gamma + 1), nctas, kSmallMaxChunks);
-    // Loads ahead of the arithmetic: where a CTA has more than one item, or one of more than 16 vectors a thread (B = 20, gamma = 6, V = 65536,
-    // Algorithm 1, 30.7 us without, 28.6 with; B = 12, gamma = 8, V = 32000, all positions, 30.7 / 28.7; B = 24, gamma = 5, V = 50257 alike, 40 to 46).  A single item of fewer waits for memory once or twice either way, and the
-    // ring only costs: B = 1, gamma = 8, V = 152064 19.1 / 20.5, B = 3, gamma = 3, V = 256000 24.7 / 25.2, B = 8, V = 32000 in 32 bits 19.2 / 19.5.
+    // Loads ahead of the arithmetic: where a CTA has more than one item, or one of more than 16 vectors a thread (B = 20, gamma = 6,
+    // V = 65536, Algorithm 1, 30.7 us without, 28.6 with; B = 12, gamma = 8, V = 32000, all positions, 30.7 / 28.7; B = 24, gamma = 5,
+    // V = 50257 alike).  A single item of fewer waits for memory once or twice either way, and the ring only costs: B = 1, gamma = 8,
+    // V = 152064 7 % more, B = 3, gamma = 3, V = 256000 2 %, B = 8, V = 32000 in 32 bits 1.5 %.
     pl.ahead = static_cast<long long>(B) * (2 * gamma + 1) * pl.nch > nctas || units / pl.nch > 16 * kSmThreads;
     pl.np = 8;           // (the most: the kernel knows how many positions there are)
     return pl;
