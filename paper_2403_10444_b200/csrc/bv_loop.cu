@@ -495,13 +495,17 @@ bool loop_fits(int V, int dtype) { return 2 * static_cast<size_t>(V) * (dtype ==
 // Within the lines 2 of 4400 calls were 3 % or more slower than the loop that this kernel replaced (3 and 6 %).  Algorithm 1, which has
 // one candidate, gains up to half as much gamma again (V = 17000: gamma = 6 / 10, B = 4 0.83 / 1.01, B = 149 0.84 / 1.01), and up to
 // twice where every sequence has an SM (V = 36864, B = 148: gamma = 16 0.84).
+// Up to 8 sequences of rows of up to 1024 stay one launch at any gamma, as the calls that launches count most for; on the device that
+// is no gain from gamma = 24 on in 16 bits: V = 1024, B = 3, 3 iterations, noise 0.2 / 0.7 / 1.5: gamma = 16 0.98 / 0.97 / 0.94, 24 1.31 / 1.08 / 0.98,
+// 64 1.25 / 1.13 / 1.12; in 32 bits 16 0.90 / 0.83 / 0.80, 24 1.04 / 0.90 / 0.86, 64 1.13 / 0.99 / 0.98.
 bool loop_pays(int V, int dtype, int B, int gamma, bool token, int sms) {
     struct Line { int V; unsigned char gamma[7]; };
-    static constexpr Line kBf16[] = {{3072, {12, 16, 16, 8, 8, 4, 3}},      {6144, {12, 32, 32, 12, 8, 8, 5}}, {10240, {16, 32, 32, 16, 16, 16, 12}},
-                                     {16384, {16, 32, 32, 32, 32, 32, 32}}, {20000, {5, 6, 16, 8, 6, 4, 3}},   {26600, {5, 6, 16, 8, 8, 6, 5}},
-                                     {32768, {5, 16, 32, 5, 4, 2, 1}},      {34816, {2, 3, 6, 2, 2, 1, 1}},    {49152, {2, 3, 8, 3, 2, 1, 1}},
-                                     {53248, {2, 3, 5, 2, 1, 1, 0}},        {INT_MAX, {}}};
-    static constexpr Line kF32s[] = {{1536, {16, 32, 32, 24, 16, 12, 8}},   {3072, {32, 32, 32, 32, 16, 16, 12}}, {6144, {32, 32, 32, 32, 16, 16, 16}},
+    static constexpr Line kBf16[] = {{1024, {64, 16, 16, 8, 8, 4, 3}},      {3072, {12, 16, 16, 8, 8, 4, 3}},  {6144, {12, 32, 32, 12, 8, 8, 5}},
+                                     {10240, {16, 32, 32, 16, 16, 16, 12}}, {16384, {16, 32, 32, 32, 32, 32, 32}},
+                                     {20000, {5, 6, 16, 8, 6, 4, 3}},       {26600, {5, 6, 16, 8, 8, 6, 5}},   {32768, {5, 16, 32, 5, 4, 2, 1}},
+                                     {34816, {2, 3, 6, 2, 2, 1, 1}},        {49152, {2, 3, 8, 3, 2, 1, 1}},    {53248, {2, 3, 5, 2, 1, 1, 0}},
+                                     {INT_MAX, {}}};
+    static constexpr Line kF32s[] = {{1024, {64, 32, 32, 24, 16, 12, 8}},   {1536, {16, 32, 32, 24, 16, 12, 8}},   {3072, {32, 32, 32, 32, 16, 16, 12}}, {6144, {32, 32, 32, 32, 16, 16, 16}},
                                      {8192, {64, 64, 64, 64, 64, 64, 64}},  {13300, {8, 16, 32, 32, 32, 32, 32}}, {16384, {8, 16, 24, 10, 8, 6, 3}},
                                      {24576, {5, 6, 16, 5, 5, 3, 2}},       {26624, {2, 2, 8, 3, 3, 2, 1}},       {INT_MAX, {}}};
     const int load = B <= 8 ? 0 : B <= 24 ? 1 : B > 4 * sms ? 6 : 2 + (B - 1) / sms;

@@ -252,7 +252,7 @@ def test_host_buffers_are_shared_by_a_device_s_calls_and_by_no_others(host, devi
 # (V, dtype, B, gamma, Algorithm 1), on both sides of the lines between the decoding loop in one kernel and in two launches an iteration
 @pytest.mark.parametrize("call,one", [((16384, BF16, 128, 5, 0), 1), ((16384, BF16, 768, 32, 0), 1), ((16384, BF16, 8, 17, 0), 0), ((16384, BF16, 8, 24, 1), 1),
                                       ((16392, BF16, 8, 5, 0), 1), ((16392, BF16, 8, 6, 0), 0), ((16392, BF16, 8, 7, 1), 1), ((16392, BF16, 9, 6, 0), 1),
-                                      ((2048, BF16, 148, 16, 0), 1), ((2048, BF16, 149, 16, 0), 0), ((2048, BF16, 592, 3, 0), 1), ((2048, BF16, 768, 4, 0), 0),
+                                      ((2048, BF16, 148, 16, 0), 1), ((1024, BF16, 8, 64, 1), 1), ((1032, BF16, 8, 13, 0), 0), ((1024, F32, 8, 64, 0), 1), ((2048, BF16, 149, 16, 0), 0), ((2048, BF16, 592, 3, 0), 1), ((2048, BF16, 768, 4, 0), 0),
                                       ((32768, BF16, 148, 32, 0), 1), ((32768, BF16, 149, 6, 0), 0), ((32768, BF16, 445, 3, 0), 0), ((51200, BF16, 24, 4, 0), 0),
                                       ((51200, BF16, 25, 5, 0), 1), ((51200, BF16, 149, 3, 0), 0), ((51200, BF16, 593, 1, 0), 0), ((53256, BF16, 100, 1, 0), 0), ((8192, F32, 768, 64, 0), 1),
                                       ((24576, F32, 592, 3, 0), 1), ((24576, F32, 593, 3, 0), 0), ((26624, F32, 1, 2, 0), 1), ((26628, F32, 1, 1, 0), 0)])
