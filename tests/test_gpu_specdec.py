@@ -53,9 +53,33 @@ def oracle_loop(tt, dt, first, u_draft, u_verify, gamma, T, algo, supply_lse):
                                             ("token", oracle.TOKEN_VERIFY, False),
                                             ("block_lse", oracle.BLOCK_VERIFY, True),
                                             ("token_lse", oracle.TOKEN_VERIFY, True)])
-# the loop in one kernel, in the sampler's two forms; in two launches an iteration, by the small-batch kernel and by the phase kernel
-@pytest.mark.parametrize("V,kernel", [(2048, 0), (16384, 0), (2048, 4), (2048, 5)])
-def test_loop_matches_the_oracle_loop(algo, oalgo, lse, V, kernel, bv_options):
+def test_loop_matches_the_oracle_loop(algo, oalgo, lse):
+    V, B, gamma, N, T = 2048, 12, 4, 6, 0.9
+    tt, dt = wl.markov_models(V, "bf16", 5, 2.0, 0.8, 1.1, "cpu")
+    first = torch.arange(B, dtype=torch.int32)
+    ud, uv = wl.loop_uniforms(N, B, gamma, 6, "cpu")
+    want = oracle_loop(tt, dt, first, ud, uv, gamma, T, oalgo, lse)
+    res = specdec.run(tt.cuda(), dt.cuda(), first.cuda(), ud.cuda(), uv.cuda(), gamma, T, algo)
+    toks, lens = res["tokens"].cpu().numpy(), res["lengths"].cpu().numpy()
+    if lse:
+        # the supplied normalisers are each side's own float32 values, which may differ in the last
+        # bit; a sequence may then part ways at a near-tie, so only agreement of most is asked
+        same = sum(list(toks[b, : lens[b]]) == want[b] for b in range(B))
+        assert same >= B - 1
+    else:
+        for b in range(B):
+            assert list(toks[b, : lens[b]]) == want[b], b
+    assert (toks[np.arange(toks.shape[1])[None, :] >= lens[:, None]] == -1).all()
+    assert N <= lens.min() and lens.max() <= N * (gamma + 1)
+
+
+@pytest.mark.parametrize("algo,oalgo,lse", [("block", oracle.BLOCK_VERIFY, False),
+                                            ("token", oracle.TOKEN_VERIFY, False),
+                                            ("block_lse", oracle.BLOCK_VERIFY, True),
+                                            ("token_lse", oracle.TOKEN_VERIFY, True)])
+# the loop in one kernel, in the sampler's other form; in two launches an iteration, by the small-batch kernel and by the phase kernel
+@pytest.mark.parametrize("V,kernel", [(16384, 0), (2048, 4), (2048, 5)])
+def test_each_form_of_the_loop_matches_the_oracle_loop(algo, oalgo, lse, V, kernel, bv_options):
     bv_options("kernel", kernel)
     B, gamma, N, T = 12, 4, 6, 0.9
     tt, dt = (x.cpu() for x in wl.markov_models(V, "bf16", 5, 2.0, 0.8, 1.1, "cpu" if V == 2048 else "cuda"))
@@ -131,7 +155,7 @@ def test_block_verification_generates_more_per_iteration():
     assert be["block"] > be["token"] and be["block_lse"] > be["token"]
 
 
-@pytest.mark.parametrize("B", [48, 12])        # of the replayed steps: the phase kernel; the small-batch kernel (both cooperative launches)
+@pytest.mark.parametrize("B", [48, 12])        # the phase kernel; the small-batch kernel (both cooperative launches)
 @pytest.mark.parametrize("algo", ["block_lse", "block", "token"])
 def test_graph_replay_generates_the_same_tokens(algo, B):
     V, N, gamma = 4096, 9, 5
@@ -145,8 +169,30 @@ def test_graph_replay_generates_the_same_tokens(algo, B):
 
 
 @pytest.mark.parametrize("algo,oalgo", [("block", oracle.BLOCK_VERIFY), ("token", oracle.TOKEN_VERIFY)])
-@pytest.mark.parametrize("kernel", [0, 4, 5])
-def test_nucleus_masked_rows_through_the_loop(algo, oalgo, kernel, bv_options):
+def test_nucleus_masked_rows_through_the_loop(algo, oalgo):
+    # top-p masked rows (-inf outside each row's nucleus, the two models' nuclei differ): tokens the
+    # target model excludes are never emitted, and the loop still equals the oracle's
+    V, B, gamma, N, T = 1024, 10, 4, 5, 0.8
+    tt, dt = wl.markov_models(V, "f32", 51, 2.0, 1.0, 1.1, "cpu")
+    tt, dt = wl.top_p_mask(tt, 0.9, T), wl.top_p_mask(dt, 0.9, T)
+    assert 0.02 < torch.isfinite(tt).float().mean() < 0.9
+    first = torch.arange(B, dtype=torch.int32)
+    ud, uv = wl.loop_uniforms(N, B, gamma, 52, "cpu")
+    want = oracle_loop(tt, dt, first, ud, uv, gamma, T, oalgo, False)
+    res = specdec.run(tt.cuda(), dt.cuda(), first.cuda(), ud.cuda(), uv.cuda(), gamma, T, algo)
+    toks, lens = res["tokens"].cpu().numpy(), res["lengths"].cpu().numpy()
+    for b in range(B):
+        got = list(toks[b, : lens[b]])
+        assert got == want[b], b
+        prev = int(first[b])
+        for x in got:
+            assert torch.isfinite(tt[prev, x]), "a token outside the target model's nucleus was emitted"
+            prev = x
+
+
+@pytest.mark.parametrize("algo,oalgo", [("block", oracle.BLOCK_VERIFY), ("token", oracle.TOKEN_VERIFY)])
+@pytest.mark.parametrize("kernel", [4, 5])
+def test_nucleus_masked_rows_through_each_form_of_the_loop(algo, oalgo, kernel, bv_options):
     # top-p masked rows (-inf outside each row's nucleus, the two models' nuclei differ): tokens the
     # target model excludes are never emitted, and the loop still equals the oracle's
     bv_options("kernel", kernel)
@@ -210,8 +256,20 @@ def test_draft_chain_ends_a_sequence_at_a_token_it_cannot_follow():
 
 
 @pytest.mark.parametrize("algo", ["block_lse", "token"])
-@pytest.mark.parametrize("kernel", [0, 4, 5])
-def test_loop_with_and_without_the_chain_kernel_generates_the_same_tokens(algo, kernel, bv_options):
+def test_loop_with_and_without_the_chain_kernel_generates_the_same_tokens(algo):
+    V, B, N, gamma = 4096, 24, 7, 5
+    tt, dt = wl.markov_models(V, "bf16", 71, 2.0, 1.0, 1.1, "cuda")
+    ud, uv = wl.loop_uniforms(N, B, gamma, 72, "cuda")
+    first = torch.arange(B, dtype=torch.int32, device="cuda")
+    a = specdec.run(tt, dt, first, ud, uv, gamma, 0.9, algo, chain=True)
+    b = specdec.run(tt, dt, first, ud, uv, gamma, 0.9, algo, chain=False)
+    for k in ("tokens", "lengths", "tau", "drafted"):
+        assert torch.equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("algo", ["block_lse", "token"])
+@pytest.mark.parametrize("kernel", [4, 5])
+def test_two_launches_and_the_steps_generate_the_same_tokens(algo, kernel, bv_options):
     bv_options("kernel", kernel)
     V, B, N, gamma = 4096, 24, 7, 5
     tt, dt = wl.markov_models(V, "bf16", 71, 2.0, 1.0, 1.1, "cuda")
@@ -223,8 +281,25 @@ def test_loop_with_and_without_the_chain_kernel_generates_the_same_tokens(algo, 
         assert torch.equal(a[k], b[k]), k
 
 
-@pytest.mark.parametrize("V,B,kernel", [(512, 5, 0), (4096, 40, 0), (512, 5, 4), (4096, 40, 5)])      # one kernel; the small-batch kernel; the phase kernel
-def test_a_fault_in_the_loop_is_an_exception_and_harms_nothing(V, B, kernel, bv_options):
+@pytest.mark.parametrize("V,B", [(512, 5), (4096, 40)])      # (both in one kernel)
+def test_a_fault_in_the_loop_is_an_exception_and_harms_nothing(V, B):
+    tt, dt = wl.markov_models(V, "bf16", 3, 2.0, 0.7, 1.1, "cuda")
+    ud, uv = wl.loop_uniforms(3, B, 3, 4, "cuda")
+    first = torch.full((B,), 2, dtype=torch.int32, device="cuda")
+    good = specdec.run(tt, dt, first, ud, uv, 3)
+    bad = dt.clone()
+    bad[2, 7] = float("nan")                # the row every chain starts from: no token can be drawn
+    for algo in specdec.ALGOS:
+        with pytest.raises(RuntimeError):
+            specdec.run(tt, bad, first, ud, uv, 3, algo=algo)
+    with pytest.raises(RuntimeError):
+        specdec.run(tt, dt, torch.full_like(first, V), ud, uv, 3)
+    again = specdec.run(tt, dt, first, ud, uv, 3)
+    assert all(torch.equal(good[k], again[k]) for k in good)
+
+
+@pytest.mark.parametrize("V,B,kernel", [(512, 5, 4), (4096, 40, 5)])      # the small-batch kernel; the phase kernel
+def test_a_fault_in_each_form_of_the_loop_is_an_exception_and_harms_nothing(V, B, kernel, bv_options):
     bv_options("kernel", kernel)
     tt, dt = wl.markov_models(V, "bf16", 3, 2.0, 0.7, 1.1, "cuda")
     ud, uv = wl.loop_uniforms(3, B, 3, 4, "cuda")
